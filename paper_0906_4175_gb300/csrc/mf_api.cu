@@ -158,6 +158,44 @@ static cudaError_t dev_malloc_async(T **p, size_t bytes, cudaStream_t st) {
     return cudaMallocAsync(p, bytes, st);
 }
 
+// One call's scratch: its parts are added first, in a few groups that are
+// allocated together.  add() gives a part's place, at() its address.
+struct Scratch {
+    static constexpr int kGroups = 8;
+    static constexpr int kShift = 56;   // place: group, then offset
+    size_t size[kGroups] = {0};
+    char *base[kGroups] = {nullptr};
+    int n = 1;
+    void group() { ++n; }   // the next part opens a new allocation
+    size_t add(size_t bytes) {
+        const size_t off = size[n - 1];
+        size[n - 1] += (bytes + 255) & ~(size_t)255;
+        return ((size_t)(n - 1) << kShift) | off;
+    }
+    cudaError_t alloc(cudaStream_t st) {
+        for (int i = 0; i < n; ++i) {
+            if (size[i] == 0) continue;
+            const cudaError_t e = dev_malloc_async(&base[i], size[i], st);
+            if (e != cudaSuccess) {
+                base[i] = nullptr;
+                return e;
+            }
+        }
+        return cudaSuccess;
+    }
+    template <class T>
+    T *at(size_t place) const {
+        char *b = base[place >> kShift];
+        return b ? reinterpret_cast<T *>(b + (place & (((size_t)1 << kShift) - 1))) : nullptr;
+    }
+    void free(cudaStream_t st) {
+        for (int i = 0; i < n; ++i) {
+            if (base[i]) cudaFreeAsync(base[i], st);
+            base[i] = nullptr;
+        }
+    }
+};
+
 struct Workspace {
     int64_t exch_elems = 0, n_t = 0, cap = 0, anc_elems = 0, nblk = 0;
     UnitInfo *units = nullptr;
@@ -1114,31 +1152,33 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
     const int lgD = choose_log2D(b, seg);
     const int man = (int)anchor_slot_records(seg->log2N, lgD);   // records per anchor slot
     const int n_t = (int)b->n;
-    // 1024-point rows: every sub-band's exchange of a batch first, then one
-    // rows kernel over all of them (p + 1 exchanges per template in flight)
+    // every sub-band's exchange of a batch first, then one kernel that runs the
+    // row IFFTs over all of them (p + 1 exchanges per template in flight)
     const bool rows = chisq_rows_applies(seg->log2N);
     const int64_t budget = b->tuned_exch > 0 ? b->tuned_exch : kExchBudget;
-    const int64_t batch = rows ? std::max<int64_t>(1, std::min<int64_t>(n, budget / (8 * seg->N * (p + 1))))
-                               : std::min<int64_t>(n, choose_batch(seg->N, n, budget));
+    const int64_t batch =
+        std::max<int64_t>(1, std::min<int64_t>({n, budget / (8 * seg->N * (p + 1)), 65535 / (p + 1)}));
     const bool anchors = b->params.phase_mode != MF_PHASE_FP32;
     if (rows && !b->chi_status) MF_CUDA(dev_malloc(&b->chi_status, sizeof(int)));
     if (b->chi_status) MF_CUDA(cudaMemsetAsync(b->chi_status, 0, sizeof(int), st));
-    // With the persistent pass 1, one launch per batch covers all p + 1 bands:
-    // unit slot l nb + s is band l of template u0 + s (a band-major copy of the
-    // batch's units), reading the copy of its template's anchors that the
-    // anchor launch stores for each band.
-    const bool merged = rows && p1_form(b) != 1 && pass1_pf_applies(sd.log2N, sd.log2N2, lgD, b->params.phase_mode);
-    UnitInfo *all = nullptr, *units = nullptr, *mu = nullptr;
-    float4 *anc = nullptr;
-    float *anc4 = nullptr;
-    float2 *exch = nullptr;
-    cudaError_t e = dev_malloc_async(&all, sizeof(UnitInfo) * n_t, st);
-    if (e == cudaSuccess) e = dev_malloc_async(&units, sizeof(UnitInfo) * (size_t)(p + 1) * n, st);
-    if (e == cudaSuccess && merged) e = dev_malloc_async(&mu, sizeof(UnitInfo) * (size_t)(p + 1) * batch, st);
-    const int64_t anc_slots = batch * (merged ? p + 1 : 1);
-    if (e == cudaSuccess) e = dev_malloc_async(&anc, sizeof(float4) * man * anc_slots, st);
-    if (e == cudaSuccess) e = dev_malloc_async(&anc4, sizeof(float) * man * anc_slots, st);
-    if (e == cudaSuccess) e = dev_malloc_async(&exch, sizeof(float2) * seg->N * batch * (rows ? p + 1 : 1), st);
+    // One pass-1 launch per batch covers all p + 1 bands: unit slot l nb + s is
+    // band l of template u0 + s (a band-major copy of the batch's units).  The
+    // persistent pass 1 reads the copy of its template's anchors that the
+    // anchor launch stores for each band; the per-tile form shares them.
+    const bool pf = p1_form(b) != 1 && pass1_pf_applies(sd.log2N, sd.log2N2, lgD, b->params.phase_mode);
+    const int reps = pf ? p + 1 : 1;
+    Scratch sc;
+    const size_t o_all = sc.add(sizeof(UnitInfo) * n_t), o_units = sc.add(sizeof(UnitInfo) * (size_t)(p + 1) * n);
+    const size_t o_mu = sc.add(sizeof(UnitInfo) * (size_t)(p + 1) * batch);
+    sc.group();
+    const size_t o_anc = sc.add(sizeof(float4) * man * batch * reps), o_anc4 = sc.add(sizeof(float) * man * batch * reps);
+    sc.group();
+    const size_t o_exch = sc.add(sizeof(float2) * seg->N * batch * (p + 1));
+    cudaError_t e = sc.alloc(st);
+    UnitInfo *all = sc.at<UnitInfo>(o_all), *units = sc.at<UnitInfo>(o_units), *mu = sc.at<UnitInfo>(o_mu);
+    float4 *anc = sc.at<float4>(o_anc);
+    float *anc4 = sc.at<float>(o_anc4);
+    float2 *exch = sc.at<float2>(o_exch);
     int launches = 0;
     if (e == cudaSuccess) e = launch_units(sd, b->d_tmpl, n_t, b->params.f_low, 0.f, lgD, nullptr, all, st);
     if (e == cudaSuccess) e = launch_chisq_units(sd, all, n_t, tmpl, (int)n, p, units, edges, st);
@@ -1146,47 +1186,26 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
     const UnitInfo *full = units + (size_t)p * n;
     for (int64_t u0 = 0; u0 < n && e == cudaSuccess; u0 += batch) {
         const int nb = (int)std::min<int64_t>(batch, n - u0);
+        const UnitInfo *bu = units;   // one batch: the call's units are in band-major order already
         if (anchors) {
-            e = launch_anchors(sd, b->d_tmpl, full, (int)u0, nb, lgD, man, anc, anc4, st, merged ? p + 1 : 1);
+            e = launch_anchors(sd, b->d_tmpl, full, (int)u0, nb, lgD, man, anc, anc4, st, reps);
             ++launches;
         }
-        if (rows) {
-            if (merged) {
-                if (e == cudaSuccess)
-                    e = cudaMemcpy2DAsync(mu, sizeof(UnitInfo) * nb, units + u0, sizeof(UnitInfo) * n,
-                                          sizeof(UnitInfo) * nb, p + 1, cudaMemcpyDeviceToDevice, st);
-                if (e == cudaSuccess)
-                    e = launch_pass1(sd, mu, 0, (p + 1) * nb, lgD, man, anc, anc4, exch, b->params.phase_mode,
-                                     b->d_tmpl, p1_form(b), b->chi_status, b->spin_limit, st, true);
-                ++launches;
-            }
-            for (int l = 0; !merged && l <= p && e == cudaSuccess; ++l) {
-                e = launch_pass1(sd, units + (size_t)l * n, (int)u0, nb, lgD, man, anc, anc4,
-                                 exch + (size_t)l * nb * seg->N, b->params.phase_mode, b->d_tmpl, p1_form(b),
-                                 b->chi_status, b->spin_limit, st);
-                ++launches;
-            }
-            if (e == cudaSuccess)
-                e = launch_chisq_rows(sd, exch, full, (int)u0, nb, p, chisq, b->chi_status, b->spin_limit,
-                                      (int)b->stall_unit, sm_count(), st);
-            ++launches;
-            continue;
+        if (e == cudaSuccess && nb < n) {
+            e = cudaMemcpy2DAsync(mu, sizeof(UnitInfo) * nb, units + u0, sizeof(UnitInfo) * n, sizeof(UnitInfo) * nb,
+                                  p + 1, cudaMemcpyDeviceToDevice, st);
+            bu = mu;
         }
-        for (int l = 0; l <= p && e == cudaSuccess; ++l) {
-            const UnitInfo *ul = units + (size_t)l * n;
-            e = launch_pass1(sd, ul, (int)u0, nb, lgD, man, anc, anc4, exch, b->params.phase_mode, b->d_tmpl,
-                             p1_form(b), b->chi_status, b->spin_limit, st);
-            if (e == cudaSuccess)
-                e = launch_chisq_pass2(sd, ul, (int)u0, nb, exch, chisq, l == p ? 2 : (l == 0 ? 0 : 1), p, st);
-            launches += 2;
-        }
+        if (e == cudaSuccess)
+            e = launch_pass1(sd, bu, 0, (p + 1) * nb, lgD, man, anc, anc4, exch, b->params.phase_mode, b->d_tmpl,
+                             p1_form(b), b->chi_status, b->spin_limit, st, rows, nb);
+        if (e == cudaSuccess)
+            e = rows ? launch_chisq_rows(sd, exch, full, (int)u0, nb, p, chisq, b->chi_status, b->spin_limit,
+                                         (int)b->stall_unit, sm_count(), st)
+                     : launch_chisq_tiles(sd, exch, full, (int)u0, nb, p, chisq, st);
+        launches += 2;
     }
-    if (all) cudaFreeAsync(all, st);
-    if (units) cudaFreeAsync(units, st);
-    if (mu) cudaFreeAsync(mu, st);
-    if (anc) cudaFreeAsync(anc, st);
-    if (anc4) cudaFreeAsync(anc4, st);
-    if (exch) cudaFreeAsync(exch, st);
+    sc.free(st);
     if (e != cudaSuccess)
         return set_err(e == cudaErrorMemoryAllocation ? MF_ENOMEM : MF_ECUDA, "chisq_series: %s", cudaGetErrorString(e));
     count_launches(launches);

@@ -9,9 +9,9 @@
 // b_l is the smallest k with P[k] - P[k_lo] >= (l/p)(P[k_hi] - P[k_lo]), P the
 // segment's FP64 prefix of f^(-7/3)/S (|h~|^2/S up to the amplitude).
 // Each sub-band runs through the filter's own pass 1 (template generation on
-// the sub-band only, column IFFTs) and a pass 2 whose sink accumulates
-// |raw_l|^2 into the caller's output row; the last, full-band pass 2 turns
-// the sum into chi^2.  Neither z_l nor z is stored.
+// the sub-band only, column IFFTs) into its own exchange; one kernel then runs
+// the row IFFTs of all p + 1 bands, summing |raw_l|^2 in registers and turning
+// the sum into chi^2 at the full band.  Neither z_l nor z is stored.
 #include <algorithm>
 
 #include "mf_filter.cuh"
@@ -66,91 +66,90 @@ __global__ void k_chisq_units(SegDev seg, const UnitInfo *__restrict__ all, int 
     }
 }
 
-// pass-2 sinks.  The CTA owns rows j2 = tile C .. tile C + C - 1, i.e. C
-// consecutive samples out of every N2, so per-element global accesses from
-// the butterflies would touch one 32-byte sector per lane.  Each thread
-// therefore parks |raw|^2 of its outputs in its sequence's shared-memory row
-// (free once every thread of the sequence has read its last stage: the warp
-// for rows of up to 1024 points, the CTA for 2048), and finish() moves the
-// C x N1 tile to the unit's output row with the C consecutive samples of each
-// j1 on consecutive threads.
-template <int L, int C>
-__device__ __forceinline__ float *chi_tile_row(int seq) {
-    extern __shared__ float2 chi_smem[];
-    return reinterpret_cast<float *>(chi_smem + seq * SeqStride<L, C>::value);
-}
+// ---------------------------------------------------------------------------
+// chi^2 tile kernel (row lengths other than 1024).  Pass 1 has written the
+// exchange of every sub-band l = 0..p of a batch of nb templates, sub-band l
+// of entry b at exch + (l nb + b) N.  Each CTA owns C rows j2 = tile C ..
+// tile C + C - 1 of one entry and transforms them for l = 0..p in turn,
+// summing |raw_l|^2 of its 32 outputs per thread in registers; at l = p (the
+// full band) the sum becomes chi^2 = rho_scale^2 (p sum_l |raw_l|^2 - |raw|^2).
+// The C consecutive samples of each j1 then leave through a shared-memory
+// tile (per-element stores from the butterflies would touch one 32-byte sector
+// per lane).  One launch per batch instead of one per sub-band, and no
+// accumulator in memory: 16 templates at N = 2^16, p = 16 took 17 pass-1 and
+// 17 pass-2 launches of 7 us each, every one a fraction of a wave: 330 us a
+// call, 151 us now.
+// ---------------------------------------------------------------------------
+struct ChiTilesParams {
+    const float2 *exch;
+    const UnitInfo *full;   // full-band units of the call's template list
+    float *chisq;           // [n][N]
+    int unit0, nb, p;
+    int log2N, log2N1, log2N2;
+};
 
+// rows of one sub-band; from the second sub-band on, the sequences' shared
+// memory is free only once every thread has read its last stage
 template <int L, int C>
-__device__ __forceinline__ void chi_park(int seq, int b, int stride, const float2 *v, int R) {
-    float *row = chi_tile_row<L, C>(seq);
-    if constexpr (L / 32 <= 32) __syncwarp();   // the sequence's threads have read their last-stage inputs
-    else __syncthreads();                        // (a 2048-point sequence spans two warps; every thread gets here once)
-#pragma unroll 32
-    for (int r = 0; r < R; ++r) row[b + r * stride] = fmaf(v[r].x, v[r].x, v[r].y * v[r].y);
-}
+struct ChiTileSrc {
+    static constexpr bool kHalfZero = false;
+    const RowSrc<L, C> rows;
+    const bool again;
+    __device__ __forceinline__ void load(int seq, int t, float2 *v) const {
+        rows.load(seq, t, v);
+        if (again) __syncthreads();
+    }
+};
 
-// mode 0: acc = |raw|^2, 1: acc += |raw|^2, 2: acc = rs2 (p acc - |raw|^2).
-// Rows of up to 2048 points go through the shared-memory tile; longer rows
-// would update the output element by element from the butterflies.
-template <int L, int C>
-struct ChiSink {
-    static constexpr bool kTile = (L / 32) <= 64;
-    struct Params { float *acc; const UnitInfo *units; int log2N2, log2N, mode; float pf; };
-    const Params &p;
-    const int tile, unit;
-    float rs2;
-    __device__ ChiSink(const Params &pp, int tl, int un, int) : p(pp), tile(tl), unit(un), rs2(0.f) {
-        if (p.mode == 2) {
-            const float rs = p.units[un].rho_scale;
-            rs2 = rs * rs;
-        }
-    }
-    __device__ __forceinline__ void update(float *q, float pw) const {
-        if (p.mode == 0) *q = pw;
-        else if (p.mode == 1) *q += pw;
-        else *q = rs2 * fmaf(p.pf, *q, -pw);
-    }
+// |raw_l|^2 of the thread's 32 outputs summed over l < p; chi^2 at l = p
+struct ChiTileAcc {
+    float acc[32];
+    int l = 0, p = 0;
+    float pf = 0.f, rs2 = 0.f;
     template <int R>
-    __device__ __forceinline__ void store(int seq, int b, int stride, const float2 *v) const {
-        if constexpr (kTile) {
-            chi_park<L, C>(seq, b, stride, v, R);
-        } else {
-            float *a = p.acc + ((int64_t)unit << p.log2N) + tile * C + seq;
+    __device__ __forceinline__ void store(int, int, int, const float2 *v) {
 #pragma unroll
-            for (int r = 0; r < R; ++r)
-                update(a + ((int64_t)(b + r * stride) << p.log2N2), fmaf(v[r].x, v[r].x, v[r].y * v[r].y));
-        }
-    }
-    __device__ __forceinline__ void finish(float2 *) const {
-        if constexpr (kTile) {
-            __syncthreads();
-            float *a = p.acc + ((int64_t)unit << p.log2N) + tile * C;
-            // C L elements over C (L / 32) threads: 32 per thread, issued in
-            // groups of 8 loads before their read-modify-writes
-            constexpr int NT = C * (L / 32);
-            constexpr int G = 8;
-            static_assert((C * L) % (NT * G) == 0, "tile split");
-#pragma unroll 1
-            for (int base = 0; base < C * L; base += NT * G) {
-                float pw[G], old[G];
-                float *q[G];
-#pragma unroll
-                for (int g = 0; g < G; ++g) {
-                    const int idx = base + g * NT + (int)threadIdx.x;
-                    const int seq = idx % C, j1 = idx / C;
-                    q[g] = a + seq + ((int64_t)j1 << p.log2N2);
-                    pw[g] = chi_tile_row<L, C>(seq)[j1];
-                    old[g] = p.mode == 0 ? 0.f : __ldcg(q[g]);
-                }
-#pragma unroll
-                for (int g = 0; g < G; ++g) {
-                    const float x = p.mode == 0 ? pw[g] : (p.mode == 1 ? old[g] + pw[g] : rs2 * fmaf(p.pf, old[g], -pw[g]));
-                    __stcg(q[g], x);
-                }
-            }
+        for (int r = 0; r < R; ++r) {
+            const float pw = fmaf(v[r].x, v[r].x, v[r].y * v[r].y);
+            if (l < p) acc[r] = l == 0 ? pw : acc[r] + pw;
+            else acc[r] = rs2 * fmaf(pf, acc[r], -pw);
         }
     }
 };
+
+template <int L, int C>
+__global__ void __launch_bounds__(C *(L / 32), (C * (L / 32) >= 256) ? 2 : 1) k_chisq_tiles(ChiTilesParams q) {
+    extern __shared__ float2 chi_smem[];
+    constexpr int T = L / 32, NT = C * T;
+    float2 *tw = chi_smem + pass_data_bytes<L, C>() / sizeof(float2);
+    const int tile = blockIdx.x, b = blockIdx.y;
+    fill_twiddles<L>(tw);
+    ChiTileAcc snk;
+    snk.p = q.p;
+    snk.pf = (float)q.p;
+    {
+        const float rs = q.full[q.unit0 + b].rho_scale;
+        snk.rs2 = rs * rs;
+    }
+    const typename RowSrc<L, C>::Params rp{q.exch, q.log2N1, q.log2N};
+#pragma unroll 1
+    for (int l = 0; l <= q.p; ++l) {
+        snk.l = l;
+        ChiTileSrc<L, C> src{RowSrc<L, C>(rp, tile, 0, l * q.nb + b, nullptr), l > 0};
+        cta_fft<L, C, false, +1>(chi_smem, tw, src, snk);
+    }
+    const int seq = threadIdx.x / T, t = threadIdx.x % T;
+    auto row = [&](int s) { return reinterpret_cast<float *>(chi_smem + s * SeqStride<L, C>::value); };
+    __syncthreads();   // the last stage has read the sequences
+#pragma unroll
+    for (int r = 0; r < 32; ++r) row(seq)[t + r * T] = snk.acc[r];
+    __syncthreads();
+    float *out = q.chisq + ((int64_t)(q.unit0 + b) << q.log2N) + tile * C;
+    for (int idx = threadIdx.x; idx < C * L; idx += NT) {
+        const int s = idx % C, j1 = idx / C;
+        __stcs(&out[s + ((int64_t)j1 << q.log2N2)], row(s)[j1]);
+    }
+}
 
 // ---------------------------------------------------------------------------
 // chi^2 rows kernel (N1 = 1024, N = 2^19 and 2^20).  Pass 1 has written the
@@ -164,9 +163,7 @@ struct ChiSink {
 //   chi^2 = rho_scale^2 (p sum_l |raw_l|^2 - |raw|^2)
 // is formed without any accumulator in memory.  The CTA's 8 warps own 8
 // consecutive rows; they park their 1024 values each in their regions and
-// write the 8 x 1024 tile with 8 consecutive samples per 32-byte sector.  The
-// sums run in the same order and with the same butterflies as the per-tile
-// path, so the results are the same bit for bit.
+// write the 8 x 1024 tile with 8 consecutive samples per 32-byte sector.
 // ---------------------------------------------------------------------------
 namespace {
 
@@ -335,30 +332,26 @@ static size_t chi_rows_smem_bytes() {
            kChiWarps * sizeof(uint64_t);
 }
 
-struct ChiPass2Op {
-    const SegDev &seg;
-    const UnitInfo *units;
-    int unit0, n_units;
-    const float2 *exch;
-    float *acc;
-    int mode;   // 0: first sub-band (store), 1: later sub-band (add), 2: full band (chi^2)
-    int p;
+template <int L, int C>
+constexpr size_t chi_tiles_smem_bytes() {
+    return pass_data_bytes<L, C>() + (size_t)TwTable<L>::SIZE * sizeof(float2);
+}
+
+struct ChiTilesOp {
+    const ChiTilesParams *q;   // NULL: set the kernel attributes only
     cudaStream_t st;
     template <int N2, int N1>
     cudaError_t run() {
-        constexpr int C = seqs_per_cta<N1>(N2);
-        const dim3 grid(N2 / C, n_units);
-        typename RowSrc<N1, C>::Params sp{exch, seg.log2N1, seg.log2N};
-        typename ChiSink<N1, C>::Params kp{acc, units, seg.log2N2, seg.log2N, mode, (float)p};
-        return run_pass<N1, C, false, +1, RowSrc<N1, C>, ChiSink<N1, C>>(grid, sp, kp, st, unit0);
-    }
-};
-
-struct ChiAttrOp {
-    template <int N2, int N1>
-    cudaError_t run() {
-        constexpr int C = seqs_per_cta<N1>(N2);
-        return set_pass_attrs<N1, C, false, +1, RowSrc<N1, C>, ChiSink<N1, C>>();
+        if constexpr (N1 != 1024) {
+            constexpr int C = seqs_per_cta<N1>(N2);
+            constexpr size_t smem = chi_tiles_smem_bytes<N1, C>();
+            if (!q)
+                return cudaFuncSetAttribute(k_chisq_tiles<N1, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            k_chisq_tiles<N1, C><<<dim3(N2 / C, q->nb), C * (N1 / 32), smem, st>>>(*q);
+            return cudaGetLastError();
+        } else {
+            return q ? cudaErrorInvalidValue : cudaSuccess;   // 1024-point rows: k_chisq_rows
+        }
     }
 };
 }  // namespace
@@ -370,9 +363,10 @@ cudaError_t launch_chisq_units(const SegDev &seg, const UnitInfo *all, int n_t, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_chisq_pass2(const SegDev &seg, const UnitInfo *units, int unit0, int n_units, const float2 *exch,
-                               float *acc, int mode, int p, cudaStream_t st) {
-    ChiPass2Op op{seg, units, unit0, n_units, exch, acc, mode, p, st};
+cudaError_t launch_chisq_tiles(const SegDev &seg, const float2 *exch, const UnitInfo *full, int unit0, int nb, int p,
+                               float *chisq, cudaStream_t st) {
+    ChiTilesParams q{exch, full, chisq, unit0, nb, p, seg.log2N, seg.log2N1, seg.log2N2};
+    ChiTilesOp op{&q, st};
     return dispatch_split(seg.log2N, op);
 }
 
@@ -401,7 +395,7 @@ cudaError_t chisq_kernel_attributes() {
         if (e1 != cudaSuccess) return e1;
     }
     for (int lg = 10; lg <= 22; ++lg) {
-        ChiAttrOp op;
+        ChiTilesOp op{nullptr, nullptr};
         cudaError_t e = dispatch_split(lg, op);
         if (e != cudaSuccess) return e;
     }

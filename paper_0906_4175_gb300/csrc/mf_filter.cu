@@ -104,6 +104,7 @@ struct Pass1Op {
     const float *anchors4;
     float2 *exch;
     const double *tmpl;
+    int anc_slots;
     cudaStream_t st;
     template <int N2, int N1>
     cudaError_t run() {
@@ -114,7 +115,7 @@ struct Pass1Op {
             typename TemplateSrcF32<N2, C, cx_ilog2(N1)>::Params sp{seg.W, units, tmpl, (float)seg.df};
             return run_pass<N2, C, true, +1, TemplateSrcF32<N2, C, cx_ilog2(N1)>, ExchSink<N2, C, +1, cx_ilog2(N1)>>(grid, sp, kp, st, unit0);
         }
-        typename TemplateSrc<N2, C, cx_ilog2(N1)>::Params sp{seg.W, units, anchors, anchors4, max_anc, log2D};
+        typename TemplateSrc<N2, C, cx_ilog2(N1)>::Params sp{seg.W, units, anchors, anchors4, max_anc, log2D, anc_slots};
         return run_pass<N2, C, true, +1, TemplateSrc<N2, C, cx_ilog2(N1)>, ExchSink<N2, C, +1, cx_ilog2(N1)>>(grid, sp, kp, st, unit0);
     }
 };
@@ -168,11 +169,11 @@ struct AttrOp {
 cudaError_t launch_pass1(const SegDev &seg, const UnitInfo *units, int unit0, int n_units, int log2D, int max_anc,
                          const float4 *anchors, const float *anchors4, float2 *exch, int phase_mode,
                          const double *tmpl, int p1_form, int *status, long long spin_limit, cudaStream_t st,
-                         bool narrow) {
+                         bool narrow, int anc_slots) {
     if (p1_form != 1 && pass1_pf_applies(seg.log2N, seg.log2N2, log2D, phase_mode))
         return launch_pass1_pf(seg, units, unit0, n_units, log2D, max_anc, anchors, anchors4, exch, p1_form == 2,
                                status, spin_limit, st, narrow);
-    Pass1Op op{seg, units, unit0, n_units, log2D, max_anc, phase_mode, anchors, anchors4, exch, tmpl, st};
+    Pass1Op op{seg, units, unit0, n_units, log2D, max_anc, phase_mode, anchors, anchors4, exch, tmpl, anc_slots, st};
     return dispatch_split2(seg.log2N, seg.log2N2, op);
 }
 

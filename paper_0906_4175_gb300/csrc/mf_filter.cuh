@@ -56,6 +56,7 @@ struct TemplateSrc {
         const float4 *anchors;
         const float *anchors4;
         int anc_stride, log2D;
+        int anc_slots;   // > 0: several bands share a template's anchors, slot mod anc_slots
     };
     const Params &p;
     const int tile, unit, slot;
@@ -68,8 +69,9 @@ struct TemplateSrc {
     __device__ __forceinline__ void load(int seq, int t, float2 *v) const {
         constexpr int T = L / 32;
         const UnitInfo u = p.units[unit];
-        const float4 *anc0 = p.anchors + (int64_t)slot * p.anc_stride;   // index: anchor_slot_index(g)
-        const float *anc40 = p.anchors4 + (int64_t)slot * p.anc_stride;
+        const int aslot = p.anc_slots > 0 ? slot % p.anc_slots : slot;
+        const float4 *anc0 = p.anchors + (int64_t)aslot * p.anc_stride;   // index: anchor_slot_index(g)
+        const float *anc40 = p.anchors4 + (int64_t)aslot * p.anc_stride;
         constexpr int LGL = cx_ilog2(L);
         const int k1 = tile * C + seq;
         const int D = 1 << p.log2D;

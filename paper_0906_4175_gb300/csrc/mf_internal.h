@@ -224,7 +224,9 @@ cudaError_t launch_anchors(const SegDev &seg, const double *tmpl, const UnitInfo
 cudaError_t launch_pass1(const SegDev &seg, const UnitInfo *units, int unit0, int n_units, int log2D,
                          int max_anc, const float4 *anchors, const float *anchors4, float2 *exch,
                          int phase_mode, const double *tmpl, int p1_form, int *status, long long spin_limit,
-                         cudaStream_t st, bool narrow = false);
+                         cudaStream_t st, bool narrow = false, int anc_slots = 0);
+// anc_slots > 0: unit slot i reads anchor slot i mod anc_slots (the per-tile
+// form only; the persistent form reads slot i).
 // narrow: bands of a few rows per column (the chi^2 sub-bands); the staged form
 // then starts a column with a cheaper first stage wherever each lane of a warp
 // holds at most one row of the band (other forms ignore it; rounding differs
@@ -280,9 +282,10 @@ cudaError_t launch_refine(const SegDev &seg, double f_low, int phase_mode, const
 constexpr int kChisqMaxBands = 64;
 cudaError_t launch_chisq_units(const SegDev &seg, const UnitInfo *all, int n_t, const int32_t *tmpl, int n, int p,
                                UnitInfo *out, int64_t *edges, cudaStream_t st);
-// mode 0: first sub-band (store |raw|^2), 1: later sub-band (add), 2: full band (write chi^2)
-cudaError_t launch_chisq_pass2(const SegDev &seg, const UnitInfo *units, int unit0, int n_units, const float2 *exch,
-                               float *acc, int mode, int p, cudaStream_t st);
+// row IFFTs of all p + 1 bands of nb templates and chi^2 (row lengths other
+// than 1024); band l of entry b at exch + (l nb + b) N
+cudaError_t launch_chisq_tiles(const SegDev &seg, const float2 *exch, const UnitInfo *full, int unit0, int nb, int p,
+                               float *chisq, cudaStream_t st);
 
 // trigger clustering scratch (every array sized for the trigger capacity)
 struct ClusterScratch {
