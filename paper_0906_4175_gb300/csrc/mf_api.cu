@@ -594,7 +594,7 @@ extern "C" int mf_segment_upload(const float *s, int64_t N, double fs, const dou
         psd_dev = g->psd;
     }
     const float *s_use = s_on_device ? s : s_dev;
-    if (e == cudaSuccess) e = launch_forward_fft64(s_use, N, exch, X, st);   // exch: 8 N bytes = N/2 complex128
+    if (e == cudaSuccess) e = launch_forward_fft64(s_use, N, exch, nullptr, X, st);   // exch: 8 N bytes = N/2 complex128
     if (e == cudaSuccess) e = launch_psd_weights(X, psd_dev, psd_f0, psd_S0, N, fs, q, st);
     if (e == cudaSuccess) e = launch_prefix_f64(q, half, g->P, btmp, st);
     if (e == cudaSuccess) e = launch_weight_data(X, psd_dev, psd_f0, psd_S0, N, fs, g->P, g->consts, g->W, g->fac, st);
@@ -642,13 +642,12 @@ extern "C" int mf_segment_refresh(mf_segment g, const float *s, int s_on_device,
     // the PSD and with it P, sigma's normalisation and the factors a_k are unchanged
     if (g->cond == MF_COND_FP32) {
         MF_CUDA(launch_forward_fft(s_use, N, g->r_exch, g->r_X, st));
-        count_launches(2);
+        MF_CUDA(launch_apply_weights(g->r_X, g->fac, N, g->W, st));
+        count_launches(3);
     } else {
-        MF_CUDA(launch_forward_fft64(s_use, N, g->r_exch, g->r_X, st));
+        MF_CUDA(launch_forward_fft64(s_use, N, g->r_exch, g->fac, g->W, st));
         count_launches(3);
     }
-    MF_CUDA(launch_apply_weights(g->r_X, g->fac, N, g->W, st));
-    count_launches(1);
     if (!s_on_device) MF_CUDA(cudaStreamSynchronize(st));   // host s consumed before return
     return MF_OK;
 }
