@@ -28,6 +28,10 @@ cudaError_t launch_chisq_rows(const SegDev &seg, const float2 *exch, const UnitI
 // batched FFT of whole sequences per CTA (mf_prep.cu), N = 1024 and 2048
 bool fft_c2c_single_pass(int64_t N);
 cudaError_t launch_fft_c2c_single(const float2 *x, float2 *y, int64_t N, int64_t batch, int sign, cudaStream_t st);
+// sequences of 4096 .. 16384 points in one CTA's shared memory (mf_seq.cu)
+bool fft_seq_applies(int64_t N);
+cudaError_t launch_fft_seq(const float2 *x, float2 *y, int64_t N, int64_t batch, int sign, cudaStream_t st);
+cudaError_t seq_kernel_attributes();
 cudaError_t synth_kernel_attributes();
 cudaError_t refine_kernel_attributes();
 cudaError_t chisq_kernel_attributes();
@@ -84,6 +88,7 @@ static int ensure_device_init() {
     MF_CUDA(filter_kernel_attributes());
     MF_CUDA(prep_kernel_attributes());
     MF_CUDA(persist_kernel_attributes());
+    MF_CUDA(seq_kernel_attributes());
     MF_CUDA(synth_kernel_attributes());
     MF_CUDA(refine_kernel_attributes());
     MF_CUDA(chisq_kernel_attributes());
@@ -1165,6 +1170,11 @@ extern "C" int mf_fft_c2c(const void *x, void *y, int64_t N, int64_t batch, int 
         return MF_OK;
     }
     if (stream_capturing(st)) return set_err(MF_EINVAL, "mf_fft_c2c allocates its exchange and cannot be captured");
+    if (fft_seq_applies(N)) {
+        MF_CUDA(launch_fft_seq((const float2 *)x, (float2 *)y, N, batch, sign, st));
+        count_launches(1);
+        return MF_OK;
+    }
     const int64_t chunk = std::min<int64_t>({batch, std::max<int64_t>(1, kScratchBudget / (8 * N)), 65535});
     Scratch sc;
     sc.add(sizeof(float2) * N * chunk);
