@@ -294,7 +294,7 @@ struct mf_bank_s {
     // order) puts the widest bands first for every segment.  pos is the inverse.
     std::vector<int> order, pos;
     int *d_order = nullptr;
-    double B1 = 0.0, B5 = 0.0, fisco_min = 0.0;
+    double B1 = 0.0, B3 = 0.0, B5 = 0.0, B7 = 0.0, fisco_min = 0.0;   // phase-derivative bounds at f_low
     int device = 0;
     Workspace ws;
     bool prof_on = false;
@@ -427,7 +427,7 @@ static int bank_create_range(const double *m1, const double *m2, int64_t n, cons
     int r0 = ensure_device_init();
     if (r0) return r0;
     std::vector<double> rec((size_t)count * kTmplStride);
-    double B1 = 0.0, B5 = 0.0, fmin = INFINITY;
+    double B1 = 0.0, B3 = 0.0, B5 = 0.0, B7 = 0.0, fmin = INFINITY;
     for (int64_t i = 0; i < n; ++i) {
         if (!(m1[i] > 0.0) || !(m2[i] > 0.0) || !isfinite(m1[i]) || !isfinite(m2[i]))
             return set_err(MF_EINVAL, "template %lld: masses must be finite and > 0", (long long)i);
@@ -437,6 +437,10 @@ static int bank_create_range(const double *m1, const double *m2, int64_t n, cons
         template_constants(m1[i], m2[i], r);
         B1 = std::max(B1, psi_deriv_bound(r, p.f_low, 1));
         B5 = std::max(B5, psi_deriv_bound(r, p.f_low, 5));
+        if (p.phase_mode == MF_PHASE_FP64) {
+            B3 = std::max(B3, psi_deriv_bound(r, p.f_low, 3));
+            B7 = std::max(B7, psi_deriv_bound(r, p.f_low, 7));
+        }
         if (mine) fmin = std::min(fmin, r[TF_FISCO]);
     }
     n = count;
@@ -445,7 +449,9 @@ static int bank_create_range(const double *m1, const double *m2, int64_t n, cons
     b->n = n;
     b->params = p;
     b->B1 = B1;
+    b->B3 = B3;
     b->B5 = B5;
+    b->B7 = B7;
     b->fisco_min = fmin;
     b->fisco.resize((size_t)n);
     for (int64_t i = 0; i < n; ++i) b->fisco[(size_t)i] = rec[(size_t)i * kTmplStride + TF_FISCO];
@@ -701,9 +707,9 @@ static SegDev seg_dev(const mf_segment_s *g, int log2N2 = -1) {
 // (<= 256) for which the quartic-Taylor remainder max|d^5 psi/dk^5| (D/2)^5/120
 // stays below 5e-7 turns and |d psi/dk| D/2 below 16 turns (FP32 magnitude of
 // the Taylor sum), both bounded at f_low over the whole bank (k-derivatives are
-// f-derivatives times df^n).
+// f-derivatives times df^n).  MF_PHASE_FP64 has its own rule (anchor_log2D64).
 static int choose_log2D(const mf_bank_s *b, const mf_segment_s *g) {
-    if (b->params.phase_mode == MF_PHASE_FP64) return 0;
+    if (b->params.phase_mode == MF_PHASE_FP64) return anchor_log2D64(b->B3, b->B7, g->fs / (double)g->N);
     return anchor_log2D(b->B1, b->B5, g->fs / (double)g->N);
 }
 
@@ -716,6 +722,9 @@ static int choose_log2D(const mf_bank_s *b, const mf_segment_s *g) {
 // allocates its exchange per call, keeps 1 GiB.
 constexpr int64_t kExchBudget = (int64_t)4 << 30;
 constexpr int64_t kScratchBudget = (int64_t)1 << 30;
+
+// 16-byte planes of an anchor record (and one float, MF_PHASE_ANCHOR)
+static int anchor_planes(const mf_bank_s *b) { return b->params.phase_mode == MF_PHASE_FP64 ? 3 : 1; }
 
 static int64_t choose_batch(int64_t N, int64_t n_t, int64_t tuned_exch) {
     int64_t b = (tuned_exch > 0 ? tuned_exch : kExchBudget) / (8 * N);
@@ -804,7 +813,7 @@ static int filter_log2n2(const mf_bank_s *b, const mf_segment_s *g) {
 }
 
 static bool use_persistent(const mf_bank_s *b, const mf_segment_s *g) {
-    if (g->log2N < 13 || b->params.phase_mode == MF_PHASE_FP32 || b->params.fft_mode != MF_FFT_FP32) return false;
+    if (g->log2N < 13 || b->params.phase_mode != MF_PHASE_ANCHOR || b->params.fft_mode != MF_FFT_FP32) return false;
     if (const char *e = getenv("MFGB_SCHED")) {
         if (strcmp(e, "batch") == 0 || strcmp(e, "fused") == 0) return false;
         if (strcmp(e, "persistent") == 0) return true;
@@ -923,7 +932,7 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
         seg_batch[(size_t)s] = bt;
         const int lgD = choose_log2D(b, segs[s]);
         exch_elems = std::max(exch_elems, bt * segs[s]->N);
-        anc_elems = std::max(anc_elems, 2 * bt * (((segs[s]->N / 2) >> lgD) + 2));   // two batches in flight
+        anc_elems = std::max(anc_elems, 2 * bt * (((segs[s]->N / 2) >> lgD) + 2) * anchor_planes(b));   // two batches in flight
         if (use_fused(b, segs[s])) {   // the ring, and the anchors of every unit
             exch_elems = std::max(exch_elems, (int64_t)fused_slots(segs[s]->N) * segs[s]->N);
             anc_elems = std::max(anc_elems, b->n * anchor_slot_records(segs[s]->log2N, lgD));
@@ -986,7 +995,8 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
                     by_anc += anc_bytes[(size_t)t];
                 }
             pi = prof_begin(b, MF_STAGE_ANCHORS, by_anc, st);
-            MF_CUDA(launch_anchors(sd, b->d_tmpl, w.units, 0, n_t, lgD, man, w.anchors, w.anchors4, st));
+            MF_CUDA(launch_anchors(sd, b->d_tmpl, w.units, 0, n_t, lgD, man, w.anchors, w.anchors4,
+                                   b->params.phase_mode, st));
             prof_end(b, pi, st);
             MF_CUDA(cudaMemsetAsync(w.ctl, 0, sizeof(unsigned) * (4 + 2 * (size_t)n_t), st));
             double split = b->split > 0.0 ? b->split : kSplit;
@@ -1086,7 +1096,7 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
             MF_CUDA(cudaEventCreateWithFlags(&b->ev_p1, cudaEventDisableTiming));
             MF_CUDA(cudaEventCreateWithFlags(&b->ev_anc, cudaEventDisableTiming));
         }
-        const int64_t slot_elems = batch * man;
+        const int64_t slot_elems = batch * man * anchor_planes(b);
         for (int u0 = 0, bi = 0; u0 < n_t; u0 += (int)batch, ++bi) {
             const int nb = (int)std::min<int64_t>(batch, n_t - u0);
             const int64_t aoff = overlap ? (bi & 1) * slot_elems : 0;
@@ -1101,7 +1111,7 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
             if (anchors && (!overlap || bi == 0)) {
                 pi = prof_begin(b, MF_STAGE_ANCHORS, by_anc, st);
                 MF_CUDA(launch_anchors(sd, b->d_tmpl, w.units, u0, nb, lgD, man, w.anchors + aoff, w.anchors4 + aoff,
-                                       st));
+                                       b->params.phase_mode, st));
                 prof_end(b, pi, st);
                 count_launches(1);
             } else if (overlap) {
@@ -1118,7 +1128,7 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
                 MF_CUDA(cudaEventRecord(b->ev_p1, st));
                 MF_CUDA(cudaStreamWaitEvent(b->side, b->ev_p1, 0));
                 MF_CUDA(launch_anchors(sd, b->d_tmpl, w.units, u1, nb1, lgD, man, w.anchors + aoff1,
-                                       w.anchors4 + aoff1, b->side));
+                                       w.anchors4 + aoff1, b->params.phase_mode, b->side));
                 MF_CUDA(cudaEventRecord(b->ev_anc, b->side));
                 count_launches(1);
             }
@@ -1233,7 +1243,7 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
     const size_t o_all = sc.add(sizeof(UnitInfo) * n_t), o_units = sc.add(sizeof(UnitInfo) * (size_t)(p + 1) * n);
     const size_t o_mu = sc.add(sizeof(UnitInfo) * (size_t)(p + 1) * batch);
     sc.group();
-    const size_t o_anc = sc.add(sizeof(float4) * man * batch * reps), o_anc4 = sc.add(sizeof(float) * man * batch * reps);
+    const size_t o_anc = sc.add(sizeof(float4) * man * batch * reps * anchor_planes(b)), o_anc4 = sc.add(sizeof(float) * man * batch * reps);
     sc.group();
     const size_t o_exch = sc.add(sizeof(float2) * seg->N * batch * (p + 1));
     cudaError_t e = sc.alloc(st);
@@ -1250,7 +1260,7 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
         const int nb = (int)std::min<int64_t>(batch, n - u0);
         const UnitInfo *bu = units;   // one batch: the call's units are in band-major order already
         if (anchors) {
-            e = launch_anchors(sd, b->d_tmpl, full, (int)u0, nb, lgD, man, anc, anc4, st, reps);
+            e = launch_anchors(sd, b->d_tmpl, full, (int)u0, nb, lgD, man, anc, anc4, b->params.phase_mode, st, reps);
             ++launches;
         }
         if (e == cudaSuccess && nb < n) {

@@ -4,6 +4,7 @@
 //              prefix table, rho and z scale factors, anchor range;
 //   k_anchors  the 2PN phase Psi/(2 pi) in FP64 at anchor bins, reduced mod 1,
 //              plus its first four k-derivatives (FP32 Taylor coefficients);
+//              k_anchors64 the records of MF_PHASE_FP64;
 //   pass 1     template generation h~_k = e^{-i Psi_k} in registers (FP32
 //              quartic Taylor from the nearest anchor, __sincosf of the reduced
 //              phase), weighting by W_k = f^(-7/6) conj(s~_k)/S_k, column IFFTs,
@@ -74,6 +75,26 @@ __global__ void k_anchors(SegDev seg, const double *__restrict__ tmpl, const Uni
     }
 }
 
+__global__ void k_anchors64(SegDev seg, const double *__restrict__ tmpl, const UnitInfo *__restrict__ units, int unit0,
+                            int log2D, int max_anc, float4 *__restrict__ anchors) {
+    const int b = blockIdx.y;
+    const UnitInfo u = units[unit0 + b];
+    const double *T = tmpl + (int64_t)u.tmpl * kTmplStride;
+    const double c1 = T[TF_C1], c2 = T[TF_C2], c3 = T[TF_C3], c5 = T[TF_C5];
+    float4 *out = anchors + (int64_t)b * 3 * max_anc;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < u.n_anc; i += gridDim.x * blockDim.x) {
+        const int64_t g = (int64_t)u.g_lo + i;
+        const Anchor64 r = anchor_record64(c1, c2, c3, c5, g, log2D, seg.df);
+        const int64_t a = anchor_slot_index(g, seg.log2N, seg.log2N1, log2D);
+        if (!MF_DBG(a >= 0 && a < max_anc, kDbgAnchor)) continue;
+        auto lo = [](unsigned long long x) { return __int_as_float((int)(unsigned)x); };
+        auto hi = [](unsigned long long x) { return __int_as_float((int)(unsigned)(x >> 32)); };
+        out[a] = make_float4(lo(r.r0), hi(r.r0), lo(r.q1), hi(r.q1));
+        out[a + max_anc] = make_float4(lo(r.q2), hi(r.q2), r.q3, r.q4);
+        out[a + 2 * (int64_t)max_anc] = make_float4(r.q5, r.q6, 0.f, 0.f);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // launches
 // ---------------------------------------------------------------------------
@@ -86,11 +107,17 @@ cudaError_t launch_units(const SegDev &seg, const double *tmpl, int n_t, double 
 }
 
 cudaError_t launch_anchors(const SegDev &seg, const double *tmpl, const UnitInfo *units, int unit0, int n_units,
-                           int log2D, int max_anc, float4 *anchors, float *anchors4, cudaStream_t st, int reps) {
+                           int log2D, int max_anc, float4 *anchors, float *anchors4, int phase_mode, cudaStream_t st,
+                           int reps) {
     if (reps < 1) return cudaErrorInvalidValue;
     const int per = 256;
     int gx = (max_anc + per - 1) / per;
     if (gx > 64) gx = 64;
+    if (phase_mode == MF_PHASE_FP64) {
+        if (reps != 1) return cudaErrorInvalidValue;
+        k_anchors64<<<dim3(gx, n_units), per, 0, st>>>(seg, tmpl, units, unit0, log2D, max_anc, anchors);
+        return cudaGetLastError();
+    }
     k_anchors<<<dim3(gx, n_units), per, 0, st>>>(seg, tmpl, units, unit0, log2D, max_anc, anchors, anchors4, reps);
     return cudaGetLastError();
 }
@@ -114,6 +141,10 @@ struct Pass1Op {
         if (phase_mode == MF_PHASE_FP32) {
             typename TemplateSrcF32<N2, C, cx_ilog2(N1)>::Params sp{seg.W, units, tmpl, (float)seg.df};
             return run_pass<N2, C, true, +1, TemplateSrcF32<N2, C, cx_ilog2(N1)>, ExchSink<N2, C, +1, cx_ilog2(N1)>>(grid, sp, kp, st, unit0);
+        }
+        if (phase_mode == MF_PHASE_FP64) {
+            typename TemplateSrc64<N2, C, cx_ilog2(N1)>::Params sp{seg.W, units, anchors, max_anc, log2D, anc_slots};
+            return run_pass<N2, C, true, +1, TemplateSrc64<N2, C, cx_ilog2(N1)>, ExchSink<N2, C, +1, cx_ilog2(N1)>>(grid, sp, kp, st, unit0);
         }
         typename TemplateSrc<N2, C, cx_ilog2(N1)>::Params sp{seg.W, units, anchors, anchors4, max_anc, log2D, anc_slots};
         return run_pass<N2, C, true, +1, TemplateSrc<N2, C, cx_ilog2(N1)>, ExchSink<N2, C, +1, cx_ilog2(N1)>>(grid, sp, kp, st, unit0);
@@ -161,6 +192,7 @@ struct AttrOp {
         cudaError_t e;
         if ((e = set_pass_attrs<N2, C1, true, +1, TemplateSrc<N2, C1, cx_ilog2(N1)>, ExchSink<N2, C1, +1, cx_ilog2(N1)>>())) return e;
         if ((e = set_pass_attrs<N2, C1, true, +1, TemplateSrcF32<N2, C1, cx_ilog2(N1)>, ExchSink<N2, C1, +1, cx_ilog2(N1)>>())) return e;
+        if ((e = set_pass_attrs<N2, C1, true, +1, TemplateSrc64<N2, C1, cx_ilog2(N1)>, ExchSink<N2, C1, +1, cx_ilog2(N1)>>())) return e;
         return set_pass_attrs<N1, C2, false, +1, RowSrc<N1, C2>, RhoSink<N1, C2>>();
     }
 };

@@ -145,6 +145,146 @@ struct TemplateSrc {
     }
 };
 
+// ---------------------------------------------------------------------------
+// MF_PHASE_FP64: the phase at 64-bit accuracy at every bin.  GB300 issues two
+// FP64 operations per SM and clock, so psi in FP64 at every bin (27 of them
+// with the unused derivatives) was two thirds of the filter's time: 1125 of
+// 1714 us for 250 templates at N = 2^18.  Between FP64 anchors the phase is
+// instead summed in turns mod 1 as 64-bit fixed point: with the integer offset
+// d from the anchor centre,
+//   psi = r0 + d (q1 + d q2)  (mod 1, exact in 2^-64 turns)  +  d^3 (q3 + d (q4 + d (q5 + d q6)))
+// where the quadratic part is two 64-bit integer multiply-adds (d is an
+// integer, so q1 and q2 count mod 1) and the small rest FP32.  anchor_log2D64
+// bounds what is left out and the size of the FP32 part, so that psi is good
+// to 4e-10 turns before it is rounded to FP32 (1.5e-8, as before) for the sincos.
+// Record: three planes of 16 bytes (r0, q1 | q2, q3, q4 | q5, q6, -, -).
+// ---------------------------------------------------------------------------
+struct Anchor64 {
+    unsigned long long r0, q1, q2;
+    float q3, q4, q5, q6;
+};
+__device__ __forceinline__ unsigned long long turns_fixed(double x) {   // x mod 1 in 2^-64 turns
+    return (unsigned long long)__double2ll_rn((x - rint(x)) * 4611686018427387904.0) << 2;   // 2^62: +-1/2 fits
+}
+__device__ __forceinline__ Anchor64 anchor_record64(double c1, double c2, double c3, double c5, int64_t g, int log2D,
+                                                    double df) {
+    const int64_t ka = (g << log2D) + ((1 << log2D) >> 1);
+    const double f = (double)ka * df;
+    double uu = (double)rcbrtf((float)f);
+    uu = uu * (4.0 - f * uu * uu * uu) * (1.0 / 3.0);
+    const double u2 = uu * uu;
+    const double psi = -0.125 + uu * (c1 + uu * (c2 + uu * (c3 + u2 * c5)));
+    const double S1 = uu * (c1 + uu * (2.0 * c2 + uu * (3.0 * c3 + u2 * (5.0 * c5))));
+    const double S2 = uu * (4.0 * c1 + uu * (10.0 * c2 + uu * (18.0 * c3 + u2 * (40.0 * c5))));
+    const double ik = 1.0 / (double)ka;
+    const float uf = (float)uu, ikf = (float)ik, ik3 = ikf * ikf * ikf;
+    const float w1 = (float)c1 * uf, w2 = (float)c2 * uf * uf, w3 = (float)c3 * uf * uf * uf;
+    const float w5 = (float)c5 * (uf * uf) * (uf * uf * uf);
+    Anchor64 a;
+    a.r0 = turns_fixed(psi);
+    a.q1 = turns_fixed(-S1 * ik * (1.0 / 3.0));
+    a.q2 = turns_fixed(S2 * ik * ik * (1.0 / 18.0));
+    a.q3 = -(28.f * w1 + 80.f * w2 + 162.f * w3 + 440.f * w5) * ik3 * (1.f / 162.f);
+    a.q4 = (280.f * w1 + 880.f * w2 + 1944.f * w3 + 6160.f * w5) * ik3 * ikf * (1.f / 1944.f);
+    a.q5 = -(3640.f * w1 + 12320.f * w2 + 29160.f * w3 + 104720.f * w5) * ik3 * (ikf * ikf) * (1.f / 29160.f);
+    a.q6 = (58240.f * w1 + 209440.f * w2 + 524880.f * w3 + 2094400.f * w5) * ik3 * ik3 * (1.f / 524880.f);
+    return a;
+}
+// phase in turns at integer offset d, d3 = d^3
+__device__ __forceinline__ float anchor_phase64(const float4 &p0, const float4 &p1, const float4 &p2, int d, float df,
+                                                float d3) {
+    const long long r0 = ((long long)__float_as_int(p0.y) << 32) | (unsigned)__float_as_int(p0.x);
+    const long long q1 = ((long long)__float_as_int(p0.w) << 32) | (unsigned)__float_as_int(p0.z);
+    const long long q2 = ((long long)__float_as_int(p1.y) << 32) | (unsigned)__float_as_int(p1.x);
+    const unsigned long long dd = (unsigned long long)(long long)d;
+    const unsigned long long t = (unsigned long long)r0 + dd * ((unsigned long long)q1 + dd * (unsigned long long)q2);
+    const float tail = d3 * fmaf(df, fmaf(df, fmaf(df, p2.y, p2.x), p1.w), p1.z);
+    // |tail| < 2^-10: added to 1.5 * 2^-9 its mantissa counts 2^-32 turns
+    const int hi = (int)(t >> 32) + (__float_as_int(tail + 0.0029296875f) - 0x3b400000);
+    return (float)hi * 2.3283064365386963e-10f;   // 2^-32: in [-1/2, 1/2], rounded once
+}
+
+// pass-1 source of MF_PHASE_FP64
+template <int L, int C, int LG1>
+struct TemplateSrc64 {
+    static constexpr bool kHalfZero = true;
+    static constexpr bool kSplitTw = true;
+    static constexpr size_t kScratchBytes = (size_t)(L / 2) * 3 * sizeof(float4);
+    struct Params {
+        const float2 *W;
+        const UnitInfo *units;
+        const float4 *anchors;   // slot: three planes of anc_stride records
+        int anc_stride, log2D, anc_slots;
+    };
+    const Params &p;
+    const int tile, unit, slot;
+    float4 *sa;
+    __device__ TemplateSrc64(const Params &pp, int tl, int un, int sl, void *scratch)
+        : p(pp), tile(tl), unit(un), slot(sl), sa((float4 *)scratch) {}
+    // All threads of the block call load() (it contains a block barrier).
+    __device__ __forceinline__ void load(int seq, int t, float2 *v) const {
+        constexpr int T = L / 32;
+        constexpr int LGL = cx_ilog2(L);
+        const UnitInfo u = p.units[unit];
+        const int aslot = p.anc_slots > 0 ? slot % p.anc_slots : slot;
+        const float4 *anc = p.anchors + (int64_t)aslot * 3 * p.anc_stride;   // index: anchor_slot_index(g)
+        const int k1 = tile * C + seq;
+        const int D = 1 << p.log2D;
+        const int k0 = k1 + (t << LG1);
+        float2 w[16];
+        bool in[16];
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+            const int k = k0 + ((r * T) << LG1);
+            in[r] = (k >= u.k_lo) && (k < u.k_hi);
+            w[r] = in[r] ? __ldg(&p.W[k]) : czero();   // no load outside the band
+        }
+        const bool shared_row = D >= C && p.log2D <= LG1;   // one record per column row, as in TemplateSrc
+        if (shared_row) {
+            const int gstep = 1 << (LG1 - p.log2D);
+            const int gcol = (tile * C) >> p.log2D;
+            const int gbase = gcol - u.g_lo;
+            const float4 *acol = anc + ((int64_t)gcol << (LGL - 1));
+            for (int n = threadIdx.x; n < L / 2; n += blockDim.x) {
+                const int a = gbase + n * gstep;
+                if (a >= 0 && a < u.n_anc && MF_DBG(((int64_t)gcol << (LGL - 1)) + n < p.anc_stride, kDbgAnchor)) {
+#pragma unroll
+                    for (int h = 0; h < 3; ++h) sa[h * (L / 2) + n] = __ldcg(&acol[(int64_t)h * p.anc_stride + n]);
+                }
+            }
+            __syncthreads();
+        }
+        const int d0 = (k1 & (D - 1)) - (D >> 1);   // the same on every row when D divides N1
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+            float4 a0, a1, a2;
+            int d = d0;
+            if (shared_row) {
+                const int n = t + r * T;
+                a0 = sa[n];
+                a1 = sa[L / 2 + n];
+                a2 = sa[L + n];
+            } else {
+                const int k = k0 + ((r * T) << LG1);
+                const int kk = in[r] ? k : u.k_lo;
+                const int g = kk >> p.log2D;
+                int64_t ai = anchor_slot_index(g, LGL + LG1, LG1, p.log2D);
+                if (!MF_DBG(ai >= 0 && ai < p.anc_stride, kDbgAnchor)) ai = 0;
+                a0 = __ldcg(&anc[ai]);
+                a1 = __ldcg(&anc[ai + p.anc_stride]);
+                a2 = __ldcg(&anc[ai + 2 * (int64_t)p.anc_stride]);
+                d = kk - ((g << p.log2D) + (D >> 1));
+            }
+            const float df = (float)d;
+            const float ph = anchor_phase64(a0, a1, a2, d, df, df * df * df);
+            float sn, cs;
+            __sincosf(6.283185307179586f * ph, &sn, &cs);
+            const float2 x = make_float2(fmaf(w[r].x, cs, w[r].y * sn), fmaf(w[r].y, cs, -w[r].x * sn));
+            v[r] = in[r] ? x : czero();   // rows outside the band read stale records
+        }
+    }
+};
+
 // FP32-only phase (precision-sweep reference): psi evaluated directly in FP32.
 template <int L, int C, int LG1>
 struct TemplateSrcF32 {

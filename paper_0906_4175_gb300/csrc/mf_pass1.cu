@@ -213,7 +213,7 @@ EncodeTiledFn encode_tiled() {
 MF_DEBUG_READER(dbg_read_pass1)
 
 bool pass1_pf_applies(int log2N, int log2N2, int log2D, int phase_mode) {
-    if (g_pf_sms <= 0 || phase_mode == MF_PHASE_FP32) return false;
+    if (g_pf_sms <= 0 || phase_mode != MF_PHASE_ANCHOR) return false;
     const char *env = std::getenv("MFGB_P1PF");   // "0": the per-tile kernel (comparisons)
     if (env && env[0] == '0') return false;
     if (log2N < 16 || log2N > 22 || log2N2 < 8 || log2N2 > 10) return false;
