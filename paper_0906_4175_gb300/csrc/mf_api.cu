@@ -93,6 +93,7 @@ static int ensure_device_init() {
     MF_CUDA(refine_kernel_attributes());
     MF_CUDA(chisq_kernel_attributes());
     MF_CUDA(rows_kernel_attributes());
+    MF_CUDA(events_kernel_attributes());
     MF_CUDA(pass1_pf_kernel_attributes());
     MF_CUDA(prep64_kernel_attributes());
     MF_CUDA(fused_kernel_attributes());
@@ -263,17 +264,15 @@ struct Workspace {
     mf_trigger *staged = nullptr;
     uint64_t *keys = nullptr, *keys_tmp = nullptr;
     uint32_t *idx_a = nullptr, *idx_b = nullptr;
-    uint32_t *ghist = nullptr;    // trigger sort: digit histograms of every pass
     uint64_t *tstat = nullptr;    // trigger sort: look-back status per (tile, digit)
-    unsigned *tickets = nullptr;  // trigger sort: tile tickets per pass
-    unsigned long long *counter = nullptr;
-    int *status = nullptr;
+    FilterCtl *fctl = nullptr;    // trigger count, status and sort control, zeroed by one memset per call
+    unsigned long long *counter = nullptr;   // fctl->counter
+    int *status = nullptr;                   // fctl->status
     unsigned *ctl = nullptr;      // persistent scheduler: [1] abort, then doneA, done1, done2 per unit
     void release() {
         cudaFree(units); cudaFree(exch); cudaFree(anchors); cudaFree(anchors4); cudaFree(partials);
         cudaFree(staged); cudaFree(keys); cudaFree(keys_tmp); cudaFree(idx_a); cudaFree(idx_b);
-        cudaFree(ghist); cudaFree(tstat); cudaFree(tickets);
-        cudaFree(counter); cudaFree(status); cudaFree(ctl);
+        cudaFree(tstat); cudaFree(fctl); cudaFree(ctl);
         *this = Workspace();
     }
 };
@@ -761,12 +760,11 @@ static int ensure_workspace(mf_bank_s *b, int64_t exch_elems, int64_t cap, int64
     MF_CUDA(dev_malloc(&w.keys_tmp, sizeof(uint64_t) * ncap));
     MF_CUDA(dev_malloc(&w.idx_a, sizeof(uint32_t) * ncap));
     MF_CUDA(dev_malloc(&w.idx_b, sizeof(uint32_t) * ncap));
-    MF_CUDA(dev_malloc(&w.ghist, sizeof(uint32_t) * 256 * 8));
     MF_CUDA(dev_malloc(&w.tstat, sizeof(uint64_t) * sort_tile_words(ncap)));
-    MF_CUDA(dev_malloc(&w.tickets, sizeof(unsigned) * 8));
-    MF_CUDA(dev_malloc(&w.counter, sizeof(unsigned long long)));
-    MF_CUDA(dev_malloc(&w.status, sizeof(int)));
-    MF_CUDA(cudaMemset(w.status, 0, sizeof(int)));
+    MF_CUDA(dev_malloc(&w.fctl, sizeof(FilterCtl)));
+    MF_CUDA(cudaMemset(w.fctl, 0, sizeof(FilterCtl)));
+    w.counter = &w.fctl->counter;
+    w.status = &w.fctl->status;
     MF_CUDA(dev_malloc(&w.ctl, sizeof(unsigned) * (4 + 3 * b->n)));
     w.exch_elems = ne; w.n_t = b->n; w.cap = ncap; w.anc_elems = na; w.nblk = nbl;
     return MF_OK;
@@ -948,8 +946,7 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
     int rc = ensure_workspace(b, exch_elems, trig_cap, anc_elems, nblk, capturing);
     if (rc) return rc;
     Workspace &w = b->ws;
-    MF_CUDA(cudaMemsetAsync(w.counter, 0, sizeof(unsigned long long), st));
-    MF_CUDA(cudaMemsetAsync(w.status, 0, sizeof(int), st));
+    MF_CUDA(cudaMemsetAsync(w.fctl, 0, sizeof(FilterCtl), st));
     const int n_t = (int)b->n;
     // descending-cost unit order (MFGB_UNIT_ORDER=bank keeps bank order); the
     // stall hook names a template, the kernels see its unit position
@@ -1158,10 +1155,10 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
     }
     int pf = prof_begin(b, MF_STAGE_FINAL, 0.0, st);
     MF_CUDA(launch_sort_triggers(w.counter, std::max<int64_t>(trig_cap, 0), key_bits, w.staged, w.keys,
-                                 w.keys_tmp, w.idx_a, w.idx_b, w.ghist, w.tstat, w.tickets, trig, nullptr, n_trig,
-                                 w.status, sm_count(), b->spin_limit, st));
+                                 w.keys_tmp, w.idx_a, w.idx_b, &w.fctl->sort, w.tstat, trig, n_trig, w.status,
+                                 sm_count(), b->spin_limit, st));
     prof_end(b, pf, st);
-    count_launches(sort_launches(key_bits));
+    count_launches(1);
     return MF_OK;
 }
 
@@ -1301,45 +1298,44 @@ extern "C" int mf_cluster_triggers(const mf_trigger *trig, const int64_t *n_trig
     if (r0) return r0;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const int64_t cap = trig_cap;
-    const int64_t nb = cluster_scan_blocks(cap);
-    ClusterScratch w;
+    ClusterScratch w{};
     Scratch sc;
     std::vector<std::pair<void **, size_t>> parts;
     auto get = [&](auto **ptr, size_t bytes) { parts.push_back({(void **)ptr, sc.add(bytes)}); };
-    get(&w.flag, sizeof(uint32_t) * cap);
-    get(&w.incl, sizeof(uint32_t) * cap);
-    sc.group();
-    get(&w.bsum, sizeof(uint32_t) * nb);
-    get(&w.members, sizeof(uint32_t) * cap);
-    get(&w.wsum, sizeof(uint32_t) * cap);
-    sc.group();
-    get(&w.rep_count, sizeof(uint32_t) * cap);
-    get(&w.idx_a, sizeof(uint32_t) * cap);
-    get(&w.idx_b, sizeof(uint32_t) * cap);
-    get(&w.perm, sizeof(uint32_t) * cap);
-    get(&w.ghist, sizeof(uint32_t) * 256 * 8);
-    sc.group();
-    get(&w.best, sizeof(unsigned long long) * cap);
-    get(&w.rep, sizeof(mf_trigger) * cap);
-    get(&w.sorted, sizeof(mf_trigger) * cap);
-    sc.group();
-    get(&w.keys, sizeof(uint64_t) * cap);
-    get(&w.keys_tmp, sizeof(uint64_t) * cap);
-    get(&w.tstat, sizeof(uint64_t) * sort_tile_words(cap));
-    get(&w.tickets, sizeof(unsigned) * 8);
+    const size_t o_status = sc.add(sizeof(int));   // zeroed with the control words after it
+    get(&w.ctl, sizeof(SortCtl));
+    const size_t zeroed = sc.size[0];
     get(&w.n_c, sizeof(int64_t));
-    get(&w.n_sorted, sizeof(int64_t));
-    get(&w.status, sizeof(int));
+    if (cap > cluster_small_limit()) {   // the one-CTA form works in shared memory
+        sc.group();
+        get(&w.members, sizeof(uint32_t) * cap);
+        get(&w.members2, sizeof(uint32_t) * cap);
+        get(&w.wsum, sizeof(uint32_t) * cap);
+        get(&w.idx_a, sizeof(uint32_t) * cap);
+        get(&w.idx_b, sizeof(uint32_t) * cap);
+        sc.group();
+        get(&w.best, sizeof(unsigned long long) * cap);
+        get(&w.best2, sizeof(unsigned long long) * cap);
+        sc.group();
+        get(&w.rep, sizeof(mf_trigger) * cap);
+        get(&w.sorted, sizeof(mf_trigger) * cap);
+        sc.group();
+        get(&w.keys, sizeof(uint64_t) * cap);
+        get(&w.keys_tmp, sizeof(uint64_t) * cap);
+        get(&w.tstat, sizeof(uint64_t) * sort_tile_words(cap));
+        get(&w.scan, sizeof(uint64_t) * cluster_scan_words(cap));
+    }
     cudaError_t e = sc.alloc(st);
     for (auto &q : parts) *q.first = sc.at<char>(q.second);
-    if (e == cudaSuccess) e = cudaMemsetAsync(w.status, 0, sizeof(int), st);
+    w.status = sc.at<int>(o_status);
+    if (e == cudaSuccess) e = cudaMemsetAsync(w.status, 0, zeroed, st);
     if (e == cudaSuccess)
         e = launch_cluster(trig, n_trig, cap, window, kl, w, events, ev_cap, n_events, sm_count(), 4000000, st);
     sc.free(st);
     if (e != cudaSuccess)
         return set_err(e == cudaErrorMemoryAllocation ? MF_ENOMEM : MF_ECUDA, "cluster_triggers: %s",
                        cudaGetErrorString(e));
-    count_launches(cluster_launches(key_bits));
+    count_launches(1);
     return MF_OK;
 }
 
@@ -1354,22 +1350,25 @@ extern "C" int mf_chisq_points(mf_bank b, const mf_segment *segs, int n_seg, con
     cudaGetDevice(&cur);
     if (b->device != cur) return set_err(MF_EINVAL, "bank lives on device %d", b->device);
     std::vector<SegDev> sd((size_t)n_seg);
+    std::vector<int> lg((size_t)n_seg);
     for (int s = 0; s < n_seg; ++s) {
         if (!segs[s] || segs[s]->device != cur) return set_err(MF_EINVAL, "segs[%d] is NULL or on another device", s);
         sd[(size_t)s] = seg_dev(segs[s]);
+        lg[(size_t)s] = b->params.phase_mode == MF_PHASE_FP64 ? 0 : choose_log2D(b, segs[s]);
     }
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const int64_t chunk = std::min<int64_t>(n, 65535);
     const int bpr = (int)std::max<int64_t>(4, std::min<int64_t>(64, (4 * (int64_t)sm_count() + chunk - 1) / chunk));
     Scratch sc;
-    sc.add(sizeof(double2) * (size_t)bpr * chunk * p);
+    const size_t o_partial = sc.add(sizeof(double2) * (size_t)bpr * chunk * p), o_pratio = sc.add(sizeof(double) * chunk);
     cudaError_t e = sc.alloc(st);
-    double2 *partial = sc.at<double2>(0);
+    double2 *partial = sc.at<double2>(o_partial);
+    double *pratio = sc.at<double>(o_pratio);
     int launches = 0;
     for (int64_t i0 = 0; i0 < n && e == cudaSuccess; i0 += chunk) {
         const int64_t m = std::min<int64_t>(chunk, n - i0);
-        e = launch_chisq_points(sd.data(), n_seg, b->d_tmpl, (int)b->n, b->params.f_low, b->params.phase_mode,
-                                rows + i0 * stride, stride, m, p, bpr, partial, chisq + i0, st);
+        e = launch_chisq_points(sd.data(), lg.data(), n_seg, b->d_tmpl, (int)b->n, b->params.f_low, rows + i0 * stride,
+                                stride, m, p, bpr, partial, pratio, chisq + i0, st);
         launches += 2;
     }
     sc.free(st);

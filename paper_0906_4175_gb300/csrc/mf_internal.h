@@ -265,14 +265,29 @@ cudaError_t launch_peaks_rows(const SegDev &seg, const UnitInfo *units, int unit
                               cudaStream_t st);
 cudaError_t launch_reduce_peaks(const SegDev &seg, const UnitInfo *units, int n_units, const float4 *partials,
                                 int nblk, int seg_idx, int n_seg, mf_peak *peaks, cudaStream_t st);
+// Control words of a sort or clustering launch, all zero before it: digit
+// histograms of every pass, and per step the tile tickets and finished tiles.
+constexpr int kSortMaxPass = 8, kSortMaxPhase = 16;
+struct SortCtl {
+    unsigned ghist[kSortMaxPass * 256];
+    unsigned ticket[kSortMaxPhase], done[kSortMaxPhase];
+    unsigned abort, pad;
+};
+// what a filter call zeroes before its first kernel
+struct FilterCtl {
+    unsigned long long counter;   // triggers found
+    int status;                   // bit 0: overflow, bit 1: a bounded wait ran out
+    int pad;
+    SortCtl sort;
+};
+constexpr int kSortTile = 4096;   // keys per tile of a sort of more than 8192 keys
+// one kernel; ctl zeroed.  (mf_sort.cuh)
 cudaError_t launch_sort_triggers(const unsigned long long *counter, int64_t cap, int key_bits,
                                  const mf_trigger *staged, const uint64_t *keys, uint64_t *keys_tmp,
-                                 uint32_t *idx_a, uint32_t *idx_b, uint32_t *ghist, uint64_t *tstat,
-                                 unsigned *tickets, mf_trigger *out, uint32_t *perm_out, int64_t *n_out,
-                                 int *status, int n_sm, int64_t spin_limit, cudaStream_t st);
-int sort_launches(int key_bits);   // kernels queued by launch_sort_triggers
-// tile status words the sort needs for cap records (one per 2048-key tile and digit)
-inline int64_t sort_tile_words(int64_t cap) { return ((cap + 2047) / 2048) * 256; }
+                                 uint32_t *idx_a, uint32_t *idx_b, SortCtl *ctl, uint64_t *tstat, mf_trigger *out,
+                                 int64_t *n_out, int *status, int n_sm, int64_t spin_limit, cudaStream_t st);
+// tile status words the sort needs for cap records (one per tile and digit)
+inline int64_t sort_tile_words(int64_t cap) { return ((cap + kSortTile - 1) / kSortTile) * 256; }
 
 // refinement (mf_refine.cu).  partial: device scratch of refine_scratch_bytes(n, bpr)
 // bytes (8 partial sums per block, then one row record of at most kRefRowBytesMax bytes per row)
@@ -290,24 +305,28 @@ cudaError_t launch_chisq_units(const SegDev &seg, const UnitInfo *all, int n_t, 
 cudaError_t launch_chisq_tiles(const SegDev &seg, const float2 *exch, const UnitInfo *full, int unit0, int nb, int p,
                                float *chisq, cudaStream_t st);
 
-// trigger clustering scratch (every array sized for the trigger capacity)
+// trigger clustering scratch (arrays sized for the trigger capacity; ctl
+// zeroed before the launch, scan: two look-back words per tile)
 struct ClusterScratch {
-    uint32_t *flag, *incl, *bsum, *members, *wsum, *rep_count, *idx_a, *idx_b, *perm, *ghist;
-    unsigned long long *best;
+    uint32_t *members, *members2, *wsum, *idx_a, *idx_b;
+    unsigned long long *best, *best2;
     mf_trigger *rep, *sorted;
-    uint64_t *keys, *keys_tmp, *tstat;
-    unsigned *tickets;
-    int64_t *n_c, *n_sorted;
+    uint64_t *keys, *keys_tmp, *tstat, *scan;
+    int64_t *n_c;
     int *status;
+    SortCtl *ctl;
 };
+inline int64_t cluster_small_limit() { return 8192; }   // triggers one CTA clusters in shared memory
+inline int64_t cluster_scan_words(int64_t cap) { return 2 * ((cap + kSortTile - 1) / kSortTile); }
 cudaError_t launch_cluster(const mf_trigger *trig, const int64_t *n_trig, int64_t cap, int window, KeyLayout kl,
-                           ClusterScratch &w, mf_event *events, int64_t ev_cap, int64_t *n_events, int n_sm,
+                           const ClusterScratch &w, mf_event *events, int64_t ev_cap, int64_t *n_events, int n_sm,
                            int64_t spin_limit, cudaStream_t st);
-int cluster_launches(int key_bits);
-int64_t cluster_scan_blocks(int64_t cap);
-cudaError_t launch_chisq_points(const SegDev *segs, int n_seg, const double *tmpl, int n_t, double f_low,
-                                int phase_mode, const int32_t *rows, int64_t stride, int64_t n, int p, int bpr,
-                                double2 *partial, float *chisq, cudaStream_t st);
+cudaError_t events_kernel_attributes();
+// lg[s]: log2 of segment s's anchor spacing (0: FP64 phase at every bin);
+// scratch: partial bpr * n * p complex128, pratio n doubles
+cudaError_t launch_chisq_points(const SegDev *segs, const int *lg, int n_seg, const double *tmpl, int n_t,
+                                double f_low, const int32_t *rows, int64_t stride, int64_t n, int p, int bpr,
+                                double2 *partial, double *pratio, float *chisq, cudaStream_t st);
 
 // segments of one mf_refine_triggers_multi call (kernel-parameter table)
 constexpr int kRefineMaxSegs = 256;
