@@ -152,19 +152,28 @@ struct TemplateSrc {
 // 1714 us for 250 templates at N = 2^18.  Between FP64 anchors the phase is
 // instead summed in turns mod 1 as 64-bit fixed point: with the integer offset
 // d from the anchor centre,
-//   psi = r0 + d (q1 + d q2)  (mod 1, exact in 2^-64 turns)  +  d^3 (q3 + d (q4 + d (q5 + d q6)))
-// where the quadratic part is two 64-bit integer multiply-adds (d is an
-// integer, so q1 and q2 count mod 1) and the small rest FP32.  anchor_log2D64
+//   psi = r0 + d (q1 + d (q2 + d q3))  (mod 1, exact in 2^-64 turns)  +  d^4 (q4 + d (q5 + d q6))
+// where the cubic part is three 64-bit integer multiply-adds (d is an integer,
+// so the coefficients count mod 1) and the small rest FP32.  anchor_log2D64
 // bounds what is left out and the size of the FP32 part, so that psi is good
 // to 4e-10 turns before it is rounded to FP32 (1.5e-8, as before) for the sincos.
-// Record: three planes of 16 bytes (r0, q1 | q2, q3, q4 | q5, q6, -, -).
+// Record: three planes of 16 bytes (r0, q1 | q2, q3 | q4, q5, q6, -).
 // ---------------------------------------------------------------------------
 struct Anchor64 {
-    unsigned long long r0, q1, q2;
-    float q3, q4, q5, q6;
+    unsigned long long r0, q1, q2, q3;
+    float q4, q5, q6;
 };
-__device__ __forceinline__ unsigned long long turns_fixed(double x) {   // x mod 1 in 2^-64 turns
-    return (unsigned long long)__double2ll_rn((x - rint(x)) * 4611686018427387904.0) << 2;   // 2^62: +-1/2 fits
+// x mod 1 in 2^-64 turns: the sum with 1.5 * 2^(52 - 30) leaves x in units of
+// 2^-30 in the mantissa, and the rest of x is exact (a conversion from FP64 to
+// a 64-bit integer is several FP64 operations)
+__device__ __forceinline__ unsigned long long turns_fixed(double x) {
+    x -= rint(x);
+    constexpr double kBig = 6291456.0;   // 1.5 * 2^22
+    const double s = x + kBig;
+    const long long hi = __double_as_longlong(s) & ((1ll << 30) - 1);   // x mod 1 in 2^-30 turns
+    const double rest = x - (s - kBig);                                  // |rest| <= 2^-31
+    const float top = (float)rest;                                       // rest to 2^-55
+    return ((unsigned long long)hi << 34) + (unsigned long long)(long long)__float2ll_rn(top * 1.8446744073709552e19f);
 }
 __device__ __forceinline__ Anchor64 anchor_record64(double c1, double c2, double c3, double c5, int64_t g, int log2D,
                                                     double df) {
@@ -176,29 +185,32 @@ __device__ __forceinline__ Anchor64 anchor_record64(double c1, double c2, double
     const double psi = -0.125 + uu * (c1 + uu * (c2 + uu * (c3 + u2 * c5)));
     const double S1 = uu * (c1 + uu * (2.0 * c2 + uu * (3.0 * c3 + u2 * (5.0 * c5))));
     const double S2 = uu * (4.0 * c1 + uu * (10.0 * c2 + uu * (18.0 * c3 + u2 * (40.0 * c5))));
-    const double ik = 1.0 / (double)ka;
-    const float uf = (float)uu, ikf = (float)ik, ik3 = ikf * ikf * ikf;
+    const double ik = df * u2 * uu;   // 1 / k_a
+    const double ik2 = ik * ik;
+    const float uf = (float)uu, ikf = (float)ik, ik4 = (ikf * ikf) * (ikf * ikf);
     const float w1 = (float)c1 * uf, w2 = (float)c2 * uf * uf, w3 = (float)c3 * uf * uf * uf;
     const float w5 = (float)c5 * (uf * uf) * (uf * uf * uf);
+    const double S3 = uu * (28.0 * c1 + uu * (80.0 * c2 + uu * (162.0 * c3 + u2 * (440.0 * c5))));
     Anchor64 a;
     a.r0 = turns_fixed(psi);
-    a.q1 = turns_fixed(-S1 * ik * (1.0 / 3.0));
-    a.q2 = turns_fixed(S2 * ik * ik * (1.0 / 18.0));
-    a.q3 = -(28.f * w1 + 80.f * w2 + 162.f * w3 + 440.f * w5) * ik3 * (1.f / 162.f);
-    a.q4 = (280.f * w1 + 880.f * w2 + 1944.f * w3 + 6160.f * w5) * ik3 * ikf * (1.f / 1944.f);
-    a.q5 = -(3640.f * w1 + 12320.f * w2 + 29160.f * w3 + 104720.f * w5) * ik3 * (ikf * ikf) * (1.f / 29160.f);
-    a.q6 = (58240.f * w1 + 209440.f * w2 + 524880.f * w3 + 2094400.f * w5) * ik3 * ik3 * (1.f / 524880.f);
+    a.q1 = turns_fixed(S1 * ik * (-1.0 / 3.0));
+    a.q2 = turns_fixed(S2 * ik2 * (1.0 / 18.0));
+    a.q3 = turns_fixed(S3 * (ik2 * ik) * (-1.0 / 162.0));
+    a.q4 = (280.f * w1 + 880.f * w2 + 1944.f * w3 + 6160.f * w5) * ik4 * (1.f / 1944.f);
+    a.q5 = -(3640.f * w1 + 12320.f * w2 + 29160.f * w3 + 104720.f * w5) * ik4 * ikf * (1.f / 29160.f);
+    a.q6 = (58240.f * w1 + 209440.f * w2 + 524880.f * w3 + 2094400.f * w5) * ik4 * (ikf * ikf) * (1.f / 524880.f);
     return a;
 }
-// phase in turns at integer offset d, d3 = d^3
+// phase in turns at integer offset d, d4 = d^4
 __device__ __forceinline__ float anchor_phase64(const float4 &p0, const float4 &p1, const float4 &p2, int d, float df,
-                                                float d3) {
-    const long long r0 = ((long long)__float_as_int(p0.y) << 32) | (unsigned)__float_as_int(p0.x);
-    const long long q1 = ((long long)__float_as_int(p0.w) << 32) | (unsigned)__float_as_int(p0.z);
-    const long long q2 = ((long long)__float_as_int(p1.y) << 32) | (unsigned)__float_as_int(p1.x);
+                                                float d4) {
+    auto word = [](float lo, float hi) {
+        return ((unsigned long long)(unsigned)__float_as_int(hi) << 32) | (unsigned)__float_as_int(lo);
+    };
     const unsigned long long dd = (unsigned long long)(long long)d;
-    const unsigned long long t = (unsigned long long)r0 + dd * ((unsigned long long)q1 + dd * (unsigned long long)q2);
-    const float tail = d3 * fmaf(df, fmaf(df, fmaf(df, p2.y, p2.x), p1.w), p1.z);
+    const unsigned long long t =
+        word(p0.x, p0.y) + dd * (word(p0.z, p0.w) + dd * (word(p1.x, p1.y) + dd * word(p1.z, p1.w)));
+    const float tail = d4 * fmaf(df, fmaf(df, p2.z, p2.y), p2.x);
     // |tail| < 2^-10: added to 1.5 * 2^-9 its mantissa counts 2^-32 turns
     const int hi = (int)(t >> 32) + (__float_as_int(tail + 0.0029296875f) - 0x3b400000);
     return (float)hi * 2.3283064365386963e-10f;   // 2^-32: in [-1/2, 1/2], rounded once
@@ -276,7 +288,7 @@ struct TemplateSrc64 {
                 d = kk - ((g << p.log2D) + (D >> 1));
             }
             const float df = (float)d;
-            const float ph = anchor_phase64(a0, a1, a2, d, df, df * df * df);
+            const float ph = anchor_phase64(a0, a1, a2, d, df, (df * df) * (df * df));
             float sn, cs;
             __sincosf(6.283185307179586f * ph, &sn, &cs);
             const float2 x = make_float2(fmaf(w[r].x, cs, w[r].y * sn), fmaf(w[r].y, cs, -w[r].x * sn));

@@ -97,16 +97,15 @@ __host__ __device__ inline int anchor_log2D(double B1, double B5, double df) {
     return lg;
 }
 
-// The same for MF_PHASE_FP64 (fixed-point quadratic part, FP32 terms 3..6): the
+// The same for MF_PHASE_FP64 (fixed-point cubic part, FP32 terms 4..6): the
 // seventh-order remainder B7 df^7 (D/2)^7 / 5040 stays <= 5e-11 turns and the
-// FP32 part, dominated by B3 df^3 (D/2)^3 / 6, <= 2^-11 turns (it is summed in
+// FP32 part, dominated by B4 df^4 (D/2)^4 / 24, <= 2^-11 turns (it is summed in
 // units of 2^-32 turns and must stay below 2^-10).
-// D <= 256 keeps the rounding of q1 and q2 (2^-62 d^2) below 2^-48.
-__host__ __device__ inline int anchor_log2D64(double B3, double B7, double df) {
+__host__ __device__ inline int anchor_log2D64(double B4, double B7, double df) {
     int lg = 0;
     while (lg < 8) {
         const double h = df * (double)(1 << (lg + 1)) / 2.0;
-        if (B7 * h * h * h * h * h * h * h / 5040.0 > 5e-11 || B3 * h * h * h / 6.0 > 1.0 / 2048.0) break;
+        if (B7 * h * h * h * h * h * h * h / 5040.0 > 5e-11 || B4 * h * h * h * h / 24.0 > 1.0 / 2048.0) break;
         ++lg;
     }
     return lg;
