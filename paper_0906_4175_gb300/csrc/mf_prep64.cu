@@ -148,33 +148,42 @@ __device__ __forceinline__ void smem_dft64(double2 *x) {
     }
 }
 
-constexpr int kNT = 256;
-
 __host__ __device__ constexpr int cx_log2(int x) { return x <= 1 ? 0 : 1 + cx_log2(x >> 1); }
 
-// sequences of length 2^LG per CTA: 1024 points in shared memory (16 KB;
-// 2048 for the longest rows), one radix-4 butterfly per thread and stage
-template <int LG>
-__host__ __device__ constexpr int seqs64() { return LG >= 10 ? 1 : (1024 >> LG); }
+// Sequences of length 2^LG per CTA.  Long transforms: 1024 points in shared
+// memory (16 KB; 2048 for the longest rows) on 256 threads.  SMALL (M <= 2^16):
+// one sequence, at least 128 points, so that the transform reaches every SM:
+// the FP64 pipe does two operations per SM and clock, and M = 2^12 on 4 CTAs of
+// 1024 points was 10 us a pass, 4 us on 32 (refresh of 2^13 samples 22 -> 12 us).
+template <int LG, bool SMALL>
+__host__ __device__ constexpr int seqs64() {
+    return SMALL ? (LG >= 7 ? 1 : (128 >> LG)) : (LG >= 10 ? 1 : (1024 >> LG));
+}
+// threads: one radix-4 butterfly each (two for the longest rows)
+template <int LG, bool SMALL>
+__host__ __device__ constexpr int threads64() {
+    return (seqs64<LG, SMALL>() << LG) / 4 < 256 ? (seqs64<LG, SMALL>() << LG) / 4 : 256;
+}
 
 // pass A: columns n1 of z (stride M1, M2 = 2^LG2 points each), ca = min(seqs64, M1) per CTA
-template <int LG2>
-__global__ void __launch_bounds__(kNT) k_fwd64_cols(const float2 *__restrict__ z, int lgM, double2 *__restrict__ E) {
-    constexpr int L = 1 << LG2, S = seqs64<LG2>();
+template <int LG2, bool SMALL>
+__global__ void __launch_bounds__(threads64<LG2, SMALL>())
+    k_fwd64_cols(const float2 *__restrict__ z, int lgM, double2 *__restrict__ E) {
+    constexpr int L = 1 << LG2, S = seqs64<LG2, SMALL>(), NT = threads64<LG2, SMALL>();
     extern __shared__ double2 sm64[];
     const int lgM1 = lgM - LG2;
     const int64_t M1 = (int64_t)1 << lgM1;
     const int lgca = lgM1 < cx_log2(S) ? lgM1 : cx_log2(S);
     const int ca = 1 << lgca;
     const int64_t n1_0 = (int64_t)blockIdx.x * ca;
-    for (int e = threadIdx.x; e < ca * L; e += kNT) {   // consecutive threads: consecutive columns
+    for (int e = threadIdx.x; e < ca * L; e += NT) {   // consecutive threads: consecutive columns
         const int c = e & (ca - 1), n2 = e >> lgca;
         const float2 v = z[n1_0 + c + n2 * M1];
         sm64[c * L + n2] = make_double2((double)v.x, (double)v.y);
     }
     __syncthreads();
-    smem_dft64<LG2, S, kNT>(sm64);   // sequences ca .. S-1 (if any) hold no data and are not stored
-    for (int e = threadIdx.x; e < ca * L; e += kNT) {
+    smem_dft64<LG2, S, NT>(sm64);   // sequences ca .. S-1 (if any) hold no data and are not stored
+    for (int e = threadIdx.x; e < ca * L; e += NT) {
         const int c = e & (ca - 1), k2 = e >> lgca;
         const int64_t n1 = n1_0 + c;
         E[(int64_t)k2 * M1 + n1] = dmul(sm64[c * L + k2], root64(n1 * k2, lgM));
@@ -182,17 +191,17 @@ __global__ void __launch_bounds__(kNT) k_fwd64_cols(const float2 *__restrict__ z
 }
 
 // pass B: rows k2 of E (M1 = 2^LG1 points each, contiguous), cb = min(seqs64, M2) per CTA, in place
-template <int LG1>
-__global__ void __launch_bounds__(kNT) k_fwd64_rows(double2 *__restrict__ E, int lgM) {
-    constexpr int L = 1 << LG1, S = seqs64<LG1>();
+template <int LG1, bool SMALL>
+__global__ void __launch_bounds__(threads64<LG1, SMALL>()) k_fwd64_rows(double2 *__restrict__ E, int lgM) {
+    constexpr int L = 1 << LG1, S = seqs64<LG1, SMALL>(), NT = threads64<LG1, SMALL>();
     extern __shared__ double2 sm64[];
     const int64_t M2 = (int64_t)1 << (lgM - LG1);
     const int cb = M2 < S ? (int)M2 : S;
     double2 *row = E + (int64_t)blockIdx.x * cb * L;
-    for (int e = threadIdx.x; e < cb * L; e += kNT) sm64[e] = row[e];
+    for (int e = threadIdx.x; e < cb * L; e += NT) sm64[e] = row[e];
     __syncthreads();
-    smem_dft64<LG1, S, kNT>(sm64);
-    for (int e = threadIdx.x; e < cb * L; e += kNT) row[e] = sm64[e];
+    smem_dft64<LG1, S, NT>(sm64);
+    for (int e = threadIdx.x; e < cb * L; e += NT) row[e] = sm64[e];
 }
 
 // X_k, k = 0 .. M, from Z (Z_k at E[(k mod M2) M1 + k div M2]); a thread forms
@@ -229,52 +238,54 @@ __global__ void k_fwd64_split(const double2 *__restrict__ Z, int lgM, const floa
     }
 }
 
-template <int LG>
-constexpr size_t smem64_bytes() { return (size_t)seqs64<LG>() * (1 << LG) * sizeof(double2); }
+template <int LG, bool SMALL>
+constexpr size_t smem64_bytes() { return (size_t)seqs64<LG, SMALL>() * (1 << LG) * sizeof(double2); }
 
-template <int LG2>
+template <int LG2, bool SMALL>
 cudaError_t launch_cols(const float2 *z, int lgM, double2 *E, cudaStream_t st, bool attrs) {
     if (attrs)
-        return cudaFuncSetAttribute(k_fwd64_cols<LG2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem64_bytes<LG2>());
+        return cudaFuncSetAttribute(k_fwd64_cols<LG2, SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)smem64_bytes<LG2, SMALL>());
     const int64_t M1 = (int64_t)1 << (lgM - LG2);
-    const int64_t ca = std::min<int64_t>(M1, seqs64<LG2>());
-    k_fwd64_cols<LG2><<<(unsigned)(M1 / ca), kNT, smem64_bytes<LG2>(), st>>>(z, lgM, E);
+    const int64_t ca = std::min<int64_t>(M1, seqs64<LG2, SMALL>());
+    k_fwd64_cols<LG2, SMALL>
+        <<<(unsigned)(M1 / ca), threads64<LG2, SMALL>(), smem64_bytes<LG2, SMALL>(), st>>>(z, lgM, E);
     return cudaGetLastError();
 }
-template <int LG1>
+template <int LG1, bool SMALL>
 cudaError_t launch_rows(double2 *E, int lgM, cudaStream_t st, bool attrs) {
     if (attrs)
-        return cudaFuncSetAttribute(k_fwd64_rows<LG1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem64_bytes<LG1>());
+        return cudaFuncSetAttribute(k_fwd64_rows<LG1, SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)smem64_bytes<LG1, SMALL>());
     const int64_t M2 = (int64_t)1 << (lgM - LG1);
-    const int64_t cb = std::min<int64_t>(M2, seqs64<LG1>());
-    k_fwd64_rows<LG1><<<(unsigned)(M2 / cb), kNT, smem64_bytes<LG1>(), st>>>(E, lgM);
+    const int64_t cb = std::min<int64_t>(M2, seqs64<LG1, SMALL>());
+    k_fwd64_rows<LG1, SMALL><<<(unsigned)(M2 / cb), threads64<LG1, SMALL>(), smem64_bytes<LG1, SMALL>(), st>>>(E, lgM);
     return cudaGetLastError();
 }
 
-// M = 2^lgM, lgM = 9 .. 21: column length 2^(lgM/2), row length 2^(lgM - lgM/2)
+// M = 2^lgM, lgM = 9 .. 21: column length 2^(lgM/2), row length 2^(lgM - lgM/2);
+// the SMALL kernels up to M = 2^16 (lengths 2^4 .. 2^8)
 cudaError_t fwd64_passes(const float2 *z, int lgM, double2 *E, cudaStream_t st, bool attrs) {
     cudaError_t e = cudaSuccess;
     switch (lgM / 2) {
-        case 4: e = launch_cols<4>(z, lgM, E, st, attrs); break;
-        case 5: e = launch_cols<5>(z, lgM, E, st, attrs); break;
-        case 6: e = launch_cols<6>(z, lgM, E, st, attrs); break;
-        case 7: e = launch_cols<7>(z, lgM, E, st, attrs); break;
-        case 8: e = launch_cols<8>(z, lgM, E, st, attrs); break;
-        case 9: e = launch_cols<9>(z, lgM, E, st, attrs); break;
-        case 10: e = launch_cols<10>(z, lgM, E, st, attrs); break;
+        case 4: e = launch_cols<4, true>(z, lgM, E, st, attrs); break;
+        case 5: e = launch_cols<5, true>(z, lgM, E, st, attrs); break;
+        case 6: e = launch_cols<6, true>(z, lgM, E, st, attrs); break;
+        case 7: e = launch_cols<7, true>(z, lgM, E, st, attrs); break;
+        case 8: e = lgM <= 16 ? launch_cols<8, true>(z, lgM, E, st, attrs) : launch_cols<8, false>(z, lgM, E, st, attrs); break;
+        case 9: e = launch_cols<9, false>(z, lgM, E, st, attrs); break;
+        case 10: e = launch_cols<10, false>(z, lgM, E, st, attrs); break;
         default: return cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;
     switch (lgM - lgM / 2) {
-        case 5: return launch_rows<5>(E, lgM, st, attrs);
-        case 6: return launch_rows<6>(E, lgM, st, attrs);
-        case 7: return launch_rows<7>(E, lgM, st, attrs);
-        case 8: return launch_rows<8>(E, lgM, st, attrs);
-        case 9: return launch_rows<9>(E, lgM, st, attrs);
-        case 10: return launch_rows<10>(E, lgM, st, attrs);
-        case 11: return launch_rows<11>(E, lgM, st, attrs);
+        case 5: return launch_rows<5, true>(E, lgM, st, attrs);
+        case 6: return launch_rows<6, true>(E, lgM, st, attrs);
+        case 7: return launch_rows<7, true>(E, lgM, st, attrs);
+        case 8: return launch_rows<8, true>(E, lgM, st, attrs);
+        case 9: return launch_rows<9, false>(E, lgM, st, attrs);
+        case 10: return launch_rows<10, false>(E, lgM, st, attrs);
+        case 11: return launch_rows<11, false>(E, lgM, st, attrs);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -294,10 +305,11 @@ cudaError_t launch_forward_fft64(const float *s, int64_t N, void *scratch, const
     cudaError_t e = fwd64_passes(reinterpret_cast<const float2 *>(s), lgM, E, st, false);
     if (e != cudaSuccess) return e;
     const int64_t M = N / 2;
-    int blocks = (int)((M / 2 + 1 + 255) / 256);
+    const int threads = lgM <= 16 ? 64 : 256;   // short transforms: more SMs
+    int blocks = (int)((M / 2 + 1 + threads - 1) / threads);
     if (blocks > 4096) blocks = 4096;
-    if (fac) k_fwd64_split<true><<<blocks, 256, 0, st>>>(E, lgM, fac, out);
-    else k_fwd64_split<false><<<blocks, 256, 0, st>>>(E, lgM, nullptr, out);
+    if (fac) k_fwd64_split<true><<<blocks, threads, 0, st>>>(E, lgM, fac, out);
+    else k_fwd64_split<false><<<blocks, threads, 0, st>>>(E, lgM, nullptr, out);
     return cudaGetLastError();
 }
 
