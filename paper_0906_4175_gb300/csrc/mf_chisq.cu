@@ -36,24 +36,17 @@ __global__ void k_chisq_units(SegDev seg, const UnitInfo *__restrict__ all, int 
     }
     const int64_t lo = full.k_lo, hi = full.k_hi;
     const double P0 = seg.P[lo], Q = seg.P[hi] - P0;
-    for (int l = threadIdx.x; l <= p; l += blockDim.x) {
-        int64_t e;
-        if (l == 0) {
-            e = lo;
-        } else if (l == p) {
-            e = hi;
-        } else {
+    const int lane = threadIdx.x & 31;
+    for (int l = threadIdx.x >> 5; l <= p; l += blockDim.x >> 5) {   // one warp per edge, 32 probes a step
+        int64_t a = l == p ? hi : lo;
+        if (l > 0 && l < p) {
             const double target = ((double)l / (double)p) * Q;
-            int64_t a = lo, c = hi;   // smallest k in [a, c] with P[k] - P0 >= target
-            while (a < c) {
-                const int64_t m = a + ((c - a) >> 1);
-                if (seg.P[m] - P0 >= target) c = m;
-                else a = m + 1;
-            }
-            e = a;
+            a = edge_search(seg.P, P0, target, lo, hi, lane);
         }
-        b[l] = e;
-        if (edges) edges[(int64_t)u * (p + 1) + l] = e;
+        if (lane == 0) {
+            b[l] = a;
+            if (edges) edges[(int64_t)u * (p + 1) + l] = a;
+        }
     }
     __syncthreads();
     for (int l = threadIdx.x; l <= p; l += blockDim.x) {
@@ -359,7 +352,7 @@ struct ChiTilesOp {
 cudaError_t launch_chisq_units(const SegDev &seg, const UnitInfo *all, int n_t, const int32_t *tmpl, int n, int p,
                                UnitInfo *out, int64_t *edges, cudaStream_t st) {
     if (p < 1 || p > kChisqMaxBands) return cudaErrorInvalidValue;
-    k_chisq_units<<<n, 128, 0, st>>>(seg, all, n_t, tmpl, n, p, out, edges);
+    k_chisq_units<<<n, p >= 8 ? 256 : 128, 0, st>>>(seg, all, n_t, tmpl, n, p, out, edges);
     return cudaGetLastError();
 }
 

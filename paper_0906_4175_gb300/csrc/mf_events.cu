@@ -431,24 +431,9 @@ __device__ void cp_row_edges(const SegDev &seg, int p, int64_t r0, int64_t r1, C
     const double P0 = seg.P[lo], Q = seg.P[hi] - P0, C0 = seg.P[r0] - P0, C1 = seg.P[r1] - P0;
     for (int l = 1 + (threadIdx.x >> 5); l < p; l += kCpWarps) {
         const double target = ((double)l / (double)p) * Q;
-        int64_t a = r0, c = r1;   // P[c] reaches the target (or the edge is beyond r1)
-        if (C0 >= target) c = r0;
-        else if (C1 < target) a = r1;
-        while (a < c) {
-            const int64_t step = (c - a + 31) / 32;
-            const int64_t k = a + lane * step;
-            const bool reach = k < c && seg.P[k] - P0 >= target;
-            const unsigned m = __ballot_sync(0xffffffffu, reach);
-            const int first = m ? __ffs(m) - 1 : 32;   // P does not decrease: the first probe that reaches it
-            if (first < 32) {
-                const int64_t top = a + first * step;
-                a = first == 0 ? top : top - step + 1;
-                c = top;
-            } else {   // none of the probes below c: past the last one
-                const int64_t last = a + ((c - 1 - a) / step) * step;
-                a = last + 1;
-            }
-        }
+        int64_t a = r0;
+        if (C1 < target) a = r1;
+        else if (C0 < target) a = edge_search(seg.P, P0, target, r0, r1, lane);
         if (lane == 0) r.b[l] = a;
     }
 }

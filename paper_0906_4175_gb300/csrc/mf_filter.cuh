@@ -40,6 +40,26 @@ __device__ __forceinline__ void anchor_record(double c1, double c2, double c3, d
     rec4 = S4 * ik2 * ik2 * (1.f / 1944.f);
 }
 
+// Smallest k in [a, c] with P[k] - P0 >= target, or c (P does not decrease), by
+// one warp: 32 probes a step, so four dependent loads for 2^19 bins instead of
+// twenty.  All lanes call it with the same arguments and get the result.
+__device__ __forceinline__ int64_t edge_search(const double *P, double P0, double target, int64_t a, int64_t c, int lane) {
+    while (a < c) {
+        const int64_t step = (c - a + 31) / 32;
+        const int64_t k = a + lane * step;
+        const bool reach = k < c && P[k] - P0 >= target;
+        const unsigned m = __ballot_sync(0xffffffffu, reach);
+        if (m) {   // the first probe that reaches it
+            const int first = __ffs(m) - 1;
+            c = a + first * step;
+            if (first > 0) a = c - step + 1;
+        } else {   // none of the probes below c: past the last one
+            a += ((c - 1 - a) / step) * step + 1;
+        }
+    }
+    return a;
+}
+
 // ---------------------------------------------------------------------------
 // pass-1 source: X_k = W_k e^{-i Psi_k} on the band, 0 elsewhere; k >= N/2 is
 // always outside (one-sided spectrum), so the upper half of every column is 0.
@@ -110,7 +130,7 @@ struct TemplateSrc {
             for (int r = 0; r < 16; ++r) {
                 const int n = t + r * T;
                 float2 x = czero();
-                if (in[r]) {
+                if (__any_sync(0xffffffffu, in[r])) {   // rows outside the band of the whole warp cost nothing
                     const float4 a = sa[n];
                     const float a4 = sa4[n];
                     float ph = fmaf(fmaf(fmaf(fmaf(a4, d, a.w), d, a.z), d, a.y), d, a.x);
@@ -119,13 +139,17 @@ struct TemplateSrc {
                     __sincosf(6.283185307179586f * ph, &sn, &cs);
                     x = make_float2(fmaf(w[r].x, cs, w[r].y * sn), fmaf(w[r].y, cs, -w[r].x * sn));  // W e^{-i 2 pi ph}
                 }
-                v[r] = x;
+                v[r] = in[r] ? x : czero();
             }
         } else {
             release_hook(rel);
             const int half = D >> 1;
 #pragma unroll
             for (int r = 0; r < 16; ++r) {
+                if (!__any_sync(0xffffffffu, in[r])) {
+                    v[r] = czero();
+                    continue;
+                }
                 const int k = k0 + ((r * T) << LG1);
                 const int kk = in[r] ? k : u.k_lo;
                 const int g = kk >> p.log2D;
@@ -269,6 +293,10 @@ struct TemplateSrc64 {
         const int d0 = (k1 & (D - 1)) - (D >> 1);   // the same on every row when D divides N1
 #pragma unroll
         for (int r = 0; r < 16; ++r) {
+            if (!__any_sync(0xffffffffu, in[r])) {
+                v[r] = czero();
+                continue;
+            }
             float4 a0, a1, a2;
             int d = d0;
             if (shared_row) {
