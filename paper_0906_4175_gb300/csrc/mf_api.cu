@@ -293,7 +293,7 @@ struct mf_bank_s {
     // order) puts the widest bands first for every segment.  pos is the inverse.
     std::vector<int> order, pos;
     int *d_order = nullptr;
-    double B1 = 0.0, B4 = 0.0, B5 = 0.0, B7 = 0.0, fisco_min = 0.0;   // phase-derivative bounds at f_low
+    double B1 = 0.0, B4 = 0.0, B5 = 0.0, B8 = 0.0, fisco_min = 0.0;   // phase-derivative bounds at f_low
     int device = 0;
     Workspace ws;
     bool prof_on = false;
@@ -426,7 +426,7 @@ static int bank_create_range(const double *m1, const double *m2, int64_t n, cons
     int r0 = ensure_device_init();
     if (r0) return r0;
     std::vector<double> rec((size_t)count * kTmplStride);
-    double B1 = 0.0, B4 = 0.0, B5 = 0.0, B7 = 0.0, fmin = INFINITY;
+    double B1 = 0.0, B4 = 0.0, B5 = 0.0, B8 = 0.0, fmin = INFINITY;
     for (int64_t i = 0; i < n; ++i) {
         if (!(m1[i] > 0.0) || !(m2[i] > 0.0) || !isfinite(m1[i]) || !isfinite(m2[i]))
             return set_err(MF_EINVAL, "template %lld: masses must be finite and > 0", (long long)i);
@@ -438,7 +438,7 @@ static int bank_create_range(const double *m1, const double *m2, int64_t n, cons
         B5 = std::max(B5, psi_deriv_bound(r, p.f_low, 5));
         if (p.phase_mode == MF_PHASE_FP64) {
             B4 = std::max(B4, psi_deriv_bound(r, p.f_low, 4));
-            B7 = std::max(B7, psi_deriv_bound(r, p.f_low, 7));
+            B8 = std::max(B8, psi_deriv_bound(r, p.f_low, 8));
         }
         if (mine) fmin = std::min(fmin, r[TF_FISCO]);
     }
@@ -450,7 +450,7 @@ static int bank_create_range(const double *m1, const double *m2, int64_t n, cons
     b->B1 = B1;
     b->B4 = B4;
     b->B5 = B5;
-    b->B7 = B7;
+    b->B8 = B8;
     b->fisco_min = fmin;
     b->fisco.resize((size_t)n);
     for (int64_t i = 0; i < n; ++i) b->fisco[(size_t)i] = rec[(size_t)i * kTmplStride + TF_FISCO];
@@ -708,7 +708,7 @@ static SegDev seg_dev(const mf_segment_s *g, int log2N2 = -1) {
 // the Taylor sum), both bounded at f_low over the whole bank (k-derivatives are
 // f-derivatives times df^n).  MF_PHASE_FP64 has its own rule (anchor_log2D64).
 static int choose_log2D(const mf_bank_s *b, const mf_segment_s *g) {
-    if (b->params.phase_mode == MF_PHASE_FP64) return anchor_log2D64(b->B4, b->B7, g->fs / (double)g->N);
+    if (b->params.phase_mode == MF_PHASE_FP64) return anchor_log2D64(b->B4, b->B8, g->fs / (double)g->N);
     return anchor_log2D(b->B1, b->B5, g->fs / (double)g->N);
 }
 

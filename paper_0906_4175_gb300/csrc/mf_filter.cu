@@ -92,7 +92,7 @@ __global__ void k_anchors64(SegDev seg, const double *__restrict__ tmpl, const U
         auto hi = [](unsigned long long x) { return __int_as_float((int)(unsigned)(x >> 32)); };
         out[a] = make_float4(lo(r.r0), hi(r.r0), lo(r.q1), hi(r.q1));
         out[a + max_anc] = make_float4(lo(r.q2), hi(r.q2), lo(r.q3), hi(r.q3));
-        out[a + 2 * (int64_t)max_anc] = make_float4(r.q4, r.q5, r.q6, 0.f);
+        out[a + 2 * (int64_t)max_anc] = make_float4(r.q4, r.q5, r.q6, r.q7);
     }
 }
 

@@ -176,16 +176,16 @@ struct TemplateSrc {
 // 1714 us for 250 templates at N = 2^18.  Between FP64 anchors the phase is
 // instead summed in turns mod 1 as 64-bit fixed point: with the integer offset
 // d from the anchor centre,
-//   psi = r0 + d (q1 + d (q2 + d q3))  (mod 1, exact in 2^-64 turns)  +  d^4 (q4 + d (q5 + d q6))
+//   psi = r0 + d (q1 + d (q2 + d q3))  (mod 1, exact in 2^-64 turns)  +  d^4 (q4 + d (q5 + d (q6 + d q7)))
 // where the cubic part is three 64-bit integer multiply-adds (d is an integer,
 // so the coefficients count mod 1) and the small rest FP32.  anchor_log2D64
 // bounds what is left out and the size of the FP32 part, so that psi is good
 // to 4e-10 turns before it is rounded to FP32 (1.5e-8, as before) for the sincos.
-// Record: three planes of 16 bytes (r0, q1 | q2, q3 | q4, q5, q6, -).
+// Record: three planes of 16 bytes (r0, q1 | q2, q3 | q4, q5, q6, q7).
 // ---------------------------------------------------------------------------
 struct Anchor64 {
     unsigned long long r0, q1, q2, q3;
-    float q4, q5, q6;
+    float q4, q5, q6, q7;
 };
 // x mod 1 in 2^-64 turns: the sum with 1.5 * 2^(52 - 30) leaves x in units of
 // 2^-30 in the mantissa, and the rest of x is exact (a conversion from FP64 to
@@ -223,6 +223,8 @@ __device__ __forceinline__ Anchor64 anchor_record64(double c1, double c2, double
     a.q4 = (280.f * w1 + 880.f * w2 + 1944.f * w3 + 6160.f * w5) * ik4 * (1.f / 1944.f);
     a.q5 = -(3640.f * w1 + 12320.f * w2 + 29160.f * w3 + 104720.f * w5) * ik4 * ikf * (1.f / 29160.f);
     a.q6 = (58240.f * w1 + 209440.f * w2 + 524880.f * w3 + 2094400.f * w5) * ik4 * (ikf * ikf) * (1.f / 524880.f);
+    a.q7 = -(1106560.f * w1 + 4188800.f * w2 + 11022480.f * w3 + 48171200.f * w5) * ik4 * (ikf * ikf * ikf) *
+           (1.f / 11022480.f);
     return a;
 }
 // phase in turns at integer offset d, d4 = d^4
@@ -234,7 +236,7 @@ __device__ __forceinline__ float anchor_phase64(const float4 &p0, const float4 &
     const unsigned long long dd = (unsigned long long)(long long)d;
     const unsigned long long t =
         word(p0.x, p0.y) + dd * (word(p0.z, p0.w) + dd * (word(p1.x, p1.y) + dd * word(p1.z, p1.w)));
-    const float tail = d4 * fmaf(df, fmaf(df, p2.z, p2.y), p2.x);
+    const float tail = d4 * fmaf(df, fmaf(df, fmaf(df, p2.w, p2.z), p2.y), p2.x);
     // |tail| < 2^-10: added to 1.5 * 2^-9 its mantissa counts 2^-32 turns
     const int hi = (int)(t >> 32) + (__float_as_int(tail + 0.0029296875f) - 0x3b400000);
     return (float)hi * 2.3283064365386963e-10f;   // 2^-32: in [-1/2, 1/2], rounded once

@@ -97,15 +97,15 @@ __host__ __device__ inline int anchor_log2D(double B1, double B5, double df) {
     return lg;
 }
 
-// The same for MF_PHASE_FP64 (fixed-point cubic part, FP32 terms 4..6): the
-// seventh-order remainder B7 df^7 (D/2)^7 / 5040 stays <= 5e-11 turns and the
+// The same for MF_PHASE_FP64 (fixed-point cubic part, FP32 terms 4..7): the
+// eighth-order remainder B8 df^8 (D/2)^8 / 40320 stays <= 5e-11 turns and the
 // FP32 part, dominated by B4 df^4 (D/2)^4 / 24, <= 2^-11 turns (it is summed in
 // units of 2^-32 turns and must stay below 2^-10).
-__host__ __device__ inline int anchor_log2D64(double B4, double B7, double df) {
+__host__ __device__ inline int anchor_log2D64(double B4, double B8, double df) {
     int lg = 0;
     while (lg < 8) {
-        const double h = df * (double)(1 << (lg + 1)) / 2.0;
-        if (B7 * h * h * h * h * h * h * h / 5040.0 > 5e-11 || B4 * h * h * h * h / 24.0 > 1.0 / 2048.0) break;
+        const double h = df * (double)(1 << (lg + 1)) / 2.0, h2 = h * h, h4 = h2 * h2;
+        if (B8 * h4 * h4 / 40320.0 > 5e-11 || B4 * h4 / 24.0 > 1.0 / 2048.0) break;
         ++lg;
     }
     return lg;
