@@ -946,7 +946,6 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
     int rc = ensure_workspace(b, exch_elems, trig_cap, anc_elems, nblk, capturing);
     if (rc) return rc;
     Workspace &w = b->ws;
-    MF_CUDA(cudaMemsetAsync(w.fctl, 0, sizeof(FilterCtl), st));
     const int n_t = (int)b->n;
     // descending-cost unit order (MFGB_UNIT_ORDER=bank keeps bank order); the
     // stall hook names a template, the kernels see its unit position
@@ -980,8 +979,17 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
                 anc_bytes[(size_t)t] = anchors ? 16.0 * (double)(((hi - 1) >> lgD) - (lo >> lgD) + 1) : 0.0;
             }
         }
+        // the first kernel of the call zeroes the control words; a small bank's
+        // units and anchors come from one launch (stage profiling keeps two)
+        FilterCtl *clear = s == 0 ? w.fctl : nullptr;
+        const bool merged = !b->prof_on && !use_persistent(b, segs[s]) && seg_batch[(size_t)s] >= n_t &&
+                            units_anchors_applies(n_t, man, b->params.phase_mode, sm_count());
         int pi = prof_begin(b, MF_STAGE_SETUP, 48.0 * n_t, st);
-        MF_CUDA(launch_units(sd, b->d_tmpl, n_t, b->params.f_low, threshold, lgD, unit_order, w.units, st));
+        if (merged)
+            MF_CUDA(launch_units_anchors(sd, b->d_tmpl, n_t, b->params.f_low, threshold, lgD, unit_order, w.units, man,
+                                         w.anchors, w.anchors4, clear, sm_count(), st));
+        else
+            MF_CUDA(launch_units(sd, b->d_tmpl, n_t, b->params.f_low, threshold, lgD, unit_order, w.units, clear, st));
         prof_end(b, pi, st);
         count_launches(1);
         if (use_fused(b, segs[s])) {
@@ -991,10 +999,12 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
                     by_band += band_bytes[(size_t)t];
                     by_anc += anc_bytes[(size_t)t];
                 }
-            pi = prof_begin(b, MF_STAGE_ANCHORS, by_anc, st);
-            MF_CUDA(launch_anchors(sd, b->d_tmpl, w.units, 0, n_t, lgD, man, w.anchors, w.anchors4,
-                                   b->params.phase_mode, st));
-            prof_end(b, pi, st);
+            if (!merged) {
+                pi = prof_begin(b, MF_STAGE_ANCHORS, by_anc, st);
+                MF_CUDA(launch_anchors(sd, b->d_tmpl, w.units, 0, n_t, lgD, man, w.anchors, w.anchors4,
+                                       b->params.phase_mode, st));
+                prof_end(b, pi, st);
+            }
             MF_CUDA(cudaMemsetAsync(w.ctl, 0, sizeof(unsigned) * (4 + 2 * (size_t)n_t), st));
             double split = b->split > 0.0 ? b->split : kSplit;
             if (const char *e = getenv("MFGB_SPLIT")) split = atof(e);
@@ -1006,7 +1016,7 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
             pi = prof_begin(b, MF_STAGE_FINAL, 16.0 * nbk * n_t, st);
             MF_CUDA(launch_reduce_peaks(sd, w.units, n_t, w.partials, nbk, s, n_seg, peaks, st));
             prof_end(b, pi, st);
-            count_launches(3);
+            count_launches(merged ? 2 : 3);
             continue;
         }
         PersistParams P;
@@ -1105,7 +1115,7 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
                     by_anc += anc_bytes[t];
                 }
             const double exch_bytes = 8.0 * (double)sd.N * nb;
-            if (anchors && (!overlap || bi == 0)) {
+            if (anchors && !merged && (!overlap || bi == 0)) {
                 pi = prof_begin(b, MF_STAGE_ANCHORS, by_anc, st);
                 MF_CUDA(launch_anchors(sd, b->d_tmpl, w.units, u0, nb, lgD, man, w.anchors + aoff, w.anchors4 + aoff,
                                        b->params.phase_mode, st));
@@ -1249,7 +1259,7 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
     float *anc4 = sc.at<float>(o_anc4);
     float2 *exch = sc.at<float2>(o_exch);
     int launches = 0;
-    if (e == cudaSuccess) e = launch_units(sd, b->d_tmpl, n_t, b->params.f_low, 0.f, lgD, nullptr, all, st);
+    if (e == cudaSuccess) e = launch_units(sd, b->d_tmpl, n_t, b->params.f_low, 0.f, lgD, nullptr, all, nullptr, st);
     if (e == cudaSuccess) e = launch_chisq_units(sd, all, n_t, tmpl, (int)n, p, units, edges, st);
     launches += 2;
     const UnitInfo *full = units + (size_t)p * n;

@@ -22,13 +22,8 @@ namespace mf {
 // ---------------------------------------------------------------------------
 // per-unit set-up
 // ---------------------------------------------------------------------------
-// Unit i of a segment is template order[i] (bank order when order is NULL).
-__global__ void k_units(SegDev seg, const double *__restrict__ tmpl, int n_t, double f_low, float thr,
-                        int log2D, const int *__restrict__ order, UnitInfo *__restrict__ units) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_t) return;
-    const int t = order ? order[i] : i;
-    const double *T = tmpl + (int64_t)t * kTmplStride;
+// Unit of template t: band, scale factors, threshold, anchor range.
+__device__ UnitInfo unit_info(const SegDev &seg, const double *T, int t, double f_low, float thr, int log2D) {
     const double N = (double)seg.N, fs = seg.fs;
     const double fisco = T[TF_FISCO];
     const double fc = fisco < 0.5 * fs ? fisco : 0.5 * fs;
@@ -49,20 +44,32 @@ __global__ void k_units(SegDev seg, const double *__restrict__ tmpl, int n_t, do
     u.thr2 = (float)(th * th);
     u.z_scale = (float)(4.0 * seg.df * T[TF_AMP] / seg.consts->alpha);
     u.tmpl = t;
-    units[i] = u;
+    return u;
 }
 
-__global__ void k_anchors(SegDev seg, const double *__restrict__ tmpl, const UnitInfo *__restrict__ units,
-                          int unit0, int log2D, int max_anc, float4 *__restrict__ anchors,
-                          float *__restrict__ anchors4, int reps) {
-    const int b = blockIdx.y;
-    const UnitInfo u = units[unit0 + b];
-    const double *T = tmpl + (int64_t)u.tmpl * kTmplStride;
+// the call's control words, zeroed by the first kernel of the call (one block
+// of it calls this; a memset would be one more launch)
+__device__ __forceinline__ void clear_ctl(FilterCtl *ctl) {
+    unsigned *w = reinterpret_cast<unsigned *>(ctl);
+    for (unsigned i = threadIdx.x; i < sizeof(FilterCtl) / 4; i += blockDim.x) w[i] = 0u;
+}
+
+// Unit i of a segment is template order[i] (bank order when order is NULL).
+__global__ void k_units(SegDev seg, const double *__restrict__ tmpl, int n_t, double f_low, float thr,
+                        int log2D, const int *__restrict__ order, UnitInfo *__restrict__ units, FilterCtl *clear) {
+    if (clear && blockIdx.x == 0) clear_ctl(clear);
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n_t) return;
+    const int t = order ? order[i] : i;
+    units[i] = unit_info(seg, tmpl + (int64_t)t * kTmplStride, t, f_low, thr, log2D);
+}
+
+// the anchor records of one unit, blocks bx of nbx
+__device__ __forceinline__ void unit_anchors(const SegDev &seg, const double *T, const UnitInfo &u, int log2D,
+                                             int max_anc, float4 *out, float *out4, int reps, int64_t rep_stride,
+                                             int bx, int nbx) {
     const double c1 = T[TF_C1], c2 = T[TF_C2], c3 = T[TF_C3], c5 = T[TF_C5];
-    float4 *out = anchors + (int64_t)b * max_anc;
-    float *out4 = anchors4 + (int64_t)b * max_anc;
-    const int64_t rep_stride = (int64_t)gridDim.y * max_anc;   // copy k of slot b is slot b + k n_units
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < u.n_anc; i += gridDim.x * blockDim.x) {
+    for (int i = bx * blockDim.x + threadIdx.x; i < u.n_anc; i += nbx * blockDim.x) {
         float4 r;
         float r4;
         const int64_t g = (int64_t)u.g_lo + i;
@@ -74,6 +81,35 @@ __global__ void k_anchors(SegDev seg, const double *__restrict__ tmpl, const Uni
             out4[a + k * rep_stride] = r4;
         }
     }
+}
+
+__global__ void k_anchors(SegDev seg, const double *__restrict__ tmpl, const UnitInfo *__restrict__ units,
+                          int unit0, int log2D, int max_anc, float4 *__restrict__ anchors,
+                          float *__restrict__ anchors4, int reps) {
+    const int b = blockIdx.y;
+    const UnitInfo u = units[unit0 + b];
+    unit_anchors(seg, tmpl + (int64_t)u.tmpl * kTmplStride, u, log2D, max_anc, anchors + (int64_t)b * max_anc,
+                 anchors4 + (int64_t)b * max_anc, reps, (int64_t)gridDim.y * max_anc,   // copy k of slot b: slot b + k n_units
+                 blockIdx.x, gridDim.x);
+}
+
+// k_units and k_anchors of a small bank in one launch: every block of a unit
+// forms its UnitInfo anew (some 60 FP64 operations of one thread), which pays
+// while all blocks are resident at once: two launches of 4 and 7 us, 8 us here.
+__global__ void k_units_anchors(SegDev seg, const double *__restrict__ tmpl, double f_low, float thr, int log2D,
+                                const int *__restrict__ order, UnitInfo *__restrict__ units, int max_anc,
+                                float4 *__restrict__ anchors, float *__restrict__ anchors4, FilterCtl *clear) {
+    __shared__ UnitInfo su;
+    const int b = blockIdx.y, t = order ? order[b] : b;
+    const double *T = tmpl + (int64_t)t * kTmplStride;
+    if (clear && blockIdx.x == 0 && b == 0) clear_ctl(clear);
+    if (threadIdx.x == 0) {
+        su = unit_info(seg, T, t, f_low, thr, log2D);
+        if (blockIdx.x == 0) units[b] = su;
+    }
+    __syncthreads();
+    unit_anchors(seg, T, su, log2D, max_anc, anchors + (int64_t)b * max_anc, anchors4 + (int64_t)b * max_anc, 1, 0,
+                 blockIdx.x, gridDim.x);
 }
 
 __global__ void k_anchors64(SegDev seg, const double *__restrict__ tmpl, const UnitInfo *__restrict__ units, int unit0,
@@ -102,8 +138,30 @@ __global__ void k_anchors64(SegDev seg, const double *__restrict__ tmpl, const U
 MF_DEBUG_READER(dbg_read_filter)
 
 cudaError_t launch_units(const SegDev &seg, const double *tmpl, int n_t, double f_low, float thr, int log2D,
-                         const int *order, UnitInfo *units, cudaStream_t st) {
-    k_units<<<(n_t + 255) / 256, 256, 0, st>>>(seg, tmpl, n_t, f_low, thr, log2D, order, units);
+                         const int *order, UnitInfo *units, FilterCtl *clear, cudaStream_t st) {
+    k_units<<<(n_t + 255) / 256, 256, 0, st>>>(seg, tmpl, n_t, f_low, thr, log2D, order, units, clear);
+    return cudaGetLastError();
+}
+
+// Blocks per unit of the merged launch, or 0 where the two launches are better:
+// at most eight blocks of 256 threads per SM.
+static int units_anchors_blocks(int n_t, int max_anc, int n_sm) {
+    const int most = 8 * n_sm / (n_t > 0 ? n_t : 1);
+    const int want = (max_anc + 255) / 256;
+    return most < 1 ? 0 : (want < most ? want : most);
+}
+
+bool units_anchors_applies(int n_t, int max_anc, int phase_mode, int n_sm) {
+    return phase_mode == MF_PHASE_ANCHOR && units_anchors_blocks(n_t, max_anc, n_sm) > 0;
+}
+
+cudaError_t launch_units_anchors(const SegDev &seg, const double *tmpl, int n_t, double f_low, float thr, int log2D,
+                                 const int *order, UnitInfo *units, int max_anc, float4 *anchors, float *anchors4,
+                                 FilterCtl *clear, int n_sm, cudaStream_t st) {
+    const int gx = units_anchors_blocks(n_t, max_anc, n_sm);
+    if (gx < 1) return cudaErrorInvalidValue;
+    k_units_anchors<<<dim3(gx, n_t), 256, 0, st>>>(seg, tmpl, f_low, thr, log2D, order, units, max_anc, anchors,
+                                                   anchors4, clear);
     return cudaGetLastError();
 }
 

@@ -210,9 +210,16 @@ cudaError_t launch_inverse_real_fft(const float2 *Y, int64_t N, double scale, fl
                                     cudaStream_t st);
 
 // filter (mf_filter.cu)
-// units[i] <- template order[i] (order NULL: template i)
+// units[i] <- template order[i] (order NULL: template i); clear (may be NULL):
+// control words to zero
+struct FilterCtl;
 cudaError_t launch_units(const SegDev &seg, const double *tmpl, int n_t, double f_low, float thr,
-                         int log2D, const int *order, UnitInfo *units, cudaStream_t st);
+                         int log2D, const int *order, UnitInfo *units, FilterCtl *clear, cudaStream_t st);
+// units and the anchors of all of them in one launch (small banks, MF_PHASE_ANCHOR)
+bool units_anchors_applies(int n_t, int max_anc, int phase_mode, int n_sm);
+cudaError_t launch_units_anchors(const SegDev &seg, const double *tmpl, int n_t, double f_low, float thr, int log2D,
+                                 const int *order, UnitInfo *units, int max_anc, float4 *anchors, float *anchors4,
+                                 FilterCtl *clear, int n_sm, cudaStream_t st);
 cudaError_t launch_anchors(const SegDev &seg, const double *tmpl, const UnitInfo *units, int unit0,
                            int n_units, int log2D, int max_anc, float4 *anchors, float *anchors4, int phase_mode,
                            cudaStream_t st, int reps = 1);
