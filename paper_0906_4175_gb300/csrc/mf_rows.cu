@@ -181,6 +181,227 @@ __global__ void __launch_bounds__(kWarps * 32) k_peaks_rows(const float2 *__rest
 }
 
 // ---------------------------------------------------------------------------
+// Rows of L = 128, 256 and 512 points (N = 2^15 .. 2^18 and the 1024 x 512
+// split of 2^19): a warp takes 1024 / L consecutive rows at a time, L / 32 lanes
+// each, with the two-stage schedule of the per-tile kernel (bit-identical).  As
+// in k_pass2_rows the next rows are copied in under the last stage and no CTA
+// barrier separates the stages, which a CTA per tile of 8192 points pays three
+// times per tile.  The rows land, and are held between the stages, L + L/32
+// apart: a half-warp's L / 32 lanes of each row then meet different banks in
+// every access.  512-point rows, 250 templates at N = 2^18: 140 us per tile, 85
+// here.
+// ---------------------------------------------------------------------------
+template <int L>
+struct ShortRows {
+    static constexpr int T = L / 32, RPW = 1024 / L;   // lanes per row, rows per warp
+    static constexpr int RS = L + L / 32;              // row stride in the region, T (mod 16)
+    static constexpr int REGION = RPW * RS;
+    static constexpr size_t SMEM =
+        (size_t)kWarps * REGION * sizeof(float2) + (size_t)TwTable<L>::SIZE * sizeof(float2) + kWarps * sizeof(uint64_t);
+    static_assert(RS % 16 == T % 16 && RS % 2 == 0, "bank spread, 16-byte copies");
+};
+
+// the warp starts the copies of rows r .. r + RPW - 1 into its region (all lanes call it)
+template <int L>
+__device__ __forceinline__ void short_rows_copy(const RowsParams &p, int64_t r, float2 *region, uint64_t *bar) {
+    using R = ShortRows<L>;
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) mbar_expect_tx(bar, R::RPW * L * sizeof(float2));
+    __syncwarp();
+    if (lane < R::RPW) bulk_copy_g2s(region + lane * R::RS, row_src<L>(p, r + lane), L * sizeof(float2), bar);
+}
+
+template <int L, bool FULL>
+struct ShortRhoSink : GroupRhoSink<L, 1, FULL> {
+    using Base = GroupRhoSink<L, 1, FULL>;
+    int64_t next;   // first row of the warp's next group, or -1
+    __device__ ShortRhoSink(const RowsParams &pp, const UnitInfo &uu, int jj, float2 *rg, uint64_t *br, int64_t nx)
+        : Base(pp, uu, jj, rg, br, nullptr), next(nx) {}
+    __device__ __forceinline__ void after_loads() {
+        __syncwarp();
+        fence_proxy_async();
+        if (next >= 0) short_rows_copy<L>(this->p, next, this->region, this->bar);
+    }
+    // the row's partial, from its L / 32 lanes
+    __device__ __forceinline__ void finish_row(float4 *out) {
+        constexpr int T = L / 32;
+        if constexpr (!FULL) {
+#pragma unroll
+            for (int o = T / 2; o > 0; o >>= 1) this->bp = fmaxf(this->bp, __shfl_xor_sync(0xffffffffu, this->bp, o));
+            if ((threadIdx.x & (T - 1)) == 0) *out = make_float4(this->bp, __int_as_float(-1), 0.f, 0.f);
+        } else {
+#pragma unroll
+            for (int o = T / 2; o > 0; o >>= 1) {
+                const float op = __shfl_xor_sync(0xffffffffu, this->bp, o);
+                const int oj = __shfl_xor_sync(0xffffffffu, this->bj, o);
+                const float ox = __shfl_xor_sync(0xffffffffu, this->bz.x, o);
+                const float oy = __shfl_xor_sync(0xffffffffu, this->bz.y, o);
+                if (op > this->bp || (op == this->bp && oj < this->bj)) {
+                    this->bp = op;
+                    this->bj = oj;
+                    this->bz = make_float2(ox, oy);
+                }
+            }
+            if ((threadIdx.x & (T - 1)) == 0)
+                *out = make_float4(this->bp, __int_as_float(this->bj), this->bz.x, this->bz.y);
+        }
+    }
+};
+
+// stages of the warp's rows from the landed region; the sink gets outputs t + (L/32) q of its row
+template <int L, class Snk>
+__device__ __forceinline__ void short_rows_transform(float2 *region, const float2 *tw, Snk &snk) {
+    using R = ShortRows<L>;
+    const int lane = threadIdx.x & 31, t = lane & (R::T - 1);
+    float2 *sq = region + (lane / R::T) * R::RS;
+    float2 v[32];
+#pragma unroll
+    for (int q = 0; q < 32; ++q) v[q] = sq[t + R::T * q];
+    Dft<32, +1>::run(v);
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 32; ++q) sq[spad(32 * t + q)] = v[q];
+    __syncwarp();
+    stockham_stage<L, FftShape<L>::R1, 32, +1, true, Snk, GroupSync<1>>(sq, tw, 0, t, snk);
+}
+
+template <int L, bool FULL>
+__global__ void __launch_bounds__(kWarps * 32, 2) k_pass2_rows_short(RowsParams p) {
+    using R = ShortRows<L>;
+    static_assert(FftShape<L>::NST == 2, "two-stage row lengths");
+    extern __shared__ __align__(16) float2 rows_smem[];
+    float2 *tw = rows_smem + kWarps * R::REGION;
+    uint64_t *bars = reinterpret_cast<uint64_t *>(tw + TwTable<L>::SIZE);
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float2 *region = rows_smem + w * R::REGION;
+    fill_twiddles<L>(tw);
+    if (lane == 0) mbar_init(&bars[w], 1);
+    mbar_fence_init();
+    __syncthreads();
+    const int64_t total = (int64_t)p.n_units << p.log2N2;   // rows, a multiple of RPW per unit
+    const int64_t step = (int64_t)gridDim.x * kWarps * R::RPW;
+    int64_t r = ((int64_t)blockIdx.x * kWarps + w) * R::RPW;
+    if (r < total && !row_withheld(p, r)) short_rows_copy<L>(p, r, region, &bars[w]);
+    uint32_t parity = 0;
+    for (; r < total; r += step) {
+        long long it = 0;
+        bool ok = true;
+        while (!mbar_try_wait(&bars[w], parity)) {
+            if (++it > p.spin_limit) { ok = false; break; }
+        }
+        if (!__all_sync(0xffffffffu, ok)) {
+            if (lane == 0) atomicOr(p.status, 2);
+            return;   // the copies into this warp's region never completed; nothing else is in flight
+        }
+        parity ^= 1u;
+        const int slot = (int)(r >> p.log2N2);
+        const int j2 = (int)(r & (((int64_t)1 << p.log2N2) - 1)) + lane / R::T;
+        const int unit = p.unit0 + slot;
+        const UnitInfo u = p.units[unit];
+        const int64_t rn = r + step;
+        ShortRhoSink<L, FULL> snk(p, u, j2, region, &bars[w], rn < total && !row_withheld(p, rn) ? rn : -1);
+        short_rows_transform<L>(region, tw, snk);
+        if (MF_DBG(slot < p.n_units && j2 < (1 << p.log2N2), kDbgRows))
+            snk.finish_row(&p.partials[((int64_t)unit << p.log2N2) + j2]);
+    }
+}
+
+// k_peaks_rows for the short rows: a row that reaches the unit's maximum is
+// transformed again together with the other rows of its group.
+template <int L>
+__global__ void __launch_bounds__(kWarps * 32) k_peaks_rows_short(const float2 *__restrict__ exch,
+                                                                  const UnitInfo *__restrict__ units, int unit0,
+                                                                  int n_units, int n_all, int log2N, int log2N2,
+                                                                  const float4 *__restrict__ partials, int seg_idx,
+                                                                  int n_seg, mf_peak *__restrict__ peaks) {
+    using R = ShortRows<L>;
+    extern __shared__ __align__(16) float2 rows_smem[];
+    float2 *tw = rows_smem + kWarps * R::REGION;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, t = lane & (R::T - 1), sub = lane / R::T;
+    float2 *region = rows_smem + w * R::REGION;
+    fill_twiddles<L>(tw);
+    __syncthreads();
+    const int b = blockIdx.x * kWarps + w;   // unit within the batch
+    if (b >= n_units) return;
+    const int unit = unit0 + b;
+    const int n2 = 1 << log2N2;
+    const float4 *pp = partials + ((int64_t)unit << log2N2);
+    float M = -1.f;
+    for (int j2 = lane; j2 < n2; j2 += 32) M = fmaxf(M, pp[j2].x);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    int bj = 0x7fffffff;
+    float2 bz = make_float2(0.f, 0.f);
+    for (int r0 = 0; r0 < n2; r0 += 32) {   // n2 >= 32 rows, RPW divides 32
+        const unsigned cand = __ballot_sync(0xffffffffu, pp[r0 + lane].x == M);
+        for (int g = 0; g < 32 / R::RPW; ++g) {
+            const unsigned mine = (cand >> (g * R::RPW)) & ((1u << R::RPW) - 1u);
+            if (mine == 0u) continue;   // warp-uniform
+            const int j2 = r0 + g * R::RPW + sub;
+            if (!MF_DBG(b < n_units && (int64_t)(j2 + 1) * L <= ((int64_t)1 << log2N), kDbgRows)) continue;
+            const float2 *row = exch + ((int64_t)b << log2N) + (int64_t)j2 * L;
+            float2 *sq = region + sub * R::RS;
+#pragma unroll
+            for (int q = 0; q < 32; ++q) sq[t + R::T * q] = row[t + R::T * q];   // read back by the same lane
+            CaptureSink cs;
+            short_rows_transform<L>(region, tw, cs);
+            if ((mine >> sub) & 1u) {
+#pragma unroll
+                for (int q = 0; q < 32; ++q) {   // outputs t + T q of the row (j increases with q)
+                    const float pw = fmaf(cs.v[q].x, cs.v[q].x, cs.v[q].y * cs.v[q].y);
+                    const int j = j2 + ((t + R::T * q) << log2N2);
+                    if (pw == M && j < bj) {
+                        bj = j;
+                        bz = cs.v[q];
+                    }
+                }
+            }
+            __syncwarp();   // the region is read before the next candidate rows overwrite it
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+        const float ox = __shfl_xor_sync(0xffffffffu, bz.x, o);
+        const float oy = __shfl_xor_sync(0xffffffffu, bz.y, o);
+        if (oj < bj) {
+            bj = oj;
+            bz = make_float2(ox, oy);
+        }
+    }
+    if (lane == 0) {
+        const UnitInfo u = units[unit];
+        mf_peak pk;
+        pk.rho = sqrtf(M) * u.rho_scale;
+        pk.j = bj;
+        pk.z_re = bz.x * u.z_scale;
+        pk.z_im = bz.y * u.z_scale;
+        if (MF_DBG(u.tmpl >= 0 && u.tmpl < n_all && seg_idx < n_seg, kDbgOut))
+            peaks[(int64_t)u.tmpl * n_seg + seg_idx] = pk;
+    }
+}
+
+template <int L>
+static cudaError_t short_rows_attrs() {
+    cudaError_t e = cudaFuncSetAttribute(k_pass2_rows_short<L, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)ShortRows<L>::SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_pass2_rows_short<L, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)ShortRows<L>::SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_peaks_rows_short<L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)ShortRows<L>::SMEM);
+    return e;
+}
+template <int L>
+static void short_rows_launch(const RowsParams &p, int64_t rows, int n_sm, bool peaks_later, cudaStream_t st) {
+    const int64_t per = kWarps * ShortRows<L>::RPW;
+    const unsigned gr = (unsigned)std::max<int64_t>(1, std::min<int64_t>(2 * (int64_t)n_sm, (rows + per - 1) / per));
+    if (peaks_later) k_pass2_rows_short<L, false><<<gr, kWarps * 32, ShortRows<L>::SMEM, st>>>(p);
+    else k_pass2_rows_short<L, true><<<gr, kWarps * 32, ShortRows<L>::SMEM, st>>>(p);
+}
+
+// ---------------------------------------------------------------------------
 // Rows of L = 1024 G points on a group of G = 2 or 4 warps: 2048-point rows
 // (N = 2^21, 2^22, and the 512 x 2048 split of 2^20) and 4096-point rows (the
 // 1024 x 4096 split of 2^22), with the arithmetic of the radix 32 x 32 x G
@@ -686,7 +907,7 @@ static size_t rows_smem_tc() {
 
 MF_DEBUG_READER(dbg_read_rows)
 
-bool pass2_rows_applies(int log2N1) { return log2N1 >= 10 && log2N1 <= 12; }
+bool pass2_rows_applies(int log2N1) { return log2N1 >= 7 && log2N1 <= 12; }
 
 int pass2_rows_partials(int log2N, int log2N2) {   // partials per unit: one per row and warp
     const int lg1 = log2N - log2N2;
@@ -729,6 +950,12 @@ cudaError_t launch_pass2_rows(const SegDev &seg, const UnitInfo *units, int unit
             k_pass2_rows<1024, false><<<gr, kWarps * 32, rows_smem<1024>(), st>>>(p);
         else
             k_pass2_rows<1024, true><<<gr, kWarps * 32, rows_smem<1024>(), st>>>(p);
+    } else if (seg.log2N1 == 7) {
+        short_rows_launch<128>(p, rows, n_sm, peaks_later, st);
+    } else if (seg.log2N1 == 8) {
+        short_rows_launch<256>(p, rows, n_sm, peaks_later, st);
+    } else if (seg.log2N1 == 9) {
+        short_rows_launch<512>(p, rows, n_sm, peaks_later, st);
     } else if (seg.log2N1 == 11) {
         int64_t grid = std::min<int64_t>(2 * (int64_t)n_sm, (rows + kWarps / 2 - 1) / (kWarps / 2));
         const unsigned gr = (unsigned)std::max<int64_t>(grid, 1);
@@ -744,7 +971,7 @@ cudaError_t launch_pass2_rows(const SegDev &seg, const UnitInfo *units, int unit
 }
 
 bool pass2_rows_peaks_later(int log2N1, int fft_mode) {
-    return log2N1 >= 10 && log2N1 <= 12 && fft_mode == MF_FFT_FP32;
+    return pass2_rows_applies(log2N1) && fft_mode == MF_FFT_FP32;
 }
 
 cudaError_t launch_peaks_rows(const SegDev &seg, const UnitInfo *units, int unit0, int n_units, int n_all,
@@ -755,6 +982,15 @@ cudaError_t launch_peaks_rows(const SegDev &seg, const UnitInfo *units, int unit
         const unsigned grid = (unsigned)((n_units + kWarps - 1) / kWarps);
         k_peaks_rows<<<grid, kWarps * 32, rows_smem<1024>(), st>>>(exch, units, unit0, n_units, n_all, seg.log2N,
                                                                    seg.log2N2, partials, seg_idx, n_seg, peaks);
+    } else if (seg.log2N1 >= 7 && seg.log2N1 <= 9) {
+        const unsigned grid = (unsigned)((n_units + kWarps - 1) / kWarps);
+        auto run = [&](auto kernel, size_t smem) {
+            kernel<<<grid, kWarps * 32, smem, st>>>(exch, units, unit0, n_units, n_all, seg.log2N, seg.log2N2, partials,
+                                                    seg_idx, n_seg, peaks);
+        };
+        if (seg.log2N1 == 7) run(k_peaks_rows_short<128>, ShortRows<128>::SMEM);
+        else if (seg.log2N1 == 8) run(k_peaks_rows_short<256>, ShortRows<256>::SMEM);
+        else run(k_peaks_rows_short<512>, ShortRows<512>::SMEM);
     } else if (seg.log2N1 == 11) {
         const unsigned grid = (unsigned)((n_units + kWarps / 2 - 1) / (kWarps / 2));
         k_peaks_rows_group<2><<<grid, kWarps * 32, rows_group_smem<2>(), st>>>(
@@ -782,6 +1018,9 @@ cudaError_t rows_kernel_attributes() {
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_peaks_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rows_smem<1024>());
     if (e != cudaSuccess) return e;
+    if ((e = short_rows_attrs<128>()) != cudaSuccess || (e = short_rows_attrs<256>()) != cudaSuccess ||
+        (e = short_rows_attrs<512>()) != cudaSuccess)
+        return e;
     e = cudaFuncSetAttribute(k_pass2_rows_tc<MF_FFT_TC_FP16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)rows_smem_tc());
     if (e != cudaSuccess) return e;
