@@ -652,6 +652,7 @@ extern "C" int mf_segment_refresh(mf_segment g, const float *s, int s_on_device,
         MF_CUDA(cudaMemcpyAsync(g->r_s, s, sizeof(float) * N, cudaMemcpyHostToDevice, st));
         s_use = g->r_s;
     }
+    ChainScope chain(true);
     // the PSD and with it P, sigma's normalisation and the factors a_k are unchanged
     if (g->cond == MF_COND_FP32) {
         MF_CUDA(launch_forward_fft(s_use, N, g->r_exch, g->r_X, st));
@@ -956,6 +957,12 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
     const int *unit_order = (uo && !strcmp(uo, "bank")) ? nullptr : b->d_order;
     const int stall_pos =
         b->stall_unit < 0 ? -1 : (unit_order ? b->pos[(size_t)b->stall_unit] : (int)b->stall_unit);
+    // Chained launches where the call stays on one stream, kernel after kernel
+    bool one_stream = !b->prof_on;
+    for (int s = 0; s < n_seg; ++s)
+        one_stream = one_stream && !use_persistent(b, segs[s]) && !use_fused(b, segs[s]) &&
+                     (seg_batch[(size_t)s] >= n_t || b->params.phase_mode == MF_PHASE_FP32);
+    ChainScope chain(one_stream);
     for (int s = 0; s < n_seg; ++s) {
         const SegDev sd = seg_dev(segs[s], filter_log2n2(b, segs[s]));
         const int lgD = choose_log2D(b, segs[s]);
@@ -1264,6 +1271,7 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
     float *anc4 = sc.at<float>(o_anc4);
     float2 *exch = sc.at<float2>(o_exch);
     int launches = 0;
+    ChainScope chain(true);
     if (e == cudaSuccess) e = launch_units(sd, b->d_tmpl, n_t, b->params.f_low, 0.f, lgD, nullptr, all, nullptr, st);
     if (e == cudaSuccess) e = launch_chisq_units(sd, all, n_t, tmpl, (int)n, p, units, edges, st);
     launches += 2;
@@ -1379,6 +1387,7 @@ extern "C" int mf_chisq_points(mf_bank b, const mf_segment *segs, int n_seg, con
     cudaError_t e = sc.alloc(st);
     double2 *partial = sc.at<double2>(o_partial);
     double *pratio = sc.at<double>(o_pratio);
+    ChainScope chain(true);
     int launches = 0;
     for (int64_t i0 = 0; i0 < n && e == cudaSuccess; i0 += chunk) {
         const int64_t m = std::min<int64_t>(chunk, n - i0);

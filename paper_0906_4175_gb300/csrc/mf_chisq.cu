@@ -25,7 +25,8 @@ namespace mf {
 __global__ void k_chisq_units(SegDev seg, const UnitInfo *__restrict__ all, int n_t, const int32_t *__restrict__ tmpl,
                               int n, int p, UnitInfo *__restrict__ out, int64_t *__restrict__ edges) {
     __shared__ int64_t b[kChisqMaxBands + 1];
-    const int u = blockIdx.x;
+    int u = blockIdx.x;
+    chain_wait(u);
     const int t = tmpl[u];
     UnitInfo full;
     if (t >= 0 && t < n_t) {
@@ -115,8 +116,9 @@ __global__ void __launch_bounds__(C *(L / 32), (C * (L / 32) >= 256) ? 2 : 1) k_
     extern __shared__ float2 chi_smem[];
     constexpr int T = L / 32, NT = C * T;
     float2 *tw = chi_smem + pass_data_bytes<L, C>() / sizeof(float2);
-    const int tile = blockIdx.x, b = blockIdx.y;
+    int tile = blockIdx.x, b = blockIdx.y;
     fill_twiddles<L>(tw);
+    chain_wait(tile, b);
     ChiTileAcc snk;
     snk.p = q.p;
     snk.pf = (float)q.p;
@@ -252,11 +254,12 @@ __global__ void __launch_bounds__(kChiWarps * 32, 2) k_chisq_rows(ChiRowsParams 
     if (t == 0) cs_mbar_init(&bars[w]);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncthreads();
+    int64_t r0 = (int64_t)blockIdx.x * kChiWarps;
+    chain_wait_async(r0);
     // rows of the batch: nb N2, a multiple of 8 (N2 >= 512), so every warp has a row in every round
     const int64_t total = (int64_t)p.nb << p.log2N2;
     const int64_t step = (int64_t)gridDim.x * kChiWarps;
     const float pf = (float)p.p;
-    int64_t r0 = (int64_t)blockIdx.x * kChiWarps;
     if (r0 < total && t == 0 && !chi_withheld(p, r0 + w)) cs_row_copy(region, chi_row_src(p, r0 + w, 0), &bars[w]);
     uint32_t parity = 0;
     // a warp whose wait ran out stops waiting and issues no further copies
@@ -340,8 +343,7 @@ struct ChiTilesOp {
             constexpr size_t smem = chi_tiles_smem_bytes<N1, C>();
             if (!q)
                 return cudaFuncSetAttribute(k_chisq_tiles<N1, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            k_chisq_tiles<N1, C><<<dim3(N2 / C, q->nb), C * (N1 / 32), smem, st>>>(*q);
-            return cudaGetLastError();
+            return launch(k_chisq_tiles<N1, C>, dim3(N2 / C, q->nb), C * (N1 / 32), smem, st, *q);
         } else {
             return q ? cudaErrorInvalidValue : cudaSuccess;   // 1024-point rows: k_chisq_rows
         }
@@ -352,8 +354,7 @@ struct ChiTilesOp {
 cudaError_t launch_chisq_units(const SegDev &seg, const UnitInfo *all, int n_t, const int32_t *tmpl, int n, int p,
                                UnitInfo *out, int64_t *edges, cudaStream_t st) {
     if (p < 1 || p > kChisqMaxBands) return cudaErrorInvalidValue;
-    k_chisq_units<<<n, p >= 8 ? 256 : 128, 0, st>>>(seg, all, n_t, tmpl, n, p, out, edges);
-    return cudaGetLastError();
+    return launch(k_chisq_units, dim3(n), p >= 8 ? 256 : 128, 0, st, seg, all, n_t, tmpl, n, p, out, edges);
 }
 
 cudaError_t launch_chisq_tiles(const SegDev &seg, const float2 *exch, const UnitInfo *full, int unit0, int nb, int p,
@@ -371,8 +372,7 @@ cudaError_t launch_chisq_rows(const SegDev &seg, const float2 *exch, const UnitI
     ChiRowsParams q{exch, full, chisq, unit0, nb, p, seg.log2N, seg.log2N2, status, spin_limit, stall};
     const int64_t rounds = ((int64_t)nb << seg.log2N2) / kChiWarps;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(2 * (int64_t)n_sm, rounds));
-    k_chisq_rows<<<grid, kChiWarps * 32, chi_rows_smem_bytes(), st>>>(q);
-    return cudaGetLastError();
+    return launch(k_chisq_rows, dim3(grid), kChiWarps * 32, chi_rows_smem_bytes(), st, q);
 }
 
 MF_DEBUG_READER(dbg_read_chisq)

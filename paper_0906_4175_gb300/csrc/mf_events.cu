@@ -452,7 +452,8 @@ __global__ void __launch_bounds__(kCpThreads)
     __shared__ float4 sanc[kCpAnchors];
     __shared__ float sanc4[kCpAnchors];
     __shared__ double red[2][kCpWarps];
-    const int64_t i = blockIdx.y;
+    int64_t i = blockIdx.y;
+    chain_wait(i);
     const int32_t t = rows[i * stride], sg = rows[i * stride + 1], jj = rows[i * stride + 2];
     const int si = sg >= 0 && sg < segs.n ? sg : 0;
     const SegDev &seg = segs.s[si];
@@ -560,8 +561,9 @@ __global__ void __launch_bounds__(kCpThreads)
                          int64_t stride, int p, const double2 *__restrict__ partial, const double *__restrict__ pratio,
                          int bpr, float *__restrict__ chisq) {
     __shared__ double2 R[kChisqMaxBands];
-    const int64_t i = blockIdx.x;
+    int64_t i = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    chain_wait(i);
     const int32_t t = rows[i * stride], sg = rows[i * stride + 1], jj = rows[i * stride + 2];
     if (!cp_row_valid(t, n_t, sg, segs.n, jj, segs.s[sg >= 0 && sg < segs.n ? sg : 0])) {
         if (threadIdx.x == 0) chisq[i] = __int_as_float(0x7fc00000);
@@ -618,12 +620,11 @@ static cudaError_t chisq_points_run(const SegDev *segs, const int *lg, int n_seg
         tab.lg[s] = lg[s];
     }
     tab.n = n_seg;
-    k_chisq_points<NS><<<dim3((unsigned)bpr, (unsigned)n), kCpThreads, 0, st>>>(tab, tmpl, n_t, f_low, rows, stride,
-                                                                               p, partial, pratio);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch(k_chisq_points<NS>, dim3((unsigned)bpr, (unsigned)n), kCpThreads, 0, st, tab, tmpl, n_t,
+                                 f_low, rows, stride, p, partial, pratio);
     if (e != cudaSuccess) return e;
-    k_chisq_points_final<NS><<<(unsigned)n, kCpThreads, 0, st>>>(tab, n_t, rows, stride, p, partial, pratio, bpr, chisq);
-    return cudaGetLastError();
+    return launch(k_chisq_points_final<NS>, dim3((unsigned)n), kCpThreads, 0, st, tab, n_t, rows, stride, p, partial, pratio,
+                  bpr, chisq);
 }
 
 cudaError_t launch_chisq_points(const SegDev *segs, const int *lg, int n_seg, const double *tmpl, int n_t,

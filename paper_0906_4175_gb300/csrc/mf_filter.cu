@@ -57,8 +57,9 @@ __device__ __forceinline__ void clear_ctl(FilterCtl *ctl) {
 // Unit i of a segment is template order[i] (bank order when order is NULL).
 __global__ void k_units(SegDev seg, const double *__restrict__ tmpl, int n_t, double f_low, float thr,
                         int log2D, const int *__restrict__ order, UnitInfo *__restrict__ units, FilterCtl *clear) {
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    chain_wait(i);
     if (clear && blockIdx.x == 0) clear_ctl(clear);
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_t) return;
     const int t = order ? order[i] : i;
     units[i] = unit_info(seg, tmpl + (int64_t)t * kTmplStride, t, f_low, thr, log2D);
@@ -86,7 +87,8 @@ __device__ __forceinline__ void unit_anchors(const SegDev &seg, const double *T,
 __global__ void k_anchors(SegDev seg, const double *__restrict__ tmpl, const UnitInfo *__restrict__ units,
                           int unit0, int log2D, int max_anc, float4 *__restrict__ anchors,
                           float *__restrict__ anchors4, int reps) {
-    const int b = blockIdx.y;
+    int b = blockIdx.y;
+    chain_wait(b);
     const UnitInfo u = units[unit0 + b];
     unit_anchors(seg, tmpl + (int64_t)u.tmpl * kTmplStride, u, log2D, max_anc, anchors + (int64_t)b * max_anc,
                  anchors4 + (int64_t)b * max_anc, reps, (int64_t)gridDim.y * max_anc,   // copy k of slot b: slot b + k n_units
@@ -100,7 +102,9 @@ __global__ void k_units_anchors(SegDev seg, const double *__restrict__ tmpl, dou
                                 const int *__restrict__ order, UnitInfo *__restrict__ units, int max_anc,
                                 float4 *__restrict__ anchors, float *__restrict__ anchors4, FilterCtl *clear) {
     __shared__ UnitInfo su;
-    const int b = blockIdx.y, t = order ? order[b] : b;
+    int b = blockIdx.y;
+    chain_wait(b);
+    const int t = order ? order[b] : b;
     const double *T = tmpl + (int64_t)t * kTmplStride;
     if (clear && blockIdx.x == 0 && b == 0) clear_ctl(clear);
     if (threadIdx.x == 0) {
@@ -114,7 +118,8 @@ __global__ void k_units_anchors(SegDev seg, const double *__restrict__ tmpl, dou
 
 __global__ void k_anchors64(SegDev seg, const double *__restrict__ tmpl, const UnitInfo *__restrict__ units, int unit0,
                             int log2D, int max_anc, float4 *__restrict__ anchors) {
-    const int b = blockIdx.y;
+    int b = blockIdx.y;
+    chain_wait(b);
     const UnitInfo u = units[unit0 + b];
     const double *T = tmpl + (int64_t)u.tmpl * kTmplStride;
     const double c1 = T[TF_C1], c2 = T[TF_C2], c3 = T[TF_C3], c5 = T[TF_C5];
@@ -139,8 +144,7 @@ MF_DEBUG_READER(dbg_read_filter)
 
 cudaError_t launch_units(const SegDev &seg, const double *tmpl, int n_t, double f_low, float thr, int log2D,
                          const int *order, UnitInfo *units, FilterCtl *clear, cudaStream_t st) {
-    k_units<<<(n_t + 255) / 256, 256, 0, st>>>(seg, tmpl, n_t, f_low, thr, log2D, order, units, clear);
-    return cudaGetLastError();
+    return launch(k_units, dim3((n_t + 255) / 256), 256, 0, st, seg, tmpl, n_t, f_low, thr, log2D, order, units, clear);
 }
 
 // Blocks per unit of the merged launch, or 0 where the two launches are better:
@@ -160,9 +164,8 @@ cudaError_t launch_units_anchors(const SegDev &seg, const double *tmpl, int n_t,
                                  FilterCtl *clear, int n_sm, cudaStream_t st) {
     const int gx = units_anchors_blocks(n_t, max_anc, n_sm);
     if (gx < 1) return cudaErrorInvalidValue;
-    k_units_anchors<<<dim3(gx, n_t), 256, 0, st>>>(seg, tmpl, f_low, thr, log2D, order, units, max_anc, anchors,
-                                                   anchors4, clear);
-    return cudaGetLastError();
+    return launch(k_units_anchors, dim3(gx, n_t), 256, 0, st, seg, tmpl, f_low, thr, log2D, order, units, max_anc, anchors,
+                  anchors4, clear);
 }
 
 cudaError_t launch_anchors(const SegDev &seg, const double *tmpl, const UnitInfo *units, int unit0, int n_units,
@@ -174,11 +177,10 @@ cudaError_t launch_anchors(const SegDev &seg, const double *tmpl, const UnitInfo
     if (gx > 64) gx = 64;
     if (phase_mode == MF_PHASE_FP64) {
         if (reps != 1) return cudaErrorInvalidValue;
-        k_anchors64<<<dim3(gx, n_units), per, 0, st>>>(seg, tmpl, units, unit0, log2D, max_anc, anchors);
-        return cudaGetLastError();
+        return launch(k_anchors64, dim3(gx, n_units), per, 0, st, seg, tmpl, units, unit0, log2D, max_anc, anchors);
     }
-    k_anchors<<<dim3(gx, n_units), per, 0, st>>>(seg, tmpl, units, unit0, log2D, max_anc, anchors, anchors4, reps);
-    return cudaGetLastError();
+    return launch(k_anchors, dim3(gx, n_units), per, 0, st, seg, tmpl, units, unit0, log2D, max_anc, anchors, anchors4,
+                  reps);
 }
 
 namespace {
@@ -303,8 +305,9 @@ cudaError_t filter_kernel_attributes() {
 // ---------------------------------------------------------------------------
 __global__ void k_reduce_peaks(const UnitInfo *__restrict__ units, int n_units, const float4 *__restrict__ partials,
                                int nblk, int seg_idx, int n_seg, mf_peak *__restrict__ peaks) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
+    chain_wait(warp);
     if (warp >= n_units) return;
     float bp = -1.f;
     int bj = 0x7fffffff;
@@ -340,8 +343,7 @@ cudaError_t launch_reduce_peaks(const SegDev &seg, const UnitInfo *units, int n_
     (void)seg;
     const int threads = 256;
     const int blocks = (n_units * 32 + threads - 1) / threads;
-    k_reduce_peaks<<<blocks, threads, 0, st>>>(units, n_units, partials, nblk, seg_idx, n_seg, peaks);
-    return cudaGetLastError();
+    return launch(k_reduce_peaks, dim3(blocks), threads, 0, st, units, n_units, partials, nblk, seg_idx, n_seg, peaks);
 }
 
 // ---------------------------------------------------------------------------
@@ -351,12 +353,12 @@ cudaError_t launch_reduce_peaks(const SegDev &seg, const UnitInfo *units, int n_
 // one CTA sorts in shared memory and the others leave; more go through tiles.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kSortThreads, 1)
-    k_sort_triggers(const unsigned long long *__restrict__ counter, int64_t cap, int npass,
-                    const mf_trigger *__restrict__ staged, uint64_t *keys, uint64_t *keys_tmp, uint32_t *idx_a,
+    k_sort_triggers(const unsigned long long *counter, int64_t cap, int npass, const mf_trigger *staged, uint64_t *keys, uint64_t *keys_tmp, uint32_t *idx_a,
                     uint32_t *idx_b, SortCtl *ctl, uint64_t *tstat, mf_trigger *__restrict__ out,
                     int64_t *__restrict__ n_out, int *status, int64_t spin_limit) {
     extern __shared__ __align__(16) unsigned char sort_smem[];
     SortShared &sh = *reinterpret_cast<SortShared *>(sort_smem);
+    chain_wait(counter, staged);
     const unsigned long long total = *counter;
     const int64_t n = (int64_t)(total < (unsigned long long)cap ? total : (unsigned long long)cap);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -405,10 +407,8 @@ cudaError_t launch_sort_triggers(const unsigned long long *counter, int64_t cap,
     const int npass = key_bits > 0 ? (key_bits + 7) / 8 : 1;
     if (npass > kSortMaxPass) return cudaErrorInvalidValue;
     const int grid = cap <= kSortSmall ? 1 : n_sm;
-    k_sort_triggers<<<grid, kSortThreads, kSortSmemBytes, st>>>(counter, cap, npass, staged,
-                                                               const_cast<uint64_t *>(keys), keys_tmp, idx_a, idx_b,
-                                                               ctl, tstat, out, n_out, status, spin_limit);
-    return cudaGetLastError();
+    return launch(k_sort_triggers, dim3(grid), kSortThreads, kSortSmemBytes, st, counter, cap, npass, staged,
+                  const_cast<uint64_t *>(keys), keys_tmp, idx_a, idx_b, ctl, tstat, out, n_out, status, spin_limit);
 }
 
 }  // namespace mf

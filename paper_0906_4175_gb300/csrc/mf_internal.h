@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "mf_launch.h"
 #include "mfgb.h"
 
 namespace mf {

@@ -80,9 +80,10 @@ __global__ void __launch_bounds__(C *(L / 32), (C * (L / 32) >= 256) ? 2 : 3)
         }
     }
     __syncthreads();   // twiddles and the mbarrier initialised
+    int item = blockIdx.x;
+    chain_wait_async(item);
     const typename ExchSink<L, C, +1, LG1>::Params kp{p.E, LG1, p.log2N};
 
-    int item = blockIdx.x;
     uint32_t parity = 0;
     int4 band = make_int4(0, 0, 0, 0);
     if (item < p.n_items) {
@@ -138,8 +139,7 @@ cudaError_t pf_launch(const Pass1PfParams &p, const CUtensorMap &map, int n_unit
     Pass1PfParams q = p;
     q.n_items = n_units * (N1 / C);
     const int grid = (int)std::min<int64_t>(q.n_items, (int64_t)per_sm * g_pf_sms);
-    k_pass1_pf<N2, C, LG1, TMA, NARROW><<<grid, C * (N2 / 32), pf_smem_bytes<N2, C>(), st>>>(q, map);
-    return cudaGetLastError();
+    return launch(k_pass1_pf<N2, C, LG1, TMA, NARROW>, dim3(grid), C * (N2 / 32), pf_smem_bytes<N2, C>(), st, q, map);
 }
 
 struct PfOp {

@@ -37,8 +37,10 @@ __global__ void __launch_bounds__(C *(L / 32), (C * (L / 32) >= 256) ? 2 : 1)
     extern __shared__ float2 smem[];
     float2 *tw = smem + pass_data_bytes<L, C>() / sizeof(float2);
     fill_twiddles<L>(tw);
-    Src src(sp, blockIdx.x, unit0 + blockIdx.y, blockIdx.y, tw + TwTable<L>::SIZE);
-    Snk snk(kp, blockIdx.x, unit0 + blockIdx.y, blockIdx.y);
+    int tile = blockIdx.x, slot = blockIdx.y;
+    chain_wait(tile, slot);
+    Src src(sp, tile, unit0 + slot, slot, tw + TwTable<L>::SIZE);
+    Snk snk(kp, tile, unit0 + slot, slot);
     cta_fft<L, C, SEQ_FAST, SIGN>(smem, tw, src, snk);
     snk.finish(smem);
 }
@@ -53,9 +55,8 @@ cudaError_t set_pass_attrs() {
 template <int L, int C, bool SEQ_FAST, int SIGN, class Src, class Snk>
 cudaError_t run_pass(dim3 grid, const typename Src::Params &sp, const typename Snk::Params &kp,
                      cudaStream_t st, int unit0 = 0) {
-    k_fft_pass<L, C, SEQ_FAST, SIGN, Src, Snk>
-        <<<grid, C * (L / 32), pass_smem_bytes<L, C, Src>(), st>>>(sp, kp, unit0);
-    return cudaGetLastError();
+    return launch(k_fft_pass<L, C, SEQ_FAST, SIGN, Src, Snk>, grid, C * (L / 32), pass_smem_bytes<L, C, Src>(), st, sp,
+                  kp, unit0);
 }
 
 // Calls op.template run<N2, N1>() for the split of N = 2^log2N.

@@ -175,7 +175,8 @@ __global__ void __launch_bounds__(threads64<LG2, SMALL>())
     const int64_t M1 = (int64_t)1 << lgM1;
     const int lgca = lgM1 < cx_log2(S) ? lgM1 : cx_log2(S);
     const int ca = 1 << lgca;
-    const int64_t n1_0 = (int64_t)blockIdx.x * ca;
+    int64_t n1_0 = (int64_t)blockIdx.x * ca;
+    chain_wait(n1_0);
     for (int e = threadIdx.x; e < ca * L; e += NT) {   // consecutive threads: consecutive columns
         const int c = e & (ca - 1), n2 = e >> lgca;
         const float2 v = z[n1_0 + c + n2 * M1];
@@ -198,6 +199,7 @@ __global__ void __launch_bounds__(threads64<LG1, SMALL>()) k_fwd64_rows(double2 
     const int64_t M2 = (int64_t)1 << (lgM - LG1);
     const int cb = M2 < S ? (int)M2 : S;
     double2 *row = E + (int64_t)blockIdx.x * cb * L;
+    chain_wait(row);
     for (int e = threadIdx.x; e < cb * L; e += NT) sm64[e] = row[e];
     __syncthreads();
     smem_dft64<LG1, S, NT>(sm64);
@@ -215,7 +217,9 @@ __global__ void k_fwd64_split(const double2 *__restrict__ Z, int lgM, const floa
                               float2 *__restrict__ out) {
     const int lgM2 = lgM / 2, lgM1 = lgM - lgM2;
     const int64_t M = (int64_t)1 << lgM;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k <= M / 2; k += (int64_t)gridDim.x * blockDim.x) {
+    int64_t k0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    chain_wait(k0);
+    for (int64_t k = k0; k <= M / 2; k += (int64_t)gridDim.x * blockDim.x) {
         const int64_t kb = (M - k) & (M - 1);
         const double2 za = Z[((k & (((int64_t)1 << lgM2) - 1)) << lgM1) + (k >> lgM2)];
         const double2 zb = Z[((kb & (((int64_t)1 << lgM2) - 1)) << lgM1) + (kb >> lgM2)];
@@ -248,9 +252,8 @@ cudaError_t launch_cols(const float2 *z, int lgM, double2 *E, cudaStream_t st, b
                                     (int)smem64_bytes<LG2, SMALL>());
     const int64_t M1 = (int64_t)1 << (lgM - LG2);
     const int64_t ca = std::min<int64_t>(M1, seqs64<LG2, SMALL>());
-    k_fwd64_cols<LG2, SMALL>
-        <<<(unsigned)(M1 / ca), threads64<LG2, SMALL>(), smem64_bytes<LG2, SMALL>(), st>>>(z, lgM, E);
-    return cudaGetLastError();
+    return launch(k_fwd64_cols<LG2, SMALL>, dim3((unsigned)(M1 / ca)), threads64<LG2, SMALL>(),
+                  smem64_bytes<LG2, SMALL>(), st, z, lgM, E);
 }
 template <int LG1, bool SMALL>
 cudaError_t launch_rows(double2 *E, int lgM, cudaStream_t st, bool attrs) {
@@ -259,8 +262,8 @@ cudaError_t launch_rows(double2 *E, int lgM, cudaStream_t st, bool attrs) {
                                     (int)smem64_bytes<LG1, SMALL>());
     const int64_t M2 = (int64_t)1 << (lgM - LG1);
     const int64_t cb = std::min<int64_t>(M2, seqs64<LG1, SMALL>());
-    k_fwd64_rows<LG1, SMALL><<<(unsigned)(M2 / cb), threads64<LG1, SMALL>(), smem64_bytes<LG1, SMALL>(), st>>>(E, lgM);
-    return cudaGetLastError();
+    return launch(k_fwd64_rows<LG1, SMALL>, dim3((unsigned)(M2 / cb)), threads64<LG1, SMALL>(),
+                  smem64_bytes<LG1, SMALL>(), st, E, lgM);
 }
 
 // M = 2^lgM, lgM = 9 .. 21: column length 2^(lgM/2), row length 2^(lgM - lgM/2);
@@ -308,9 +311,7 @@ cudaError_t launch_forward_fft64(const float *s, int64_t N, void *scratch, const
     const int threads = lgM <= 16 ? 64 : 256;   // short transforms: more SMs
     int blocks = (int)((M / 2 + 1 + threads - 1) / threads);
     if (blocks > 4096) blocks = 4096;
-    if (fac) k_fwd64_split<true><<<blocks, threads, 0, st>>>(E, lgM, fac, out);
-    else k_fwd64_split<false><<<blocks, threads, 0, st>>>(E, lgM, nullptr, out);
-    return cudaGetLastError();
+    return launch(fac ? k_fwd64_split<true> : k_fwd64_split<false>, dim3(blocks), threads, 0, st, E, lgM, fac, out);
 }
 
 cudaError_t prep64_kernel_attributes() {

@@ -45,9 +45,10 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_pass2_rows(RowsParams p) {
     if (t == 0) mbar_init(&bars[grp], 1);
     mbar_fence_init();
     __syncthreads();
+    int64_t r = (int64_t)blockIdx.x * kWarps + grp;
+    chain_wait_async(r);
     const int64_t total = (int64_t)p.n_units << p.log2N2;
     const int64_t step = (int64_t)gridDim.x * kWarps;
-    int64_t r = (int64_t)blockIdx.x * kWarps + grp;
     if (r < total && t == 0 && !row_withheld(p, r)) {
         mbar_expect_tx(&bars[grp], L * sizeof(float2));
         bulk_copy_g2s(region, row_src<L>(p, r), L * sizeof(float2), &bars[grp]);
@@ -118,7 +119,8 @@ __global__ void __launch_bounds__(kWarps * 32) k_peaks_rows(const float2 *__rest
     float2 *region = rows_smem + w * S::STRIDE;
     fill_twiddles<L>(tw);
     __syncthreads();
-    const int b = blockIdx.x * kWarps + w;   // unit within the batch
+    int b = blockIdx.x * kWarps + w;   // unit within the batch
+    chain_wait(b);
     if (b >= n_units) return;
     const int unit = unit0 + b;
     const int n2 = 1 << log2N2;
@@ -278,9 +280,10 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_pass2_rows_short(RowsParams 
     if (lane == 0) mbar_init(&bars[w], 1);
     mbar_fence_init();
     __syncthreads();
+    int64_t r = ((int64_t)blockIdx.x * kWarps + w) * R::RPW;
+    chain_wait_async(r);
     const int64_t total = (int64_t)p.n_units << p.log2N2;   // rows, a multiple of RPW per unit
     const int64_t step = (int64_t)gridDim.x * kWarps * R::RPW;
-    int64_t r = ((int64_t)blockIdx.x * kWarps + w) * R::RPW;
     if (r < total && !row_withheld(p, r)) short_rows_copy<L>(p, r, region, &bars[w]);
     uint32_t parity = 0;
     for (; r < total; r += step) {
@@ -321,7 +324,8 @@ __global__ void __launch_bounds__(kWarps * 32) k_peaks_rows_short(const float2 *
     float2 *region = rows_smem + w * R::REGION;
     fill_twiddles<L>(tw);
     __syncthreads();
-    const int b = blockIdx.x * kWarps + w;   // unit within the batch
+    int b = blockIdx.x * kWarps + w;   // unit within the batch
+    chain_wait(b);
     if (b >= n_units) return;
     const int unit = unit0 + b;
     const int n2 = 1 << log2N2;
@@ -394,11 +398,11 @@ static cudaError_t short_rows_attrs() {
     return e;
 }
 template <int L>
-static void short_rows_launch(const RowsParams &p, int64_t rows, int n_sm, bool peaks_later, cudaStream_t st) {
+static cudaError_t short_rows_launch(const RowsParams &p, int64_t rows, int n_sm, bool peaks_later, cudaStream_t st) {
     const int64_t per = kWarps * ShortRows<L>::RPW;
     const unsigned gr = (unsigned)std::max<int64_t>(1, std::min<int64_t>(2 * (int64_t)n_sm, (rows + per - 1) / per));
-    if (peaks_later) k_pass2_rows_short<L, false><<<gr, kWarps * 32, ShortRows<L>::SMEM, st>>>(p);
-    else k_pass2_rows_short<L, true><<<gr, kWarps * 32, ShortRows<L>::SMEM, st>>>(p);
+    return launch(peaks_later ? k_pass2_rows_short<L, false> : k_pass2_rows_short<L, true>, dim3(gr), kWarps * 32,
+                  ShortRows<L>::SMEM, st, p);
 }
 
 // ---------------------------------------------------------------------------
@@ -506,9 +510,10 @@ __global__ void __launch_bounds__(kWarps * 32, 2) k_pass2_rows_group(RowsParams 
     }
     mbar_fence_init();
     __syncthreads();
+    int64_t r = (int64_t)blockIdx.x * NG + grp;
+    chain_wait_async(r);
     const int64_t total = (int64_t)p.n_units << p.log2N2;
     const int64_t step = (int64_t)gridDim.x * NG;
-    int64_t r = (int64_t)blockIdx.x * NG + grp;
     if (r < total && t == 0 && !row_withheld(p, r)) {
         mbar_expect_tx(&bars[grp], L * sizeof(float2));
         bulk_copy_g2s(region, row_src<L>(p, r), L * sizeof(float2), &bars[grp]);
@@ -576,7 +581,8 @@ __global__ void __launch_bounds__(kWarps * 32) k_peaks_rows_group(const float2 *
             tw1[m] = __ldg(&src[m < 1024 ? m : TwTable<L>::S1 + m]);
     }
     __syncthreads();
-    const int b = blockIdx.x * NG + grp;   // unit within the batch (the group's warps agree)
+    int b = blockIdx.x * NG + grp;   // unit within the batch (the group's warps agree)
+    chain_wait(b);
     if (b >= n_units) return;              // whole groups leave: no group barrier is left waiting
     const int unit = unit0 + b;
     const int n2 = 1 << log2N2;
@@ -946,26 +952,25 @@ cudaError_t launch_pass2_rows(const SegDev &seg, const UnitInfo *units, int unit
             k_pass2_rows_tc<MF_FFT_TC_FP16><<<gr, kWarps * 32, rows_smem_tc(), st>>>(p);
         else if (fft_mode == MF_FFT_TC_BF16)
             k_pass2_rows_tc<MF_FFT_TC_BF16><<<gr, kWarps * 32, rows_smem_tc(), st>>>(p);
-        else if (peaks_later)
-            k_pass2_rows<1024, false><<<gr, kWarps * 32, rows_smem<1024>(), st>>>(p);
         else
-            k_pass2_rows<1024, true><<<gr, kWarps * 32, rows_smem<1024>(), st>>>(p);
+            return launch(peaks_later ? k_pass2_rows<1024, false> : k_pass2_rows<1024, true>, dim3(gr), kWarps * 32,
+                          rows_smem<1024>(), st, p);
     } else if (seg.log2N1 == 7) {
-        short_rows_launch<128>(p, rows, n_sm, peaks_later, st);
+        return short_rows_launch<128>(p, rows, n_sm, peaks_later, st);
     } else if (seg.log2N1 == 8) {
-        short_rows_launch<256>(p, rows, n_sm, peaks_later, st);
+        return short_rows_launch<256>(p, rows, n_sm, peaks_later, st);
     } else if (seg.log2N1 == 9) {
-        short_rows_launch<512>(p, rows, n_sm, peaks_later, st);
+        return short_rows_launch<512>(p, rows, n_sm, peaks_later, st);
     } else if (seg.log2N1 == 11) {
         int64_t grid = std::min<int64_t>(2 * (int64_t)n_sm, (rows + kWarps / 2 - 1) / (kWarps / 2));
         const unsigned gr = (unsigned)std::max<int64_t>(grid, 1);
-        if (peaks_later) k_pass2_rows_group<2, false><<<gr, kWarps * 32, rows_group_smem<2>(), st>>>(p);
-        else k_pass2_rows_group<2, true><<<gr, kWarps * 32, rows_group_smem<2>(), st>>>(p);
+        return launch(peaks_later ? k_pass2_rows_group<2, false> : k_pass2_rows_group<2, true>, dim3(gr), kWarps * 32,
+                      rows_group_smem<2>(), st, p);
     } else {
         int64_t grid = std::min<int64_t>(2 * (int64_t)n_sm, (rows + kWarps / 4 - 1) / (kWarps / 4));
         const unsigned gr = (unsigned)std::max<int64_t>(grid, 1);
-        if (peaks_later) k_pass2_rows_group<4, false><<<gr, kWarps * 32, rows_group_smem<4>(), st>>>(p);
-        else k_pass2_rows_group<4, true><<<gr, kWarps * 32, rows_group_smem<4>(), st>>>(p);
+        return launch(peaks_later ? k_pass2_rows_group<4, false> : k_pass2_rows_group<4, true>, dim3(gr), kWarps * 32,
+                      rows_group_smem<4>(), st, p);
     }
     return cudaGetLastError();
 }
@@ -978,31 +983,20 @@ cudaError_t launch_peaks_rows(const SegDev &seg, const UnitInfo *units, int unit
                               const float2 *exch, const float4 *partials, int seg_idx, int n_seg, mf_peak *peaks,
                               cudaStream_t st) {
     if (n_units <= 0) return cudaSuccess;
-    if (seg.log2N1 == 10) {
-        const unsigned grid = (unsigned)((n_units + kWarps - 1) / kWarps);
-        k_peaks_rows<<<grid, kWarps * 32, rows_smem<1024>(), st>>>(exch, units, unit0, n_units, n_all, seg.log2N,
-                                                                   seg.log2N2, partials, seg_idx, n_seg, peaks);
-    } else if (seg.log2N1 >= 7 && seg.log2N1 <= 9) {
-        const unsigned grid = (unsigned)((n_units + kWarps - 1) / kWarps);
-        auto run = [&](auto kernel, size_t smem) {
-            kernel<<<grid, kWarps * 32, smem, st>>>(exch, units, unit0, n_units, n_all, seg.log2N, seg.log2N2, partials,
-                                                    seg_idx, n_seg, peaks);
-        };
-        if (seg.log2N1 == 7) run(k_peaks_rows_short<128>, ShortRows<128>::SMEM);
-        else if (seg.log2N1 == 8) run(k_peaks_rows_short<256>, ShortRows<256>::SMEM);
-        else run(k_peaks_rows_short<512>, ShortRows<512>::SMEM);
-    } else if (seg.log2N1 == 11) {
-        const unsigned grid = (unsigned)((n_units + kWarps / 2 - 1) / (kWarps / 2));
-        k_peaks_rows_group<2><<<grid, kWarps * 32, rows_group_smem<2>(), st>>>(
-            exch, units, unit0, n_units, n_all, seg.log2N, seg.log2N2, partials, seg_idx, n_seg, peaks);
-    } else if (seg.log2N1 == 12) {
-        const unsigned grid = (unsigned)((n_units + kWarps / 4 - 1) / (kWarps / 4));
-        k_peaks_rows_group<4><<<grid, kWarps * 32, rows_group_smem<4>(), st>>>(
-            exch, units, unit0, n_units, n_all, seg.log2N, seg.log2N2, partials, seg_idx, n_seg, peaks);
-    } else {
-        return cudaErrorInvalidValue;
+    // units per CTA: one warp each, or the two or four warps of a longer row
+    auto run = [&](auto kernel, int per, size_t smem) {
+        return launch(kernel, dim3((unsigned)((n_units + per - 1) / per)), kWarps * 32, smem, st, exch, units, unit0,
+                      n_units, n_all, seg.log2N, seg.log2N2, partials, seg_idx, n_seg, peaks);
+    };
+    switch (seg.log2N1) {
+        case 7: return run(k_peaks_rows_short<128>, kWarps, ShortRows<128>::SMEM);
+        case 8: return run(k_peaks_rows_short<256>, kWarps, ShortRows<256>::SMEM);
+        case 9: return run(k_peaks_rows_short<512>, kWarps, ShortRows<512>::SMEM);
+        case 10: return run(k_peaks_rows, kWarps, rows_smem<1024>());
+        case 11: return run(k_peaks_rows_group<2>, kWarps / 2, rows_group_smem<2>());
+        case 12: return run(k_peaks_rows_group<4>, kWarps / 4, rows_group_smem<4>());
+        default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 cudaError_t rows_kernel_attributes() {

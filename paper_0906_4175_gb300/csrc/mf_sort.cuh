@@ -121,6 +121,19 @@ __device__ __forceinline__ uint32_t excl_scan_256(uint32_t x, SortShared &sh) {
     return wo + incl - x;
 }
 
+// Lanes whose 8-bit digit equals this lane's, among the lanes with a digit
+// (d < 256): one vote per bit.  __match_any_sync serialises on one unit per SM
+// (the one-CTA sort of 4400 keys 27 us with it).
+__device__ __forceinline__ unsigned match_digit(uint32_t d) {
+    unsigned peers = __ballot_sync(0xffffffffu, d < 256u);
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const unsigned v = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+        peers &= ((d >> b) & 1u) ? v : ~v;
+    }
+    return peers;
+}
+
 // Ranks rows of keys held by the warps (warp w owns ROWS rows of 32 consecutive
 // keys, rows in order): lr[r] = the key's rank among the warp's equal digits,
 // sh.whist[w][d] = the warp's count of digit d.  Inactive keys carry a digit
@@ -134,7 +147,7 @@ __device__ __forceinline__ void sort_rank_rows(const uint32_t *dg, uint32_t *lr,
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) {
         if (r >= rows) break;
-        const unsigned peers = __match_any_sync(0xffffffffu, dg[r]);
+        const unsigned peers = match_digit(dg[r]);
         const uint32_t rank = (uint32_t)__popc(peers & lt_mask);
         const bool act = dg[r] < 256u;
         lr[r] = act ? sh.whist[warp][dg[r]] + rank : 0u;
