@@ -283,12 +283,9 @@ int pass2_blocks(int log2N, int log2N2) {
     return op.nblk;
 }
 
-static cudaError_t sort_kernel_attributes();
-
 cudaError_t filter_kernel_attributes() {
     {
         cudaError_t e0 = init_pass_tables();
-        if (e0 == cudaSuccess) e0 = sort_kernel_attributes();
         if (e0 != cudaSuccess) return e0;
     }
     for (int lg = 10; lg <= 22; ++lg) {
@@ -349,14 +346,15 @@ cudaError_t launch_reduce_peaks(const SegDev &seg, const UnitInfo *units, int n_
 // ---------------------------------------------------------------------------
 // Trigger compaction: the staged records into the caller's buffer in (tmpl,
 // seg, j) order, by a stable LSD radix sort of the packed keys with 8-bit
-// digits (mf_sort.cuh), the whole chain in one launch.  Up to 8192 triggers
-// one CTA sorts in shared memory and the others leave; more go through tiles.
+// digits or, up to 16384 triggers, by rank (mf_sort.cuh), in one launch.
 // ---------------------------------------------------------------------------
+constexpr size_t kRankSmem = (size_t)kRankChunk * sizeof(uint64_t) + kSortThreads * sizeof(uint32_t);
+constexpr size_t kTriggerSortSmem = sizeof(SortShared) > kRankSmem ? sizeof(SortShared) : kRankSmem;
 __global__ void __launch_bounds__(kSortThreads, 1)
-    k_sort_triggers(const unsigned long long *counter, int64_t cap, int npass, const mf_trigger *staged, uint64_t *keys, uint64_t *keys_tmp, uint32_t *idx_a,
+    k_sort_triggers(const unsigned long long *counter, int64_t cap, int key_bits, const mf_trigger *staged, uint64_t *keys, uint64_t *keys_tmp, uint32_t *idx_a,
                     uint32_t *idx_b, SortCtl *ctl, uint64_t *tstat, mf_trigger *__restrict__ out,
                     int64_t *__restrict__ n_out, int *status, int64_t spin_limit) {
-    extern __shared__ __align__(16) unsigned char sort_smem[];
+    __shared__ __align__(16) unsigned char sort_smem[kTriggerSortSmem];
     SortShared &sh = *reinterpret_cast<SortShared *>(sort_smem);
     chain_wait(counter, staged);
     const unsigned long long total = *counter;
@@ -365,15 +363,12 @@ __global__ void __launch_bounds__(kSortThreads, 1)
         *n_out = (int64_t)total;
         if (total > (unsigned long long)cap) atomicOr(status, 1);
     }
-    if (n <= kSortSmall) {
-        if (blockIdx.x == 0 && n > 0) {
-            uint64_t *skey = reinterpret_cast<uint64_t *>(sort_smem + sizeof(SortShared));
-            uint32_t *sidx = reinterpret_cast<uint32_t *>(skey + kSortSmall);
-            sort_small((int)n, npass, sh, skey, sidx, [&](int i) { return keys[i]; });
-            gather_records(staged, out, 0, n, [&](int64_t i) { return sidx[i]; });
-        }
+    if (n <= kRankMax) {
+        if (key_bits <= 32) sort_rank<uint32_t>(keys, (int)n, staged, out, sort_smem);
+        else sort_rank<uint64_t>(keys, (int)n, staged, out, sort_smem);
         return;
     }
+    const int npass = (key_bits + 7) / 8;
     const int64_t n_tiles = (n + kSortTile - 1) / kSortTile;
     if (!run_phase(ctl, 0, n_tiles, 0, sh, status, spin_limit, [&](int64_t t) {
             sort_hist_tile(ctl, tstat, t, n, npass, sh, [&](int64_t i) { return keys[i]; });
@@ -396,18 +391,12 @@ __global__ void __launch_bounds__(kSortThreads, 1)
     });
 }
 
-static cudaError_t sort_kernel_attributes() {
-    return cudaFuncSetAttribute(k_sort_triggers, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSortSmemBytes);
-}
-
 cudaError_t launch_sort_triggers(const unsigned long long *counter, int64_t cap, int key_bits,
                                  const mf_trigger *staged, const uint64_t *keys, uint64_t *keys_tmp,
                                  uint32_t *idx_a, uint32_t *idx_b, SortCtl *ctl, uint64_t *tstat, mf_trigger *out,
                                  int64_t *n_out, int *status, int n_sm, int64_t spin_limit, cudaStream_t st) {
-    const int npass = key_bits > 0 ? (key_bits + 7) / 8 : 1;
-    if (npass > kSortMaxPass) return cudaErrorInvalidValue;
-    const int grid = cap <= kSortSmall ? 1 : n_sm;
-    return launch(k_sort_triggers, dim3(grid), kSortThreads, kSortSmemBytes, st, counter, cap, npass, staged,
+    if (key_bits > 8 * kSortMaxPass || n_sm * kSortThreads < kRankMax) return cudaErrorInvalidValue;
+    return launch(k_sort_triggers, dim3(n_sm), kSortThreads, 0, st, counter, cap, key_bits, staged,
                   const_cast<uint64_t *>(keys), keys_tmp, idx_a, idx_b, ctl, tstat, out, n_out, status, spin_limit);
 }
 

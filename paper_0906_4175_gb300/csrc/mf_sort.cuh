@@ -4,11 +4,14 @@
 // A search step ends with a sort of a few thousand trigger keys, and every
 // kernel of a chain of small ones costs its launch (about 5 us of host time and
 // a gap of 2 us on the device) more than its work: the sort of 5000 keys took a
-// memset and 6 launches, 45 us; one launch takes 12 us.  So
-//   sort_small   up to 8192 keys: one CTA of 1024 threads, keys and payloads in
-//                registers between passes and in shared memory for the scatter;
+// memset and 5 launches, 45 us.  So
+//   sort_rank    up to 16384 unique keys: every CTA counts, for its share of the
+//                keys, the smaller ones among all of them, which is their place:
+//                no passes and no CTA waits for another;
 //   sort_pass    more keys: tiles of 4096 keys with decoupled look-back (Merrill
 //                & Garland's single-pass scan) per digit;
+//   sort_small   up to 8192 keys inside one CTA (clustering), keys and payloads in
+//                registers between passes and in shared memory for the scatter;
 //   run_phase    hands the tiles of one step to the CTAs by a ticket counter and
 //                lets a step's first tile of each CTA wait until every tile of
 //                the step before is done.
@@ -30,7 +33,7 @@ struct SortShared {
     uint32_t wsum[kSortWarps];
     int tile, ok;
 };
-// shared memory of a sorting kernel: SortShared, then the one-CTA sort's keys and payloads
+// shared memory of a kernel with the one-CTA sort: SortShared, then its keys and payloads
 constexpr size_t kSortSmemBytes = sizeof(SortShared) + (size_t)kSortSmall * (sizeof(uint64_t) + sizeof(uint32_t));
 static_assert(sizeof(SortShared) % 8 == 0, "the keys follow the shared block");
 
@@ -122,8 +125,8 @@ __device__ __forceinline__ uint32_t excl_scan_256(uint32_t x, SortShared &sh) {
 }
 
 // Lanes whose 8-bit digit equals this lane's, among the lanes with a digit
-// (d < 256): one vote per bit.  __match_any_sync serialises on one unit per SM
-// (the one-CTA sort of 4400 keys 27 us with it).
+// (d < 256): one vote per bit (__match_any_sync takes as long: 28 us for 4400
+// keys in one CTA either way).
 __device__ __forceinline__ unsigned match_digit(uint32_t d) {
     unsigned peers = __ballot_sync(0xffffffffu, d < 256u);
 #pragma unroll
@@ -222,6 +225,56 @@ __device__ __forceinline__ void sort_small(int n, int npass, SortShared &sh, uin
     }
 }
 
+// Rank sort of n unique keys by all CTAs of the grid (kSortThreads threads
+// each): CTA b places the records of keys [b k, b k + k), k = ceil(n / CTAs).
+// Its threads are k keys times as many parts of the comparison as fit, so few
+// keys are a few comparisons a thread and the latency of one read of the keys.
+// The limit is where n^2 comparisons catch up with the radix passes: 4400 keys
+// 28 us in one CTA's radix passes, 7 here, 180 keys 10 and 3.7; 22,800 keys 51 us
+// in tiles and 75 here, so about 38 at the limit.
+constexpr int kRankMax = 16384, kRankChunk = 4096;
+template <class K>
+__device__ __forceinline__ void sort_rank(const uint64_t *keys, int n, const mf_trigger *src, mf_trigger *dst,
+                                          unsigned char *smem) {
+    K *sk = reinterpret_cast<K *>(smem);
+    uint32_t *rank = reinterpret_cast<uint32_t *>(smem + kRankChunk * sizeof(uint64_t));   // [kSortThreads]
+    const int per = (n + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int k0 = (int)blockIdx.x * per, mine = min(per, n - k0);
+    if (mine <= 0) return;
+    const int parts = kSortThreads / per;   // per <= kSortThreads: n <= kRankMax on any GPU of 24 SMs
+    const int q = (int)threadIdx.x % per, part = (int)threadIdx.x / per;
+    const bool act = q < mine && part < parts;
+    const K my = act ? (K)keys[k0 + q] : (K)0;
+    if ((int)threadIdx.x < per) rank[threadIdx.x] = 0u;
+    uint32_t less = 0;
+    for (int c0 = 0; c0 < n; c0 += kRankChunk) {
+        const int m = min(kRankChunk, n - c0);
+        __syncthreads();
+        for (int i = threadIdx.x; i < m; i += kSortThreads) sk[i] = (K)keys[c0 + i];
+        __syncthreads();
+        const int len = ((m + parts - 1) / parts + 3) & ~3;
+        const int lo = part * len, hi = min(m, lo + len);
+        if (act) {
+            int j = lo;
+#pragma unroll 4
+            for (; j + 4 <= hi; j += 4) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) less += sk[j + e] < my ? 1u : 0u;
+            }
+            for (; j < hi; ++j) less += sk[j] < my ? 1u : 0u;
+        }
+    }
+    if (act && less) atomicAdd(&rank[q], less);
+    __syncthreads();
+    constexpr int W = sizeof(mf_trigger) / 4;
+    const uint32_t *s = reinterpret_cast<const uint32_t *>(src) + (int64_t)k0 * W;
+    uint32_t *d = reinterpret_cast<uint32_t *>(dst);
+    for (int w = threadIdx.x; w < mine * W; w += kSortThreads) {
+        const int r = w / W;
+        if (MF_DBG(rank[r] < (uint32_t)n, kDbgSort)) d[(int64_t)rank[r] * W + (w - r * W)] = s[w];
+    }
+}
+
 // Digit histograms of one tile for every pass (into ctl->ghist) and its
 // look-back words cleared.  key_of(i) gives key i < n.
 template <class KeyOf>
@@ -246,7 +299,7 @@ __device__ __forceinline__ void sort_hist_tile(SortCtl *ctl, uint64_t *tstat, in
 
 // dst[i] = src[index(i)] for i in [i0, i1), word by word with consecutive threads
 // on consecutive words: whole-record copies by one thread each touch a sector
-// per lane and word (47 us for 6000 records on one SM).  All threads call it.
+// per lane and word.  All threads call it.
 template <class Index>
 __device__ __forceinline__ void gather_records(const mf_trigger *src, mf_trigger *dst, int64_t i0, int64_t i1,
                                                Index index) {

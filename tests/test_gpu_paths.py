@@ -77,8 +77,9 @@ def test_merged_units_and_anchors(mf, lg, n):
     assert a[2] == b[2] and np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
 
 
-# every sample a trigger: 8192 records are the most one CTA sorts, then tiles of 4096
-@pytest.mark.parametrize("lg,n,segs", [(10, 1, 1), (10, 8, 1), (10, 4, 2), (10, 9, 1), (11, 5, 3), (14, 9, 2)])
+# every sample a trigger: up to 16384 records by rank, then tiles of 4096
+@pytest.mark.parametrize("lg,n,segs", [(10, 1, 1), (10, 8, 1), (10, 4, 2), (10, 9, 1), (11, 5, 3), (14, 9, 2),
+                                       (10, 16, 1), (10, 17, 1)])
 def test_trigger_order(mf, lg, n, segs):
     N = 1 << lg
     bank = mf.Bank(*_masses(n))
