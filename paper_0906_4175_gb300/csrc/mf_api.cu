@@ -1137,8 +1137,12 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
                 MF_CUDA(cudaStreamWaitEvent(st, b->ev_anc, 0));
             }
             pi = prof_begin(b, MF_STAGE_PASS1, by_band + by_anc + exch_bytes, st);
+            // units are in descending band width: half of the batch ends below fs/8
+            const size_t mid = (size_t)(u0 + nb / 2);
+            const int form =
+                b->fisco[unit_order ? (size_t)b->order[mid] : mid] <= 0.125 * sd.fs ? kBandLead : kBandPlain;
             MF_CUDA(launch_pass1(sd, w.units, u0, nb, lgD, man, w.anchors + aoff, w.anchors4 + aoff, w.exch,
-                                 b->params.phase_mode, b->d_tmpl, p1_form(b), w.status, b->spin_limit, st));
+                                 b->params.phase_mode, b->d_tmpl, p1_form(b), w.status, b->spin_limit, st, form));
             prof_end(b, pi, st);
             if (overlap && u0 + batch < n_t) {
                 const int u1 = u0 + (int)batch;
@@ -1290,7 +1294,7 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
         }
         if (e == cudaSuccess)
             e = launch_pass1(sd, bu, 0, (p + 1) * nb, lgD, man, anc, anc4, exch, b->params.phase_mode, b->d_tmpl,
-                             p1_form(b), b->chi_status, b->spin_limit, st, rows, nb);
+                             p1_form(b), b->chi_status, b->spin_limit, st, rows ? kBandNarrow : kBandPlain, nb);
         if (e == cudaSuccess)
             e = rows ? launch_chisq_rows(sd, exch, full, (int)u0, nb, p, chisq, b->chi_status, b->spin_limit,
                                          (int)b->stall_unit, sm_count(), st)

@@ -180,30 +180,51 @@ struct Dft {
     }
 };
 
-// 32-point DFT whose inputs v[16..31] are zero (upper half of a one-sided
-// spectrum): even outputs are the 16-point DFT of v, odd outputs the 16-point
-// DFT of v_r exp(SIGN 2 pi i r/32).
-template <int SIGN, int Q>
-struct HalfZeroTw {
-    static __device__ __forceinline__ void run(const float2 *v, float2 *b) {
-        if constexpr (Q < 16) {
-            b[Q] = tw_const<Q, 32, SIGN>(v[Q]);
-            HalfZeroTw<SIGN, Q + 1>::run(v, b);
+// The same with inputs v[NZ .. R - 1] zero (NZ a power of two): the sums with
+// zero terms are left out, which changes no rounding, so the outputs equal those
+// of Dft (an output that is exactly zero may differ in its sign).
+template <int R, int SIGN, int NZ>
+struct DftLead {
+    static __device__ __forceinline__ void run(float2 *v) {
+        if constexpr (NZ >= R) {
+            Dft<R, SIGN>::run(v);
+        } else if constexpr (NZ == 1) {
+#pragma unroll
+            for (int i = 1; i < R; ++i) v[i] = v[0];
+        } else {
+            float2 e[R / 2], o[R / 2];
+#pragma unroll
+            for (int i = 0; i < NZ / 2; ++i) { e[i] = v[2 * i]; o[i] = v[2 * i + 1]; }
+            DftLead<R / 2, SIGN, NZ / 2>::run(e);
+            DftLead<R / 2, SIGN, NZ / 2>::run(o);
+            Combine<R, SIGN, 0>::run(v, e, o);
         }
     }
 };
-template <int SIGN>
+
+// 32-point DFT whose inputs v[NZ..31] are zero, NZ <= 16 (the upper half of a
+// one-sided spectrum, or more of it): even outputs are the 16-point DFT of v,
+// odd outputs the 16-point DFT of v_r exp(SIGN 2 pi i r/32).
+template <int SIGN, int NZ, int Q>
+struct HalfZeroTw {
+    static __device__ __forceinline__ void run(const float2 *v, float2 *b) {
+        if constexpr (Q < NZ) {
+            b[Q] = tw_const<Q, 32, SIGN>(v[Q]);
+            HalfZeroTw<SIGN, NZ, Q + 1>::run(v, b);
+        }
+    }
+};
+template <int SIGN, int NZ = 16>
 __device__ __forceinline__ void dft32_halfzero(float2 *v) {
     float2 a[16], b[16];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) a[i] = v[i];
-    HalfZeroTw<SIGN, 0>::run(v, b);
-    Dft<16, SIGN>::run(a);
-    Dft<16, SIGN>::run(b);
+    for (int i = 0; i < NZ; ++i) a[i] = v[i];
+    HalfZeroTw<SIGN, NZ, 0>::run(v, b);
+    DftLead<16, SIGN, NZ>::run(a);
+    DftLead<16, SIGN, NZ>::run(b);
 #pragma unroll
     for (int p = 0; p < 16; ++p) { v[2 * p] = a[p]; v[2 * p + 1] = b[p]; }
 }
-
 // v[r] *= w^r for r = 1..R-1 (w^r by repeated multiplication)
 template <int R>
 __device__ __forceinline__ void twiddle_powers(float2 *v, float2 w) {

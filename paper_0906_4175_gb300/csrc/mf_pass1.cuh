@@ -135,10 +135,39 @@ __device__ __forceinline__ void dft32_single(float2 *v, float2 x, int rs, float2
 // thread's 16 rows n = t + 32 r of column k1 = tile C + seq (warps skip groups
 // of four rows outside every lane's band), the half-zero radix-32 DFT, and the
 // store into the sequence's shared-memory column sq.  Reads the staged W tile,
-// anchors and q4 terms.  NARROW (bands of a few rows, the chi^2 sub-bands):
+// anchors and q4 terms.  Narrow form (bands of a few rows, the chi^2 sub-bands):
 // where no lane of the warp holds more than one row of the band, the DFT is
 // dft32_single with w from the stage-1 table tw (exp(2 pi i r k / L), row L/64).
-template <int L, int C, int LG1, bool NARROW = false>
+// Leading form (bands that end below fs/8, four of the 16 rows: templates of 8.6 solar
+// masses and more at 4096 Hz): a warp without a bin past row 4, or past row 2,
+// leaves the rows and sums of zeros out; every output is the same.  1-34 solar
+// masses at N = 2^18 .. 2^21, pass 1 per 2^29 samples: 944 us without, 827
+// with it; in a bank of 1-3 solar masses, which has no such warp, the extra code
+// costs 2 % (1016 -> 1035 us), so it is a form of its own.
+template <int NROWS, int T, int C>
+__device__ __forceinline__ void pf_rows(int r0, int seq, int t, int rlo, int rhi, float d, const float2 *wbuf,
+                                        const float4 *abuf, const float *abuf4, float2 *v) {
+#pragma unroll
+    for (int i = 0; i < NROWS; ++i) {
+        const int r = r0 + i, n = t + r * T;
+        const float2 w = wbuf[n * C + seq];
+        const float4 a = abuf[n];
+        const float a4 = abuf4[n];
+        float ph = fmaf(fmaf(fmaf(fmaf(a4, d, a.w), d, a.z), d, a.y), d, a.x);
+        ph -= rintf(ph);
+        float sn, cs;
+        __sincosf(6.283185307179586f * ph, &sn, &cs);
+        const float2 x = make_float2(fmaf(w.x, cs, w.y * sn), fmaf(w.y, cs, -w.x * sn));  // W e^{-i 2 pi ph}
+        v[i] = (r >= rlo && r < rhi) ? x : czero();   // staging outside the band is stale
+    }
+}
+template <int NZ>
+__device__ __forceinline__ void pf_lead(float2 *v, float2 *sq, int t) {
+    dft32_halfzero<+1, NZ>(v);
+#pragma unroll
+    for (int r = 0; r < 32; ++r) sq[spad(32 * t + r)] = v[r];
+}
+template <int L, int C, int LG1, int FORM = kBandPlain>
 __device__ __forceinline__ void pf_stage1(int tile, int seq, int t, int k_lo, int k_hi, int log2D,
                                           const float2 *wbuf, const float4 *abuf, const float *abuf4, float2 *sq,
                                           const float2 *tw = nullptr) {
@@ -155,29 +184,29 @@ __device__ __forceinline__ void pf_stage1(int tile, int seq, int t, int k_lo, in
     const int rhi = k_hi <= k0 ? 0 : min(16, (k_hi - k0 + (1 << LGS) - 1) >> LGS);
     const int wlo = (int)__reduce_min_sync(0xffffffffu, (unsigned)rlo);
     const int whi = (int)__reduce_max_sync(0xffffffffu, (unsigned)rhi);
+    if constexpr (FORM == kBandLead) {
+        if (whi <= 2) {
+            pf_rows<2, T, C>(0, seq, t, rlo, rhi, d, wbuf, abuf, abuf4, v);
+            pf_lead<2>(v, sq, t);
+            return;
+        }
+        if (whi <= 4) {
+            pf_rows<4, T, C>(0, seq, t, rlo, rhi, d, wbuf, abuf, abuf4, v);
+            pf_lead<4>(v, sq, t);
+            return;
+        }
+    }
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
         if (4 * g + 4 > wlo && 4 * g < whi) {   // some lane of the warp has a bin of rows 4g..4g+3
-#pragma unroll
-            for (int r = 4 * g; r < 4 * g + 4; ++r) {
-                const int n = t + r * T;
-                const float2 w = wbuf[n * C + seq];
-                const float4 a = abuf[n];
-                const float a4 = abuf4[n];
-                float ph = fmaf(fmaf(fmaf(fmaf(a4, d, a.w), d, a.z), d, a.y), d, a.x);
-                ph -= rintf(ph);
-                float sn, cs;
-                __sincosf(6.283185307179586f * ph, &sn, &cs);
-                const float2 x = make_float2(fmaf(w.x, cs, w.y * sn), fmaf(w.y, cs, -w.x * sn));  // W e^{-i 2 pi ph}
-                v[r] = (r >= rlo && r < rhi) ? x : czero();   // staging outside the band is stale
-            }
+            pf_rows<4, T, C>(4 * g, seq, t, rlo, rhi, d, wbuf, abuf, abuf4, v + 4 * g);
         } else {
 #pragma unroll
             for (int r = 4 * g; r < 4 * g + 4; ++r) v[r] = czero();
         }
     }
     bool single = false;
-    if constexpr (NARROW) {
+    if constexpr (FORM == kBandNarrow) {
         static_assert(L >= 512, "the row L/64 of the stage-1 table holds the 32nd roots for L >= 512");
         single = __reduce_max_sync(0xffffffffu, (unsigned)(rhi > rlo ? rhi - rlo : 0)) <= 1u;
         if (single) {

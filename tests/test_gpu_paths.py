@@ -247,3 +247,18 @@ def test_scratch_of_threads_and_streams(mf):
     for t in th:
         t.join()
     assert not bad
+
+
+# bands that end below fs/8 (the leading-row form of the staged pass 1): whole and
+# mixed batches against one CTA per tile, which forms every row
+@pytest.mark.parametrize("lg,fs,m", [(16, 16384.0, 3.0), (17, 4096.0, 20.0), (18, 4096.0, 10.0), (19, 4096.0, 16.0),
+                                     (20, 4096.0, 5.0), (20, 8192.0, 8.0), (21, 4096.0, 30.0)])
+def test_leading_bands(mf, monkeypatch, lg, fs, m):
+    r = np.random.default_rng(lg)
+    m1, m2 = r.uniform(0.3 * m, 1.5 * m, (2, 21))
+    bank, seg = mf.Bank(m1, m2), _segment(mf, lg, fs)
+    a = _run(mf, bank, [seg], 4.75)
+    monkeypatch.setenv("MFGB_P1PF", "0")
+    b = _run(mf, bank, [seg], 4.75)
+    assert bank.check() == 0 and a[2] == b[2]
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
