@@ -86,6 +86,7 @@ static int ensure_device_init() {
     std::lock_guard<std::mutex> lk(mu);
     if (std::find(done.begin(), done.end(), dev) != done.end()) return MF_OK;
     MF_CUDA(filter_kernel_attributes());
+    MF_CUDA(group_kernel_attributes());
     MF_CUDA(prep_kernel_attributes());
     MF_CUDA(persist_kernel_attributes());
     MF_CUDA(seq_kernel_attributes());
@@ -256,6 +257,7 @@ struct Scratch {
 
 struct Workspace {
     int64_t exch_elems = 0, n_t = 0, cap = 0, anc_elems = 0, nblk = 0;
+    int n_set = 0;
     UnitInfo *units = nullptr;
     float2 *exch = nullptr;
     float4 *anchors = nullptr;
@@ -729,6 +731,8 @@ constexpr int64_t kScratchBudget = (int64_t)1 << 30;
 // 16-byte planes of an anchor record (and one float, MF_PHASE_ANCHOR)
 static int anchor_planes(const mf_bank_s *b) { return b->params.phase_mode == MF_PHASE_FP64 ? 3 : 1; }
 
+static int64_t exch_budget(const mf_bank_s *b) { return b->tuned_exch > 0 ? b->tuned_exch : kExchBudget; }
+
 static int64_t choose_batch(int64_t N, int64_t n_t, int64_t tuned_exch) {
     int64_t b = (tuned_exch > 0 ? tuned_exch : kExchBudget) / (8 * N);
     if (const char *env = getenv("MFGB_BATCH")) b = atoll(env);
@@ -739,12 +743,13 @@ static int64_t choose_batch(int64_t N, int64_t n_t, int64_t tuned_exch) {
 }
 
 // exch_elems: complex64 entries of the exchange ring (max over the call's
-// segments of batch * N); anc_elems: anchor records (max of batch * anchors)
+// segments of batch * N); anc_elems: anchor records (max of batch * anchors);
+// n_set: segments whose units are held at once
 static int ensure_workspace(mf_bank_s *b, int64_t exch_elems, int64_t cap, int64_t anc_elems, int64_t nblk,
-                            bool capturing) {
+                            int n_set, bool capturing) {
     Workspace &w = b->ws;
     if (w.units && w.exch_elems >= exch_elems && w.n_t >= b->n && w.cap >= cap && w.anc_elems >= anc_elems &&
-        w.nblk >= nblk)
+        w.nblk >= nblk && w.n_set >= n_set)
         return MF_OK;
     if (capturing)
         return set_err(MF_EINVAL, "the workspace must grow: call mf_filter_bank once with these segments and "
@@ -752,9 +757,10 @@ static int ensure_workspace(mf_bank_s *b, int64_t exch_elems, int64_t cap, int64
     const int64_t ne = std::max(w.exch_elems, exch_elems), ncap = std::max(std::max(w.cap, cap), (int64_t)1);
     const int64_t na = std::max(w.anc_elems, anc_elems);
     const int64_t nbl = std::max(w.nblk, nblk);
+    const int ns = std::max(w.n_set, n_set);
     MF_CUDA(cudaDeviceSynchronize());
     w.release();
-    MF_CUDA(dev_malloc(&w.units, sizeof(UnitInfo) * b->n));
+    MF_CUDA(dev_malloc(&w.units, sizeof(UnitInfo) * b->n * ns));
     MF_CUDA(dev_malloc(&w.exch, sizeof(float2) * ne));
     MF_CUDA(dev_malloc(&w.anchors, sizeof(float4) * na));
     MF_CUDA(dev_malloc(&w.anchors4, sizeof(float) * na));
@@ -770,7 +776,7 @@ static int ensure_workspace(mf_bank_s *b, int64_t exch_elems, int64_t cap, int64
     w.counter = &w.fctl->counter;
     w.status = &w.fctl->status;
     MF_CUDA(dev_malloc(&w.ctl, sizeof(unsigned) * (4 + 3 * b->n)));
-    w.exch_elems = ne; w.n_t = b->n; w.cap = ncap; w.anc_elems = na; w.nblk = nbl;
+    w.exch_elems = ne; w.n_t = b->n; w.cap = ncap; w.anc_elems = na; w.nblk = nbl; w.n_set = ns;
     return MF_OK;
 }
 
@@ -947,10 +953,61 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const bool capturing = stream_capturing(st);
     if (capturing && b->prof_on) return set_err(MF_EINVAL, "stage profiling cannot run inside a stream capture");
-    int rc = ensure_workspace(b, exch_elems, trig_cap, anc_elems, nblk, capturing);
+    // Short segments share launches (mf_group.cu): up to 16 at a time, of
+    // together at most four waves of tiles (80 MB of exchange, within L2).  4
+    // segments of 2^12 .. 2^14, 75 templates: 106 us one after the other, 62
+    // grouped.  Alone, or with a wave of tiles or more each, a segment gains
+    // nothing from it.  Stage profiling and the stall hook keep segments apart.
+    const int n_t = (int)b->n;
+    std::vector<FilterGroup> groups;
+    std::vector<char> grouped((size_t)n_seg, 0);
+    if (n_seg > 1 && !b->prof_on && b->stall_unit < 0 && b->params.phase_mode == MF_PHASE_ANCHOR &&
+        b->params.fft_mode == MF_FFT_FP32) {
+        std::vector<int> cand;
+        for (int s = 0; s < n_seg; ++s) {
+            if (group_tiles(segs[s]->log2N, n_t, sm_count()) > 0 && seg_batch[(size_t)s] >= n_t &&
+                !use_persistent(b, segs[s]) && !use_fused(b, segs[s]) &&
+                units_anchors_applies(n_t, b->params.phase_mode, sm_count()))
+                cand.push_back(s);
+        }
+        // the longest first: the tiles of the shortest, below 2^13, are less work and end a launch
+        std::stable_sort(cand.begin(), cand.end(), [&](int x, int y) { return segs[x]->N > segs[y]->N; });
+        int64_t tiles = 0;
+        for (size_t i = 0; i < cand.size() && cand.size() > 1; ++i) {
+            const mf_segment_s *g = segs[cand[i]];
+            const int lgD = choose_log2D(b, g), add = group_tiles(g->log2N, n_t, sm_count());
+            if (groups.empty() || tiles + add > 8 * (int64_t)sm_count() || groups.back().n == kGroupMax ||
+                (groups.back().exch_elems + n_t * g->N) * 8 > exch_budget(b)) {
+                groups.emplace_back();
+                groups.back().n_t = n_t;
+                tiles = 0;
+            }
+            if (!group_add(groups.back(), seg_dev(g, filter_log2n2(b, g)), cand[i], lgD,
+                           (int)anchor_slot_records(g->log2N, lgD)))
+                return set_err(MF_ECUDA, "segs[%d] does not fit its group", cand[i]);
+            tiles += add;
+            grouped[(size_t)cand[i]] = 1;
+        }
+    }
+    int rc = MF_EINVAL;
+    if (!groups.empty()) {
+        int64_t ge = exch_elems, ga = anc_elems, gn = nblk;
+        int n_set = 1;
+        for (const FilterGroup &g : groups) {
+            ge = std::max(ge, g.exch_elems);
+            ga = std::max(ga, g.anc_records);
+            gn = std::max(gn, (g.n_partials + n_t - 1) / n_t);
+            n_set = std::max(n_set, g.n);
+        }
+        rc = ensure_workspace(b, ge, trig_cap, ga, gn, n_set, capturing);
+        if (rc) {   // no room for several segments (or none may be made in a capture): one after the other
+            groups.clear();
+            std::fill(grouped.begin(), grouped.end(), 0);
+        }
+    }
+    if (rc) rc = ensure_workspace(b, exch_elems, trig_cap, anc_elems, nblk, 1, capturing);
     if (rc) return rc;
     Workspace &w = b->ws;
-    const int n_t = (int)b->n;
     // descending-cost unit order (MFGB_UNIT_ORDER=bank keeps bank order); the
     // stall hook names a template, the kernels see its unit position
     const char *uo = getenv("MFGB_UNIT_ORDER");
@@ -963,7 +1020,35 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
         one_stream = one_stream && !use_persistent(b, segs[s]) && !use_fused(b, segs[s]) &&
                      (seg_batch[(size_t)s] >= n_t || b->params.phase_mode == MF_PHASE_FP32);
     ChainScope chain(one_stream);
+    // the first kernel of the call zeroes the control words
+    FilterCtl *clear = w.fctl;
+    auto bind = [&](auto &g) {
+        g.n_seg = n_seg;
+        g.thr = threshold;
+        g.f_low = b->params.f_low;
+        g.tmpl = b->d_tmpl;
+        g.order = unit_order;
+        g.units = w.units;
+        g.anchors = w.anchors;
+        g.anchors4 = w.anchors4;
+        g.exch = w.exch;
+        g.partials = w.partials;
+        g.staged = w.staged;
+        g.keys = w.keys;
+        g.counter = w.counter;
+        g.cap = std::max<int64_t>(trig_cap, 0);
+        g.kl = kl;
+        g.peaks = peaks;
+        g.clear = clear;
+        clear = nullptr;
+    };
+    for (FilterGroup &g : groups) {
+        bind(g);
+        MF_CUDA(launch_group(g, sm_count(), st));
+        count_launches(4);
+    }
     for (int s = 0; s < n_seg; ++s) {
+        if (grouped[(size_t)s]) continue;
         const SegDev sd = seg_dev(segs[s], filter_log2n2(b, segs[s]));
         const int lgD = choose_log2D(b, segs[s]);
         const int man = (int)anchor_slot_records(segs[s]->log2N, lgD);   // records per anchor slot
@@ -991,17 +1076,20 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
                 anc_bytes[(size_t)t] = anchors ? 16.0 * (double)(((hi - 1) >> lgD) - (lo >> lgD) + 1) : 0.0;
             }
         }
-        // the first kernel of the call zeroes the control words; a small bank's
-        // units and anchors come from one launch (stage profiling keeps two)
-        FilterCtl *clear = s == 0 ? w.fctl : nullptr;
+        // a small bank's units and anchors come from one launch (stage profiling keeps two)
         const bool merged = !b->prof_on && !use_persistent(b, segs[s]) && seg_batch[(size_t)s] >= n_t &&
-                            units_anchors_applies(n_t, man, b->params.phase_mode, sm_count());
+                            units_anchors_applies(n_t, b->params.phase_mode, sm_count());
         int pi = prof_begin(b, MF_STAGE_SETUP, 48.0 * n_t, st);
-        if (merged)
-            MF_CUDA(launch_units_anchors(sd, b->d_tmpl, n_t, b->params.f_low, threshold, lgD, unit_order, w.units, man,
-                                         w.anchors, w.anchors4, clear, sm_count(), st));
-        else
+        if (merged) {
+            FilterGroupOf<1> one;
+            one.n_t = n_t;
+            bind(one);
+            group_add(one, sd, s, lgD, man);
+            MF_CUDA(launch_units_anchors(one, sm_count(), st));
+        } else {
             MF_CUDA(launch_units(sd, b->d_tmpl, n_t, b->params.f_low, threshold, lgD, unit_order, w.units, clear, st));
+            clear = nullptr;
+        }
         prof_end(b, pi, st);
         count_launches(1);
         if (use_fused(b, segs[s])) {
@@ -1417,7 +1505,7 @@ extern "C" int mf_debug_status(uint32_t *word, int *enabled) {
     if (r0) return r0;
     MF_CUDA(cudaDeviceSynchronize());
     unsigned all = 0, w = 0;
-    cudaError_t (*readers[])(unsigned *) = {dbg_read_filter, dbg_read_pass1, dbg_read_rows,
+    cudaError_t (*readers[])(unsigned *) = {dbg_read_filter, dbg_read_pass1, dbg_read_rows, dbg_read_group,
                                             dbg_read_persist, dbg_read_chisq, dbg_read_prep, dbg_read_fused};
     for (auto rd : readers) {
         MF_CUDA(rd(&w));

@@ -22,38 +22,6 @@ namespace mf {
 // ---------------------------------------------------------------------------
 // per-unit set-up
 // ---------------------------------------------------------------------------
-// Unit of template t: band, scale factors, threshold, anchor range.
-__device__ UnitInfo unit_info(const SegDev &seg, const double *T, int t, double f_low, float thr, int log2D) {
-    const double N = (double)seg.N, fs = seg.fs;
-    const double fisco = T[TF_FISCO];
-    const double fc = fisco < 0.5 * fs ? fisco : 0.5 * fs;
-    int64_t lo = (int64_t)ceil(f_low * N / fs);
-    int64_t hi = (int64_t)floor(fc * N / fs) + 1;
-    if (lo < 1) lo = 1;
-    if (hi > seg.N / 2) hi = seg.N / 2;
-    if (hi < lo) hi = lo;
-    const double Q = seg.P[hi] - seg.P[lo];              // sum_band f^(-7/3)/S  (Eq. 4 / (4 df A^2))
-    const double rs = sqrt(seg.consts->P_tot / Q);
-    UnitInfo u;
-    u.k_lo = (int32_t)lo;
-    u.k_hi = (int32_t)hi;
-    u.g_lo = (int32_t)(lo >> log2D);
-    u.n_anc = (int32_t)(((hi - 1) >> log2D) - (lo >> log2D) + 1);
-    u.rho_scale = (float)rs;
-    const double th = (double)thr / rs;
-    u.thr2 = (float)(th * th);
-    u.z_scale = (float)(4.0 * seg.df * T[TF_AMP] / seg.consts->alpha);
-    u.tmpl = t;
-    return u;
-}
-
-// the call's control words, zeroed by the first kernel of the call (one block
-// of it calls this; a memset would be one more launch)
-__device__ __forceinline__ void clear_ctl(FilterCtl *ctl) {
-    unsigned *w = reinterpret_cast<unsigned *>(ctl);
-    for (unsigned i = threadIdx.x; i < sizeof(FilterCtl) / 4; i += blockDim.x) w[i] = 0u;
-}
-
 // Unit i of a segment is template order[i] (bank order when order is NULL).
 __global__ void k_units(SegDev seg, const double *__restrict__ tmpl, int n_t, double f_low, float thr,
                         int log2D, const int *__restrict__ order, UnitInfo *__restrict__ units, FilterCtl *clear) {
@@ -65,25 +33,6 @@ __global__ void k_units(SegDev seg, const double *__restrict__ tmpl, int n_t, do
     units[i] = unit_info(seg, tmpl + (int64_t)t * kTmplStride, t, f_low, thr, log2D);
 }
 
-// the anchor records of one unit, blocks bx of nbx
-__device__ __forceinline__ void unit_anchors(const SegDev &seg, const double *T, const UnitInfo &u, int log2D,
-                                             int max_anc, float4 *out, float *out4, int reps, int64_t rep_stride,
-                                             int bx, int nbx) {
-    const double c1 = T[TF_C1], c2 = T[TF_C2], c3 = T[TF_C3], c5 = T[TF_C5];
-    for (int i = bx * blockDim.x + threadIdx.x; i < u.n_anc; i += nbx * blockDim.x) {
-        float4 r;
-        float r4;
-        const int64_t g = (int64_t)u.g_lo + i;
-        anchor_record(c1, c2, c3, c5, g, log2D, seg.df, r, r4);
-        const int64_t a = anchor_slot_index(g, seg.log2N, seg.log2N1, log2D);
-        if (!MF_DBG(a >= 0 && a < max_anc, kDbgAnchor)) continue;
-        for (int k = 0; k < reps; ++k) {
-            out[a + k * rep_stride] = r;
-            out4[a + k * rep_stride] = r4;
-        }
-    }
-}
-
 __global__ void k_anchors(SegDev seg, const double *__restrict__ tmpl, const UnitInfo *__restrict__ units,
                           int unit0, int log2D, int max_anc, float4 *__restrict__ anchors,
                           float *__restrict__ anchors4, int reps) {
@@ -92,27 +41,6 @@ __global__ void k_anchors(SegDev seg, const double *__restrict__ tmpl, const Uni
     const UnitInfo u = units[unit0 + b];
     unit_anchors(seg, tmpl + (int64_t)u.tmpl * kTmplStride, u, log2D, max_anc, anchors + (int64_t)b * max_anc,
                  anchors4 + (int64_t)b * max_anc, reps, (int64_t)gridDim.y * max_anc,   // copy k of slot b: slot b + k n_units
-                 blockIdx.x, gridDim.x);
-}
-
-// k_units and k_anchors of a small bank in one launch: every block of a unit
-// forms its UnitInfo anew (some 60 FP64 operations of one thread), which pays
-// while all blocks are resident at once: two launches of 4 and 7 us, 8 us here.
-__global__ void k_units_anchors(SegDev seg, const double *__restrict__ tmpl, double f_low, float thr, int log2D,
-                                const int *__restrict__ order, UnitInfo *__restrict__ units, int max_anc,
-                                float4 *__restrict__ anchors, float *__restrict__ anchors4, FilterCtl *clear) {
-    __shared__ UnitInfo su;
-    int b = blockIdx.y;
-    chain_wait(b);
-    const int t = order ? order[b] : b;
-    const double *T = tmpl + (int64_t)t * kTmplStride;
-    if (clear && blockIdx.x == 0 && b == 0) clear_ctl(clear);
-    if (threadIdx.x == 0) {
-        su = unit_info(seg, T, t, f_low, thr, log2D);
-        if (blockIdx.x == 0) units[b] = su;
-    }
-    __syncthreads();
-    unit_anchors(seg, T, su, log2D, max_anc, anchors + (int64_t)b * max_anc, anchors4 + (int64_t)b * max_anc, 1, 0,
                  blockIdx.x, gridDim.x);
 }
 
@@ -145,27 +73,6 @@ MF_DEBUG_READER(dbg_read_filter)
 cudaError_t launch_units(const SegDev &seg, const double *tmpl, int n_t, double f_low, float thr, int log2D,
                          const int *order, UnitInfo *units, FilterCtl *clear, cudaStream_t st) {
     return launch(k_units, dim3((n_t + 255) / 256), 256, 0, st, seg, tmpl, n_t, f_low, thr, log2D, order, units, clear);
-}
-
-// Blocks per unit of the merged launch, or 0 where the two launches are better:
-// at most eight blocks of 256 threads per SM.
-static int units_anchors_blocks(int n_t, int max_anc, int n_sm) {
-    const int most = 8 * n_sm / (n_t > 0 ? n_t : 1);
-    const int want = (max_anc + 255) / 256;
-    return most < 1 ? 0 : (want < most ? want : most);
-}
-
-bool units_anchors_applies(int n_t, int max_anc, int phase_mode, int n_sm) {
-    return phase_mode == MF_PHASE_ANCHOR && units_anchors_blocks(n_t, max_anc, n_sm) > 0;
-}
-
-cudaError_t launch_units_anchors(const SegDev &seg, const double *tmpl, int n_t, double f_low, float thr, int log2D,
-                                 const int *order, UnitInfo *units, int max_anc, float4 *anchors, float *anchors4,
-                                 FilterCtl *clear, int n_sm, cudaStream_t st) {
-    const int gx = units_anchors_blocks(n_t, max_anc, n_sm);
-    if (gx < 1) return cudaErrorInvalidValue;
-    return launch(k_units_anchors, dim3(gx, n_t), 256, 0, st, seg, tmpl, f_low, thr, log2D, order, units, max_anc, anchors,
-                  anchors4, clear);
 }
 
 cudaError_t launch_anchors(const SegDev &seg, const double *tmpl, const UnitInfo *units, int unit0, int n_units,
@@ -303,36 +210,9 @@ cudaError_t filter_kernel_attributes() {
 __global__ void k_reduce_peaks(const UnitInfo *__restrict__ units, int n_units, const float4 *__restrict__ partials,
                                int nblk, int seg_idx, int n_seg, mf_peak *__restrict__ peaks) {
     int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
     chain_wait(warp);
     if (warp >= n_units) return;
-    float bp = -1.f;
-    int bj = 0x7fffffff;
-    float bx = 0.f, by = 0.f;
-    const float4 *pp = partials + (int64_t)warp * nblk;
-    for (int i = lane; i < nblk; i += 32) {
-        const float4 c = pp[i];
-        const int cj = __float_as_int(c.y);
-        if (c.x > bp || (c.x == bp && cj < bj)) { bp = c.x; bj = cj; bx = c.z; by = c.w; }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float op = __shfl_xor_sync(0xffffffffu, bp, o);
-        const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
-        const float ox = __shfl_xor_sync(0xffffffffu, bx, o);
-        const float oy = __shfl_xor_sync(0xffffffffu, by, o);
-        if (op > bp || (op == bp && oj < bj)) { bp = op; bj = oj; bx = ox; by = oy; }
-    }
-    if (lane == 0) {
-        const UnitInfo u = units[warp];
-        mf_peak pk;
-        pk.rho = sqrtf(bp) * u.rho_scale;
-        pk.j = bj;
-        pk.z_re = bx * u.z_scale;
-        pk.z_im = by * u.z_scale;
-        if (MF_DBG(u.tmpl >= 0 && u.tmpl < n_units && seg_idx < n_seg, kDbgOut))
-            peaks[(int64_t)u.tmpl * n_seg + seg_idx] = pk;
-    }
+    unit_peak(units[warp], n_units, partials + (int64_t)warp * nblk, nblk, seg_idx, n_seg, peaks);
 }
 
 cudaError_t launch_reduce_peaks(const SegDev &seg, const UnitInfo *units, int n_units, const float4 *partials,

@@ -85,7 +85,7 @@ struct TemplateSrc {
     unsigned *rel = nullptr;   // deferred release (persistent scheduler), done by thread 0 once loads are in flight
     __device__ TemplateSrc(const Params &pp, int tl, int un, int sl, void *scratch)
         : p(pp), tile(tl), unit(un), slot(sl), sa((float4 *)scratch), sa4((float *)((float4 *)scratch + L / 2)) {}
-    // All threads of the block call load() (it contains a block barrier).
+    // All C L/32 threads of the tile call load() (it contains a block barrier).
     __device__ __forceinline__ void load(int seq, int t, float2 *v) const {
         constexpr int T = L / 32;
         const UnitInfo u = p.units[unit];
@@ -114,7 +114,7 @@ struct TemplateSrc {
             const int gbase = gcol - u.g_lo;
             const float4 *acol = anc0 + ((int64_t)gcol << (LGL - 1));
             const float *acol4 = anc40 + ((int64_t)gcol << (LGL - 1));
-            for (int n = threadIdx.x; n < L / 2; n += blockDim.x) {
+            for (int n = threadIdx.x; n < L / 2; n += C * T) {
                 const int a = gbase + n * gstep;
                 if (a >= 0 && a < u.n_anc &&
                     MF_DBG(((int64_t)gcol << (LGL - 1)) + n < p.anc_stride, kDbgAnchor)) {
@@ -259,7 +259,7 @@ struct TemplateSrc64 {
     float4 *sa;
     __device__ TemplateSrc64(const Params &pp, int tl, int un, int sl, void *scratch)
         : p(pp), tile(tl), unit(un), slot(sl), sa((float4 *)scratch) {}
-    // All threads of the block call load() (it contains a block barrier).
+    // All C L/32 threads of the tile call load() (it contains a block barrier).
     __device__ __forceinline__ void load(int seq, int t, float2 *v) const {
         constexpr int T = L / 32;
         constexpr int LGL = cx_ilog2(L);
@@ -283,7 +283,7 @@ struct TemplateSrc64 {
             const int gcol = (tile * C) >> p.log2D;
             const int gbase = gcol - u.g_lo;
             const float4 *acol = anc + ((int64_t)gcol << (LGL - 1));
-            for (int n = threadIdx.x; n < L / 2; n += blockDim.x) {
+            for (int n = threadIdx.x; n < L / 2; n += C * T) {
                 const int a = gbase + n * gstep;
                 if (a >= 0 && a < u.n_anc && MF_DBG(((int64_t)gcol << (LGL - 1)) + n < p.anc_stride, kDbgAnchor)) {
 #pragma unroll
@@ -478,7 +478,7 @@ struct RhoSink {
         if (lane == 0) red[warp] = make_float4(bp, __int_as_float(bj), bz.x, bz.y);
         __syncthreads();
         if (threadIdx.x == 0) {
-            const int nw = blockDim.x >> 5;
+            constexpr int nw = C * (L / 32) / 32;
             float4 best = red[0];
             for (int w = 1; w < nw; ++w) {
                 const float4 c = red[w];
@@ -489,5 +489,91 @@ struct RhoSink {
         }
     }
 };
+
+// ---------------------------------------------------------------------------
+// per-unit set-up and peaks
+// ---------------------------------------------------------------------------
+// Unit of template t: band, scale factors, threshold, anchor range.
+__device__ __forceinline__ UnitInfo unit_info(const SegDev &seg, const double *T, int t, double f_low, float thr, int log2D) {
+    const double N = (double)seg.N, fs = seg.fs;
+    const double fisco = T[TF_FISCO];
+    const double fc = fisco < 0.5 * fs ? fisco : 0.5 * fs;
+    int64_t lo = (int64_t)ceil(f_low * N / fs);
+    int64_t hi = (int64_t)floor(fc * N / fs) + 1;
+    if (lo < 1) lo = 1;
+    if (hi > seg.N / 2) hi = seg.N / 2;
+    if (hi < lo) hi = lo;
+    const double Q = seg.P[hi] - seg.P[lo];              // sum_band f^(-7/3)/S  (Eq. 4 / (4 df A^2))
+    const double rs = sqrt(seg.consts->P_tot / Q);
+    UnitInfo u;
+    u.k_lo = (int32_t)lo;
+    u.k_hi = (int32_t)hi;
+    u.g_lo = (int32_t)(lo >> log2D);
+    u.n_anc = (int32_t)(((hi - 1) >> log2D) - (lo >> log2D) + 1);
+    u.rho_scale = (float)rs;
+    const double th = (double)thr / rs;
+    u.thr2 = (float)(th * th);
+    u.z_scale = (float)(4.0 * seg.df * T[TF_AMP] / seg.consts->alpha);
+    u.tmpl = t;
+    return u;
+}
+
+// the call's control words, zeroed by the first kernel of the call (one block
+// of it calls this; a memset would be one more launch)
+__device__ __forceinline__ void clear_ctl(FilterCtl *ctl) {
+    unsigned *w = reinterpret_cast<unsigned *>(ctl);
+    for (unsigned i = threadIdx.x; i < sizeof(FilterCtl) / 4; i += blockDim.x) w[i] = 0u;
+}
+
+// the anchor records of one unit, blocks bx of nbx
+__device__ __forceinline__ void unit_anchors(const SegDev &seg, const double *T, const UnitInfo &u, int log2D,
+                                             int max_anc, float4 *out, float *out4, int reps, int64_t rep_stride,
+                                             int bx, int nbx) {
+    const double c1 = T[TF_C1], c2 = T[TF_C2], c3 = T[TF_C3], c5 = T[TF_C5];
+    for (int i = bx * blockDim.x + threadIdx.x; i < u.n_anc; i += nbx * blockDim.x) {
+        float4 r;
+        float r4;
+        const int64_t g = (int64_t)u.g_lo + i;
+        anchor_record(c1, c2, c3, c5, g, log2D, seg.df, r, r4);
+        const int64_t a = anchor_slot_index(g, seg.log2N, seg.log2N1, log2D);
+        if (!MF_DBG(a >= 0 && a < max_anc, kDbgAnchor)) continue;
+        for (int k = 0; k < reps; ++k) {
+            out[a + k * rep_stride] = r;
+            out4[a + k * rep_stride] = r4;
+        }
+    }
+}
+
+// The peak of one unit from its pass-2 partials, by one warp: the loudest
+// sample, the first of equal ones.
+__device__ __forceinline__ void unit_peak(const UnitInfo &u, int n_all, const float4 *pp, int nblk, int seg_idx,
+                                          int n_seg, mf_peak *peaks) {
+    const int lane = threadIdx.x & 31;
+    float bp = -1.f;
+    int bj = 0x7fffffff;
+    float bx = 0.f, by = 0.f;
+    for (int i = lane; i < nblk; i += 32) {
+        const float4 c = pp[i];
+        const int cj = __float_as_int(c.y);
+        if (c.x > bp || (c.x == bp && cj < bj)) { bp = c.x; bj = cj; bx = c.z; by = c.w; }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float op = __shfl_xor_sync(0xffffffffu, bp, o);
+        const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+        const float ox = __shfl_xor_sync(0xffffffffu, bx, o);
+        const float oy = __shfl_xor_sync(0xffffffffu, by, o);
+        if (op > bp || (op == bp && oj < bj)) { bp = op; bj = oj; bx = ox; by = oy; }
+    }
+    if (lane == 0) {
+        mf_peak pk;
+        pk.rho = sqrtf(bp) * u.rho_scale;
+        pk.j = bj;
+        pk.z_re = bx * u.z_scale;
+        pk.z_im = by * u.z_scale;
+        if (MF_DBG(u.tmpl >= 0 && u.tmpl < n_all && seg_idx < n_seg, kDbgOut))
+            peaks[(int64_t)u.tmpl * n_seg + seg_idx] = pk;
+    }
+}
 
 }  // namespace mf

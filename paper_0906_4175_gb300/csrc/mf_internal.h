@@ -129,6 +129,7 @@ __device__ __forceinline__ bool mf_dbg_ok(bool c, unsigned bit) {
 cudaError_t dbg_read_filter(unsigned *w);
 cudaError_t dbg_read_pass1(unsigned *w);
 cudaError_t dbg_read_rows(unsigned *w);
+cudaError_t dbg_read_group(unsigned *w);
 cudaError_t dbg_read_persist(unsigned *w);
 cudaError_t dbg_read_chisq(unsigned *w);
 cudaError_t dbg_read_prep(unsigned *w);
@@ -216,11 +217,6 @@ cudaError_t launch_inverse_real_fft(const float2 *Y, int64_t N, double scale, fl
 struct FilterCtl;
 cudaError_t launch_units(const SegDev &seg, const double *tmpl, int n_t, double f_low, float thr,
                          int log2D, const int *order, UnitInfo *units, FilterCtl *clear, cudaStream_t st);
-// units and the anchors of all of them in one launch (small banks, MF_PHASE_ANCHOR)
-bool units_anchors_applies(int n_t, int max_anc, int phase_mode, int n_sm);
-cudaError_t launch_units_anchors(const SegDev &seg, const double *tmpl, int n_t, double f_low, float thr, int log2D,
-                                 const int *order, UnitInfo *units, int max_anc, float4 *anchors, float *anchors4,
-                                 FilterCtl *clear, int n_sm, cudaStream_t st);
 cudaError_t launch_anchors(const SegDev &seg, const double *tmpl, const UnitInfo *units, int unit0,
                            int n_units, int log2D, int max_anc, float4 *anchors, float *anchors4, int phase_mode,
                            cudaStream_t st, int reps = 1);
@@ -291,6 +287,53 @@ struct FilterCtl {
     int pad;
     SortCtl sort;
 };
+// Segments of one filter call that share launches (mf_group.cu), passed to the
+// kernels by value.  Offsets into the call's workspace are per segment.  CAP 1:
+// the units and anchors of one segment (3 KB of parameters are 0.6 us a launch).
+constexpr int kGroupMax = 16;
+struct GroupSeg {
+    SegDev seg;
+    int seg_idx, log2D, max_anc, anc_blocks;   // anc_blocks: blocks per unit of k_units_anchors
+    int unit0, tiles1, tiles2, pad;            // first unit; tiles per unit of the two passes
+    int64_t anc0, exch0, part0;
+};
+template <int CAP>
+struct FilterGroupOf {
+    GroupSeg s[CAP];
+    int end_anc[CAP], end1[CAP], end2[CAP];   // running block counts of the launches
+    int n = 0, n_t = 0, n_seg = 0;
+    float thr = 0.f;
+    double f_low = 0.0;
+    const double *tmpl = nullptr;
+    const int *order = nullptr;
+    UnitInfo *units = nullptr;
+    float4 *anchors = nullptr;
+    float *anchors4 = nullptr;
+    float2 *exch = nullptr;
+    float4 *partials = nullptr;
+    mf_trigger *staged = nullptr;
+    uint64_t *keys = nullptr;
+    unsigned long long *counter = nullptr;
+    int64_t cap = 0;
+    KeyLayout kl = {};
+    mf_peak *peaks = nullptr;
+    FilterCtl *clear = nullptr;
+    int64_t anc_records = 0, exch_elems = 0, n_partials = 0;   // workspace the group takes
+};
+using FilterGroup = FilterGroupOf<kGroupMax>;
+static_assert(sizeof(FilterGroup) <= 4000, "kernel parameter space");
+// tiles of 8192 samples of a segment that may be grouped, or 0: N <= 2^16 and
+// at most one wave of tiles (2 per SM)
+int group_tiles(int log2N, int n_t, int n_sm);
+template <int CAP>
+bool group_add(FilterGroupOf<CAP> &p, const SegDev &seg, int seg_idx, int log2D, int max_anc);   // p.n_t is set
+cudaError_t launch_group(FilterGroup &p, int n_sm, cudaStream_t st);   // units, anchors, passes and peaks
+// units and the anchors of all of them in one launch (small banks, MF_PHASE_ANCHOR)
+bool units_anchors_applies(int n_t, int phase_mode, int n_sm);
+template <int CAP>
+cudaError_t launch_units_anchors(FilterGroupOf<CAP> &p, int n_sm, cudaStream_t st);
+cudaError_t group_kernel_attributes();
+
 constexpr int kSortTile = 4096;   // keys per tile of a sort of more than 8192 keys
 // one kernel; ctl zeroed.  (mf_sort.cuh)
 cudaError_t launch_sort_triggers(const unsigned long long *counter, int64_t cap, int key_bits,

@@ -97,6 +97,57 @@ def test_trigger_order(mf, lg, n, segs):
         assert np.array_equal(t["z_im"].reshape(n, segs, N)[:, s].ravel(), one["z_im"])
 
 
+# short segments share launches (16 at most, four waves of tiles): as each alone,
+# with longer segments between them, one wave of tiles and one tile more, and
+# trigger keys of more than 32 bits
+@pytest.mark.parametrize("lgs,n,thr", [((10, 11, 12, 13, 14, 15, 16), 3, 4.0), ((12, 13, 13, 14), 75, 4.5),
+                                       ((13, 17, 10, 20, 16), 5, 4.5), ((13, 13), 304, 4.75), ((13, 13), 305, 4.75),
+                                       ((16, 16, 15), 38, 4.75), ((14,) * 9, 152, 4.75), ((10,) * 33, 2, 3.5),
+                                       ((20,) + (10,) * 1024, 3, 4.0)])
+def test_short_segments_together(mf, lgs, n, thr):
+    bank = mf.Bank(*_masses(n))
+    pool = {}
+    for i, lg in enumerate(lgs):
+        if (lg, i % 5) not in pool:
+            pool[lg, i % 5] = _segment(mf, lg, seed=i % 5)
+    segs = [pool[lg, i % 5] for i, lg in enumerate(lgs)]
+    peaks, trig, nt = mf.filter_bank(bank, segs, thr, trig_cap=1 << 20)
+    assert bank.check() == 0
+    peaks, trig = peaks.cpu().numpy().view(np.uint8).reshape(n, len(segs), -1), mf.triggers_to_numpy(trig, nt)
+    key = (trig["tmpl"].astype(np.int64) * len(segs) + trig["seg"]) << 22 | trig["j"]
+    assert np.all(np.diff(key) > 0)
+    one, alone = mf.Bank(*_masses(n)), {}
+    for i, s in enumerate(segs):
+        if id(s) not in alone:
+            p1, t1, n1 = mf.filter_bank(one, [s], thr, trig_cap=1 << 20)
+            alone[id(s)] = p1.cpu().numpy().view(np.uint8).reshape(n, -1).copy(), mf.triggers_to_numpy(t1, n1).copy()
+        p1, t1 = alone[id(s)]
+        mine = trig[trig["seg"] == i]
+        assert np.array_equal(peaks[:, i], p1) and mine.size == t1.size
+        for f in ("tmpl", "j", "rho", "z_re", "z_im"):
+            assert np.array_equal(mine[f], t1[f]), f
+
+
+# a capture whose workspace was made by calls on single segments takes them one by one
+def test_short_segments_in_a_capture(mf):
+    import torch
+    bank, segs = mf.Bank(*_masses(20)), [_segment(mf, lg) for lg in (12, 15, 13)]
+    ref = _run(mf, mf.Bank(*_masses(20)), segs, 4.25)
+    for warm in ([[s] for s in segs], [segs]):
+        for w in warm:
+            mf.filter_bank(bank, w, 4.25, trig_cap=1 << 20)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            out = mf.filter_bank(bank, segs, 4.25, trig_cap=1 << 20)
+        for _ in range(2):
+            g.replay()
+            torch.cuda.synchronize()
+            nt = int(out[2][0])
+            assert nt == ref[2] and np.array_equal(out[0].cpu().numpy().view(np.uint8), ref[0])
+            assert np.array_equal(out[1][:nt].cpu().numpy().view(np.uint8), ref[1])
+
+
 def test_trigger_overflow_of_both_sorts(mf):
     bank, seg = mf.Bank(*_masses(9)), _segment(mf, 12)
     full = mf.triggers_to_numpy(*mf.filter_bank(bank, [seg], 0.0, trig_cap=9 << 12)[1:])
