@@ -142,28 +142,43 @@ struct TemplateSrc {
                 v[r] = in[r] ? x : czero();
             }
         } else {
+            // Several anchor groups per row of the tile (short segments): each
+            // element reads its record.  The records of four rows are loaded
+            // before the first is used: a row at a time, one after the other
+            // behind its test, is 16 trips to L2 a tile (16 templates at N =
+            // 2^16, D = 16, all tiles resident: 11.1 us, 9.4 so).
             release_hook(rel);
             const int half = D >> 1;
 #pragma unroll
-            for (int r = 0; r < 16; ++r) {
-                if (!__any_sync(0xffffffffu, in[r])) {
-                    v[r] = czero();
+            for (int c = 0; c < 16; c += 4) {
+                if (!__any_sync(0xffffffffu, in[c] || in[c + 1] || in[c + 2] || in[c + 3])) {
+#pragma unroll
+                    for (int r = c; r < c + 4; ++r) v[r] = czero();
                     continue;
                 }
-                const int k = k0 + ((r * T) << LG1);
-                const int kk = in[r] ? k : u.k_lo;
-                const int g = kk >> p.log2D;
-                int64_t ai = anchor_slot_index(g, LGL + LG1, LG1, p.log2D);
-                if (!MF_DBG(ai >= 0 && ai < p.anc_stride, kDbgAnchor)) ai = 0;
-                const float4 a = __ldcg(&anc0[ai]);
-                const float a4 = __ldcg(&anc40[ai]);
-                const float d = (float)(kk - ((g << p.log2D) + half));
-                float ph = fmaf(fmaf(fmaf(fmaf(a4, d, a.w), d, a.z), d, a.y), d, a.x);
-                ph -= rintf(ph);
-                float sn, cs;
-                __sincosf(6.283185307179586f * ph, &sn, &cs);
-                const float2 x = make_float2(fmaf(w[r].x, cs, w[r].y * sn), fmaf(w[r].y, cs, -w[r].x * sn));
-                v[r] = in[r] ? x : czero();
+                float4 a[4];
+                float a4[4], d[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int k = k0 + (((c + i) * T) << LG1);
+                    const int kk = in[c + i] ? k : u.k_lo;
+                    const int g = kk >> p.log2D;
+                    int64_t ai = anchor_slot_index(g, LGL + LG1, LG1, p.log2D);
+                    if (!MF_DBG(ai >= 0 && ai < p.anc_stride, kDbgAnchor)) ai = 0;
+                    a[i] = __ldcg(&anc0[ai]);
+                    a4[i] = __ldcg(&anc40[ai]);
+                    d[i] = (float)(kk - ((g << p.log2D) + half));
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = c + i;
+                    float ph = fmaf(fmaf(fmaf(fmaf(a4[i], d[i], a[i].w), d[i], a[i].z), d[i], a[i].y), d[i], a[i].x);
+                    ph -= rintf(ph);
+                    float sn, cs;
+                    __sincosf(6.283185307179586f * ph, &sn, &cs);
+                    const float2 x = make_float2(fmaf(w[r].x, cs, w[r].y * sn), fmaf(w[r].y, cs, -w[r].x * sn));
+                    v[r] = in[r] ? x : czero();
+                }
             }
         }
     }

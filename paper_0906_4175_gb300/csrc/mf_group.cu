@@ -109,12 +109,13 @@ __device__ __forceinline__ void group_dispatch(int log2N, const Op &op) {
 template <int CAP>
 __global__ void __launch_bounds__(kGroupThreads) k_units_anchors(__grid_constant__ const FilterGroupOf<CAP> p) {
     __shared__ UnitInfo su;
-    int b = blockIdx.x;
-    chain_wait(b);
-    if (p.clear && b == 0) clear_ctl(p.clear);
-    const int s = group_find(p.end_anc, p.n, b);
+    int b = blockIdx.x, i = blockIdx.y;
+    chain_wait(b, i);
+    if (p.clear && b == 0 && i == 0) clear_ctl(p.clear);
+    const int s = CAP > 1 ? group_find(p.end_anc, p.n, b) : 0;
     const GroupSeg &g = p.s[s];
-    const int i = b / g.anc_blocks, bx = b - i * g.anc_blocks;
+    if (CAP > 1) i = b / g.anc_blocks;
+    const int bx = CAP > 1 ? b - i * g.anc_blocks : b;
     const int t = p.order ? p.order[i] : i;
     const double *T = p.tmpl + (int64_t)t * kTmplStride;
     if (threadIdx.x == 0) {
@@ -207,7 +208,7 @@ cudaError_t launch_units_anchors(FilterGroupOf<CAP> &p, int n_sm, cudaStream_t s
         g.anc_blocks = std::min(most, std::max(coarse, std::min(fine, fill)));
         p.end_anc[i] = blocks += p.n_t * g.anc_blocks;
     }
-    return launch(k_units_anchors<CAP>, dim3(blocks), kGroupThreads, 0, st, p);
+    return launch(k_units_anchors<CAP>, CAP > 1 ? dim3(blocks) : dim3(p.s[0].anc_blocks, p.n_t), kGroupThreads, 0, st, p);
 }
 template cudaError_t launch_units_anchors(FilterGroupOf<1> &, int, cudaStream_t);
 
