@@ -1382,7 +1382,7 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
         }
         if (e == cudaSuccess)
             e = launch_pass1(sd, bu, 0, (p + 1) * nb, lgD, man, anc, anc4, exch, b->params.phase_mode, b->d_tmpl,
-                             p1_form(b), b->chi_status, b->spin_limit, st, rows ? kBandNarrow : kBandPlain, nb);
+                             p1_form(b), b->chi_status, b->spin_limit, st, kBandNarrow, nb);
         if (e == cudaSuccess)
             e = rows ? launch_chisq_rows(sd, exch, full, (int)u0, nb, p, chisq, b->chi_status, b->spin_limit,
                                          (int)b->stall_unit, sm_count(), st)

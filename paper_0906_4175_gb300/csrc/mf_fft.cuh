@@ -444,6 +444,42 @@ struct uses_split_tw { static constexpr bool value = false; };
 template <class T>
 struct uses_split_tw<T, decltype((void)T::kSplitTw, void())> { static constexpr bool value = T::kSplitTw; };
 
+// 32-point DFT X_q = sum_r v_r e^{2 pi i r q / 32} of a vector whose only
+// non-zero entry is x at r = rs < 16; roots: e^{2 pi i k / 64}, k < 32.  X_q =
+// x w^q, w = e^{2 pi i rs / 32}, for q < 8 from w, w^2 and w^4, three products at
+// most (a running product of seven doubles chi^2's distance from 64 bits, a root
+// for every q costs pass 1 of the chi^2 sub-bands 1 %), then X_{q+8} = i^rs X_q
+// and X_{q+16} = (-1)^rs X_q, both exact.
+__device__ __forceinline__ void dft32_single(float2 *v, float2 x, int rs, const float2 *roots) {
+    float2 w[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int e = rs << i;
+        w[i] = roots[2 * (e & 15)];   // half the circle
+        if (e & 16) w[i] = make_float2(-w[i].x, -w[i].y);
+    }
+    v[0] = x;
+    v[1] = cmul(x, w[0]);
+    v[2] = cmul(x, w[1]);
+    v[3] = cmul(v[1], w[1]);
+#pragma unroll
+    for (int q = 4; q < 8; ++q) v[q] = cmul(v[q - 4], w[2]);
+    const int k = rs & 3;   // i^rs = c + i s
+    const float c = k == 0 ? 1.f : (k == 2 ? -1.f : 0.f), s = k == 1 ? 1.f : (k == 3 ? -1.f : 0.f);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q + 8] = make_float2(c * v[q].x - s * v[q].y, c * v[q].y + s * v[q].x);
+    const float sg = (rs & 1) ? -1.f : 1.f;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) v[q + 16] = make_float2(sg * v[q].x, sg * v[q].y);
+}
+
+// Sources of narrow bands (kNarrow): after load(), single says that no lane of
+// the warp holds more than one non-zero input, v[0] is it and rs its place.
+template <class T, class = void>
+struct is_narrow { static constexpr bool value = false; };
+template <class T>
+struct is_narrow<T, decltype((void)&T::single, void())> { static constexpr bool value = true; };
+
 // Full CTA FFT.  tw: the TwTable<L> twiddles in shared memory, filled and
 // made visible before the call (or filled before it with no intervening
 // shared-memory write, the first stage barrier publishes them).
@@ -466,7 +502,10 @@ __device__ __forceinline__ void cta_fft(float2 *smem, const float2 *tw, Src &src
     {
         float2 v[32];
         src.load(seq, t, v);
-        if constexpr (Src::kHalfZero) dft32_halfzero<SIGN>(v);
+        if constexpr (is_narrow<Src>::value) {
+            if (src.single) dft32_single(v, v[0], src.rs, g_tw_tables + tw_offset<64>() + 32);   // row 1 of that table
+            else dft32_halfzero<SIGN>(v);
+        } else if constexpr (Src::kHalfZero) dft32_halfzero<SIGN>(v);
         else Dft<32, SIGN>::run(v);
         if constexpr (S::NST == 1) {
             snk.template store<32>(seq, t, T, v);

@@ -100,6 +100,7 @@ struct Pass1Op {
     float2 *exch;
     const double *tmpl;
     int anc_slots;
+    bool narrow;
     cudaStream_t st;
     template <int N2, int N1>
     cudaError_t run() {
@@ -115,6 +116,8 @@ struct Pass1Op {
             return run_pass<N2, C, true, +1, TemplateSrc64<N2, C, cx_ilog2(N1)>, ExchSink<N2, C, +1, cx_ilog2(N1)>>(grid, sp, kp, st, unit0);
         }
         typename TemplateSrc<N2, C, cx_ilog2(N1)>::Params sp{seg.W, units, anchors, anchors4, max_anc, log2D, anc_slots};
+        if (narrow)
+            return run_pass<N2, C, true, +1, TemplateSrcNarrow<N2, C, cx_ilog2(N1)>, ExchSink<N2, C, +1, cx_ilog2(N1)>>(grid, sp, kp, st, unit0);
         return run_pass<N2, C, true, +1, TemplateSrc<N2, C, cx_ilog2(N1)>, ExchSink<N2, C, +1, cx_ilog2(N1)>>(grid, sp, kp, st, unit0);
     }
 };
@@ -159,6 +162,7 @@ struct AttrOp {
         constexpr int C2 = seqs_per_cta<N1>(N2);
         cudaError_t e;
         if ((e = set_pass_attrs<N2, C1, true, +1, TemplateSrc<N2, C1, cx_ilog2(N1)>, ExchSink<N2, C1, +1, cx_ilog2(N1)>>())) return e;
+        if ((e = set_pass_attrs<N2, C1, true, +1, TemplateSrcNarrow<N2, C1, cx_ilog2(N1)>, ExchSink<N2, C1, +1, cx_ilog2(N1)>>())) return e;
         if ((e = set_pass_attrs<N2, C1, true, +1, TemplateSrcF32<N2, C1, cx_ilog2(N1)>, ExchSink<N2, C1, +1, cx_ilog2(N1)>>())) return e;
         if ((e = set_pass_attrs<N2, C1, true, +1, TemplateSrc64<N2, C1, cx_ilog2(N1)>, ExchSink<N2, C1, +1, cx_ilog2(N1)>>())) return e;
         return set_pass_attrs<N1, C2, false, +1, RowSrc<N1, C2>, RhoSink<N1, C2>>();
@@ -173,7 +177,7 @@ cudaError_t launch_pass1(const SegDev &seg, const UnitInfo *units, int unit0, in
     if (p1_form != 1 && pass1_pf_applies(seg.log2N, seg.log2N2, log2D, phase_mode))
         return launch_pass1_pf(seg, units, unit0, n_units, log2D, max_anc, anchors, anchors4, exch, p1_form == 2,
                                status, spin_limit, st, form);
-    Pass1Op op{seg, units, unit0, n_units, log2D, max_anc, phase_mode, anchors, anchors4, exch, tmpl, anc_slots, st};
+    Pass1Op op{seg, units, unit0, n_units, log2D, max_anc, phase_mode, anchors, anchors4, exch, tmpl, anc_slots, form == kBandNarrow, st};
     return dispatch_split2(seg.log2N, seg.log2N2, op);
 }
 

@@ -236,11 +236,12 @@ cudaError_t launch_pass1(const SegDev &seg, const UnitInfo *units, int unit0, in
 // anc_slots > 0: unit slot i reads anchor slot i mod anc_slots (the per-tile
 // form only; the persistent form reads slot i).
 // form: a hint on the bands.  kBandNarrow, bands of a few rows per column (the
-// chi^2 sub-bands): the staged form then starts a column with a cheaper first
-// stage wherever each lane of a warp holds at most one row of the band (rounding
-// differs from the half-zero DFT, within the FP32 error of the transform).
+// chi^2 sub-bands): the staged form (N2 >= 512) and the per-tile form then start a
+// column with a cheaper first stage wherever each lane of a warp (a tile) holds
+// at most one row of the band (rounding differs from the half-zero DFT, within the
+// FP32 error of the transform).
 // kBandLead, bands that end below fs / 8: the staged form leaves out the rows and
-// sums of zeros (bit-identical).  Other forms of the kernel ignore them.
+// sums of zeros (bit-identical).  Where a form does not apply it is ignored.
 cudaError_t launch_pass2(const SegDev &seg, const UnitInfo *units, int unit0, int n_units,
                          const float2 *exch, float4 *partials, int seg_idx, KeyLayout kl,
                          mf_trigger *staged, uint64_t *keys, unsigned long long *counter, int64_t cap,
