@@ -1386,7 +1386,7 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
         if (e == cudaSuccess)
             e = rows ? launch_chisq_rows(sd, exch, full, (int)u0, nb, p, chisq, b->chi_status, b->spin_limit,
                                          (int)b->stall_unit, sm_count(), st)
-                     : launch_chisq_tiles(sd, exch, full, (int)u0, nb, p, chisq, st);
+                     : launch_chisq_tiles(sd, exch, full, (int)u0, nb, p, chisq, sm_count(), st);
         launches += 2;
     }
     sc.free(st);

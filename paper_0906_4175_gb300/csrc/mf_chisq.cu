@@ -12,7 +12,10 @@
 // the sub-band only, column IFFTs) into its own exchange; one kernel then runs
 // the row IFFTs of all p + 1 bands, summing |raw_l|^2 in registers and turning
 // the sum into chi^2 at the full band.  Neither z_l nor z is stored.
+#include <cooperative_groups.h>
+
 #include <algorithm>
+#include <type_traits>
 
 #include "mf_filter.cuh"
 
@@ -72,7 +75,7 @@ __global__ void k_chisq_units(SegDev seg, const UnitInfo *__restrict__ all, int 
 // per lane).  One launch per batch instead of one per sub-band, and no
 // accumulator in memory: 16 templates at N = 2^16, p = 16 took 17 pass-1 and
 // 17 pass-2 launches of 7 us each, every one a fraction of a wave: 330 us a
-// call, 151 us now.
+// call, 104 us now.
 // ---------------------------------------------------------------------------
 struct ChiTilesParams {
     const float2 *exch;
@@ -84,65 +87,97 @@ struct ChiTilesParams {
 
 // rows of one sub-band; from the second sub-band on, the sequences' shared
 // memory is free only once every thread has read its last stage
-template <int L, int C>
+template <int L, int C, class Sync>
 struct ChiTileSrc {
     static constexpr bool kHalfZero = false;
     const RowSrc<L, C> rows;
     const bool again;
     __device__ __forceinline__ void load(int seq, int t, float2 *v) const {
         rows.load(seq, t, v);
-        if (again) __syncthreads();
+        if (again) Sync::sync();
     }
 };
+struct ChiWarpSync {
+    static __device__ __forceinline__ void sync() { __syncwarp(); }
+};
 
-// |raw_l|^2 of the thread's 32 outputs summed over l < p; chi^2 at l = p
+// p |raw_l|^2 of the thread's 32 outputs summed over the CTA's l < p, less
+// |raw|^2 of the full band l = p.  The bands are taken in descending order, the
+// one pass 1 wrote last first: of an exchange somewhat larger than L2 the
+// ascending order finds nothing left.
 struct ChiTileAcc {
     float acc[32];
     int l = 0, p = 0;
-    float pf = 0.f, rs2 = 0.f;
+    float pf = 0.f;
     template <int R>
     __device__ __forceinline__ void store(int, int, int, const float2 *v) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const float pw = fmaf(v[r].x, v[r].x, v[r].y * v[r].y);
-            if (l < p) acc[r] = l == 0 ? pw : acc[r] + pw;
-            else acc[r] = rs2 * fmaf(pf, acc[r], -pw);
+            acc[r] = l == p ? -pw : fmaf(pf, pw, acc[r]);
         }
     }
 };
 
-template <int L, int C>
+// S > 1: a cluster of S CTAs shares a tile, CTA c taking the sub-bands [c q, c q + q)
+// of the p + 1, q = ceil((p + 1) / S); each sums its own, and the CTAs add the
+// sums through distributed shared memory, 1 / S of the tile each.  A tile a CTA
+// leaves the GPU to a few: 16 templates at N = 2^16, p = 16, are 128 tiles, 17
+// transforms of 3.6 us one after the other, 61 us; 50 us in pairs of CTAs whose warps (with their own
+// rows) do not wait for one another: 59 with CTA barriers, 53 in ascending order.
+template <int L, int C, int S>
 __global__ void __launch_bounds__(C *(L / 32), (C * (L / 32) >= 256) ? 2 : 1) k_chisq_tiles(ChiTilesParams q) {
     extern __shared__ float2 chi_smem[];
     constexpr int T = L / 32, NT = C * T;
+    // rows of up to 1024 points lie within a warp: no barrier holds the warps together
+    using Sync = std::conditional_t<(L <= 1024), ChiWarpSync, CtaSync>;
     float2 *tw = chi_smem + pass_data_bytes<L, C>() / sizeof(float2);
-    int tile = blockIdx.x, b = blockIdx.y;
+    int tile = blockIdx.x / S, b = blockIdx.y;
+    const int c = S > 1 ? (int)(blockIdx.x % S) : 0;   // rank in the cluster
     fill_twiddles<L>(tw);
     chain_wait(tile, b);
+    const int per = (q.p + S) / S, l0 = min(c * per, q.p + 1), l1 = min(l0 + per, q.p + 1);
+    const float rs = q.full[q.unit0 + b].rho_scale, rs2 = rs * rs;
     ChiTileAcc snk;
     snk.p = q.p;
     snk.pf = (float)q.p;
-    {
-        const float rs = q.full[q.unit0 + b].rho_scale;
-        snk.rs2 = rs * rs;
-    }
+#pragma unroll
+    for (int r = 0; r < 32; ++r) snk.acc[r] = 0.f;
     const typename RowSrc<L, C>::Params rp{q.exch, q.log2N1, q.log2N};
+    __syncthreads();   // twiddles
 #pragma unroll 1
-    for (int l = 0; l <= q.p; ++l) {
+    for (int l = l1 - 1; l >= l0; --l) {
         snk.l = l;
-        ChiTileSrc<L, C> src{RowSrc<L, C>(rp, tile, 0, l * q.nb + b, nullptr), l > 0};
-        cta_fft<L, C, false, +1>(chi_smem, tw, src, snk);
+        ChiTileSrc<L, C, Sync> src{RowSrc<L, C>(rp, tile, 0, l * q.nb + b, nullptr), l < l1 - 1};
+        cta_fft<L, C, false, +1, ChiTileSrc<L, C, Sync>, ChiTileAcc, Sync>(chi_smem, tw, src, snk);
     }
     const int seq = threadIdx.x / T, t = threadIdx.x % T;
     auto row = [&](int s) { return reinterpret_cast<float *>(chi_smem + s * SeqStride<L, C>::value); };
     __syncthreads();   // the last stage has read the sequences
-#pragma unroll
-    for (int r = 0; r < 32; ++r) row(seq)[t + r * T] = snk.acc[r];
-    __syncthreads();
     float *out = q.chisq + ((int64_t)(q.unit0 + b) << q.log2N) + tile * C;
-    for (int idx = threadIdx.x; idx < C * L; idx += NT) {
-        const int s = idx % C, j1 = idx / C;
-        __stcs(&out[s + ((int64_t)j1 << q.log2N2)], row(s)[j1]);
+    const float scale = S == 1 ? rs2 : 1.f;
+#pragma unroll
+    for (int r = 0; r < 32; ++r) row(seq)[t + r * T] = scale * snk.acc[r];
+    if constexpr (S == 1) {
+        __syncthreads();
+        for (int idx = threadIdx.x; idx < C * L; idx += NT) {
+            const int s = idx % C, j1 = idx / C;
+            __stcs(&out[s + ((int64_t)j1 << q.log2N2)], row(s)[j1]);
+        }
+    } else {
+        cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+        const float2 *peer[S];
+#pragma unroll
+        for (int i = 0; i < S; ++i) peer[i] = cl.map_shared_rank(chi_smem, i);
+        cl.sync();
+        for (int idx = c * (C * L / S) + threadIdx.x; idx < (c + 1) * (C * L / S); idx += NT) {
+            const int s = idx % C, j1 = idx / C;
+            float a = 0.f;
+#pragma unroll
+            for (int i = 0; i < S; ++i) a += reinterpret_cast<const float *>(peer[i] + s * SeqStride<L, C>::value)[j1];
+            __stcs(&out[s + ((int64_t)j1 << q.log2N2)], rs2 * a);
+        }
+        cl.sync();   // no CTA leaves while its sums are being read
     }
 }
 
@@ -188,10 +223,6 @@ __device__ __forceinline__ void cs_row_copy(float2 *dst, const float2 *src, uint
                  "l"(src), "r"(bytes), "r"(cs_addr(bar))
                  : "memory");
 }
-
-struct ChiWarpSync {
-    static __device__ __forceinline__ void sync() { __syncwarp(); }
-};
 
 constexpr int kChiWarps = 8;
 
@@ -335,15 +366,34 @@ constexpr size_t chi_tiles_smem_bytes() {
 
 struct ChiTilesOp {
     const ChiTilesParams *q;   // NULL: set the kernel attributes only
+    int n_sm;
     cudaStream_t st;
     template <int N2, int N1>
     cudaError_t run() {
         if constexpr (N1 != 1024) {
             constexpr int C = seqs_per_cta<N1>(N2);
             constexpr size_t smem = chi_tiles_smem_bytes<N1, C>();
-            if (!q)
-                return cudaFuncSetAttribute(k_chisq_tiles<N1, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            return launch(k_chisq_tiles<N1, C>, dim3(N2 / C, q->nb), C * (N1 / 32), smem, st, *q);
+            constexpr unsigned threads = C * (N1 / 32);
+            auto attr = [&](auto kernel) {
+                return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            };
+            if constexpr (N1 <= 512) {   // a template of 2048-point rows is 256 tiles and more
+                if (!q) {
+                    cudaError_t e = attr(k_chisq_tiles<N1, C, 2>);
+                    if (e == cudaSuccess) e = attr(k_chisq_tiles<N1, C, 4>);
+                    if (e != cudaSuccess) return e;
+                } else {
+                    // as many CTAs per tile as keep the launch within one wave (two per
+                    // SM), with two sub-bands or more each
+                    const int64_t tiles = (int64_t)(N2 / C) * q->nb, wave = 2 * (int64_t)n_sm;
+                    if (4 * tiles <= wave && q->p >= 7)
+                        return launch_cluster(k_chisq_tiles<N1, C, 4>, dim3(4 * (N2 / C), q->nb), threads, 4, smem, st, *q);
+                    if (2 * tiles <= wave && q->p >= 3)
+                        return launch_cluster(k_chisq_tiles<N1, C, 2>, dim3(2 * (N2 / C), q->nb), threads, 2, smem, st, *q);
+                }
+            }
+            if (!q) return attr(k_chisq_tiles<N1, C, 1>);
+            return launch(k_chisq_tiles<N1, C, 1>, dim3(N2 / C, q->nb), threads, smem, st, *q);
         } else {
             return q ? cudaErrorInvalidValue : cudaSuccess;   // 1024-point rows: k_chisq_rows
         }
@@ -358,9 +408,9 @@ cudaError_t launch_chisq_units(const SegDev &seg, const UnitInfo *all, int n_t, 
 }
 
 cudaError_t launch_chisq_tiles(const SegDev &seg, const float2 *exch, const UnitInfo *full, int unit0, int nb, int p,
-                               float *chisq, cudaStream_t st) {
+                               float *chisq, int n_sm, cudaStream_t st) {
     ChiTilesParams q{exch, full, chisq, unit0, nb, p, seg.log2N, seg.log2N1, seg.log2N2};
-    ChiTilesOp op{&q, st};
+    ChiTilesOp op{&q, n_sm, st};
     return dispatch_split(seg.log2N, op);
 }
 
@@ -388,7 +438,7 @@ cudaError_t chisq_kernel_attributes() {
         if (e1 != cudaSuccess) return e1;
     }
     for (int lg = 10; lg <= 22; ++lg) {
-        ChiTilesOp op{nullptr, nullptr};
+        ChiTilesOp op{nullptr, 0, nullptr};
         cudaError_t e = dispatch_split(lg, op);
         if (e != cudaSuccess) return e;
     }

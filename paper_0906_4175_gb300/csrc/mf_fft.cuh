@@ -490,7 +490,9 @@ struct is_narrow<T, decltype((void)&T::single, void())> { static constexpr bool 
 // The last stage does not synchronise: a sink that reuses shared memory
 // afterwards must __syncthreads() first.
 // smem: C * SeqStride<L, C>::value float2.  Must be called by all C*T threads.
-template <int L, int C, bool SEQ_FAST, int SIGN, class Src, class Snk>
+// Sync: the barrier between the stages; a warp's own where it holds whole
+// sequences (SEQ_FAST false, L <= 1024) and the caller has synchronised tw.
+template <int L, int C, bool SEQ_FAST, int SIGN, class Src, class Snk, class Sync = CtaSync>
 __device__ __forceinline__ void cta_fft(float2 *smem, const float2 *tw, Src &src, Snk &snk) {
     using S = FftShape<L>;
     constexpr int T = S::T;
@@ -515,13 +517,13 @@ __device__ __forceinline__ void cta_fft(float2 *smem, const float2 *tw, Src &src
             for (int r = 0; r < 32; ++r) sq[spad(32 * t + r)] = v[r];
         }
     }
-    __syncthreads();
+    Sync::sync();
     if constexpr (S::NST == 2) {
         if constexpr (L == 1024 && uses_split_tw<Src>::value) last_stage_1024_split<SIGN>(sq, tw, seq, t, snk);
-        else stockham_stage<L, S::R1, 32, SIGN, true>(sq, tw, seq, t, snk);
+        else stockham_stage<L, S::R1, 32, SIGN, true, Snk, Sync>(sq, tw, seq, t, snk);
     } else if constexpr (S::NST == 3) {
-        stockham_stage<L, S::R1, 32, SIGN, false>(sq, tw, seq, t, snk);
-        stockham_stage<L, S::R2, 32 * S::R1, SIGN, true>(sq, tw + TwTable<L>::S1, seq, t, snk);
+        stockham_stage<L, S::R1, 32, SIGN, false, Snk, Sync>(sq, tw, seq, t, snk);
+        stockham_stage<L, S::R2, 32 * S::R1, SIGN, true, Snk, Sync>(sq, tw + TwTable<L>::S1, seq, t, snk);
     }
 }
 

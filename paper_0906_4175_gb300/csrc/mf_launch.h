@@ -37,19 +37,32 @@ struct ChainScope {
     ChainScope &operator=(const ChainScope &) = delete;
 };
 
+// in clusters of `cluster` CTAs along x (0: none)
 template <class... P, class... A>
-inline cudaError_t launch(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A &&...args) {
+inline cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, unsigned threads, unsigned cluster, size_t smem,
+                                  cudaStream_t st, A &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute at[2];
     cfg.attrs = at;
-    cfg.numAttrs = t_chain ? 1 : 0;
+    if (t_chain) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster) {
+        at[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        at[cfg.numAttrs].val.clusterDim.x = cluster;
+        at[cfg.numAttrs].val.clusterDim.y = 1;
+        at[cfg.numAttrs++].val.clusterDim.z = 1;
+    }
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+template <class... P, class... A>
+inline cudaError_t launch(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A &&...args) {
+    return launch_cluster(kernel, grid, threads, 0, smem, st, std::forward<A>(args)...);
 }
 
 __device__ __forceinline__ void chain_opaque(int &x) { asm volatile("" : "+r"(x)::"memory"); }

@@ -313,3 +313,18 @@ def test_leading_bands(mf, monkeypatch, lg, fs, m):
     b = _run(mf, bank, [seg], 4.75)
     assert bank.check() == 0 and a[2] == b[2]
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
+# chi^2 tiles in clusters of four and two and alone (at most one wave of two blocks
+# per SM, two sub-bands or more per block): one template, whose tiles are few,
+# against the same template among many
+@pytest.mark.parametrize("lg,p,n", [(10, 3, 400), (10, 7, 80), (12, 16, 200), (14, 2, 3), (14, 6, 30), (14, 7, 30),
+                                    (14, 16, 170), (16, 16, 20), (16, 64, 12), (17, 9, 9), (18, 16, 12)])
+def test_chisq_tiles_in_clusters(mf, lg, p, n):
+    bank, seg = mf.Bank(*_masses(n)), _segment(mf, lg)
+    many = mf.chisq_series(bank, seg, list(range(n)), p=p)[0].cpu().numpy()
+    assert bank.check() == 0
+    for t in {0, n // 2, n - 1}:
+        one = mf.chisq_series(bank, seg, [t], p=p)[0].cpu().numpy()[0]
+        # both are FP32 sums of p + 1 squares of size rho^2 <= chi^2 + rho^2 terms
+        assert np.max(np.abs(one - many[t])) <= 1e-4 * max(1.0, float(np.max(many[t])))
