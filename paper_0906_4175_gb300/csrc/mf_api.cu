@@ -320,7 +320,7 @@ struct mf_bank_s {
     // split N = N1 * N2 (alt_log2n2) instead of the balanced one.  Until
     // mf_autotune measures the bank only 2^22 does: its balanced 2048-point
     // columns do not fit the staged pass 1 (128 templates: pass 1 2170 us per
-    // tile, pass 2 876), 4096 x 1024 does (1025 + 930).
+    // tile, pass 2 876), 4096 x 1024 does (1023 + 980).
     unsigned char alt_split[23] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 1};
     int *chi_status = nullptr;        // status of the last mf_chisq_series (bit 2: a bounded wait ran out)
 };

@@ -390,7 +390,7 @@ cudaError_t events_kernel_attributes() {
 // filter), the sub-band edges from a 32-way search by one warp per edge (4
 // dependent loads instead of 20), sub-bands outside a block's bins cost
 // nothing, and the row's total is one warp per sub-band instead of one thread
-// per row.  9 rows at N = 2^20, p = 16: 85 + 175 us before, 24 + 5 us now.
+// per row.  9 rows at N = 2^20, p = 16: 85 + 175 us before, 36 + 7 us now.
 constexpr int kCpThreads = 256, kCpWarps = kCpThreads / 32;
 constexpr int kCpAnchors = kCpThreads;
 

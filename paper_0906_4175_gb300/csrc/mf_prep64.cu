@@ -154,7 +154,7 @@ __host__ __device__ constexpr int cx_log2(int x) { return x <= 1 ? 0 : 1 + cx_lo
 // memory (16 KB; 2048 for the longest rows) on 256 threads.  SMALL (M <= 2^16):
 // one sequence, at least 128 points, so that the transform reaches every SM:
 // the FP64 pipe does two operations per SM and clock, and M = 2^12 on 4 CTAs of
-// 1024 points was 10 us a pass, 4 us on 32 (refresh of 2^13 samples 22 -> 12 us).
+// 1024 points was 10 us a pass, 6.3 and 5.6 us on 32 (refresh of 2^13 samples 22 -> 15 us).
 template <int LG, bool SMALL>
 __host__ __device__ constexpr int seqs64() {
     return SMALL ? (LG >= 7 ? 1 : (128 >> LG)) : (LG >= 10 ? 1 : (1024 >> LG));

@@ -183,14 +183,14 @@ __global__ void __launch_bounds__(kWarps * 32) k_peaks_rows(const float2 *__rest
 }
 
 // ---------------------------------------------------------------------------
-// Rows of L = 128, 256 and 512 points (N = 2^15 .. 2^18 and the 1024 x 512
+// Rows of L = 128, 256 and 512 points (N = 2^13 .. 2^18 and the 1024 x 512
 // split of 2^19): a warp takes 1024 / L consecutive rows at a time, L / 32 lanes
 // each, with the two-stage schedule of the per-tile kernel (bit-identical).  As
 // in k_pass2_rows the next rows are copied in under the last stage and no CTA
 // barrier separates the stages, which a CTA per tile of 8192 points pays three
 // times per tile.  The rows land, and are held between the stages, L + L/32
 // apart: a half-warp's L / 32 lanes of each row then meet different banks in
-// every access.  512-point rows, 250 templates at N = 2^18: 140 us per tile, 85
+// every access.  512-point rows, 250 templates at N = 2^18: 140 us per tile, 104
 // here.
 // ---------------------------------------------------------------------------
 template <int L>
