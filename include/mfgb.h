@@ -54,7 +54,8 @@ typedef struct {
 } mf_bank_params;
 
 #define MF_PHASE_ANCHOR 0  /* default: Psi in FP64 at anchor bins, reduced mod 2 pi, FP32 cubic Taylor between them */
-#define MF_PHASE_FP64   1  /* Psi in FP64 at every bin (anchor spacing 1) */
+#define MF_PHASE_FP64   1  /* Psi to 4e-10 turns at every bin: FP64 anchors, between them the Taylor series to 7th
+                              order, its cubic part in 64-bit fixed-point turns; per-batch launches always */
 #define MF_PHASE_FP32   2  /* Psi in FP32 only, no FP64 reduction (precision-sweep reference; loses accuracy) */
 #define MF_FFT_FP32     0  /* default: every FFT stage in FP32 on the CUDA cores */
 /* Precision-sweep forms (config "FFT in FP32 vs a tensor-core DFT-GEMM radix stage"): the first radix-32
@@ -209,10 +210,13 @@ int mf_segment_info(mf_segment seg, int64_t *N, double *fs);
  * The first call for a given (segment length, bank size, trig_cap) allocates
  * the bank's workspace (mostly the exchange of the templates in flight:
  * min(bank size, 4 GiB / 8N) x 8N bytes by default, the autotuned budget after
- * mf_autotune); later calls allocate nothing and queue only kernels
- * and memsets, so a call may be captured in a CUDA graph once an identical
- * call has run outside the capture (the graph keeps the segment, output and
- * workspace pointers; replays recompute from the segments' current contents).
+ * mf_autotune; segments of up to 2^16 samples with at most two tiles of 8192
+ * samples per SM share launches, up to 16 and 80 MB of exchange at a time, where
+ * the workspace can hold them); later calls allocate nothing and queue only
+ * kernels and memsets, so a call may be captured in a CUDA graph once an
+ * identical call has run outside the capture (the graph keeps the segment,
+ * output and workspace pointers; replays recompute from the segments' current
+ * contents).
  * Errors: MF_EINVAL (f_low >= f_cut for some pair, bad sizes, a workspace that
  * would have to grow or stage profiling switched on inside a stream capture),
  * MF_ENOMEM, MF_ECUDA. */
@@ -227,8 +231,9 @@ int mf_filter_bank(mf_bank bank, const mf_segment *segs, int n_seg, float thresh
  * 8-byte aligned), batch entries N apart; y may equal x (in place).
  * N a power of two in [2^10, 2^22]; sign = -1 (forward) or +1.  N = 2^10 and
  * 2^11: one kernel holding whole sequences per CTA, no allocation (capturable).
- * Larger N: the four-step passes through a complex64 exchange of up to 1 GiB
- * allocated on cuda_stream (not capturable), two kernels per 1 GiB of batch.
+ * N = 2^12 .. 2^14: one kernel too, but not capturable.  Larger N: the four-step
+ * passes through a complex64 exchange of up to 1 GiB allocated on cuda_stream
+ * (not capturable), two kernels per 1 GiB of batch.
  * Returns without synchronising.
  * Errors: MF_EINVAL (NULL, size, sign, alignment, N > 2^11 inside a capture),
  * MF_ENOMEM, MF_ECUDA. */
@@ -245,9 +250,9 @@ int mf_fft_c2c(const void *x, void *y, int64_t N, int64_t batch, int sign, void 
  * chisq: device FP32 [n][N] (row i for template tmpl[i]); edges: NULL or
  * device int64 [n][p+1] receiving b_0..b_p.  A template index outside the
  * bank gives an empty band (a zero row).  1 <= p <= 64, 1 <= n <= 2^24.
- * Cost: p + 1 inverse FFTs of length N per template (at N = 2^19, 2^20 the
- * first passes of a batch's p + 1 bands run as one launch and the second
- * passes as one kernel that sums the sub-bands in registers).
+ * Cost: p + 1 inverse FFTs of length N per template (the first passes of a
+ * batch's p + 1 bands run as one launch and the second passes as one kernel that
+ * sums the sub-bands in registers).
  * Allocates scratch on cuda_stream (p + 1 exchanges of 8 N bytes per
  * template of a batch, batches sized to the bank's exchange budget: 4 GiB
  * unless mf_autotune chose another), so it cannot be captured in a graph, and
@@ -270,9 +275,12 @@ int mf_chisq_series(mf_bank bank, mf_segment seg, const int32_t *tmpl, int64_t n
  * array of ev_cap records, written sorted by (seg, j); *n_events (device)
  * receives the true event count (compare with ev_cap for truncation).
  * n_tmpl, n_seg, max_N: the bank size, segment count and largest segment
- * length of the filter call (they size the sort keys).  Allocates scratch
- * (about 100 bytes per trigger of trig_cap) on cuda_stream; does not
+ * length of the filter call (they size the sort keys).  One launch.  Allocates
+ * scratch (about 100 bytes per trigger of trig_cap) on cuda_stream; does not
  * synchronise.
+ * The scratch of this call, mf_chisq_* and mf_fft_c2c comes from a
+ * stream-ordered pool of the library's own on the device, which keeps up to 4.5 GiB
+ * between calls and is trimmed when the last handle is destroyed.
  * Errors: MF_EINVAL (NULL, negative window, sizes), MF_ENOMEM, MF_ECUDA. */
 int mf_cluster_triggers(const mf_trigger *trig, const int64_t *n_trig, int64_t trig_cap, int64_t n_tmpl,
                         int n_seg, int64_t max_N, int32_t window, mf_event *events, int64_t ev_cap,
@@ -307,7 +315,8 @@ int mf_bank_check(mf_bank bank, void *cuda_stream);
  * (the CTA tile), or one CTA per column tile; pass 2 in warp-owned rows
  * with bulk-copy prefetch, or one CTA per row tile) and keeps the fastest in
  * the bank for later calls (the default is per-batch launches with 4 GiB, the
- * staged pass 1 and the row pass 2 where they apply).  Before those it picks,
+ * staged pass 1 and the row pass 2 where they apply, and the alternative split
+ * below for 2^22).  Before those it picks,
  * per segment length N = 2^18 .. 2^22, the four-step split N = N1 x N2 of the
  * per-batch schedule: the balanced one (N2 = 2^floor(log2 N / 2) columns) or
  * an alternative (2^18: 1024 x 256, 2^19: 512 x 1024, 2^20: 2048 x 512,
