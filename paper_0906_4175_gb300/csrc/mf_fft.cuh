@@ -125,14 +125,14 @@ __host__ __device__ constexpr double cx_abs(double x) { return x < 0 ? -x : x; }
 // multiply-add form of Linzer & Feig (1993): w o = c (o (1 + i s/c)) when
 // |c| >= |s|, else s (o (c/s + i)); the inner product takes 2 FMAs and the
 // scaled add/subtract 4, i.e. 6 instead of 8 instructions.
-template <int R, int SIGN, int Q>
+template <int R, int SIGN, int Q, bool PACK = true>
 struct Combine {
     static __device__ __forceinline__ void run(float2 *v, const float2 *e, const float2 *o) {
         if constexpr (Q < R / 2) {
             constexpr long long g = Q % R;
             if constexpr (g == 0) {
-                v[Q] = cadd(e[Q], o[Q]);
-                v[Q + R / 2] = csub(e[Q], o[Q]);
+                v[Q] = PACK ? cadd(e[Q], o[Q]) : make_float2(e[Q].x + o[Q].x, e[Q].y + o[Q].y);
+                v[Q + R / 2] = PACK ? csub(e[Q], o[Q]) : make_float2(e[Q].x - o[Q].x, e[Q].y - o[Q].y);
             } else if constexpr (4 * g == R) {   // the swapped operand is no register pair: scalar
                 const float2 t = tw_const<Q, R, SIGN>(o[Q]);
                 v[Q] = make_float2(e[Q].x + t.x, e[Q].y + t.y);
@@ -155,27 +155,27 @@ struct Combine {
                 v[Q] = make_float2(fmaf(k, b.x, e[Q].x), fmaf(k, b.y, e[Q].y));
                 v[Q + R / 2] = make_float2(fmaf(-k, b.x, e[Q].x), fmaf(-k, b.y, e[Q].y));
             }
-            Combine<R, SIGN, Q + 1>::run(v, e, o);
+            Combine<R, SIGN, Q + 1, PACK>::run(v, e, o);
         }
     }
 };
 
-template <int R, int SIGN>
+template <int R, int SIGN, bool PACK = true>
 struct Dft {
     static __device__ __forceinline__ void run(float2 *v) {
         if constexpr (R == 1) {
             return;
         } else if constexpr (R == 2) {
             float2 a = v[0], b = v[1];
-            v[0] = cadd(a, b);
-            v[1] = csub(a, b);
+            v[0] = PACK ? cadd(a, b) : make_float2(a.x + b.x, a.y + b.y);
+            v[1] = PACK ? csub(a, b) : make_float2(a.x - b.x, a.y - b.y);
         } else {
             float2 e[R / 2], o[R / 2];
 #pragma unroll
             for (int i = 0; i < R / 2; ++i) { e[i] = v[2 * i]; o[i] = v[2 * i + 1]; }
-            Dft<R / 2, SIGN>::run(e);
-            Dft<R / 2, SIGN>::run(o);
-            Combine<R, SIGN, 0>::run(v, e, o);
+            Dft<R / 2, SIGN, PACK>::run(e);
+            Dft<R / 2, SIGN, PACK>::run(o);
+            Combine<R, SIGN, 0, PACK>::run(v, e, o);
         }
     }
 };
@@ -361,7 +361,7 @@ struct CtaSync {
 
 // One Stockham stage reading from and (unless LAST) writing to shared memory.
 // Ns = product of earlier radices; each thread runs 32/R butterflies b = t + i*T.
-template <int L, int R, int Ns, int SIGN, bool LAST, class Snk, class Sync = CtaSync>
+template <int L, int R, int Ns, int SIGN, bool LAST, class Snk, class Sync = CtaSync, bool PACK = true>
 __device__ __forceinline__ void stockham_stage(float2 *sq, const float2 *tw, int seq, int t, Snk &snk) {
     constexpr int T = L / 32;
     constexpr int NB = 32 / R;
@@ -387,7 +387,7 @@ __device__ __forceinline__ void stockham_stage(float2 *sq, const float2 *tw, int
                 v[i * R + r] = cmul(v[i * R + r], w);
             }
         }
-        Dft<R, SIGN>::run(v + i * R);
+        Dft<R, SIGN, PACK>::run(v + i * R);
         if constexpr (!LAST) {
             const int idxD = (b / Ns) * Ns * R + k;
 #pragma unroll
@@ -480,6 +480,14 @@ struct is_narrow { static constexpr bool value = false; };
 template <class T>
 struct is_narrow<T, decltype((void)&T::single, void())> { static constexpr bool value = true; };
 
+// Sources and sinks with kScalarAdd = true have the plain additions of their
+// transform as scalar instructions (the same bits): where a kernel is not bound
+// by issue the packed ones only cost moves into register pairs.
+template <class T, class = void>
+struct scalar_adds { static constexpr bool value = false; };
+template <class T>
+struct scalar_adds<T, decltype((void)T::kScalarAdd, void())> { static constexpr bool value = T::kScalarAdd; };
+
 // Full CTA FFT.  tw: the TwTable<L> twiddles in shared memory, filled and
 // made visible before the call (or filled before it with no intervening
 // shared-memory write, the first stage barrier publishes them).
@@ -495,6 +503,7 @@ struct is_narrow<T, decltype((void)&T::single, void())> { static constexpr bool 
 template <int L, int C, bool SEQ_FAST, int SIGN, class Src, class Snk, class Sync = CtaSync>
 __device__ __forceinline__ void cta_fft(float2 *smem, const float2 *tw, Src &src, Snk &snk) {
     using S = FftShape<L>;
+    constexpr bool PACK = !scalar_adds<Src>::value && !scalar_adds<Snk>::value;
     constexpr int T = S::T;
     const int tid = threadIdx.x;
     const int seq = SEQ_FAST ? (tid % C) : (tid / T);
@@ -508,7 +517,7 @@ __device__ __forceinline__ void cta_fft(float2 *smem, const float2 *tw, Src &src
             if (src.single) dft32_single(v, v[0], src.rs, g_tw_tables + tw_offset<64>() + 32);   // row 1 of that table
             else dft32_halfzero<SIGN>(v);
         } else if constexpr (Src::kHalfZero) dft32_halfzero<SIGN>(v);
-        else Dft<32, SIGN>::run(v);
+        else Dft<32, SIGN, PACK>::run(v);
         if constexpr (S::NST == 1) {
             snk.template store<32>(seq, t, T, v);
             return;
@@ -520,10 +529,10 @@ __device__ __forceinline__ void cta_fft(float2 *smem, const float2 *tw, Src &src
     Sync::sync();
     if constexpr (S::NST == 2) {
         if constexpr (L == 1024 && uses_split_tw<Src>::value) last_stage_1024_split<SIGN>(sq, tw, seq, t, snk);
-        else stockham_stage<L, S::R1, 32, SIGN, true, Snk, Sync>(sq, tw, seq, t, snk);
+        else stockham_stage<L, S::R1, 32, SIGN, true, Snk, Sync, PACK>(sq, tw, seq, t, snk);
     } else if constexpr (S::NST == 3) {
-        stockham_stage<L, S::R1, 32, SIGN, false, Snk, Sync>(sq, tw, seq, t, snk);
-        stockham_stage<L, S::R2, 32 * S::R1, SIGN, true, Snk, Sync>(sq, tw + TwTable<L>::S1, seq, t, snk);
+        stockham_stage<L, S::R1, 32, SIGN, false, Snk, Sync, PACK>(sq, tw, seq, t, snk);
+        stockham_stage<L, S::R2, 32 * S::R1, SIGN, true, Snk, Sync, PACK>(sq, tw + TwTable<L>::S1, seq, t, snk);
     }
 }
 
