@@ -29,7 +29,8 @@ def mf():
 def _segment(mf, lg, fs=4096.0, seed=5):
     import torch
     g = torch.Generator(device="cuda").manual_seed(seed)
-    return mf.Segment(torch.randn(1 << lg, dtype=torch.float32, device="cuda", generator=g), fs)
+    x = 70.0 * torch.randn(1 << lg, dtype=torch.float32, device="cuda", generator=g)   # loudest rho about 4 .. 7
+    return mf.Segment(x, fs)
 
 
 def _run(mf, bank, segs, thr, cap=1 << 20):
@@ -328,3 +329,27 @@ def test_chisq_tiles_in_clusters(mf, lg, p, n):
         one = mf.chisq_series(bank, seg, [t], p=p)[0].cpu().numpy()[0]
         # both are FP32 sums of p + 1 squares of size rho^2 <= chi^2 + rho^2 terms
         assert np.max(np.abs(one - many[t])) <= 1e-4 * max(1.0, float(np.max(many[t])))
+
+
+# clustering and the chi^2 of single samples allocate scratch in stream order, in a
+# capture as allocation nodes of the graph
+def test_events_in_a_capture(mf):
+    import torch
+    bank, seg = mf.Bank(*_masses(12)), _segment(mf, 16)
+    loudest = float(mf.filter_bank(bank, [seg], 1e9, trig_cap=1 << 16)[0].view(-1, 4)[:, 0].max())
+    _, trig, nt = mf.filter_bank(bank, [seg], 0.75 * loudest, trig_cap=1 << 16)
+    ev, n_ev = mf.cluster_triggers(trig, nt, bank.n, 1, seg.N, 40)
+    n = int(n_ev.item())
+    assert n > 1
+    rows = ev[:n].clone()
+    chi = mf.chisq_points(bank, [seg], rows, p=8)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        ev2, n2 = mf.cluster_triggers(trig, nt, bank.n, 1, seg.N, 40)
+        chi2 = mf.chisq_points(bank, [seg], rows, p=8)
+    for _ in range(3):
+        g.replay()
+        torch.cuda.synchronize()
+        assert int(n2.item()) == n and torch.equal(ev2[:n].view(torch.int32), ev[:n].view(torch.int32))
+        assert torch.equal(chi2, chi)
