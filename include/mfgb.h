@@ -280,7 +280,7 @@ int mf_chisq_series(mf_bank bank, mf_segment seg, const int32_t *tmpl, int64_t n
  * synchronise.
  * The scratch of this call, mf_chisq_* and mf_fft_c2c comes from a
  * stream-ordered pool of the library's own on the device, which keeps up to 4.5 GiB
- * between calls and is trimmed when the last handle is destroyed.
+ * between calls and is trimmed when the last bank or segment is destroyed.
  * Errors: MF_EINVAL (NULL, negative window, sizes), MF_ENOMEM, MF_ECUDA. */
 int mf_cluster_triggers(const mf_trigger *trig, const int64_t *n_trig, int64_t trig_cap, int64_t n_tmpl,
                         int n_seg, int64_t max_N, int32_t window, mf_event *events, int64_t ev_cap,
@@ -490,6 +490,11 @@ int mf_bank_debug_stall(mf_bank bank, int64_t unit, int64_t spin_limit);
  * workspace is released and regrown by the next call) and the hook disarms.
  * countdown < 0 disarms it.  Never fails. */
 int mf_debug_fail_alloc(int64_t countdown);
+
+/* mf_debug_scratch_reserved -- bytes of device memory that the library's
+ * scratch pools hold in this process, in use or kept for later calls (*bytes,
+ * host).  Errors: MF_EINVAL, MF_ECUDA. */
+int mf_debug_scratch_reserved(int64_t *bytes);
 int mf_bank_profile_read(mf_bank bank, double *ms, double *bytes, int64_t *launches);
 
 #ifdef __cplusplus

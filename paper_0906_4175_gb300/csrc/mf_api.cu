@@ -172,7 +172,8 @@ static cudaError_t dev_malloc_async(T **p, size_t bytes, cudaStream_t st) {
 // that waits for each call's result paid the mapping of its scratch again on
 // every call (chi^2 series of 64 templates at 2^20: 4 GiB, 12.7 ms instead of
 // 4.0 ms a call).  This pool keeps at most kScratchKeep bytes between calls
-// and gives everything back when the last bank and segment are destroyed.
+// and gives everything back when the last handle (bank or segment, counted
+// where each is handed out) is destroyed.
 // Stream order and thread safety are the pool's (cudaMallocFromPoolAsync).
 constexpr uint64_t kScratchKeep = (uint64_t)4608 << 20;   // the 4 GiB exchange budget and its companions
 static std::mutex g_pool_mu;
@@ -623,6 +624,7 @@ extern "C" int mf_segment_upload(const float *s, int64_t N, double fs, const dou
         return set_err(e == cudaErrorMemoryAllocation ? MF_ENOMEM : MF_ECUDA, "segment_upload: %s",
                        cudaGetErrorString(e));
     }
+    handle_created();
     *out = g;
     return MF_OK;
 }
@@ -1938,5 +1940,17 @@ extern "C" int mf_refine_triggers_static(mf_segment seg, const mf_bank_params *p
 
 extern "C" int mf_debug_fail_alloc(int64_t countdown) {
     g_fail_alloc.store(countdown < 0 ? -1 : countdown);
+    return MF_OK;
+}
+
+extern "C" int mf_debug_scratch_reserved(int64_t *bytes) {
+    if (!bytes) return set_err(MF_EINVAL, "NULL argument");
+    *bytes = 0;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    for (auto &q : g_pools) {
+        uint64_t v = 0;
+        MF_CUDA(cudaMemPoolGetAttribute(q.second, cudaMemPoolAttrReservedMemCurrent, &v));
+        *bytes += (int64_t)v;
+    }
     return MF_OK;
 }

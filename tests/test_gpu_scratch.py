@@ -1,0 +1,57 @@
+"""Scratch that outlives a call: what the library's pool keeps, and when it goes
+back to the system.  Handles are counted per process, so each case runs in a
+process of its own."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+PRELUDE = """
+import ctypes, gc
+import numpy as np, torch
+from paper_0906_4175_gb300 import build
+build.build()
+import paper_0906_4175_gb300 as mf
+L = mf._native.lib()
+MB = 1 << 20
+
+def reserved():
+    torch.cuda.synchronize()
+    v = ctypes.c_int64()
+    assert L.mf_debug_scratch_reserved(ctypes.byref(v)) == 0
+    return v.value
+
+def bank(n=4):
+    m = np.random.default_rng(1).uniform(1.2, 3.0, n)
+    return mf.Bank(m, m[::-1].copy())
+
+def segment(lg=16, seed=1):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return mf.Segment(torch.randn(1 << lg, dtype=torch.float32, device="cuda", generator=g), 4096.0)
+"""
+
+
+def _child(body):
+    env = dict(os.environ, PYTHONPATH=ROOT)
+    r = subprocess.run([sys.executable, "-c", PRELUDE + body], capture_output=True, text=True, timeout=300, env=env)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("order", ["b a c", "a c b", "a b c", "c b a"])
+def test_scratch_is_kept_while_a_handle_lives(order):
+    """One bank and two segments, destroyed in several orders: the pool keeps
+    the chi^2 series' scratch until the last of them is gone, twice over."""
+    _child("""
+for cycle in range(2):
+    h = {"b": bank(), "a": segment(seed=2), "c": segment(seed=3)}
+    mf.chisq_series(h["b"], h["a"], [0, 1, 2, 3], p=16)     # 4 x 17 exchanges of 512 KB
+    for name in %r.split():
+        assert reserved() >= 32 * MB, (cycle, name, reserved())
+        h[name].close()
+    assert reserved() == 0, (cycle, reserved())
+""" % order)
