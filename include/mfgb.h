@@ -280,11 +280,19 @@ int mf_chisq_series(mf_bank bank, mf_segment seg, const int32_t *tmpl, int64_t n
  * synchronise.
  * The scratch of this call, mf_chisq_* and mf_fft_c2c comes from a
  * stream-ordered pool of the library's own on the device, which keeps up to 4.5 GiB
- * between calls and is trimmed when the last bank or segment is destroyed.
+ * between calls and is trimmed when the last bank or segment is destroyed, or
+ * by mf_release_scratch.
  * Errors: MF_EINVAL (NULL, negative window, sizes), MF_ENOMEM, MF_ECUDA. */
 int mf_cluster_triggers(const mf_trigger *trig, const int64_t *n_trig, int64_t trig_cap, int64_t n_tmpl,
                         int n_seg, int64_t max_N, int32_t window, mf_event *events, int64_t ev_cap,
                         int64_t *n_events, void *cuda_stream);
+
+/* mf_release_scratch -- gives the scratch that the library keeps between calls
+ * back to the system: what calls that have finished used.  For programs that
+ * need the memory elsewhere, above all those that make no bank and no segment
+ * (mf_fft_c2c and mf_cluster_triggers alone: up to 1 GiB and 100 bytes per
+ * trigger of trig_cap).  Does not synchronise.  Errors: MF_ECUDA. */
+int mf_release_scratch(void);
 
 /* mf_chisq_points -- Eq. (5) at single samples: for each row i the template
  * rows[i*stride], segment segs[rows[i*stride+1]] and sample j =

@@ -20,8 +20,8 @@ from ._native import (EVENT_DTYPE, INJ_DTYPE, MF_EINVAL, MF_EOVERFLOW, MF_ETIMEO
                       MF_PHASE_FP32, MF_PHASE_FP64, PEAK_DTYPE, TRIG_DTYPE, BankParams, MFError, check)
 
 __all__ = ["Bank", "Segment", "filter_bank", "chisq_series", "chisq_points", "cluster_triggers",
-           "events_to_numpy", "EVENT_DTYPE", "fft", "autotune", "synth_segment", "refine", "RefineFn", "MFError",
-           "PEAK_DTYPE", "TRIG_DTYPE", "INJ_DTYPE", "MF_PHASE_ANCHOR", "MF_PHASE_FP64", "MF_PHASE_FP32",
+           "events_to_numpy", "EVENT_DTYPE", "fft", "release_scratch", "autotune", "synth_segment", "refine",
+           "RefineFn", "MFError", "PEAK_DTYPE", "TRIG_DTYPE", "INJ_DTYPE", "MF_PHASE_ANCHOR", "MF_PHASE_FP64", "MF_PHASE_FP32",
            "MF_FFT_FP32", "MF_FFT_TC_FP16", "MF_FFT_TC_BF16",
            "peaks_to_numpy", "triggers_to_numpy", "version"]
 
@@ -221,6 +221,12 @@ def fft(x, sign: int = -1, out=None, stream=None):
     y = torch.empty_like(x) if out is None else out
     check(_native.lib().mf_fft_c2c(x.data_ptr(), y.data_ptr(), N, batch, int(sign), _stream_ptr(stream)))
     return y
+
+
+def release_scratch():
+    """mf_release_scratch: give the scratch that finished calls left in the
+    library's pool back to the system (synchronise first)."""
+    check(_native.lib().mf_release_scratch())
 
 
 def cluster_triggers(trig, n_trig, n_tmpl: int, n_seg: int, max_N: int, window: int, ev_cap: int = None,

@@ -48,6 +48,7 @@ SIGNATURES = {
     "mf_refine_triggers": (_I, [_P, _P, _P, _I64, _P, _P, _P, _P]),
     "mf_fft_c2c": (_I, [_P, _P, _I64, _I64, _I, _P]),
     "mf_cluster_triggers": (_I, [_P, _P, _I64, _I64, _I, _I64, ctypes.c_int32, _P, _I64, _P, _P]),
+    "mf_release_scratch": (_I, []),
     "mf_chisq_points": (_I, [_P, _P, _I, _P, _I64, _I64, _I, _P, _P]),
     "mf_chisq_series": (_I, [_P, _P, _P, _I64, _I, _P, _P, _P]),
     "mf_refine_triggers_multi": (_I, [_P, _I, _P, _P, _P, _I64, _P, _P, _P, _P]),

@@ -173,7 +173,8 @@ static cudaError_t dev_malloc_async(T **p, size_t bytes, cudaStream_t st) {
 // every call (chi^2 series of 64 templates at 2^20: 4 GiB, 12.7 ms instead of
 // 4.0 ms a call).  This pool keeps at most kScratchKeep bytes between calls
 // and gives everything back when the last handle (bank or segment, counted
-// where each is handed out) is destroyed.
+// where each is handed out) is destroyed, or when mf_release_scratch asks: a
+// program that only transforms or clusters has no handle.
 // Stream order and thread safety are the pool's (cudaMallocFromPoolAsync).
 constexpr uint64_t kScratchKeep = (uint64_t)4608 << 20;   // the 4 GiB exchange budget and its companions
 static std::mutex g_pool_mu;
@@ -209,10 +210,17 @@ static cudaError_t scratch_pool(cudaMemPool_t *out) {
     return cudaSuccess;
 }
 static void handle_created() { g_handles.fetch_add(1); }
-static void handle_destroyed() {
-    if (g_handles.fetch_sub(1) != 1) return;
+static cudaError_t trim_pools() {   // what no queued call uses goes back to the system
     std::lock_guard<std::mutex> lk(g_pool_mu);
-    for (auto &q : g_pools) cudaMemPoolTrimTo(q.second, 0);
+    cudaError_t e = cudaSuccess;
+    for (auto &q : g_pools) {
+        const cudaError_t t = cudaMemPoolTrimTo(q.second, 0);
+        if (e == cudaSuccess) e = t;
+    }
+    return e;
+}
+static void handle_destroyed() {
+    if (g_handles.fetch_sub(1) == 1) trim_pools();
 }
 
 // One call's scratch: its parts are added first, in a few groups that are
@@ -1940,6 +1948,11 @@ extern "C" int mf_refine_triggers_static(mf_segment seg, const mf_bank_params *p
 
 extern "C" int mf_debug_fail_alloc(int64_t countdown) {
     g_fail_alloc.store(countdown < 0 ? -1 : countdown);
+    return MF_OK;
+}
+
+extern "C" int mf_release_scratch(void) {
+    MF_CUDA(trim_pools());
     return MF_OK;
 }
 

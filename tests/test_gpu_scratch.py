@@ -55,3 +55,19 @@ for cycle in range(2):
         h[name].close()
     assert reserved() == 0, (cycle, reserved())
 """ % order)
+
+
+def test_release_of_scratch_without_handles():
+    """A program that only transforms makes no handle: its scratch goes back
+    when it asks, and later calls work as before."""
+    _child("""
+x = torch.randn(8, 1 << 20, dtype=torch.complex64, device="cuda")     # exchange of 64 MB
+y = mf.fft(x)
+assert reserved() >= 64 * MB
+mf.release_scratch()
+assert reserved() == 0
+assert torch.equal(mf.fft(x), y)
+torch.cuda.synchronize()
+mf.release_scratch()
+assert reserved() == 0
+""")
