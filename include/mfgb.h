@@ -499,6 +499,13 @@ int mf_bank_debug_stall(mf_bank bank, int64_t unit, int64_t spin_limit);
  * countdown < 0 disarms it.  Never fails. */
 int mf_debug_fail_alloc(int64_t countdown);
 
+/* mf_debug_alloc_limit -- test hook for calls that find little memory.  With
+ * bytes >= 0 every later device allocation of the library of more than `bytes`
+ * (allocations outside the scratch pools: of more than `bytes` together with
+ * what the pools hold) is answered by the CUDA runtime as out of memory;
+ * bytes < 0 lifts the limit.  Never fails. */
+int mf_debug_alloc_limit(int64_t bytes);
+
 /* mf_debug_scratch_reserved -- bytes of device memory that the library's
  * scratch pools hold in this process, in use or kept for later calls (*bytes,
  * host).  Errors: MF_EINVAL, MF_ECUDA. */

@@ -136,35 +136,6 @@ static double psi_deriv_bound(const double *rec, double f, int n) {
 // ---------------------------------------------------------------------------
 // handles
 // ---------------------------------------------------------------------------
-// Device allocations of the library go through these two wrappers so that
-// mf_debug_fail_alloc can make one of them fail as if the device were out of
-// memory (a host-side fault injection for the error paths): after `countdown`
-// further allocations succeed, the next one returns cudaErrorMemoryAllocation
-// without allocating, and the hook disarms.  -1 = disarmed.
-static std::atomic<int64_t> g_fail_alloc{-1};
-static bool alloc_fault() {
-    int64_t v = g_fail_alloc.load();
-    while (v >= 0)
-        if (g_fail_alloc.compare_exchange_weak(v, v - 1)) return v == 0;
-    return false;
-}
-template <class T>
-static cudaError_t dev_malloc(T **p, size_t bytes) {
-    if (alloc_fault()) {
-        *p = nullptr;
-        return cudaErrorMemoryAllocation;
-    }
-    return cudaMalloc(p, bytes);
-}
-template <class T>
-static cudaError_t dev_malloc_async(T **p, size_t bytes, cudaStream_t st) {
-    if (alloc_fault()) {
-        *p = nullptr;
-        return cudaErrorMemoryAllocation;
-    }
-    return cudaMallocAsync(p, bytes, st);
-}
-
 // Scratch of the calls that allocate per call (chi^2, clustering, the batched
 // FFT, segment upload): one stream-ordered allocation per call from the
 // library's own pool of each device.  The default pool gives its memory back
@@ -219,8 +190,73 @@ static cudaError_t trim_pools() {   // what no queued call uses goes back to the
     }
     return e;
 }
+static cudaError_t pools_reserved(int64_t *bytes) {   // in use or kept
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    *bytes = 0;
+    for (auto &q : g_pools) {
+        uint64_t v = 0;
+        const cudaError_t e = cudaMemPoolGetAttribute(q.second, cudaMemPoolAttrReservedMemCurrent, &v);
+        if (e != cudaSuccess) return e;
+        *bytes += (int64_t)v;
+    }
+    return cudaSuccess;
+}
 static void handle_destroyed() {
     if (g_handles.fetch_sub(1) == 1) trim_pools();
+}
+
+// Device allocations of the library go through allocate().  If there is no room,
+// the calls queued so far are waited for, what the scratch pools keep goes back
+// to the system, and the allocation is tried once more: memory kept for later
+// calls makes no call fail.  A failed attempt leaves no error behind for the
+// next launch's cudaGetLastError.
+//
+// Two hooks make allocations fail (the error paths' tests).  mf_debug_fail_alloc:
+// after `countdown` further allocations succeed, the next one returns
+// cudaErrorMemoryAllocation without being attempted, and the hook disarms
+// (-1 = disarmed).  mf_debug_alloc_limit: an allocation past the limit asks the
+// runtime for more than any device holds, at every attempt.
+static std::atomic<int64_t> g_fail_alloc{-1}, g_alloc_limit{-1};
+static bool alloc_fault() {
+    int64_t v = g_fail_alloc.load();
+    while (v >= 0)
+        if (g_fail_alloc.compare_exchange_weak(v, v - 1)) return v == 0;
+    return false;
+}
+static size_t limited(size_t bytes, bool pooled) {
+    const int64_t limit = g_alloc_limit.load();
+    if (limit < 0) return bytes;
+    int64_t held = 0;
+    if (!pooled && pools_reserved(&held) != cudaSuccess) held = 0;
+    return (int64_t)bytes + held > limit ? (size_t)1 << 60 : bytes;
+}
+static bool stream_capturing(cudaStream_t st);
+static bool stream_done(cudaStream_t st) { return !stream_capturing(st) && cudaStreamSynchronize(st) == cudaSuccess; }
+// wait: true once the caller's queued work is done (and it may be waited for)
+template <class W, class F>
+static cudaError_t allocate(size_t bytes, bool pooled, W wait, F get) {
+    if (alloc_fault()) return cudaErrorMemoryAllocation;
+    cudaError_t e = get(limited(bytes, pooled));
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    if (!wait() || trim_pools() != cudaSuccess) return e;
+    e = get(limited(bytes, pooled));
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+    return e;
+}
+template <class T>
+static cudaError_t dev_malloc(T **p, size_t bytes) {
+    const cudaError_t e = allocate(
+        bytes, false, [] { return cudaDeviceSynchronize() == cudaSuccess; }, [&](size_t n) { return cudaMalloc(p, n); });
+    if (e != cudaSuccess) *p = nullptr;
+    return e;
+}
+template <class T>
+static cudaError_t dev_malloc_async(T **p, size_t bytes, cudaStream_t st) {
+    const cudaError_t e = allocate(
+        bytes, false, [&] { return stream_done(st); }, [&](size_t n) { return cudaMallocAsync(p, n, st); });
+    if (e != cudaSuccess) *p = nullptr;
+    return e;
 }
 
 // One call's scratch: its parts are added first, in a few groups that are
@@ -240,10 +276,12 @@ struct Scratch {
     cudaError_t alloc(cudaStream_t st) {
         for (int i = 0; i < n; ++i) {
             if (size[i] == 0) continue;
-            cudaError_t e = alloc_fault() ? cudaErrorMemoryAllocation : cudaSuccess;
             cudaMemPool_t pool;
-            if (e == cudaSuccess) e = scratch_pool(&pool);
-            if (e == cudaSuccess) e = cudaMallocFromPoolAsync((void **)&base[i], size[i], pool, st);
+            cudaError_t e = scratch_pool(&pool);
+            if (e == cudaSuccess)
+                e = allocate(
+                    size[i], true, [&] { return stream_done(st); },
+                    [&](size_t bytes) { return cudaMallocFromPoolAsync((void **)&base[i], bytes, pool, st); });
             if (e != cudaSuccess) {
                 base[i] = nullptr;
                 return e;
@@ -1951,6 +1989,11 @@ extern "C" int mf_debug_fail_alloc(int64_t countdown) {
     return MF_OK;
 }
 
+extern "C" int mf_debug_alloc_limit(int64_t bytes) {
+    g_alloc_limit.store(bytes < 0 ? -1 : bytes);
+    return MF_OK;
+}
+
 extern "C" int mf_release_scratch(void) {
     MF_CUDA(trim_pools());
     return MF_OK;
@@ -1958,12 +2001,6 @@ extern "C" int mf_release_scratch(void) {
 
 extern "C" int mf_debug_scratch_reserved(int64_t *bytes) {
     if (!bytes) return set_err(MF_EINVAL, "NULL argument");
-    *bytes = 0;
-    std::lock_guard<std::mutex> lk(g_pool_mu);
-    for (auto &q : g_pools) {
-        uint64_t v = 0;
-        MF_CUDA(cudaMemPoolGetAttribute(q.second, cudaMemPoolAttrReservedMemCurrent, &v));
-        *bytes += (int64_t)v;
-    }
+    MF_CUDA(pools_reserved(bytes));
     return MF_OK;
 }

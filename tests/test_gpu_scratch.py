@@ -71,3 +71,40 @@ torch.cuda.synchronize()
 mf.release_scratch()
 assert reserved() == 0
 """)
+
+
+def test_kept_scratch_makes_room():
+    """A bank's workspace that fits only without what the pool keeps."""
+    _child("""
+b, s = bank(8), segment(20)
+ref = mf.filter_bank(bank(8), [s], 4.0, trig_cap=1 << 12)
+mf.chisq_series(b, s, list(range(8)), p=8)              # 72 exchanges of 8 MB
+held = reserved()
+assert held >= 512 * MB
+L.mf_debug_alloc_limit(held + 32 * MB)                  # the workspace's exchange is 64 MB
+got = mf.filter_bank(b, [s], 4.0, trig_cap=1 << 12)
+L.mf_debug_alloc_limit(-1)
+n = int(ref[2].item())
+assert b.check() == 0 and int(got[2].item()) == n
+assert torch.equal(got[0], ref[0]) and torch.equal(got[1][:n], ref[1][:n])
+assert reserved() == 0
+""")
+
+
+def test_a_refused_allocation_leaves_no_error_behind():
+    """MF_ENOMEM from one call; the next one's launches are its own."""
+    _child("""
+b, s = bank(), segment()
+_, trig, nt = mf.filter_bank(b, [s], 3.0, trig_cap=1 << 14)
+for refused in (lambda: mf.filter_bank(b, [s], 3.0, trig_cap=1 << 20), lambda: mf.chisq_series(b, s, [0, 1], p=8),
+                lambda: mf.synth_segment(np.zeros(1 << 20), 1 << 20, 4096.0)):
+    L.mf_debug_alloc_limit(1 << 16)
+    try:
+        refused()
+        raise SystemExit("not refused")
+    except mf.MFError as e:
+        assert e.code == mf._native.MF_ENOMEM, e
+    L.mf_debug_alloc_limit(-1)
+    mf.cluster_triggers(trig, nt, b.n, 1, s.N, 40)
+    torch.cuda.synchronize()
+""")
