@@ -216,7 +216,8 @@ int mf_segment_info(mf_segment seg, int64_t *N, double *fs);
  * kernels and memsets, so a call may be captured in a CUDA graph once an
  * identical call has run outside the capture (the graph keeps the segment,
  * output and workspace pointers; replays recompute from the segments' current
- * contents).
+ * contents).  After a capture the workspace grows only for a longer segment or a
+ * larger trig_cap, which ends the use of that graph.
  * Errors: MF_EINVAL (f_low >= f_cut for some pair, bad sizes, a workspace that
  * would have to grow or stage profiling switched on inside a stream capture),
  * MF_ENOMEM, MF_ECUDA. */

@@ -369,6 +369,8 @@ struct mf_bank_s {
     // columns do not fit the staged pass 1 (128 templates: pass 1 2170 us per
     // tile, pass 2 876), 4096 x 1024 does (1023 + 980).
     unsigned char alt_split[23] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 1};
+    bool captured = false;        // a graph may hold the workspace's pointers
+    bool group_no_room = false;   // the larger workspace of grouped segments could not be allocated
     int *chi_status = nullptr;        // status of the last mf_chisq_series (bit 2: a bounded wait ran out)
 };
 
@@ -790,41 +792,68 @@ static int64_t choose_batch(int64_t N, int64_t n_t, int64_t tuned_exch) {
     return b;
 }
 
-// exch_elems: complex64 entries of the exchange ring (max over the call's
-// segments of batch * N); anc_elems: anchor records (max of batch * anchors);
-// n_set: segments whose units are held at once
-static int ensure_workspace(mf_bank_s *b, int64_t exch_elems, int64_t cap, int64_t anc_elems, int64_t nblk,
-                            int n_set, bool capturing) {
-    Workspace &w = b->ws;
-    if (w.units && w.exch_elems >= exch_elems && w.n_t >= b->n && w.cap >= cap && w.anc_elems >= anc_elems &&
-        w.nblk >= nblk && w.n_set >= n_set)
+// What a call takes of the bank's workspace.  exch_elems: complex64 entries of
+// the exchange ring (max over the call's segments of batch * N); anc_elems:
+// anchor records (max of batch * anchors); n_set: segments whose units are held
+// at once
+struct WorkspaceNeed {
+    int64_t exch_elems, cap, anc_elems, nblk;
+    int n_set;
+};
+static bool workspace_holds(const mf_bank_s *b, const WorkspaceNeed &q) {
+    const Workspace &w = b->ws;
+    return w.units && w.exch_elems >= q.exch_elems && w.n_t >= b->n && w.cap >= q.cap && w.anc_elems >= q.anc_elems &&
+           w.nblk >= q.nblk && w.n_set >= q.n_set;
+}
+// w (empty): a workspace of that size; all or nothing
+static int make_workspace(Workspace &w, int64_t n, const WorkspaceNeed &q) {
+    auto get = [&]() -> int {
+        MF_CUDA(dev_malloc(&w.units, sizeof(UnitInfo) * n * q.n_set));
+        MF_CUDA(dev_malloc(&w.exch, sizeof(float2) * q.exch_elems));
+        MF_CUDA(dev_malloc(&w.anchors, sizeof(float4) * q.anc_elems));
+        MF_CUDA(dev_malloc(&w.anchors4, sizeof(float) * q.anc_elems));
+        MF_CUDA(dev_malloc(&w.partials, sizeof(float4) * q.nblk * n));
+        MF_CUDA(dev_malloc(&w.staged, sizeof(mf_trigger) * q.cap));
+        MF_CUDA(dev_malloc(&w.keys, sizeof(uint64_t) * q.cap));
+        MF_CUDA(dev_malloc(&w.keys_tmp, sizeof(uint64_t) * q.cap));
+        MF_CUDA(dev_malloc(&w.idx_a, sizeof(uint32_t) * q.cap));
+        MF_CUDA(dev_malloc(&w.idx_b, sizeof(uint32_t) * q.cap));
+        MF_CUDA(dev_malloc(&w.tstat, sizeof(uint64_t) * sort_tile_words(q.cap)));
+        MF_CUDA(dev_malloc(&w.fctl, sizeof(FilterCtl)));
+        MF_CUDA(cudaMemset(w.fctl, 0, sizeof(FilterCtl)));
+        MF_CUDA(dev_malloc(&w.ctl, sizeof(unsigned) * (4 + 3 * n)));
         return MF_OK;
+    };
+    const int rc = get();
+    if (rc) {
+        w.release();
+        return rc;
+    }
+    w.counter = &w.fctl->counter;
+    w.status = &w.fctl->status;
+    w.exch_elems = q.exch_elems; w.n_t = n; w.cap = q.cap; w.anc_elems = q.anc_elems; w.nblk = q.nblk; w.n_set = q.n_set;
+    return MF_OK;
+}
+// keep: the old workspace goes only once the new one is there
+static int ensure_workspace(mf_bank_s *b, const WorkspaceNeed &need, bool capturing, bool keep) {
+    if (workspace_holds(b, need)) return MF_OK;
     if (capturing)
         return set_err(MF_EINVAL, "the workspace must grow: call mf_filter_bank once with these segments and "
                                   "trig_cap before capturing it");
-    const int64_t ne = std::max(w.exch_elems, exch_elems), ncap = std::max(std::max(w.cap, cap), (int64_t)1);
-    const int64_t na = std::max(w.anc_elems, anc_elems);
-    const int64_t nbl = std::max(w.nblk, nblk);
-    const int ns = std::max(w.n_set, n_set);
+    Workspace &w = b->ws;
+    const WorkspaceNeed q{std::max(w.exch_elems, need.exch_elems), std::max(std::max(w.cap, need.cap), (int64_t)1),
+                          std::max(w.anc_elems, need.anc_elems), std::max(w.nblk, need.nblk),
+                          std::max(w.n_set, need.n_set)};
     MF_CUDA(cudaDeviceSynchronize());
+    if (!keep) {
+        w.release();
+        return make_workspace(w, b->n, q);
+    }
+    Workspace grown;
+    const int rc = make_workspace(grown, b->n, q);
+    if (rc) return rc;
     w.release();
-    MF_CUDA(dev_malloc(&w.units, sizeof(UnitInfo) * b->n * ns));
-    MF_CUDA(dev_malloc(&w.exch, sizeof(float2) * ne));
-    MF_CUDA(dev_malloc(&w.anchors, sizeof(float4) * na));
-    MF_CUDA(dev_malloc(&w.anchors4, sizeof(float) * na));
-    MF_CUDA(dev_malloc(&w.partials, sizeof(float4) * nbl * b->n));
-    MF_CUDA(dev_malloc(&w.staged, sizeof(mf_trigger) * ncap));
-    MF_CUDA(dev_malloc(&w.keys, sizeof(uint64_t) * ncap));
-    MF_CUDA(dev_malloc(&w.keys_tmp, sizeof(uint64_t) * ncap));
-    MF_CUDA(dev_malloc(&w.idx_a, sizeof(uint32_t) * ncap));
-    MF_CUDA(dev_malloc(&w.idx_b, sizeof(uint32_t) * ncap));
-    MF_CUDA(dev_malloc(&w.tstat, sizeof(uint64_t) * sort_tile_words(ncap)));
-    MF_CUDA(dev_malloc(&w.fctl, sizeof(FilterCtl)));
-    MF_CUDA(cudaMemset(w.fctl, 0, sizeof(FilterCtl)));
-    w.counter = &w.fctl->counter;
-    w.status = &w.fctl->status;
-    MF_CUDA(dev_malloc(&w.ctl, sizeof(unsigned) * (4 + 3 * b->n)));
-    w.exch_elems = ne; w.n_t = b->n; w.cap = ncap; w.anc_elems = na; w.nblk = nbl; w.n_set = ns;
+    w = grown;
     return MF_OK;
 }
 
@@ -1037,24 +1066,32 @@ extern "C" int mf_filter_bank(mf_bank b, const mf_segment *segs, int n_seg, floa
             grouped[(size_t)cand[i]] = 1;
         }
     }
-    int rc = MF_EINVAL;
+    const WorkspaceNeed need{exch_elems, trig_cap, anc_elems, nblk, 1};
     if (!groups.empty()) {
-        int64_t ge = exch_elems, ga = anc_elems, gn = nblk;
-        int n_set = 1;
+        WorkspaceNeed gneed = need;
         for (const FilterGroup &g : groups) {
-            ge = std::max(ge, g.exch_elems);
-            ga = std::max(ga, g.anc_records);
-            gn = std::max(gn, (g.n_partials + n_t - 1) / n_t);
-            n_set = std::max(n_set, g.n);
+            gneed.exch_elems = std::max(gneed.exch_elems, g.exch_elems);
+            gneed.anc_elems = std::max(gneed.anc_elems, g.anc_records);
+            gneed.nblk = std::max(gneed.nblk, (g.n_partials + n_t - 1) / n_t);
+            gneed.n_set = std::max(gneed.n_set, g.n);
         }
-        rc = ensure_workspace(b, ge, trig_cap, ga, gn, n_set, capturing);
-        if (rc) {   // no room for several segments (or none may be made in a capture): one after the other
+        // Groups take a larger workspace only where that costs nothing: not once
+        // a graph may hold the present one's pointers, and not again after there
+        // was no room.  One after the other, the segments need no more than the
+        // longest of them, so a call that ran before runs without growing it.
+        bool together = workspace_holds(b, gneed);
+        if (!together && !capturing && !b->captured && !b->group_no_room) {
+            together = ensure_workspace(b, gneed, false, true) == MF_OK;
+            b->group_no_room = !together;
+        }
+        if (!together) {
             groups.clear();
             std::fill(grouped.begin(), grouped.end(), 0);
         }
     }
-    if (rc) rc = ensure_workspace(b, exch_elems, trig_cap, anc_elems, nblk, 1, capturing);
+    const int rc = ensure_workspace(b, need, capturing, false);
     if (rc) return rc;
+    b->captured = b->captured || capturing;
     Workspace &w = b->ws;
     // descending-cost unit order (MFGB_UNIT_ORDER=bank keeps bank order); the
     // stall hook names a template, the kernels see its unit position

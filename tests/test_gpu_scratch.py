@@ -108,3 +108,77 @@ for refused in (lambda: mf.filter_bank(b, [s], 3.0, trig_cap=1 << 20), lambda: m
     mf.cluster_triggers(trig, nt, b.n, 1, s.N, 40)
     torch.cuda.synchronize()
 """)
+
+
+GRAPH = """
+def loud(lg, seed):     # loudest rho about 4 .. 7
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return mf.Segment(70.0 * torch.randn(1 << lg, dtype=torch.float32, device="cuda", generator=g), 4096.0)
+
+def run(b, segs):
+    return mf.filter_bank(b, segs, 3.5, trig_cap=1 << 16)
+
+def host(out):
+    torch.cuda.synchronize()
+    n = int(out[2].item())
+    return n, out[0].cpu().numpy().tobytes(), out[1][:n].cpu().numpy().tobytes()
+
+def alone_allocates_nothing(call):
+    # the hook fails the next allocation, whoever makes it: still armed afterwards
+    L.mf_debug_fail_alloc(0)
+    out = call()
+    try:
+        bank()
+        raise SystemExit("the call allocated")
+    except mf.MFError as e:
+        assert e.code == mf._native.MF_ENOMEM
+    finally:
+        L.mf_debug_fail_alloc(-1)
+    return out
+"""
+
+
+@pytest.mark.parametrize("captured", ["[s[0]]", "s[:2]", "s"])
+def test_calls_after_a_capture_keep_its_workspace(captured):
+    """A graph of short segments, captured after calls on single ones: eager
+    calls on several allocate nothing, so its replays stay valid."""
+    _child(GRAPH + """
+s = [loud(lg, lg) for lg in (15, 12, 13)]
+ref = host(run(bank(20), s))
+assert 0 < ref[0] <= 1 << 16
+b = bank(20)
+for one in s:
+    run(b, [one])
+part = %s
+want = host(run(bank(20), part))
+torch.cuda.synchronize()
+g = torch.cuda.CUDAGraph()
+with torch.cuda.graph(g):
+    out = run(b, part)
+for _ in range(2):
+    assert host(alone_allocates_nothing(lambda: run(b, s))) == ref
+    out[0].zero_(); out[1].zero_()
+    g.replay()
+    assert host(out) == want
+assert b.check() == 0
+""" % captured)
+
+
+def test_no_room_for_segments_together():
+    """The grouped workspace cannot be had: one after the other, in the one that
+    is there, and later calls do not try again."""
+    _child(GRAPH + """
+s = [loud(lg, lg) for lg in (15, 12, 13)]
+ref = host(run(bank(20), s))
+assert 0 < ref[0] <= 1 << 16
+for k in range(13):                  # every allocation of the larger workspace
+    b = bank(20)
+    for one in s:
+        run(b, [one])
+    torch.cuda.synchronize()
+    L.mf_debug_fail_alloc(k)
+    assert host(run(b, s)) == ref, k
+    L.mf_debug_fail_alloc(-1)
+    assert host(alone_allocates_nothing(lambda: run(b, s))) == ref, k
+    assert b.check() == 0
+""")
