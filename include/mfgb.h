@@ -274,7 +274,9 @@ int mf_chisq_series(mf_bank bank, mf_segment seg, const int32_t *tmpl, int64_t n
  * members of all templates of one segment the same way.  Each event is the
  * loudest member (rho; ties: lower j, then lower template).  events: device
  * array of ev_cap records, written sorted by (seg, j); *n_events (device)
- * receives the true event count (compare with ev_cap for truncation).
+ * receives the true event count (compare with ev_cap for truncation), or -1 if
+ * a bounded device wait ran out (more than 8192 triggers): events then holds no
+ * result.
  * n_tmpl, n_seg, max_N: the bank size, segment count and largest segment
  * length of the filter call (they size the sort keys).  One launch.  Allocates
  * scratch (about 100 bytes per trigger of trig_cap) on cuda_stream; does not
@@ -506,6 +508,11 @@ int mf_debug_fail_alloc(int64_t countdown);
  * what the pools hold) is answered by the CUDA runtime as out of memory;
  * bytes < 0 lifts the limit.  Never fails. */
 int mf_debug_alloc_limit(int64_t bytes);
+
+/* mf_debug_cluster_spin -- test hook: back-off iterations after which a wait
+ * inside mf_cluster_triggers gives up (<= 0 restores the default of 4e6).  Never
+ * fails. */
+int mf_debug_cluster_spin(int64_t limit);
 
 /* mf_debug_scratch_reserved -- bytes of device memory that the library's
  * scratch pools hold in this process, in use or kept for later calls (*bytes,

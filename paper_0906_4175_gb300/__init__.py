@@ -233,7 +233,8 @@ def cluster_triggers(trig, n_trig, n_tmpl: int, n_seg: int, max_N: int, window: 
                      stream=None):
     """mf_cluster_triggers: events from (tmpl, seg, j)-sorted triggers (the
     filter_bank outputs).  Returns (events float32 cuda [ev_cap, 8] laid out
-    as EVENT_DTYPE, n_events int64 cuda [1], the true count)."""
+    as EVENT_DTYPE, n_events int64 cuda [1], the true count, or -1 where a
+    bounded device wait ran out and there is no result)."""
     torch = _torch()
     dev = trig.device
     cap = int(trig.shape[0])
@@ -248,6 +249,8 @@ def cluster_triggers(trig, n_trig, n_tmpl: int, n_seg: int, max_N: int, window: 
 
 def events_to_numpy(ev, n_ev) -> np.ndarray:
     n = int(n_ev.item()) if hasattr(n_ev, "item") else int(n_ev)
+    if n < 0:
+        raise MFError(MF_ETIMEOUT, "a bounded device wait expired in mf_cluster_triggers")
     n = min(n, ev.shape[0])
     return ev[:n].detach().cpu().contiguous().numpy().view(EVENT_DTYPE).reshape(-1)
 

@@ -1481,6 +1481,12 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
     return MF_OK;
 }
 
+static std::atomic<int64_t> g_cluster_spin{4000000};   // limit of a clustering CTA's waits
+extern "C" int mf_debug_cluster_spin(int64_t limit) {
+    g_cluster_spin.store(limit > 0 ? limit : 4000000);
+    return MF_OK;
+}
+
 extern "C" int mf_cluster_triggers(const mf_trigger *trig, const int64_t *n_trig, int64_t trig_cap, int64_t n_tmpl,
                                    int n_seg, int64_t max_N, int32_t window, mf_event *events, int64_t ev_cap,
                                    int64_t *n_events, void *cuda_stream) {
@@ -1505,7 +1511,7 @@ extern "C" int mf_cluster_triggers(const mf_trigger *trig, const int64_t *n_trig
     const size_t o_status = sc.add(sizeof(int));   // zeroed with the control words after it
     get(&w.ctl, sizeof(SortCtl));
     const size_t zeroed = sc.size[0];
-    get(&w.n_c, sizeof(int64_t));
+    get(&w.n_c, 2 * sizeof(int64_t));
     if (cap > cluster_small_limit()) {   // the one-CTA form works in shared memory
         sc.group();
         get(&w.members, sizeof(uint32_t) * cap);
@@ -1530,7 +1536,7 @@ extern "C" int mf_cluster_triggers(const mf_trigger *trig, const int64_t *n_trig
     w.status = sc.at<int>(o_status);
     if (e == cudaSuccess) e = cudaMemsetAsync(w.status, 0, zeroed, st);
     if (e == cudaSuccess)
-        e = launch_cluster(trig, n_trig, cap, window, kl, w, events, ev_cap, n_events, sm_count(), 4000000, st);
+        e = launch_cluster(trig, n_trig, cap, window, kl, w, events, ev_cap, n_events, sm_count(), g_cluster_spin.load(), st);
     sc.free(st);
     if (e != cudaSuccess)
         return set_err(e == cudaErrorMemoryAllocation ? MF_ENOMEM : MF_ECUDA, "cluster_triggers: %s",

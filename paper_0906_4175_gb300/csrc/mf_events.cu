@@ -275,21 +275,10 @@ __device__ __forceinline__ bool cl_scan_tile(const ClusterParams &p, const mf_tr
     return true;
 }
 
-__global__ void __launch_bounds__(kSortThreads, 1) k_cluster(const __grid_constant__ ClusterParams p) {
-    extern __shared__ __align__(16) unsigned char cl_smem[];
-    const int64_t nt = *p.n_trig;
-    const int64_t n = nt < p.cap ? (nt > 0 ? nt : 0) : p.cap;
-    if (n <= kSortSmall) {
-        if (blockIdx.x == 0) {
-            if (n == 0) {
-                if (threadIdx.x == 0) *p.n_events = 0;
-            } else {
-                cluster_small(p, (int)n, cl_smem);
-            }
-        }
-        return;
-    }
-    SortShared &sh = *reinterpret_cast<SortShared *>(cl_smem);
+// The steps of a call of more than kSortSmall records, as tiles.  A CTA whose
+// wait runs out sets ctl->abort and returns.
+__device__ __forceinline__ void cluster_tiles(const ClusterParams &p, int64_t n, unsigned char *smem) {
+    SortShared &sh = *reinterpret_cast<SortShared *>(smem);
     const ClusterScratch &w = p.w;
     const int64_t tn = (n + kSortTile - 1) / kSortTile;
     auto items = [&](int64_t t, int64_t count, auto f) {
@@ -351,17 +340,44 @@ __global__ void __launch_bounds__(kSortThreads, 1) k_cluster(const __grid_consta
     // pass 2: across templates within a segment
     ++ph;
     if (!run_phase(w.ctl, ph, tc, tc, sh, w.status, p.spin_limit, [&](int64_t t) {
-            return cl_scan_tile(p, w.sorted, nc, t, tc, 2, scan2, w.best2, w.members2, w.wsum, perm, p.n_events, sh);
+            return cl_scan_tile(p, w.sorted, nc, t, tc, 2, scan2, w.best2, w.members2, w.wsum, perm, w.n_c + 1, sh);
         }))
         return;
     if (!phase_wait(w.ctl, ph, (unsigned)tc, sh, w.status, p.spin_limit)) return;
-    const int64_t ne = __ldcg(p.n_events), m = ne < p.ev_cap ? ne : p.ev_cap;
+    const int64_t ne = __ldcg(w.n_c + 1), m = ne < p.ev_cap ? ne : p.ev_cap;
     ++ph;
     run_phase(w.ctl, ph, (m + kSortTile - 1) / kSortTile, tc, sh, w.status, p.spin_limit, [&](int64_t t) {
         return items(t, m, [&](int64_t c) {
             p.events[c] = cl_event(w.sorted[cl_index(__ldcg(&w.best2[c]))], __ldcg(&w.wsum[c]), __ldcg(&w.members2[c]));
         });
     });
+}
+
+__global__ void __launch_bounds__(kSortThreads, 1) k_cluster(const __grid_constant__ ClusterParams p) {
+    extern __shared__ __align__(16) unsigned char cl_smem[];
+    const int64_t nt = *p.n_trig;
+    const int64_t n = nt < p.cap ? (nt > 0 ? nt : 0) : p.cap;
+    if (n <= kSortSmall) {
+        if (blockIdx.x == 0) {
+            if (n == 0) {
+                if (threadIdx.x == 0) *p.n_events = 0;
+            } else {
+                cluster_small(p, (int)n, cl_smem);
+            }
+        }
+        return;
+    }
+    cluster_tiles(p, n, cl_smem);
+    // The last CTA to leave writes the count, or -1 where any of them gave up:
+    // the caller sees that there is no result, whatever stage it was lost in.
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&p.w.ctl->left, 1u) == gridDim.x - 1) {
+            __threadfence();
+            *p.n_events = ld_acquire(&p.w.ctl->abort) ? -1 : __ldcg(p.w.n_c + 1);
+        }
+    }
 }
 
 constexpr size_t kClusterSmem = kSortSmemBytes + 2 * (size_t)kSortSmall * sizeof(uint32_t);

@@ -279,7 +279,7 @@ constexpr int kSortMaxPass = 8, kSortMaxPhase = 16;
 struct SortCtl {
     unsigned ghist[kSortMaxPass * 256];
     unsigned ticket[kSortMaxPhase], done[kSortMaxPhase];
-    unsigned abort, pad;
+    unsigned abort, left;   // a wait ran out; CTAs that are done (clustering)
 };
 // what a filter call zeroes before its first kernel
 struct FilterCtl {
@@ -367,7 +367,7 @@ struct ClusterScratch {
     unsigned long long *best, *best2;
     mf_trigger *rep, *sorted;
     uint64_t *keys, *keys_tmp, *tstat, *scan;
-    int64_t *n_c;
+    int64_t *n_c;   // clusters of the first pass, events
     int *status;
     SortCtl *ctl;
 };
