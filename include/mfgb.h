@@ -54,8 +54,10 @@ typedef struct {
 } mf_bank_params;
 
 #define MF_PHASE_ANCHOR 0  /* default: Psi in FP64 at anchor bins, reduced mod 2 pi, FP32 cubic Taylor between them */
-#define MF_PHASE_FP64   1  /* Psi to 4e-10 turns at every bin: FP64 anchors, between them the Taylor series to 7th
-                              order, its cubic part in 64-bit fixed-point turns; per-batch launches always */
+#define MF_PHASE_FP64   1  /* FP64 accuracy at every bin: the filter and the chi^2 series sum the 7th-order Taylor
+                              series about FP64 anchors (its cubic part in 64-bit fixed-point turns), which hands the
+                              sincos Psi to 8e-9 turns, twice as close as FP64 rounded to FP32 (1.5e-8); mf_chisq_points
+                              and mf_refine_* evaluate Psi in FP64 at every bin.  Per-batch launches always */
 #define MF_PHASE_FP32   2  /* Psi in FP32 only, no FP64 reduction (precision-sweep reference; loses accuracy) */
 #define MF_FFT_FP32     0  /* default: every FFT stage in FP32 on the CUDA cores */
 /* Precision-sweep forms (config "FFT in FP32 vs a tensor-core DFT-GEMM radix stage"): the first radix-32
@@ -508,6 +510,12 @@ int mf_debug_fail_alloc(int64_t countdown);
  * what the pools hold) is answered by the CUDA runtime as out of memory;
  * bytes < 0 lifts the limit.  Never fails. */
 int mf_debug_alloc_limit(int64_t bytes);
+
+/* mf_debug_phase -- the phase of template `tmpl` that the filter of an
+ * MF_PHASE_FP64 bank hands to its sincos, in turns mod 1, at every bin of the
+ * segment (turns: device double [N/2]; 0 outside the band).  Errors: MF_EINVAL
+ * (NULL, range, another phase mode, devices), MF_ECUDA. */
+int mf_debug_phase(mf_bank bank, mf_segment seg, int64_t tmpl, double *turns, void *cuda_stream);
 
 /* mf_debug_cluster_spin -- test hook: back-off iterations after which a wait
  * inside mf_cluster_triggers gives up (<= 0 restores the default of 4e6).  Never

@@ -60,6 +60,7 @@ SIGNATURES = {
     "mf_bank_debug_stall": (_I, [_P, _I64, _I64]),
     "mf_debug_fail_alloc": (_I, [_I64]),
     "mf_debug_alloc_limit": (_I, [_I64]),
+    "mf_debug_phase": (_I, [_P, _P, _I64, _P, _P]),
     "mf_debug_cluster_spin": (_I, [_I64]),
     "mf_debug_scratch_reserved": (_I, [_P]),
     "mf_autotune": (_I, [_P, _P, _I, _F, _I, ctypes.c_char_p, _P]),

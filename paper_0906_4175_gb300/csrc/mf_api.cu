@@ -2032,6 +2032,19 @@ extern "C" int mf_debug_fail_alloc(int64_t countdown) {
     return MF_OK;
 }
 
+extern "C" int mf_debug_phase(mf_bank b, mf_segment seg, int64_t tmpl, double *turns, void *cuda_stream) {
+    if (!b || !seg || !turns) return set_err(MF_EINVAL, "NULL argument");
+    if (tmpl < 0 || tmpl >= b->n) return set_err(MF_EINVAL, "template out of range");
+    if (b->params.phase_mode != MF_PHASE_FP64) return set_err(MF_EINVAL, "the bank's phase mode is not MF_PHASE_FP64");
+    int cur = 0;
+    MF_CUDA(cudaGetDevice(&cur));
+    if (b->device != cur || seg->device != cur) return set_err(MF_EINVAL, "bank or segment on another device");
+    MF_CUDA(launch_phase64(seg_dev(seg), b->d_tmpl, (int)tmpl, b->params.f_low, choose_log2D(b, seg), turns,
+                           (cudaStream_t)cuda_stream));
+    count_launches(1);
+    return MF_OK;
+}
+
 extern "C" int mf_debug_alloc_limit(int64_t bytes) {
     g_alloc_limit.store(bytes < 0 ? -1 : bytes);
     return MF_OK;

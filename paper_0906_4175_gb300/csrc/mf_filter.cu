@@ -65,6 +65,33 @@ __global__ void k_anchors64(SegDev seg, const double *__restrict__ tmpl, const U
     }
 }
 
+// turns[k], k < N/2: the phase that pass 1 of MF_PHASE_FP64 hands to its sincos
+// (mf_debug_phase), from the same two functions; 0 outside the template's band
+__global__ void k_phase64(SegDev seg, const double *__restrict__ tmpl, int t, double f_low, int log2D,
+                          double *__restrict__ turns) {
+    int64_t k0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    chain_wait(k0);
+    const double *T = tmpl + (int64_t)t * kTmplStride;
+    const UnitInfo u = unit_info(seg, T, t, f_low, 0.f, log2D);
+    for (int64_t k = k0; k < seg.N / 2; k += (int64_t)gridDim.x * blockDim.x) {
+        double out = 0.0;
+        if (k >= u.k_lo && k < u.k_hi) {
+            const int64_t g = k >> log2D;
+            const Anchor64 r = anchor_record64(T[TF_C1], T[TF_C2], T[TF_C3], T[TF_C5], g, log2D, seg.df);
+            auto lo = [](unsigned long long x) { return __int_as_float((int)(unsigned)x); };
+            auto hi = [](unsigned long long x) { return __int_as_float((int)(unsigned)(x >> 32)); };
+            const int d = (int)(k - ((g << log2D) + ((1 << log2D) >> 1)));
+            const float df = (float)d;
+            unsigned sign;
+            out = (double)anchor_phase64(make_float4(lo(r.r0), hi(r.r0), lo(r.q1), hi(r.q1)),
+                                         make_float4(lo(r.q2), hi(r.q2), lo(r.q3), hi(r.q3)),
+                                         make_float4(r.q4, r.q5, r.q6, r.q7), d, df, (df * df) * (df * df), sign);
+            if (sign) out += 0.5;
+        }
+        turns[k] = out;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // launches
 // ---------------------------------------------------------------------------
@@ -88,6 +115,11 @@ cudaError_t launch_anchors(const SegDev &seg, const double *tmpl, const UnitInfo
     }
     return launch(k_anchors, dim3(gx, n_units), per, 0, st, seg, tmpl, units, unit0, log2D, max_anc, anchors, anchors4,
                   reps);
+}
+
+cudaError_t launch_phase64(const SegDev &seg, const double *tmpl, int t, double f_low, int log2D, double *turns,
+                           cudaStream_t st) {
+    return launch(k_phase64, dim3((unsigned)((seg.N / 2 + 255) / 256)), 256, 0, st, seg, tmpl, t, f_low, log2D, turns);
 }
 
 namespace {

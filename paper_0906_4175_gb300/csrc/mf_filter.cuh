@@ -239,9 +239,19 @@ struct TemplateSrcNarrow : TemplateSrc<L, C, LG1> {
 //   psi = r0 + d (q1 + d (q2 + d q3))  (mod 1, exact in 2^-64 turns)  +  d^4 (q4 + d (q5 + d (q6 + d q7)))
 // where the cubic part is three 64-bit integer multiply-adds (d is an integer,
 // so the coefficients count mod 1) and the small rest FP32.  anchor_log2D64
-// bounds what is left out and the size of the FP32 part, so that psi is good
-// to 4e-10 turns before it is rounded to FP32 (1.5e-8, as before) for the sincos.
-// Record: three planes of 16 bytes (r0, q1 | q2, q3 | q4, q5, q6, q7).
+// bounds what is left out and the size of the FP32 part: the sum, in 2^-32
+// turns, is off by 2^-33 (the low word, rounded) + 2^-33 (the FP32 part in those
+// units) + its own rounding, 1e-10, + 5e-11 left out: 4e-10 turns at most.
+// u comes from two Newton steps: one leaves 4e-14 of u, up to 4e-10 turns of a
+// light template at 10 Hz.  What counts is the phase the sincos gets.  psi in
+// FP64 at every bin, rounded to FP32 in [-1/2, 1/2], is off by up to 1.5e-8
+// turns; half turns are taken off first here (they change signs only), so the
+// rounding is 2^-27 at most and the whole 7.9e-9.  Over 1-34 solar masses, 10 to
+// 40 Hz, N = 2^10 .. 2^22: 7.7e-9 and 3.3e-9 rms; FP64 at every bin 1.5e-8 and
+// 6.5e-9.  The distance of the z series from 64 bits, 2^14 .. 2^20, is 0.4 to
+// 1.3 % below that of FP64 at every bin (sincos and FFT make up most of it).
+// Record: three planes of 16 bytes (r0, q1 | q2, q3 | q4, q5, q6, q7), r0 with
+// the half unit that rounds the low word.
 // ---------------------------------------------------------------------------
 struct Anchor64 {
     unsigned long long r0, q1, q2, q3;
@@ -264,7 +274,8 @@ __device__ __forceinline__ Anchor64 anchor_record64(double c1, double c2, double
     const int64_t ka = (g << log2D) + ((1 << log2D) >> 1);
     const double f = (double)ka * df;
     double uu = (double)rcbrtf((float)f);
-    uu = uu * (4.0 - f * uu * uu * uu) * (1.0 / 3.0);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) uu = uu * (4.0 - f * uu * uu * uu) * (1.0 / 3.0);
     const double u2 = uu * uu;
     const double psi = -0.125 + uu * (c1 + uu * (c2 + uu * (c3 + u2 * c5)));
     const double S1 = uu * (c1 + uu * (2.0 * c2 + uu * (3.0 * c3 + u2 * (5.0 * c5))));
@@ -276,7 +287,7 @@ __device__ __forceinline__ Anchor64 anchor_record64(double c1, double c2, double
     const float w5 = (float)c5 * (uf * uf) * (uf * uf * uf);
     const double S3 = uu * (28.0 * c1 + uu * (80.0 * c2 + uu * (162.0 * c3 + u2 * (440.0 * c5))));
     Anchor64 a;
-    a.r0 = turns_fixed(psi);
+    a.r0 = turns_fixed(psi) + (1ull << 31);
     a.q1 = turns_fixed(S1 * ik * (-1.0 / 3.0));
     a.q2 = turns_fixed(S2 * ik2 * (1.0 / 18.0));
     a.q3 = turns_fixed(S3 * (ik2 * ik) * (-1.0 / 162.0));
@@ -287,9 +298,10 @@ __device__ __forceinline__ Anchor64 anchor_record64(double c1, double c2, double
            (1.f / 11022480.f);
     return a;
 }
-// phase in turns at integer offset d, d4 = d^4
+// phase in turns at integer offset d, d4 = d^4, less the half turn that sign
+// says (bit 31: it belongs on the sine and the cosine): in [-1/4, 1/4]
 __device__ __forceinline__ float anchor_phase64(const float4 &p0, const float4 &p1, const float4 &p2, int d, float df,
-                                                float d4) {
+                                                float d4, unsigned &sign) {
     auto word = [](float lo, float hi) {
         return ((unsigned long long)(unsigned)__float_as_int(hi) << 32) | (unsigned)__float_as_int(lo);
     };
@@ -298,9 +310,12 @@ __device__ __forceinline__ float anchor_phase64(const float4 &p0, const float4 &
         word(p0.x, p0.y) + dd * (word(p0.z, p0.w) + dd * (word(p1.x, p1.y) + dd * word(p1.z, p1.w)));
     const float tail = d4 * fmaf(df, fmaf(df, fmaf(df, p2.w, p2.z), p2.y), p2.x);
     // |tail| < 2^-10: added to 1.5 * 2^-9 its mantissa counts 2^-32 turns
-    const int hi = (int)(t >> 32) + (__float_as_int(tail + 0.0029296875f) - 0x3b400000);
-    return (float)hi * 2.3283064365386963e-10f;   // 2^-32: in [-1/2, 1/2], rounded once
+    const unsigned hi = (unsigned)(t >> 32) + (unsigned)(__float_as_int(tail + 0.0029296875f) - 0x3b400000);
+    const int rest = (int)(hi << 1) >> 1;   // mod half a turn
+    sign = (hi ^ (unsigned)rest) & 0x80000000u;
+    return (float)rest * 2.3283064365386963e-10f;   // 2^-32; rounded once
 }
+__device__ __forceinline__ float flip_sign(float x, unsigned sign) { return __int_as_float(__float_as_int(x) ^ (int)sign); }
 
 // pass-1 source of MF_PHASE_FP64
 template <int L, int C, int LG1>
@@ -378,9 +393,12 @@ struct TemplateSrc64 {
                 d = kk - ((g << p.log2D) + (D >> 1));
             }
             const float df = (float)d;
-            const float ph = anchor_phase64(a0, a1, a2, d, df, (df * df) * (df * df));
+            unsigned sign;
+            const float ph = anchor_phase64(a0, a1, a2, d, df, (df * df) * (df * df), sign);
             float sn, cs;
             __sincosf(6.283185307179586f * ph, &sn, &cs);
+            sn = flip_sign(sn, sign);
+            cs = flip_sign(cs, sign);
             const float2 x = make_float2(fmaf(w[r].x, cs, w[r].y * sn), fmaf(w[r].y, cs, -w[r].x * sn));
             v[r] = in[r] ? x : czero();   // rows outside the band read stale records
         }

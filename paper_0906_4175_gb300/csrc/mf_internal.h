@@ -220,6 +220,8 @@ cudaError_t launch_units(const SegDev &seg, const double *tmpl, int n_t, double 
 cudaError_t launch_anchors(const SegDev &seg, const double *tmpl, const UnitInfo *units, int unit0,
                            int n_units, int log2D, int max_anc, float4 *anchors, float *anchors4, int phase_mode,
                            cudaStream_t st, int reps = 1);
+cudaError_t launch_phase64(const SegDev &seg, const double *tmpl, int t, double f_low, int log2D, double *turns,
+                           cudaStream_t st);
 // MF_PHASE_FP64: slots of three planes of max_anc 16-byte records, anchors4 unused, reps = 1.
 // (reps > 1: every record is also stored reps - 1 more times, n_units slots
 // apart, for launches that cover several bands of the same templates)
