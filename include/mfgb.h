@@ -255,7 +255,8 @@ int mf_fft_c2c(const void *x, void *y, int64_t N, int64_t batch, int sign, void 
  * bank gives an empty band (a zero row).  1 <= p <= 64, 1 <= n <= 2^24.
  * Cost: p + 1 inverse FFTs of length N per template (the first passes of a
  * batch's p + 1 bands run as one launch and the second passes as one kernel that
- * sums the sub-bands in registers).
+ * sums the sub-bands in registers).  The row of a template has the same bits
+ * alone and in any list.
  * Allocates scratch on cuda_stream (p + 1 exchanges of 8 N bytes per
  * template of a batch, batches sized to the bank's exchange budget: 4 GiB
  * unless mf_autotune chose another), so it cannot be captured in a graph, and

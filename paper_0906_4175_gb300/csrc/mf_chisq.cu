@@ -78,7 +78,7 @@ __global__ void k_chisq_units(SegDev seg, const UnitInfo *__restrict__ all, int 
 // call, 104 us now.
 // ---------------------------------------------------------------------------
 struct ChiTilesParams {
-    const float2 *exch;
+    float2 *exch;           // group sums are kept over bands already read
     const UnitInfo *full;   // full-band units of the call's template list
     float *chisq;           // [n][N]
     int unit0, nb, p;
@@ -101,14 +101,18 @@ struct ChiWarpSync {
     static __device__ __forceinline__ void sync() { __syncwarp(); }
 };
 
-// p |raw_l|^2 of the thread's 32 outputs summed over the CTA's l < p, less
-// |raw|^2 of the full band l = p.  The bands are taken in descending order, the
-// one pass 1 wrote last first: of an exchange somewhat larger than L2 the
-// ascending order finds nothing left.
+// p |raw_l|^2 of the thread's 32 outputs summed over the bands l < p it has seen
+// since the last start, less |raw|^2 of the full band l = p.  The bands are taken
+// in descending order, the one pass 1 wrote last first: of an exchange somewhat
+// larger than L2 the ascending order finds nothing left.
 struct ChiTileAcc {
     float acc[32];
     int l = 0, p = 0;
     float pf = 0.f;
+    __device__ __forceinline__ void start() {
+#pragma unroll
+        for (int r = 0; r < 32; ++r) acc[r] = 0.f;
+    }
     template <int R>
     __device__ __forceinline__ void store(int, int, int, const float2 *v) {
 #pragma unroll
@@ -117,18 +121,52 @@ struct ChiTileAcc {
             acc[r] = l == p ? -pw : fmaf(pf, pw, acc[r]);
         }
     }
+    // kept in 16 float2 of this thread, T apart
+    template <int T>
+    __device__ __forceinline__ void put(float2 *x) const {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) __stcg(&x[i * T], make_float2(acc[2 * i], acc[2 * i + 1]));
+    }
+    template <int T>
+    __device__ __forceinline__ void add(const float2 *x) {   // acc = x + acc
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const float2 v = __ldcg(&x[i * T]);
+            acc[2 * i] = v.x + acc[2 * i];
+            acc[2 * i + 1] = v.y + acc[2 * i + 1];
+        }
+    }
 };
 
-// S > 1: a cluster of S CTAs shares a tile, CTA c taking the sub-bands [c q, c q + q)
-// of the p + 1, q = ceil((p + 1) / S); each sums its own, and the CTAs add the
-// sums through distributed shared memory, 1 / S of the tile each.  A tile a CTA
-// leaves the GPU to a few: 16 templates at N = 2^16, p = 16, are 128 tiles, 17
-// transforms of 3.6 us one after the other, 61 us; 50 us in pairs of CTAs whose warps (with their own
-// rows) do not wait for one another: 59 with CTA barriers, 53 in ascending order.
+// Rows of up to 512 points: a sample's sum has one order whatever CTAs form it, so
+// a template's chi^2 has the same bits alone and in every list.  The bands form
+// four groups from p = 7 on, two from p = 3 on, each summed in descending order;
+// the sum is (G3 + G2) + (G1 + G0) or G1 + G0.
+template <int L>
+__host__ __device__ constexpr bool chi_ordered() { return L <= 512; }
+__host__ __device__ __forceinline__ int chi_groups(int p) { return p >= 7 ? 4 : (p >= 3 ? 2 : 1); }
+__device__ __forceinline__ int chi_start(int g, int of, int p) { return (g * (p + 1) + of - 1) / of; }
+
+// S > 1: a cluster of S CTAs shares a tile, CTA c taking the groups of part c of
+// S; the CTAs add their sums through distributed shared memory, 1 / S of the tile
+// each.  A CTA with several groups keeps the sums of all but its last where it
+// has just read the band that begins the group: each thread over its own 32
+// points of the exchange, which nothing reads again.  A sum kept is 64 KB a tile
+// more to move, 1 % of a call (200 templates at 2^16, p = 16: 881 us in one sum,
+// 910 in four; pairs keep one each, 16 templates 103.7 -> 105.5; fours none, 9
+// templates 89 -> 87).  Kept in 32 KB of shared memory the L1 that is left cannot
+// hold the loads in flight (72 us for the 50 below), 32 more registers a thread
+// would spill, and one sum in order over four CTAs, the lower ones adding their
+// bands late, was 94 -> 105 us for 30 templates at 2^14.
+// A tile a CTA leaves the GPU to a few: 16 templates at N = 2^16, p = 16, are 128
+// tiles, 17 transforms of 3.6 us one after the other, 61 us; 50 us in pairs of CTAs
+// whose warps (with their own rows) do not wait for one another: 59 with CTA
+// barriers, 53 in ascending order.
 template <int L, int C, int S>
 __global__ void __launch_bounds__(C *(L / 32), (C * (L / 32) >= 256) ? 2 : 1) k_chisq_tiles(ChiTilesParams q) {
     extern __shared__ float2 chi_smem[];
     constexpr int T = L / 32, NT = C * T;
+    static_assert(chi_ordered<L>() || S == 1, "clusters keep the order of the sum");
     // rows of up to 1024 points lie within a warp: no barrier holds the warps together
     using Sync = std::conditional_t<(L <= 1024), ChiWarpSync, CtaSync>;
     float2 *tw = chi_smem + pass_data_bytes<L, C>() / sizeof(float2);
@@ -136,13 +174,18 @@ __global__ void __launch_bounds__(C *(L / 32), (C * (L / 32) >= 256) ? 2 : 1) k_
     const int c = S > 1 ? (int)(blockIdx.x % S) : 0;   // rank in the cluster
     fill_twiddles<L>(tw);
     chain_wait(tile, b);
-    const int per = (q.p + S) / S, l0 = min(c * per, q.p + 1), l1 = min(l0 + per, q.p + 1);
+    const int groups = chi_ordered<L>() ? chi_groups(q.p) : 1;
+    const int l0 = chi_start(c, S, q.p), l1 = chi_start(c + 1, S, q.p);
+    // the bands that begin the groups 1, 2 (or the upper of two) and 3; a CTA's last group ends with l0
+    const int b1 = groups == 4 ? chi_start(1, 4, q.p) : -1, b3 = groups == 4 ? chi_start(3, 4, q.p) : -1;
+    const int b2 = groups > 1 ? chi_start(1, 2, q.p) : -1;
     const float rs = q.full[q.unit0 + b].rho_scale, rs2 = rs * rs;
     ChiTileAcc snk;
     snk.p = q.p;
     snk.pf = (float)q.p;
-#pragma unroll
-    for (int r = 0; r < 32; ++r) snk.acc[r] = 0.f;
+    snk.start();
+    const int seq = threadIdx.x / T, t = threadIdx.x % T;
+    auto kept = [&](int l) { return q.exch + ((int64_t)(l * q.nb + b) << q.log2N) + (int64_t)(tile * C + seq) * L + t; };
     const typename RowSrc<L, C>::Params rp{q.exch, q.log2N1, q.log2N};
     __syncthreads();   // twiddles
 #pragma unroll 1
@@ -150,8 +193,20 @@ __global__ void __launch_bounds__(C *(L / 32), (C * (L / 32) >= 256) ? 2 : 1) k_
         snk.l = l;
         ChiTileSrc<L, C, Sync> src{RowSrc<L, C>(rp, tile, 0, l * q.nb + b, nullptr), l < l1 - 1};
         cta_fft<L, C, false, +1, ChiTileSrc<L, C, Sync>, ChiTileAcc, Sync>(chi_smem, tw, src, snk);
+        if (chi_ordered<L>() && S < 4 && l > l0 && (l == b1 || l == b2 || l == b3)) {
+            if (S == 1 && groups == 4 && l == b2) {   // G3 + G2, in the place of G3
+                snk.template add<T>(kept(b3));
+                snk.template put<T>(kept(b3));
+            } else {
+                snk.template put<T>(kept(l));
+            }
+            snk.start();
+        }
     }
-    const int seq = threadIdx.x / T, t = threadIdx.x % T;
+    if (chi_ordered<L>() && S < 4) {
+        if (groups == 4) snk.template add<T>(kept(c > 0 ? b3 : b1));
+        if (S == 1 && groups > 1) snk.template add<T>(kept(groups == 4 ? b3 : b2));
+    }
     auto row = [&](int s) { return reinterpret_cast<float *>(chi_smem + s * SeqStride<L, C>::value); };
     __syncthreads();   // the last stage has read the sequences
     float *out = q.chisq + ((int64_t)(q.unit0 + b) << q.log2N) + tile * C;
@@ -172,9 +227,9 @@ __global__ void __launch_bounds__(C *(L / 32), (C * (L / 32) >= 256) ? 2 : 1) k_
         cl.sync();
         for (int idx = c * (C * L / S) + threadIdx.x; idx < (c + 1) * (C * L / S); idx += NT) {
             const int s = idx % C, j1 = idx / C;
-            float a = 0.f;
-#pragma unroll
-            for (int i = 0; i < S; ++i) a += reinterpret_cast<const float *>(peer[i] + s * SeqStride<L, C>::value)[j1];
+            auto sum = [&](int i) { return reinterpret_cast<const float *>(peer[i] + s * SeqStride<L, C>::value)[j1]; };
+            float a = sum(1) + sum(0);
+            if constexpr (S == 4) a = (sum(3) + sum(2)) + a;
             __stcs(&out[s + ((int64_t)j1 << q.log2N2)], rs2 * a);
         }
         cl.sync();   // no CTA leaves while its sums are being read
@@ -368,32 +423,31 @@ struct ChiTilesOp {
     const ChiTilesParams *q;   // NULL: set the kernel attributes only
     int n_sm;
     cudaStream_t st;
+    template <int N2, int N1, int S>
+    cudaError_t tiles() {
+        constexpr int C = seqs_per_cta<N1>(N2);
+        constexpr size_t smem = chi_tiles_smem_bytes<N1, C>();
+        if (!q)
+            return cudaFuncSetAttribute(k_chisq_tiles<N1, C, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        return launch_cluster(k_chisq_tiles<N1, C, S>, dim3(S * (N2 / C), q->nb), C * (N1 / 32), S > 1 ? S : 0, smem, st, *q);
+    }
     template <int N2, int N1>
     cudaError_t run() {
         if constexpr (N1 != 1024) {
-            constexpr int C = seqs_per_cta<N1>(N2);
-            constexpr size_t smem = chi_tiles_smem_bytes<N1, C>();
-            constexpr unsigned threads = C * (N1 / 32);
-            auto attr = [&](auto kernel) {
-                return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            };
-            if constexpr (N1 <= 512) {   // a template of 2048-point rows is 256 tiles and more
+            if constexpr (chi_ordered<N1>()) {   // a template of 2048-point rows is 256 tiles and more
                 if (!q) {
-                    cudaError_t e = attr(k_chisq_tiles<N1, C, 2>);
-                    if (e == cudaSuccess) e = attr(k_chisq_tiles<N1, C, 4>);
+                    cudaError_t e = tiles<N2, N1, 2>();
+                    if (e == cudaSuccess) e = tiles<N2, N1, 4>();
                     if (e != cudaSuccess) return e;
                 } else {
                     // as many CTAs per tile as keep the launch within one wave (two per
-                    // SM), with two sub-bands or more each
-                    const int64_t tiles = (int64_t)(N2 / C) * q->nb, wave = 2 * (int64_t)n_sm;
-                    if (4 * tiles <= wave && q->p >= 7)
-                        return launch_cluster(k_chisq_tiles<N1, C, 4>, dim3(4 * (N2 / C), q->nb), threads, 4, smem, st, *q);
-                    if (2 * tiles <= wave && q->p >= 3)
-                        return launch_cluster(k_chisq_tiles<N1, C, 2>, dim3(2 * (N2 / C), q->nb), threads, 2, smem, st, *q);
+                    // SM), with a group each, of two sub-bands or more
+                    const int64_t n = (int64_t)(N2 / seqs_per_cta<N1>(N2)) * q->nb, wave = 2 * (int64_t)n_sm;
+                    if (4 * n <= wave && chi_groups(q->p) == 4) return tiles<N2, N1, 4>();
+                    if (2 * n <= wave && chi_groups(q->p) >= 2) return tiles<N2, N1, 2>();
                 }
             }
-            if (!q) return attr(k_chisq_tiles<N1, C, 1>);
-            return launch(k_chisq_tiles<N1, C, 1>, dim3(N2 / C, q->nb), threads, smem, st, *q);
+            return tiles<N2, N1, 1>();
         } else {
             return q ? cudaErrorInvalidValue : cudaSuccess;   // 1024-point rows: k_chisq_rows
         }
@@ -407,7 +461,7 @@ cudaError_t launch_chisq_units(const SegDev &seg, const UnitInfo *all, int n_t, 
     return launch(k_chisq_units, dim3(n), p >= 8 ? 256 : 128, 0, st, seg, all, n_t, tmpl, n, p, out, edges);
 }
 
-cudaError_t launch_chisq_tiles(const SegDev &seg, const float2 *exch, const UnitInfo *full, int unit0, int nb, int p,
+cudaError_t launch_chisq_tiles(const SegDev &seg, float2 *exch, const UnitInfo *full, int unit0, int nb, int p,
                                float *chisq, int n_sm, cudaStream_t st) {
     ChiTilesParams q{exch, full, chisq, unit0, nb, p, seg.log2N, seg.log2N1, seg.log2N2};
     ChiTilesOp op{&q, n_sm, st};

@@ -359,7 +359,7 @@ cudaError_t launch_chisq_units(const SegDev &seg, const UnitInfo *all, int n_t, 
                                UnitInfo *out, int64_t *edges, cudaStream_t st);
 // row IFFTs of all p + 1 bands of nb templates and chi^2 (row lengths other
 // than 1024); band l of entry b at exch + (l nb + b) N
-cudaError_t launch_chisq_tiles(const SegDev &seg, const float2 *exch, const UnitInfo *full, int unit0, int nb, int p,
+cudaError_t launch_chisq_tiles(const SegDev &seg, float2 *exch, const UnitInfo *full, int unit0, int nb, int p,
                                float *chisq, int n_sm, cudaStream_t st);
 
 // trigger clustering scratch (arrays sized for the trigger capacity; ctl
