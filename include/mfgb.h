@@ -260,9 +260,9 @@ int mf_fft_c2c(const void *x, void *y, int64_t N, int64_t batch, int sign, void 
  * Allocates scratch on cuda_stream (p + 1 exchanges of 8 N bytes per
  * template of a batch, batches sized to the bank's exchange budget: 4 GiB
  * unless mf_autotune chose another), so it cannot be captured in a graph, and
- * returns without synchronising.  A bounded device wait that runs out (row
- * copies of the N = 2^19, 2^20 kernel) makes the next mf_bank_check on this
- * bank return MF_ETIMEOUT.
+ * returns without synchronising.  A bounded device wait that runs out (copies
+ * of the staged first pass where it runs and of the N = 2^19, 2^20 rows kernel)
+ * makes the next mf_bank_check on this bank return MF_ETIMEOUT.
  * Errors: MF_EINVAL (NULL, sizes, devices, f_low >= f_cut, inside a capture),
  * MF_ENOMEM, MF_ECUDA. */
 int mf_chisq_series(mf_bank bank, mf_segment seg, const int32_t *tmpl, int64_t n, int p,

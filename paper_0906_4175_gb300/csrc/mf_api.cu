@@ -1427,8 +1427,9 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
     const int64_t batch =
         std::max<int64_t>(1, std::min<int64_t>({n, budget / (8 * seg->N * (p + 1)), 65535 / (p + 1)}));
     const bool anchors = b->params.phase_mode != MF_PHASE_FP32;
-    if (rows && !b->chi_status) MF_CUDA(dev_malloc(&b->chi_status, sizeof(int)));
-    if (b->chi_status) MF_CUDA(cudaMemsetAsync(b->chi_status, 0, sizeof(int), st));
+    // the staged pass 1 and the rows kernel report waits that run out here
+    if (!b->chi_status) MF_CUDA(dev_malloc(&b->chi_status, sizeof(int)));
+    MF_CUDA(cudaMemsetAsync(b->chi_status, 0, sizeof(int), st));
     // One pass-1 launch per batch covers all p + 1 bands: unit slot l nb + s is
     // band l of template u0 + s (a band-major copy of the batch's units).  The
     // persistent pass 1 reads the copy of its template's anchors that the

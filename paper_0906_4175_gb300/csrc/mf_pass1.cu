@@ -253,6 +253,7 @@ cudaError_t launch_pass1_pf(const SegDev &seg, const UnitInfo *units, int unit0,
                             int max_anc, const float4 *anchors, const float *anchors4, float2 *exch, bool half_tile,
                             int *status, long long spin_limit, cudaStream_t st, int form) {
     if (n_units <= 0) return cudaSuccess;
+    if (!status) return cudaErrorInvalidValue;   // where a wait that runs out is reported
     Pass1PfParams p{seg.W, units, anchors, anchors4, exch, max_anc, log2D, seg.log2N, unit0, 0, status, spin_limit};
     PfOp op{&p, (const CUtensorMap *)seg.w_tmap, n_units, half_tile, st, false, form};
     return dispatch_split2(seg.log2N, seg.log2N2, op);

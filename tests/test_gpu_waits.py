@@ -44,3 +44,14 @@ def test_clustering_that_gives_up_says_so(mf, n):
     assert e.value.code == mf.MF_ETIMEOUT
     ev2, n_ev = mf.cluster_triggers(trig, nt, 1, 1, 1 << 20, 3)
     assert int(n_ev.item()) == n and torch.equal(ev2.view(torch.int32), ev.view(torch.int32))
+
+
+@pytest.mark.parametrize("lg", [16, 17, 18, 19, 21, 22])
+def test_chisq_reports_waits_at_every_length(mf, lg):
+    """The staged first pass needs a place for the status of a wait that runs
+    out, and refuses to start without one; a new bank's first call has it."""
+    import torch
+    bank = mf.Bank([1.4, 2.0], [1.3, 1.7])
+    seg = mf.Segment(torch.randn(1 << lg, dtype=torch.float32, device="cuda"), 4096.0)
+    chi, _ = mf.chisq_series(bank, seg, [0, 1], p=2)
+    assert bank.check() == 0 and bool(torch.isfinite(chi).all())
