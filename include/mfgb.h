@@ -259,7 +259,9 @@ int mf_fft_c2c(const void *x, void *y, int64_t N, int64_t batch, int sign, void 
  * alone and in any list.
  * Allocates scratch on cuda_stream (p + 1 exchanges of 8 N bytes per
  * template of a batch, batches sized to the bank's exchange budget: 4 GiB
- * unless mf_autotune chose another), so it cannot be captured in a graph, and
+ * unless mf_autotune chose another; where that finds no room, smaller batches,
+ * and except at N = 2^19 and 2^20 one template's bands in turn through 20 N
+ * bytes, with the same results), so it cannot be captured in a graph, and
  * returns without synchronising.  A bounded device wait that runs out (copies
  * of the staged first pass where it runs and of the N = 2^19, 2^20 rows kernel)
  * makes the next mf_bank_check on this bank return MF_ETIMEOUT.

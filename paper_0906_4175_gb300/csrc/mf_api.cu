@@ -217,6 +217,7 @@ static void handle_destroyed() {
 // (-1 = disarmed).  mf_debug_alloc_limit: an allocation past the limit asks the
 // runtime for more than any device holds, at every attempt.
 static std::atomic<int64_t> g_fail_alloc{-1}, g_alloc_limit{-1};
+static thread_local bool t_fault_injected = false;   // the thread's last failed attempt was mf_debug_fail_alloc's
 static bool alloc_fault() {
     int64_t v = g_fail_alloc.load();
     while (v >= 0)
@@ -235,7 +236,8 @@ static bool stream_done(cudaStream_t st) { return !stream_capturing(st) && cudaS
 // wait: true once the caller's queued work is done (and it may be waited for)
 template <class W, class F>
 static cudaError_t allocate(size_t bytes, bool pooled, W wait, F get) {
-    if (alloc_fault()) return cudaErrorMemoryAllocation;
+    t_fault_injected = alloc_fault();
+    if (t_fault_injected) return cudaErrorMemoryAllocation;
     cudaError_t e = get(limited(bytes, pooled));
     if (e != cudaErrorMemoryAllocation) return e;
     cudaGetLastError();
@@ -1421,11 +1423,14 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
     const int man = (int)anchor_slot_records(seg->log2N, lgD);   // records per anchor slot
     const int n_t = (int)b->n;
     // every sub-band's exchange of a batch first, then one kernel that runs the
-    // row IFFTs over all of them (p + 1 exchanges per template in flight)
+    // row IFFTs over all of them (p + 1 exchanges per template in flight).  Where
+    // there is no room for that, fewer templates at a time, and for the last one,
+    // unless its rows have 1024 points, band after band through one exchange:
+    // 20 N bytes instead of 8 N (p + 1), as many launches more, the same bits.
     const bool rows = chisq_rows_applies(seg->log2N);
     const int64_t budget = b->tuned_exch > 0 ? b->tuned_exch : kExchBudget;
-    const int64_t batch =
-        std::max<int64_t>(1, std::min<int64_t>({n, budget / (8 * seg->N * (p + 1)), 65535 / (p + 1)}));
+    int64_t batch = std::max<int64_t>(1, std::min<int64_t>({n, budget / (8 * seg->N * (p + 1)), 65535 / (p + 1)}));
+    bool stepwise = false;
     const bool anchors = b->params.phase_mode != MF_PHASE_FP32;
     // the staged pass 1 and the rows kernel report waits that run out here
     if (!b->chi_status) MF_CUDA(dev_malloc(&b->chi_status, sizeof(int)));
@@ -1435,15 +1440,26 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
     // persistent pass 1 reads the copy of its template's anchors that the
     // anchor launch stores for each band; the per-tile form shares them.
     const bool pf = p1_form(b) != 1 && pass1_pf_applies(sd.log2N, sd.log2N2, lgD, b->params.phase_mode);
-    const int reps = pf ? p + 1 : 1;
     Scratch sc;
-    const size_t o_all = sc.add(sizeof(UnitInfo) * n_t), o_units = sc.add(sizeof(UnitInfo) * (size_t)(p + 1) * n);
-    const size_t o_mu = sc.add(sizeof(UnitInfo) * (size_t)(p + 1) * batch);
-    sc.group();
-    const size_t o_anc = sc.add(sizeof(float4) * man * batch * reps * anchor_planes(b)), o_anc4 = sc.add(sizeof(float) * man * batch * reps);
-    sc.group();
-    const size_t o_exch = sc.add(sizeof(float2) * seg->N * batch * (p + 1));
-    cudaError_t e = sc.alloc(st);
+    size_t o_all, o_units, o_mu, o_anc, o_anc4, o_exch, o_sums;
+    int reps;
+    cudaError_t e;
+    for (;;) {
+        reps = pf && !stepwise ? p + 1 : 1;
+        sc = Scratch();
+        o_all = sc.add(sizeof(UnitInfo) * n_t), o_units = sc.add(sizeof(UnitInfo) * (size_t)(p + 1) * n);
+        o_mu = sc.add(sizeof(UnitInfo) * (size_t)(p + 1) * batch);
+        sc.group();
+        o_anc = sc.add(sizeof(float4) * man * batch * reps * anchor_planes(b)), o_anc4 = sc.add(sizeof(float) * man * batch * reps);
+        sc.group();
+        o_exch = sc.add(sizeof(float2) * seg->N * (stepwise ? 1 : batch * (p + 1)));
+        o_sums = sc.add(stepwise ? 3 * sizeof(float) * seg->N : 0);
+        e = sc.alloc(st);
+        if (e != cudaErrorMemoryAllocation || t_fault_injected || (batch == 1 && (stepwise || rows))) break;
+        sc.free(st);
+        stepwise = batch == 1;
+        batch = std::max<int64_t>(1, batch / 2);
+    }
     UnitInfo *all = sc.at<UnitInfo>(o_all), *units = sc.at<UnitInfo>(o_units), *mu = sc.at<UnitInfo>(o_mu);
     float4 *anc = sc.at<float4>(o_anc);
     float *anc4 = sc.at<float>(o_anc4);
@@ -1461,6 +1477,14 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
             e = launch_anchors(sd, b->d_tmpl, full, (int)u0, nb, lgD, man, anc, anc4, b->params.phase_mode, st, reps);
             ++launches;
         }
+        for (int l = p; stepwise && l >= 0 && e == cudaSuccess; --l) {
+            e = launch_pass1(sd, units + (size_t)l * n + u0, 0, 1, lgD, man, anc, anc4, exch, b->params.phase_mode,
+                             b->d_tmpl, p1_form(b), b->chi_status, b->spin_limit, st, kBandNarrow, 1);
+            if (e == cudaSuccess)
+                e = launch_chisq_step(sd, exch, full, (int)u0, l, p, sc.at<float2>(o_sums), chisq, st);
+            launches += 2;
+        }
+        if (stepwise) continue;
         if (e == cudaSuccess && nb < n) {
             e = cudaMemcpy2DAsync(mu, sizeof(UnitInfo) * nb, units + u0, sizeof(UnitInfo) * n, sizeof(UnitInfo) * nb,
                                   p + 1, cudaMemcpyDeviceToDevice, st);

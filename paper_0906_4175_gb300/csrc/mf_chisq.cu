@@ -236,6 +236,55 @@ __global__ void __launch_bounds__(C *(L / 32), (C * (L / 32) >= 256) ? 2 : 1) k_
     }
 }
 
+// One band of one template (little memory: no p + 1 exchanges), l = p .. 0 in turn:
+// the sums stay in sums[3][N] between the launches, the group's own, G3 (+ G2) or
+// the upper of two, and G1.  The order of the sum is k_chisq_tiles'.
+template <int L, int C>
+__global__ void __launch_bounds__(C *(L / 32), (C * (L / 32) >= 256) ? 2 : 1)
+    k_chisq_step(ChiTilesParams q, int l, float2 *sums) {
+    extern __shared__ float2 chi_smem[];
+    constexpr int T = L / 32, NT = C * T;
+    using Sync = std::conditional_t<(L <= 1024), ChiWarpSync, CtaSync>;
+    float2 *tw = chi_smem + pass_data_bytes<L, C>() / sizeof(float2);
+    int tile = blockIdx.x;
+    fill_twiddles<L>(tw);
+    chain_wait(tile);
+    const int groups = chi_ordered<L>() ? chi_groups(q.p) : 1;
+    const int b1 = groups == 4 ? chi_start(1, 4, q.p) : -1, b3 = groups == 4 ? chi_start(3, 4, q.p) : -1;
+    const int b2 = groups > 1 ? chi_start(1, 2, q.p) : -1;
+    const float rs = q.full[q.unit0].rho_scale, rs2 = rs * rs;
+    const int64_t half_n = (int64_t)1 << (q.log2N - 1);   // float2 of one of the sums
+    float2 *own = sums + (int64_t)tile * (C * L / 2) + threadIdx.x, *hi = own + half_n, *lo = hi + half_n;
+    ChiTileAcc snk;
+    snk.l = l;
+    snk.p = q.p;
+    snk.pf = (float)q.p;
+    snk.start();
+    if (l < q.p && l + 1 != b1 && l + 1 != b2 && l + 1 != b3) snk.template add<NT>(own);   // 0 + x
+    const typename RowSrc<L, C>::Params rp{q.exch, q.log2N1, q.log2N};
+    __syncthreads();   // twiddles
+    ChiTileSrc<L, C, Sync> src{RowSrc<L, C>(rp, tile, 0, 0, nullptr), false};
+    cta_fft<L, C, false, +1, ChiTileSrc<L, C, Sync>, ChiTileAcc, Sync>(chi_smem, tw, src, snk);
+    if (l > 0) {
+        if (groups == 4 && l == b2) snk.template add<NT>(hi);
+        snk.template put<NT>(l == b1 ? lo : (l == b2 || l == b3 ? hi : own));
+        return;
+    }
+    if (groups == 4) snk.template add<NT>(lo);
+    if (groups > 1) snk.template add<NT>(hi);
+    const int seq = threadIdx.x / T, t = threadIdx.x % T;
+    auto row = [&](int s) { return reinterpret_cast<float *>(chi_smem + s * SeqStride<L, C>::value); };
+    __syncthreads();   // the last stage has read the sequences
+#pragma unroll
+    for (int r = 0; r < 32; ++r) row(seq)[t + r * T] = rs2 * snk.acc[r];
+    __syncthreads();
+    float *out = q.chisq + ((int64_t)q.unit0 << q.log2N) + tile * C;
+    for (int idx = threadIdx.x; idx < C * L; idx += NT) {
+        const int s = idx % C, j1 = idx / C;
+        __stcs(&out[s + ((int64_t)j1 << q.log2N2)], row(s)[j1]);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // chi^2 rows kernel (N1 = 1024, N = 2^19 and 2^20).  Pass 1 has written the
 // exchange of every sub-band l = 0..p of a batch of nb templates, sub-band l
@@ -423,6 +472,8 @@ struct ChiTilesOp {
     const ChiTilesParams *q;   // NULL: set the kernel attributes only
     int n_sm;
     cudaStream_t st;
+    int step = -1;             // >= 0: this band alone, with sums
+    float2 *sums = nullptr;
     template <int N2, int N1, int S>
     cudaError_t tiles() {
         constexpr int C = seqs_per_cta<N1>(N2);
@@ -434,6 +485,14 @@ struct ChiTilesOp {
     template <int N2, int N1>
     cudaError_t run() {
         if constexpr (N1 != 1024) {
+            constexpr int C = seqs_per_cta<N1>(N2);
+            constexpr size_t smem = chi_tiles_smem_bytes<N1, C>();
+            if (q && step >= 0)
+                return launch(k_chisq_step<N1, C>, dim3(N2 / C), C * (N1 / 32), smem, st, *q, step, sums);
+            if (!q) {
+                cudaError_t e = cudaFuncSetAttribute(k_chisq_step<N1, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (e != cudaSuccess) return e;
+            }
             if constexpr (chi_ordered<N1>()) {   // a template of 2048-point rows is 256 tiles and more
                 if (!q) {
                     cudaError_t e = tiles<N2, N1, 2>();
@@ -442,7 +501,7 @@ struct ChiTilesOp {
                 } else {
                     // as many CTAs per tile as keep the launch within one wave (two per
                     // SM), with a group each, of two sub-bands or more
-                    const int64_t n = (int64_t)(N2 / seqs_per_cta<N1>(N2)) * q->nb, wave = 2 * (int64_t)n_sm;
+                    const int64_t n = (int64_t)(N2 / C) * q->nb, wave = 2 * (int64_t)n_sm;
                     if (4 * n <= wave && chi_groups(q->p) == 4) return tiles<N2, N1, 4>();
                     if (2 * n <= wave && chi_groups(q->p) >= 2) return tiles<N2, N1, 2>();
                 }
@@ -469,6 +528,13 @@ cudaError_t launch_chisq_tiles(const SegDev &seg, float2 *exch, const UnitInfo *
 }
 
 bool chisq_rows_applies(int log2N) { return log2N - log2_n2(log2N) == 10; }
+
+cudaError_t launch_chisq_step(const SegDev &seg, float2 *exch, const UnitInfo *full, int unit, int l, int p, float2 *sums,
+                              float *chisq, cudaStream_t st) {
+    ChiTilesParams q{exch, full, chisq, unit, 1, p, seg.log2N, seg.log2N1, seg.log2N2};
+    ChiTilesOp op{&q, 0, st, l, sums};
+    return dispatch_split(seg.log2N, op);
+}
 
 cudaError_t launch_chisq_rows(const SegDev &seg, const float2 *exch, const UnitInfo *full, int unit0, int nb, int p,
                               float *chisq, int *status, long long spin_limit, int stall, int n_sm, cudaStream_t st) {

@@ -361,6 +361,10 @@ cudaError_t launch_chisq_units(const SegDev &seg, const UnitInfo *all, int n_t, 
 // than 1024); band l of entry b at exch + (l nb + b) N
 cudaError_t launch_chisq_tiles(const SegDev &seg, float2 *exch, const UnitInfo *full, int unit0, int nb, int p,
                                float *chisq, int n_sm, cudaStream_t st);
+// the same for one template, band by band (l = p .. 0, exch of one band), with
+// the same bits; sums: 12 N bytes kept between the launches
+cudaError_t launch_chisq_step(const SegDev &seg, float2 *exch, const UnitInfo *full, int unit, int l, int p, float2 *sums,
+                              float *chisq, cudaStream_t st);
 
 // trigger clustering scratch (arrays sized for the trigger capacity; ctl
 // zeroed before the launch, scan: two look-back words per tile)

@@ -37,3 +37,29 @@ def test_same_bits_in_every_list(mf, lg, n, p):
     for k in sorted({1, max(1, n // 5), n // 2}):
         some = mf.chisq_series(bank, seg, list(range(n - k, n)), p=p)[0].cpu().numpy().view(np.uint32)
         assert np.array_equal(some, many[n - k:]), k
+
+
+# the allocation limits leave room for some of the templates' p + 1 exchanges, for
+# one template's, and for one band of one template's (1024-point rows need p + 1)
+@pytest.mark.parametrize("lg,p", [(10, 1), (12, 16), (13, 2), (14, 3), (15, 7), (16, 6), (17, 16), (18, 5), (19, 4), (21, 8),
+                                  (22, 3)])
+def test_little_memory(mf, lg, p):
+    import torch
+    n = 3 if lg > 18 else 7
+    bank, seg = _case(mf, lg, n)
+    want, edges = (x.cpu().numpy() for x in mf.chisq_series(bank, seg, list(range(n)), p=p))
+    L = mf._native.lib()
+    one = 8 * seg.N * (p + 1)
+    for limit in (3 * one, one + (1 << 16), 20 * seg.N + (1 << 16)):
+        L.mf_debug_alloc_limit(limit)
+        try:
+            if lg in (19, 20) and limit < one:
+                with pytest.raises(mf.MFError) as e:
+                    mf.chisq_series(bank, seg, list(range(n)), p=p)
+                assert e.value.code == mf._native.MF_ENOMEM
+                continue
+            got, ge = (x.cpu().numpy() for x in mf.chisq_series(bank, seg, list(range(n)), p=p))
+        finally:
+            L.mf_debug_alloc_limit(-1)
+        assert bank.check() == 0
+        assert np.array_equal(ge, edges) and np.array_equal(got.view(np.uint32), want.view(np.uint32)), limit
