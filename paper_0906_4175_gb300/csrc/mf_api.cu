@@ -373,7 +373,7 @@ struct mf_bank_s {
     unsigned char alt_split[23] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 1};
     bool captured = false;        // a graph may hold the workspace's pointers
     bool group_no_room = false;   // the larger workspace of grouped segments could not be allocated
-    int *chi_status = nullptr;        // status of the last mf_chisq_series (bit 2: a bounded wait ran out)
+    FilterCtl *chi_ctl = nullptr;     // its status is that of the last mf_chisq_series (bit 2: a bounded wait ran out)
 };
 
 // Records an event before a launch when profiling; returns the record index or -1.
@@ -593,7 +593,7 @@ extern "C" int mf_bank_destroy(mf_bank b) {
     b->ws.release();
     cudaFree(b->d_tmpl);
     cudaFree(b->d_order);
-    cudaFree(b->chi_status);
+    cudaFree(b->chi_ctl);
     if (b->ev_p1) cudaEventDestroy(b->ev_p1);
     if (b->ev_anc) cudaEventDestroy(b->ev_anc);
     if (b->side) cudaStreamDestroy(b->side);
@@ -1432,9 +1432,13 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
     int64_t batch = std::max<int64_t>(1, std::min<int64_t>({n, budget / (8 * seg->N * (p + 1)), 65535 / (p + 1)}));
     bool stepwise = false;
     const bool anchors = b->params.phase_mode != MF_PHASE_FP32;
-    // the staged pass 1 and the rows kernel report waits that run out here
-    if (!b->chi_status) MF_CUDA(dev_malloc(&b->chi_status, sizeof(int)));
-    MF_CUDA(cudaMemsetAsync(b->chi_status, 0, sizeof(int), st));
+    // the staged pass 1 and the rows kernel report waits that run out here; the
+    // call's first kernel zeroes it (a memset before it is 4 us of a short call)
+    if (!b->chi_ctl) {
+        MF_CUDA(dev_malloc(&b->chi_ctl, sizeof(FilterCtl)));
+        MF_CUDA(cudaMemsetAsync(b->chi_ctl, 0, sizeof(FilterCtl), st));
+    }
+    int *const status = &b->chi_ctl->status;
     // One pass-1 launch per batch covers all p + 1 bands: unit slot l nb + s is
     // band l of template u0 + s (a band-major copy of the batch's units).  The
     // persistent pass 1 reads the copy of its template's anchors that the
@@ -1466,7 +1470,7 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
     float2 *exch = sc.at<float2>(o_exch);
     int launches = 0;
     ChainScope chain(true);
-    if (e == cudaSuccess) e = launch_units(sd, b->d_tmpl, n_t, b->params.f_low, 0.f, lgD, nullptr, all, nullptr, st);
+    if (e == cudaSuccess) e = launch_units(sd, b->d_tmpl, n_t, b->params.f_low, 0.f, lgD, nullptr, all, b->chi_ctl, st);
     if (e == cudaSuccess) e = launch_chisq_units(sd, all, n_t, tmpl, (int)n, p, units, edges, st);
     launches += 2;
     const UnitInfo *full = units + (size_t)p * n;
@@ -1479,7 +1483,7 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
         }
         for (int l = p; stepwise && l >= 0 && e == cudaSuccess; --l) {
             e = launch_pass1(sd, units + (size_t)l * n + u0, 0, 1, lgD, man, anc, anc4, exch, b->params.phase_mode,
-                             b->d_tmpl, p1_form(b), b->chi_status, b->spin_limit, st, kBandNarrow, 1);
+                             b->d_tmpl, p1_form(b), status, b->spin_limit, st, kBandNarrow, 1);
             if (e == cudaSuccess)
                 e = launch_chisq_step(sd, exch, full, (int)u0, l, p, sc.at<float2>(o_sums), chisq, st);
             launches += 2;
@@ -1492,9 +1496,9 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
         }
         if (e == cudaSuccess)
             e = launch_pass1(sd, bu, 0, (p + 1) * nb, lgD, man, anc, anc4, exch, b->params.phase_mode, b->d_tmpl,
-                             p1_form(b), b->chi_status, b->spin_limit, st, kBandNarrow, nb);
+                             p1_form(b), status, b->spin_limit, st, kBandNarrow, nb);
         if (e == cudaSuccess)
-            e = rows ? launch_chisq_rows(sd, exch, full, (int)u0, nb, p, chisq, b->chi_status, b->spin_limit,
+            e = rows ? launch_chisq_rows(sd, exch, full, (int)u0, nb, p, chisq, status, b->spin_limit,
                                          (int)b->stall_unit, sm_count(), st)
                      : launch_chisq_tiles(sd, exch, full, (int)u0, nb, p, chisq, sm_count(), st);
         launches += 2;
@@ -1665,9 +1669,9 @@ extern "C" int mf_bank_profile_read(mf_bank b, double *ms, double *bytes, int64_
 extern "C" int mf_bank_check(mf_bank b, void *cuda_stream) {
     if (!b) return set_err(MF_EINVAL, "NULL bank");
     MF_CUDA(cudaStreamSynchronize((cudaStream_t)cuda_stream));
-    if (b->chi_status) {
+    if (b->chi_ctl) {
         int cs = 0;
-        MF_CUDA(cudaMemcpy(&cs, b->chi_status, sizeof(int), cudaMemcpyDeviceToHost));
+        MF_CUDA(cudaMemcpy(&cs, &b->chi_ctl->status, sizeof(int), cudaMemcpyDeviceToHost));
         if (cs & 2) return set_err(MF_ETIMEOUT, "a bounded device wait expired in the last mf_chisq_series");
     }
     if (!b->ws.status) return MF_OK;
