@@ -1694,7 +1694,17 @@ extern "C" int mf_autotune(mf_bank b, const mf_segment *segs, int n_seg, float t
     if (repeats < 1) repeats = 2;
     struct Cand { int sched; int64_t exch; double split; int p1, p2; };
     std::vector<Cand> cands;
-    if (b->params.fft_mode == MF_FFT_FP32)   // the tensor-core stage runs in the per-batch rows kernel only
+    // the persistent scheduler, where it takes some segment of the call (as below for
+    // the fused one): not the phase forms without its source, nor the tensor-core
+    // stage, which runs in the per-batch rows kernel only
+    bool any_persistent = false;
+    for (int s = 0; s < n_seg; ++s) {
+        const int saved = b->sched;
+        b->sched = 0;
+        any_persistent = any_persistent || use_persistent(b, segs[s]);
+        b->sched = saved;
+    }
+    if (any_persistent)
         for (double sp : {0.55, 0.60, 0.65}) cands.push_back({0, 0, sp, 0, 0});
     int64_t maxN = 0;
     for (int s = 0; s < n_seg; ++s) maxN = std::max(maxN, segs[s]->N);
