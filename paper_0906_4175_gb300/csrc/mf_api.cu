@@ -422,7 +422,7 @@ struct mf_segment_s {
     double *psd = nullptr;
     double psd_f0 = 0.0, psd_S0 = 0.0;
     float *fac = nullptr;          // a_k = alpha f^(-7/6) dt / S_k: W_k = a_k conj(X_k) for new samples
-    float2 *r_exch = nullptr, *r_X = nullptr;
+    float2 *r_exch = nullptr;
     float *r_s = nullptr;
     int cond = MF_COND_FP64;       // precision of the forward DFT in mf_segment_refresh
     // CUtensorMaps over W for pass 1 (boxes of C and C/2 columns), for the
@@ -431,9 +431,9 @@ struct mf_segment_s {
     bool has_tmap[2] = {false, false};
     void release() {
         cudaFree(W); cudaFree(P); cudaFree(consts); cudaFree(psd); cudaFree(fac);
-        cudaFree(r_exch); cudaFree(r_X); cudaFree(r_s);
+        cudaFree(r_exch); cudaFree(r_s);
         W = nullptr; P = nullptr; consts = nullptr; psd = nullptr; fac = nullptr;
-        r_exch = nullptr; r_X = nullptr; r_s = nullptr;
+        r_exch = nullptr; r_s = nullptr;
     }
 };
 
@@ -639,7 +639,7 @@ extern "C" int mf_segment_upload(const float *s, int64_t N, double fs, const dou
     const size_t o_q = sc.add(sizeof(double) * half), o_btmp = sc.add(sizeof(double) * nbt);
     const size_t o_s = s_on_device ? (size_t)0 : sc.add(sizeof(float) * N);
     const double *psd_dev = nullptr;
-    cudaError_t e = dev_malloc(&g->W, sizeof(float2) * half);
+    cudaError_t e = dev_malloc(&g->W, sizeof(float2) * (half + 1));   // a refresh in FP32 forms X here
     if (e == cudaSuccess) {   // pass 1's TMA views of W, both splits
         g->has_tmap[0] = make_w_tensor_maps(g->W, g->log2N, log2_n2(g->log2N), g->w_tmap[0]);
         g->has_tmap[1] = alt_log2n2(g->log2N) > 0 && make_w_tensor_maps(g->W, g->log2N, alt_log2n2(g->log2N), g->w_tmap[1]);
@@ -687,17 +687,10 @@ extern "C" int mf_segment_refresh(mf_segment g, const float *s, int s_on_device,
     if (cur != g->device) return set_err(MF_EINVAL, "segment lives on device %d, current is %d", g->device, cur);
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const bool capturing = stream_capturing(st);
-    const int64_t N = g->N, half = N / 2;
+    const int64_t N = g->N;
     if (!g->r_exch) {
         if (capturing) return set_err(MF_EINVAL, "the first mf_segment_refresh of a segment must precede stream capture");
-        cudaError_t e = dev_malloc(&g->r_exch, sizeof(float2) * N);
-        if (e == cudaSuccess) e = dev_malloc(&g->r_X, sizeof(float2) * (half + 1));
-        if (e != cudaSuccess) {
-            cudaFree(g->r_exch); cudaFree(g->r_X);
-            g->r_exch = nullptr; g->r_X = nullptr;
-            return set_err(e == cudaErrorMemoryAllocation ? MF_ENOMEM : MF_ECUDA, "segment_refresh: %s",
-                           cudaGetErrorString(e));
-        }
+        MF_CUDA(dev_malloc(&g->r_exch, sizeof(float2) * N));
     }
     const float *s_use = s;
     if (!s_on_device) {
@@ -709,8 +702,8 @@ extern "C" int mf_segment_refresh(mf_segment g, const float *s, int s_on_device,
     ChainScope chain(true);
     // the PSD and with it P, sigma's normalisation and the factors a_k are unchanged
     if (g->cond == MF_COND_FP32) {
-        MF_CUDA(launch_forward_fft(s_use, N, g->r_exch, g->r_X, st));
-        MF_CUDA(launch_apply_weights(g->r_X, g->fac, N, g->W, st));
+        MF_CUDA(launch_forward_fft(s_use, N, g->r_exch, g->W, st));   // X, N/2 + 1 entries
+        MF_CUDA(launch_apply_weights(g->W, g->fac, N, st));
         count_launches(3);
     } else {
         MF_CUDA(launch_forward_fft64(s_use, N, g->r_exch, g->fac, g->W, st));
@@ -780,7 +773,7 @@ static int choose_log2D(const mf_bank_s *b, const mf_segment_s *g) {
 constexpr int64_t kExchBudget = (int64_t)4 << 30;
 constexpr int64_t kScratchBudget = (int64_t)1 << 30;
 
-// 16-byte planes of an anchor record (and one float, MF_PHASE_ANCHOR)
+// 16-byte planes of an anchor record: one (and a float in anchors4), or three (MF_PHASE_FP64)
 static int anchor_planes(const mf_bank_s *b) { return b->params.phase_mode == MF_PHASE_FP64 ? 3 : 1; }
 
 static int64_t exch_budget(const mf_bank_s *b) { return b->tuned_exch > 0 ? b->tuned_exch : kExchBudget; }
@@ -808,12 +801,13 @@ static bool workspace_holds(const mf_bank_s *b, const WorkspaceNeed &q) {
            w.nblk >= q.nblk && w.n_set >= q.n_set;
 }
 // w (empty): a workspace of that size; all or nothing
-static int make_workspace(Workspace &w, int64_t n, const WorkspaceNeed &q) {
+static int make_workspace(Workspace &w, const mf_bank_s *b, const WorkspaceNeed &q) {
+    const int64_t n = b->n;
     auto get = [&]() -> int {
         MF_CUDA(dev_malloc(&w.units, sizeof(UnitInfo) * n * q.n_set));
         MF_CUDA(dev_malloc(&w.exch, sizeof(float2) * q.exch_elems));
         MF_CUDA(dev_malloc(&w.anchors, sizeof(float4) * q.anc_elems));
-        MF_CUDA(dev_malloc(&w.anchors4, sizeof(float) * q.anc_elems));
+        if (anchor_planes(b) == 1) MF_CUDA(dev_malloc(&w.anchors4, sizeof(float) * q.anc_elems));
         MF_CUDA(dev_malloc(&w.partials, sizeof(float4) * q.nblk * n));
         MF_CUDA(dev_malloc(&w.staged, sizeof(mf_trigger) * q.cap));
         MF_CUDA(dev_malloc(&w.keys, sizeof(uint64_t) * q.cap));
@@ -849,10 +843,10 @@ static int ensure_workspace(mf_bank_s *b, const WorkspaceNeed &need, bool captur
     MF_CUDA(cudaDeviceSynchronize());
     if (!keep) {
         w.release();
-        return make_workspace(w, b->n, q);
+        return make_workspace(w, b, q);
     }
     Workspace grown;
-    const int rc = make_workspace(grown, b->n, q);
+    const int rc = make_workspace(grown, b, q);
     if (rc) return rc;
     w.release();
     w = grown;
@@ -1454,7 +1448,8 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
         o_all = sc.add(sizeof(UnitInfo) * n_t), o_units = sc.add(sizeof(UnitInfo) * (size_t)(p + 1) * n);
         o_mu = sc.add(sizeof(UnitInfo) * (size_t)(p + 1) * batch);
         sc.group();
-        o_anc = sc.add(sizeof(float4) * man * batch * reps * anchor_planes(b)), o_anc4 = sc.add(sizeof(float) * man * batch * reps);
+        o_anc = sc.add(sizeof(float4) * man * batch * reps * anchor_planes(b));
+        o_anc4 = sc.add(anchor_planes(b) == 1 ? sizeof(float) * man * batch * reps : 0);
         sc.group();
         o_exch = sc.add(sizeof(float2) * seg->N * (stepwise ? 1 : batch * (p + 1)));
         o_sums = sc.add(stepwise ? 3 * sizeof(float) * seg->N : 0);

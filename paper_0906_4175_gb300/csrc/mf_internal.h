@@ -201,7 +201,7 @@ cudaError_t launch_prefix_f64(const double *q, int64_t n, double *P, double *blo
 cudaError_t launch_weight_data(const float2 *X, const double *psd, double psd_f0, double psd_S0,
                                int64_t N, double fs, const double *P, SegConsts *consts, float2 *W, float *fac,
                                cudaStream_t st);
-cudaError_t launch_apply_weights(const float2 *X, const float *fac, int64_t N, float2 *W, cudaStream_t st);
+cudaError_t launch_apply_weights(float2 *W, const float *fac, int64_t N, cudaStream_t st);
 int64_t prefix_block_tmp_count(int64_t n);
 
 // synthesis (mf_synth.cu)

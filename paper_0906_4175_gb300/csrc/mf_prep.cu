@@ -341,21 +341,20 @@ cudaError_t launch_weight_data(const float2 *X, const double *psd, double psd_f0
     return cudaGetLastError();
 }
 
-// W_k = a_k conj(X_k) with the segment's kept factors (new samples, same PSD)
-__global__ void k_apply_weights(const float2 *__restrict__ X, const float *__restrict__ fac, int64_t half,
-                                float2 *__restrict__ W) {
+// W_k = a_k conj(X_k) with the segment's kept factors (new samples, same PSD), in place
+__global__ void k_apply_weights(float2 *W, const float *__restrict__ fac, int64_t half) {
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < half; k += (int64_t)gridDim.x * blockDim.x) {
         const float a = fac[k];
-        const float2 x = X[k];
+        const float2 x = W[k];
         W[k] = make_float2(a * x.x, -a * x.y);
     }
 }
 
-cudaError_t launch_apply_weights(const float2 *X, const float *fac, int64_t N, float2 *W, cudaStream_t st) {
+cudaError_t launch_apply_weights(float2 *W, const float *fac, int64_t N, cudaStream_t st) {
     const int64_t half = N / 2;
     int blocks = (int)((half + 255) / 256);
     if (blocks > 4096) blocks = 4096;
-    k_apply_weights<<<blocks, 256, 0, st>>>(X, fac, half, W);
+    k_apply_weights<<<blocks, 256, 0, st>>>(W, fac, half);
     return cudaGetLastError();
 }
 

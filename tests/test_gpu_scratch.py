@@ -182,3 +182,24 @@ for k in range(13):                  # every allocation of the larger workspace
     assert host(alone_allocates_nothing(lambda: run(b, s))) == ref, k
     assert b.check() == 0
 """)
+
+
+@pytest.mark.parametrize("cond", ["fp64", "fp32"])
+def test_refresh_keeps_one_exchange(cond):
+    """The first refresh of a segment of 2^22 samples keeps its exchange of 32 MB
+    and nothing else; FP32 conditioning forms the spectrum in the weights' place."""
+    _child("""
+s = segment(22)
+x = torch.randn(1 << 22, dtype=torch.float32, device="cuda")
+s.set_conditioning("%s")
+torch.cuda.synchronize()
+free = torch.cuda.mem_get_info()[0]
+s.refresh(x)
+torch.cuda.synchronize()
+assert free - torch.cuda.mem_get_info()[0] <= 34 * MB
+b = bank()
+one = [t.cpu() for t in mf.filter_bank(b, [s], 0.1, trig_cap=1 << 10)]
+s.refresh(x)
+two = [t.cpu() for t in mf.filter_bank(b, [s], 0.1, trig_cap=1 << 10)]
+assert torch.equal(one[0].view(torch.int32), two[0].view(torch.int32)) and torch.equal(one[2], two[2])
+""" % cond)
