@@ -114,7 +114,11 @@ __device__ __forceinline__ void release_hook(unsigned *ctr) {
 // ---------------------------------------------------------------------------
 template <int L, int C, bool HALF_ZERO, int LG1>
 struct ColComplexSrc {      // X[k], zero for k >= N/2 when HALF_ZERO; LG1 = log2 N1
-    static constexpr bool kScalarAdd = L == 256 && LG1 == 8;   // 512 transforms of 2^16: 209 us packed, 204 scalar
+    // Columns of 256 points (N = 2^16, 2^17): 2^27 points in 749 and 672 us packed,
+    // 733 and 663 scalar.  Other lengths lose or tie with scalar additions: 2^26
+    // points at 2^15 375 packed, 378 scalar, 2^18 .. 2^21 352, 368, 396 and 470
+    // against 352, 367, 398 and 471, 2^22 564 against 583.
+    static constexpr bool kScalarAdd = L == 256;
     static constexpr bool kHalfZero = HALF_ZERO;
     static constexpr size_t kScratchBytes = 0;
     struct Params { const float2 *X; int log2N1; int64_t batch_stride; };

@@ -90,7 +90,6 @@ struct C2CAttrOp {
 template <int L, int C>
 struct SeqSrc {
     static constexpr bool kHalfZero = false;
-    static constexpr bool kScalarAdd = L == 1024;   // 2^25 points: 1024-point transforms 100.0 us packed, 98.5 scalar; 2048: 113.1, 122
     static constexpr size_t kScratchBytes = 0;
     struct Params { const float2 *x; int64_t n_seq; };
     const Params &p;
