@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kSortThreads, 1)
         *n_out = (int64_t)total;
         if (total > (unsigned long long)cap) atomicOr(status, 1);
     }
-    if (n <= kRankMax) {
+    if (n <= kRankMax && n <= (int64_t)gridDim.x * kSortThreads) {
         if (key_bits <= 32) sort_rank<uint32_t>(keys, (int)n, staged, out, sort_smem);
         else sort_rank<uint64_t>(keys, (int)n, staged, out, sort_smem);
         return;
@@ -311,7 +311,7 @@ cudaError_t launch_sort_triggers(const unsigned long long *counter, int64_t cap,
                                  const mf_trigger *staged, const uint64_t *keys, uint64_t *keys_tmp,
                                  uint32_t *idx_a, uint32_t *idx_b, SortCtl *ctl, uint64_t *tstat, mf_trigger *out,
                                  int64_t *n_out, int *status, int n_sm, int64_t spin_limit, cudaStream_t st) {
-    if (key_bits > 8 * kSortMaxPass || n_sm * kSortThreads < kRankMax) return cudaErrorInvalidValue;
+    if (key_bits > 8 * kSortMaxPass) return cudaErrorInvalidValue;
     return launch(k_sort_triggers, dim3(n_sm), kSortThreads, 0, st, counter, cap, key_bits, staged,
                   const_cast<uint64_t *>(keys), keys_tmp, idx_a, idx_b, ctl, tstat, out, n_out, status, spin_limit);
 }

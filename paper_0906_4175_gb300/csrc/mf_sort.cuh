@@ -241,7 +241,7 @@ __device__ __forceinline__ void sort_rank(const uint64_t *keys, int n, const mf_
     const int per = (n + (int)gridDim.x - 1) / (int)gridDim.x;
     const int k0 = (int)blockIdx.x * per, mine = min(per, n - k0);
     if (mine <= 0) return;
-    const int parts = kSortThreads / per;   // per <= kSortThreads: n <= kRankMax on any GPU of 24 SMs
+    const int parts = kSortThreads / per;   // the caller has n <= CTAs kSortThreads, so per <= kSortThreads
     const int q = (int)threadIdx.x % per, part = (int)threadIdx.x / per;
     const bool act = q < mine && part < parts;
     const K my = act ? (K)keys[k0 + q] : (K)0;
