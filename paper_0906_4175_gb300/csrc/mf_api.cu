@@ -316,7 +316,7 @@ struct Workspace {
     uint64_t *keys = nullptr, *keys_tmp = nullptr;
     uint32_t *idx_a = nullptr, *idx_b = nullptr;
     uint64_t *tstat = nullptr;    // trigger sort: look-back status per (tile, digit)
-    FilterCtl *fctl = nullptr;    // trigger count, status and sort control, zeroed by one memset per call
+    FilterCtl *fctl = nullptr;    // trigger count, status and sort control, zeroed by the call's first kernel
     unsigned long long *counter = nullptr;   // fctl->counter
     int *status = nullptr;                   // fctl->status
     unsigned *ctl = nullptr;      // persistent scheduler: [1] abort, then doneA, done1, done2 per unit
@@ -868,7 +868,7 @@ static int p1_form(const mf_bank_s *b) {
     return b->p1_kind;
 }
 
-// Pass 2 as whole rows per warp (row length 1024 or 2048) unless MFGB_P2ROWS=0.
+// Pass 2 in whole rows (128 .. 4096 points) unless MFGB_P2ROWS=0.
 static bool use_rows(const mf_bank_s *b, const mf_segment_s *g, int log2N1) {
     (void)g;
     if (!pass2_rows_applies(log2N1)) return false;

@@ -75,7 +75,7 @@ __global__ void k_chisq_units(SegDev seg, const UnitInfo *__restrict__ all, int 
 // per lane).  One launch per batch instead of one per sub-band, and no
 // accumulator in memory: 16 templates at N = 2^16, p = 16 took 17 pass-1 and
 // 17 pass-2 launches of 7 us each, every one a fraction of a wave: 330 us a
-// call, 104 us now.
+// call, 105 us now.
 // ---------------------------------------------------------------------------
 struct ChiTilesParams {
     float2 *exch;           // group sums are kept over bands already read
@@ -480,7 +480,7 @@ struct ChiTilesOp {
         constexpr size_t smem = chi_tiles_smem_bytes<N1, C>();
         if (!q)
             return cudaFuncSetAttribute(k_chisq_tiles<N1, C, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        return launch_cluster(k_chisq_tiles<N1, C, S>, dim3(S * (N2 / C), q->nb), C * (N1 / 32), S > 1 ? S : 0, smem, st, *q);
+        return launch_in_clusters(k_chisq_tiles<N1, C, S>, dim3(S * (N2 / C), q->nb), C * (N1 / 32), S > 1 ? S : 0, smem, st, *q);
     }
     template <int N2, int N1>
     cudaError_t run() {

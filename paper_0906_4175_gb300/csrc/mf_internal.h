@@ -260,14 +260,15 @@ cudaError_t launch_pass1_pf(const SegDev &seg, const UnitInfo *units, int unit0,
 // 2^16..2^21) or they cannot be made
 bool make_w_tensor_maps(const float2 *W, int log2N, int log2N2, void *maps_out);
 cudaError_t pass1_pf_kernel_attributes();
-// pass 2 with whole rows per warp and bulk-copy prefetch (row length 1024 only)
+// pass 2 in whole rows with bulk-copy prefetch: several rows a warp (128 .. 512
+// points), one (1024), or two or four warps a row (2048, 4096)
 bool pass2_rows_applies(int log2N1);                 // row length N1 = 2^log2N1
-int pass2_rows_partials(int log2N, int log2N2);        // partials per unit: one per row and warp
+int pass2_rows_partials(int log2N, int log2N2);        // partials per unit: one per row and warp that shares it
 cudaError_t launch_pass2_rows(const SegDev &seg, const UnitInfo *units, int unit0, int n_units, const float2 *exch,
                               float4 *partials, int seg_idx, KeyLayout kl, mf_trigger *staged, uint64_t *keys,
                               unsigned long long *counter, int64_t cap, int *status, long long spin_limit, int n_sm,
                               int fft_mode, int stall_unit, bool peaks_later, cudaStream_t st);
-// peaks_later: 1024-point FP32 rows keep only each row's maximum, and the
+// peaks_later: FP32 rows (128 .. 4096 points) keep only each row's maximum, and the
 // batch's peaks come from launch_peaks_rows (before the exchange is reused)
 bool pass2_rows_peaks_later(int log2N1, int fft_mode);
 cudaError_t launch_peaks_rows(const SegDev &seg, const UnitInfo *units, int unit0, int n_units, int n_all,
@@ -283,7 +284,7 @@ struct SortCtl {
     unsigned ticket[kSortMaxPhase], done[kSortMaxPhase];
     unsigned abort, left;   // a wait ran out; CTAs that are done (clustering)
 };
-// what a filter call zeroes before its first kernel
+// what the first kernel of a filter call (or of a chi^2 series) zeroes
 struct FilterCtl {
     unsigned long long counter;   // triggers found
     int status;                   // bit 0: overflow, bit 1: a bounded wait ran out
@@ -337,7 +338,7 @@ template <int CAP>
 cudaError_t launch_units_anchors(FilterGroupOf<CAP> &p, int n_sm, cudaStream_t st);
 cudaError_t group_kernel_attributes();
 
-constexpr int kSortTile = 4096;   // keys per tile of a sort of more than 8192 keys
+constexpr int kSortTile = 4096;   // keys per tile of the tiled sorts (more than 16384 triggers, 8192 cluster records)
 // one kernel; ctl zeroed.  (mf_sort.cuh)
 cudaError_t launch_sort_triggers(const unsigned long long *counter, int64_t cap, int key_bits,
                                  const mf_trigger *staged, const uint64_t *keys, uint64_t *keys_tmp,

@@ -39,7 +39,7 @@ struct ChainScope {
 
 // in clusters of `cluster` CTAs along x (0: none)
 template <class... P, class... A>
-inline cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, unsigned threads, unsigned cluster, size_t smem,
+inline cudaError_t launch_in_clusters(void (*kernel)(P...), dim3 grid, unsigned threads, unsigned cluster, size_t smem,
                                   cudaStream_t st, A &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -62,7 +62,7 @@ inline cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, unsigned thre
 }
 template <class... P, class... A>
 inline cudaError_t launch(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, A &&...args) {
-    return launch_cluster(kernel, grid, threads, 0, smem, st, std::forward<A>(args)...);
+    return launch_in_clusters(kernel, grid, threads, 0, smem, st, std::forward<A>(args)...);
 }
 
 __device__ __forceinline__ void chain_opaque(int &x) { asm volatile("" : "+r"(x)::"memory"); }
