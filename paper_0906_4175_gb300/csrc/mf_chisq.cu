@@ -150,7 +150,7 @@ __device__ __forceinline__ int chi_start(int g, int of, int p) { return (g * (p 
 // S > 1: a cluster of S CTAs shares a tile, CTA c taking the groups of part c of
 // S; the CTAs add their sums through distributed shared memory, 1 / S of the tile
 // each.  A CTA with several groups keeps the sums of all but its last where it
-// has just read the band that begins the group: each thread over its own 32
+// has just read the band that begins the group: each warp over its own 1024
 // points of the exchange, which nothing reads again.  A sum kept is 64 KB a tile
 // more to move, 1 % of a call (200 templates at 2^16, p = 16: 881 us in one sum,
 // 910 in four; pairs keep one each, 16 templates 103.7 -> 105.5; fours none, 9
@@ -185,7 +185,9 @@ __global__ void __launch_bounds__(C *(L / 32), (C * (L / 32) >= 256) ? 2 : 1) k_
     snk.pf = (float)q.p;
     snk.start();
     const int seq = threadIdx.x / T, t = threadIdx.x % T;
-    auto kept = [&](int l) { return q.exch + ((int64_t)(l * q.nb + b) << q.log2N) + (int64_t)(tile * C + seq) * L + t; };
+    auto kept = [&](int l) {   // over the 1024 points of the warp's rows, 256 bytes at a time
+        return q.exch + ((int64_t)(l * q.nb + b) << q.log2N) + tile * C * L + ((int)threadIdx.x & ~31) * 32 + (threadIdx.x & 31);
+    };
     const typename RowSrc<L, C>::Params rp{q.exch, q.log2N1, q.log2N};
     __syncthreads();   // twiddles
 #pragma unroll 1
@@ -195,17 +197,17 @@ __global__ void __launch_bounds__(C *(L / 32), (C * (L / 32) >= 256) ? 2 : 1) k_
         cta_fft<L, C, false, +1, ChiTileSrc<L, C, Sync>, ChiTileAcc, Sync>(chi_smem, tw, src, snk);
         if (chi_ordered<L>() && S < 4 && l > l0 && (l == b1 || l == b2 || l == b3)) {
             if (S == 1 && groups == 4 && l == b2) {   // G3 + G2, in the place of G3
-                snk.template add<T>(kept(b3));
-                snk.template put<T>(kept(b3));
+                snk.template add<32>(kept(b3));
+                snk.template put<32>(kept(b3));
             } else {
-                snk.template put<T>(kept(l));
+                snk.template put<32>(kept(l));
             }
             snk.start();
         }
     }
     if (chi_ordered<L>() && S < 4) {
-        if (groups == 4) snk.template add<T>(kept(c > 0 ? b3 : b1));
-        if (S == 1 && groups > 1) snk.template add<T>(kept(groups == 4 ? b3 : b2));
+        if (groups == 4) snk.template add<32>(kept(c > 0 ? b3 : b1));
+        if (S == 1 && groups > 1) snk.template add<32>(kept(groups == 4 ? b3 : b2));
     }
     auto row = [&](int s) { return reinterpret_cast<float *>(chi_smem + s * SeqStride<L, C>::value); };
     __syncthreads();   // the last stage has read the sequences
