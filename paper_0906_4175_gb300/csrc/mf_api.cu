@@ -373,7 +373,8 @@ struct mf_bank_s {
     unsigned char alt_split[23] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 1};
     bool captured = false;        // a graph may hold the workspace's pointers
     bool group_no_room = false;   // the larger workspace of grouped segments could not be allocated
-    FilterCtl *chi_ctl = nullptr;     // its status is that of the last mf_chisq_series (bit 2: a bounded wait ran out)
+    int *chi_status = nullptr;    // of the last mf_chisq_series (bit 2: a bounded wait ran out), behind the templates
+    bool chi_ran = false;
 };
 
 // Records an event before a launch when profiling; returns the record index or -1.
@@ -517,11 +518,13 @@ static int bank_create_range(const double *m1, const double *m2, int64_t n, cons
                      [&](int x, int y) { return b->fisco[(size_t)x] > b->fisco[(size_t)y]; });
     for (int64_t i = 0; i < n; ++i) b->pos[(size_t)b->order[(size_t)i]] = (int)i;
     cudaGetDevice(&b->device);
+    rec.push_back(0.0);   // chi_status
     cudaError_t e = dev_malloc(&b->d_tmpl, sizeof(double) * rec.size());
     if (e == cudaSuccess) e = cudaMemcpy(b->d_tmpl, rec.data(), sizeof(double) * rec.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = dev_malloc(&b->d_order, sizeof(int) * (size_t)n);
     if (e == cudaSuccess)
         e = cudaMemcpy(b->d_order, b->order.data(), sizeof(int) * (size_t)n, cudaMemcpyHostToDevice);
+    b->chi_status = reinterpret_cast<int *>(b->d_tmpl + n * kTmplStride);
     if (e != cudaSuccess) {
         cudaFree(b->d_tmpl);
         cudaFree(b->d_order);
@@ -593,7 +596,6 @@ extern "C" int mf_bank_destroy(mf_bank b) {
     b->ws.release();
     cudaFree(b->d_tmpl);
     cudaFree(b->d_order);
-    cudaFree(b->chi_ctl);
     if (b->ev_p1) cudaEventDestroy(b->ev_p1);
     if (b->ev_anc) cudaEventDestroy(b->ev_anc);
     if (b->side) cudaStreamDestroy(b->side);
@@ -1428,11 +1430,8 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
     const bool anchors = b->params.phase_mode != MF_PHASE_FP32;
     // the staged pass 1 and the rows kernel report waits that run out here; the
     // call's first kernel zeroes it (a memset before it is 4 us of a short call)
-    if (!b->chi_ctl) {
-        MF_CUDA(dev_malloc(&b->chi_ctl, sizeof(FilterCtl)));
-        MF_CUDA(cudaMemsetAsync(b->chi_ctl, 0, sizeof(FilterCtl), st));
-    }
-    int *const status = &b->chi_ctl->status;
+    int *const status = b->chi_status;
+    b->chi_ran = true;
     // One pass-1 launch per batch covers all p + 1 bands: unit slot l nb + s is
     // band l of template u0 + s (a band-major copy of the batch's units).  The
     // persistent pass 1 reads the copy of its template's anchors that the
@@ -1465,7 +1464,7 @@ extern "C" int mf_chisq_series(mf_bank b, mf_segment seg, const int32_t *tmpl, i
     float2 *exch = sc.at<float2>(o_exch);
     int launches = 0;
     ChainScope chain(true);
-    if (e == cudaSuccess) e = launch_units(sd, b->d_tmpl, n_t, b->params.f_low, 0.f, lgD, nullptr, all, b->chi_ctl, st);
+    if (e == cudaSuccess) e = launch_units(sd, b->d_tmpl, n_t, b->params.f_low, 0.f, lgD, nullptr, all, nullptr, st, status);
     if (e == cudaSuccess) e = launch_chisq_units(sd, all, n_t, tmpl, (int)n, p, units, edges, st);
     launches += 2;
     const UnitInfo *full = units + (size_t)p * n;
@@ -1664,9 +1663,9 @@ extern "C" int mf_bank_profile_read(mf_bank b, double *ms, double *bytes, int64_
 extern "C" int mf_bank_check(mf_bank b, void *cuda_stream) {
     if (!b) return set_err(MF_EINVAL, "NULL bank");
     MF_CUDA(cudaStreamSynchronize((cudaStream_t)cuda_stream));
-    if (b->chi_ctl) {
+    if (b->chi_ran) {
         int cs = 0;
-        MF_CUDA(cudaMemcpy(&cs, &b->chi_ctl->status, sizeof(int), cudaMemcpyDeviceToHost));
+        MF_CUDA(cudaMemcpy(&cs, b->chi_status, sizeof(int), cudaMemcpyDeviceToHost));
         if (cs & 2) return set_err(MF_ETIMEOUT, "a bounded device wait expired in the last mf_chisq_series");
     }
     if (!b->ws.status) return MF_OK;

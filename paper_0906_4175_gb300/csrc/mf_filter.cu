@@ -24,10 +24,12 @@ namespace mf {
 // ---------------------------------------------------------------------------
 // Unit i of a segment is template order[i] (bank order when order is NULL).
 __global__ void k_units(SegDev seg, const double *__restrict__ tmpl, int n_t, double f_low, float thr,
-                        int log2D, const int *__restrict__ order, UnitInfo *__restrict__ units, FilterCtl *clear) {
+                        int log2D, const int *__restrict__ order, UnitInfo *__restrict__ units, FilterCtl *clear,
+                        int *zero) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     chain_wait(i);
     if (clear && blockIdx.x == 0) clear_ctl(clear);
+    if (zero && i == 0) *zero = 0;
     if (i >= n_t) return;
     const int t = order ? order[i] : i;
     units[i] = unit_info(seg, tmpl + (int64_t)t * kTmplStride, t, f_low, thr, log2D);
@@ -98,8 +100,9 @@ __global__ void k_phase64(SegDev seg, const double *__restrict__ tmpl, int t, do
 MF_DEBUG_READER(dbg_read_filter)
 
 cudaError_t launch_units(const SegDev &seg, const double *tmpl, int n_t, double f_low, float thr, int log2D,
-                         const int *order, UnitInfo *units, FilterCtl *clear, cudaStream_t st) {
-    return launch(k_units, dim3((n_t + 255) / 256), 256, 0, st, seg, tmpl, n_t, f_low, thr, log2D, order, units, clear);
+                         const int *order, UnitInfo *units, FilterCtl *clear, cudaStream_t st, int *zero) {
+    return launch(k_units, dim3((n_t + 255) / 256), 256, 0, st, seg, tmpl, n_t, f_low, thr, log2D, order, units, clear,
+                  zero);
 }
 
 cudaError_t launch_anchors(const SegDev &seg, const double *tmpl, const UnitInfo *units, int unit0, int n_units,

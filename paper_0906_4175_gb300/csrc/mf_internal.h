@@ -213,10 +213,11 @@ cudaError_t launch_inverse_real_fft(const float2 *Y, int64_t N, double scale, fl
 
 // filter (mf_filter.cu)
 // units[i] <- template order[i] (order NULL: template i); clear (may be NULL):
-// control words to zero
+// control words to zero, zero (may be NULL): one more word
 struct FilterCtl;
 cudaError_t launch_units(const SegDev &seg, const double *tmpl, int n_t, double f_low, float thr,
-                         int log2D, const int *order, UnitInfo *units, FilterCtl *clear, cudaStream_t st);
+                         int log2D, const int *order, UnitInfo *units, FilterCtl *clear, cudaStream_t st,
+                         int *zero = nullptr);
 cudaError_t launch_anchors(const SegDev &seg, const double *tmpl, const UnitInfo *units, int unit0,
                            int n_units, int log2D, int max_anc, float4 *anchors, float *anchors4, int phase_mode,
                            cudaStream_t st, int reps = 1);
@@ -284,7 +285,7 @@ struct SortCtl {
     unsigned ticket[kSortMaxPhase], done[kSortMaxPhase];
     unsigned abort, left;   // a wait ran out; CTAs that are done (clustering)
 };
-// what the first kernel of a filter call (or of a chi^2 series) zeroes
+// what the first kernel of a filter call zeroes
 struct FilterCtl {
     unsigned long long counter;   // triggers found
     int status;                   // bit 0: overflow, bit 1: a bounded wait ran out
