@@ -242,8 +242,9 @@ struct TemplateSrcNarrow : TemplateSrc<L, C, LG1> {
 // bounds what is left out and the size of the FP32 part: the sum, in 2^-32
 // turns, is off by 2^-33 (the low word, rounded) + 2^-33 (the FP32 part in those
 // units) + its own rounding, 1e-10, + 5e-11 left out: 4e-10 turns at most.
-// u comes from two Newton steps: one leaves 4e-14 of u, up to 4e-10 turns of a
-// light template at 10 Hz.  What counts is the phase the sincos gets.  psi in
+// u comes from a step of third order, u (1 + e/3 + 2 e^2/9) with e = 1 - f u^3,
+// as many operations as a Newton step, which leaves 4e-14 of u, up to 4e-10 turns
+// of a light template at 10 Hz.  What counts is the phase the sincos gets.  psi in
 // FP64 at every bin, rounded to FP32 in [-1/2, 1/2], is off by up to 1.5e-8
 // turns; half turns are taken off first here (they change signs only), so the
 // rounding is 2^-27 at most and the whole 7.9e-9.  Over 1-34 solar masses, 10 to
@@ -274,8 +275,8 @@ __device__ __forceinline__ Anchor64 anchor_record64(double c1, double c2, double
     const int64_t ka = (g << log2D) + ((1 << log2D) >> 1);
     const double f = (double)ka * df;
     double uu = (double)rcbrtf((float)f);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) uu = uu * (4.0 - f * uu * uu * uu) * (1.0 / 3.0);
+    const double e = fma(-f, uu * uu * uu, 1.0);
+    uu = fma(uu, e * fma(e, 2.0 / 9.0, 1.0 / 3.0), uu);
     const double u2 = uu * uu;
     const double psi = -0.125 + uu * (c1 + uu * (c2 + uu * (c3 + u2 * c5)));
     const double S1 = uu * (c1 + uu * (2.0 * c2 + uu * (3.0 * c3 + u2 * (5.0 * c5))));
