@@ -504,6 +504,8 @@ int mf_bank_debug_stall(mf_bank bank, int64_t unit, int64_t spin_limit);
  * device were out of memory: that call returns MF_ENOMEM, frees what it had
  * allocated, leaves its handles as they were before the call (a bank's
  * workspace is released and regrown by the next call) and the hook disarms.
+ * (The larger workspace of short segments that share launches is the exception:
+ * without it the call goes on, one segment after the other.)
  * countdown < 0 disarms it.  Never fails. */
 int mf_debug_fail_alloc(int64_t countdown);
 
