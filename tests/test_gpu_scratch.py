@@ -189,9 +189,11 @@ def test_refresh_keeps_one_exchange(cond):
     """The first refresh of a segment of 2^22 samples keeps its exchange of 32 MB
     and nothing else; FP32 conditioning forms the spectrum in the weights' place."""
     _child("""
-s = segment(22)
+s, other = segment(22), segment(22, seed=2)
 x = torch.randn(1 << 22, dtype=torch.float32, device="cuda")
-s.set_conditioning("%s")
+for one in (other, s):
+    one.set_conditioning("%s")
+other.refresh(x)                    # the kernels are loaded
 torch.cuda.synchronize()
 free = torch.cuda.mem_get_info()[0]
 s.refresh(x)
