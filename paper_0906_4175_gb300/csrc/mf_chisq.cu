@@ -153,8 +153,8 @@ __device__ __forceinline__ int chi_start(int g, int of, int p) { return (g * (p 
 // has just read the band that begins the group: each warp over its own 1024
 // points of the exchange, which nothing reads again.  A sum kept is 64 KB a tile
 // more to move, 1 % of a call (200 templates at 2^16, p = 16: 881 us in one sum,
-// 910 in four; pairs keep one each, 16 templates 103.7 -> 105.5; fours none, 9
-// templates 89 -> 87).  Kept in 32 KB of shared memory the L1 that is left cannot
+// 902 in four; pairs keep one each, 16 templates 103.7 -> 105.2; fours none, 9
+// templates 89 -> 86).  Kept in 32 KB of shared memory the L1 that is left cannot
 // hold the loads in flight (72 us for the 50 below), 32 more registers a thread
 // would spill, and one sum in order over four CTAs, the lower ones adding their
 // bands late, was 94 -> 105 us for 30 templates at 2^14.
